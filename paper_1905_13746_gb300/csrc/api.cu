@@ -131,6 +131,42 @@ static nb_status alloc_model(nb_model* m) {
   return NB_OK;
 }
 
+// A fit right after a synchronisation pays the driver for mapping pool memory
+// again when its scratch was returned to the pool before it (some 100 us and
+// more); a model that is re-fitted keeps one workspace instead.  A workspace
+// baked into a captured graph could be outgrown and freed before a replay, so
+// captures take memory that the graph owns.
+nb_status FitScratch::take(size_t bytes, void** p) {
+  *p = nullptr;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  NB_TRY_CUDA(cudaStreamIsCapturing(st_, &cs), "cudaStreamIsCapturing");
+  if (m_->refit && cs == cudaStreamCaptureStatusNone && bytes <= kKeepWork) {
+    if (m_->work_bytes < bytes) {
+      if (m_->work) {
+        void* old = m_->work;
+        m_->work = nullptr;
+        m_->work_bytes = 0;
+        NB_TRY_CUDA(cudaFreeAsync(old, st_), "cudaFreeAsync(fit workspace)");
+      }
+      NB_TRY_CUDA(cudaMallocAsync(&m_->work, bytes, st_), "cudaMallocAsync(fit workspace)");
+      m_->work_bytes = bytes;
+    }
+    *p = m_->work;
+    return NB_OK;
+  }
+  NB_TRY_CUDA(cudaMallocAsync(&own_, bytes, st_), "cudaMallocAsync(fit scratch)");
+  *p = own_;
+  return NB_OK;
+}
+
+nb_status FitScratch::release() {
+  if (!own_) return NB_OK;
+  void* p = own_;
+  own_ = nullptr;
+  NB_TRY_CUDA(cudaFreeAsync(p, st_), "cudaFreeAsync(fit scratch)");
+  return NB_OK;
+}
+
 nb_status status_from_word(int w) {
   if (w & ST_TIMEOUT) {
     set_error("a bounded device wait ran out");
@@ -224,13 +260,22 @@ static nb_status check_fit_args(nb_kind kind, const void* X, nb_dtype dtype, int
   return NB_OK;
 }
 
+static nb_status fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld,
+                              const int32_t* y, bool prior_given, cudaStream_t st) {
+  FitScratch fs(m, st);
+  void* scratch = nullptr;
+  nb_status s = fs.take(gauss_scratch_bytes(n, m->F, m->C), &scratch);
+  if (s != NB_OK) return s;
+  s = launch_fit_gaussian(m, X, n, ld, y, prior_given, scratch, st);
+  const nb_status f = fs.release();
+  return s != NB_OK ? s : f;
+}
+
 // launch the fit of an allocated model; optionally wait and report bad data
 static nb_status fit_into(nb_model* m, const void* X, nb_dtype dtype, int64_t n, int64_t ld,
                           const int32_t* y, const double* prior, const nb_aux* aux, int no_sync,
                           cudaStream_t st) {
-  // the multinomial fit clears the status word together with its counts
-  if (m->kind != NB_MULTINOMIAL)
-    NB_TRY_CUDA(cudaMemsetAsync(m->d.status, 0, sizeof(int), st), "memset(status)");
+  // both kinds clear the status word together with their counts
   double* prior_dev = nullptr;
   if (prior) {
     // stage the host priors in the model's own log_pi slot
@@ -243,7 +288,7 @@ static nb_status fit_into(nb_model* m, const void* X, nb_dtype dtype, int64_t n,
   if (m->kind == NB_MULTINOMIAL)
     s = launch_fit_multinomial(m, X, dtype, n, ld, y, aux, prior_dev, st);
   else
-    s = launch_fit_gaussian(m, static_cast<const float*>(X), n, ld, y, prior_dev, st);
+    s = fit_gaussian(m, static_cast<const float*>(X), n, ld, y, prior != nullptr, st);
   if (s != NB_OK) return s;
   if (!no_sync) {
     int w = 0;
@@ -302,6 +347,7 @@ extern "C" nb_status nb_fit(nb_kind kind, const void* X, nb_dtype dtype, int64_t
     delete m;
     return s;
   }
+  m->refit = true;
   *out = m;
   return NB_OK;
 }
@@ -397,6 +443,7 @@ extern "C" nb_status nb_model_info(const nb_model* m, int32_t* kind, int32_t* C,
 extern "C" void nb_model_free(nb_model* m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
+  if (m->work) cudaFree(m->work);
   cudaFree(m->mem);
   delete m;
 }

@@ -9,11 +9,7 @@
 // sums runs of rows of one class in registers and adds each feature's total
 // to N_cj with one 64-bit atomic per run; integer sums do not depend on the
 // order of the additions, so the counts are exact and reproducible.
-//
-// Gaussian (real-valued features): per-class means and maximum-likelihood
-// variances in FP64 by two passes (mean, then squared deviations about it),
-// each pass as fixed per-chunk partial sums reduced in a fixed order, so the
-// result is bit-reproducible.  eps = var_smoothing * max_j Var(x_.j).
+// The Gaussian fit is in gauss_fit.cu.
 #include <cuda_fp16.h>
 #include <math.h>
 
@@ -886,205 +882,6 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
     NB_TRY_CUDA(cudaGetLastError(), "k_derive_general");
   }
   if (d.tc_w) return launch_derive_tc(m, st);
-  return NB_OK;
-}
-
-// ---------------------------------------------------------------------------
-// Gaussian fit
-// ---------------------------------------------------------------------------
-
-// pass 0: sums of x; pass 1: sums of (x - mean)^2.  Slot C = all rows.
-__global__ void __launch_bounds__(256) k_gauss_partial(const float* X, int64_t ld, int64_t n,
-                                                       int F, int C, const int32_t* y, int pass,
-                                                       const double* mu_c, const double* mu_all,
-                                                       double* partial, int64_t chunk_rows,
-                                                       int tile, int* status) {
-  // partial layout: [chunk][slot 0..C][F]
-  extern __shared__ double acc[];   // [8 warps][C+1][tile]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j0 = blockIdx.y * tile;
-  const int64_t r0 = (int64_t)blockIdx.x * chunk_rows;
-  int64_t r1 = r0 + chunk_rows;
-  if (r1 > n) r1 = n;
-  const int S = C + 1;
-  for (int k = threadIdx.x; k < 8 * S * tile; k += blockDim.x) acc[k] = 0.0;
-  __syncthreads();
-  double* my = acc + (size_t)warp * S * tile;
-  for (int64_t i = r0 + warp; i < r1; i += 8) {
-    const int c = y[i];
-    if (c < 0 || c >= C) {
-      if (lane == 0) atomicOr(status, ST_BAD_LABEL);
-      continue;
-    }
-    for (int jj = lane; jj < tile; jj += 32) {
-      const int j = j0 + jj;
-      if (j >= F) break;
-      const double x = (double)X[i * ld + j];
-      if (!isfinite(x)) atomicOr(status, ST_BAD_VALUE);
-      if (pass == 0) {
-        my[c * tile + jj] += x;
-        my[C * tile + jj] += x;
-      } else {
-        const double dc = x - mu_c[(int64_t)c * F + j];
-        const double da = x - mu_all[j];
-        my[c * tile + jj] += dc * dc;
-        my[C * tile + jj] += da * da;
-      }
-    }
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < S * tile; k += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += acc[(size_t)w * S * tile + k];
-    const int slot = k / tile, jj = k % tile, j = j0 + jj;
-    if (j < F) partial[((int64_t)blockIdx.x * S + slot) * F + j] = s;
-  }
-}
-
-// sum the per-chunk partials in chunk order; pass 0 -> means, pass 1 -> variances
-__global__ void k_gauss_reduce(const double* partial, int nchunk, int F, int C,
-                               const unsigned long long* nc, int64_t n, int pass, double* mu_c,
-                               double* mu_all, double* m2_c, double* m2_all) {
-  const int S = C + 1;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < S * F; k += gridDim.x * blockDim.x) {
-    const int slot = k / F, j = k % F;
-    double s = 0.0;
-    for (int ch = 0; ch < nchunk; ++ch) s += partial[((int64_t)ch * S + slot) * F + j];
-    const double cnt = slot < C ? (double)nc[slot] : (double)n;
-    const double v = cnt > 0 ? s / cnt : 0.0;
-    if (pass == 0) {
-      if (slot < C) mu_c[(int64_t)slot * F + j] = v; else mu_all[j] = v;
-    } else {
-      if (slot < C) m2_c[(int64_t)slot * F + j] = v; else m2_all[j] = v;
-    }
-  }
-}
-
-// var += eps, log prior, Gaussian constants and FP32 tables.  One block of
-// 256 threads; reductions by warp shuffles and one pass over the warp results.
-__global__ void __launch_bounds__(256) k_gauss_finalize(
-    const double* m2_all, int F, int F_pad, int C, double var_smoothing,
-    const unsigned long long* nc, int64_t n, int prior_given, const double* mu, double* var,
-    double* log_pi, double* gconst, float* g_mu, float* g_ivar, float* g_const, int* status) {
-  __shared__ double red[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double mx = 0.0;
-  for (int j = threadIdx.x; j < F; j += blockDim.x) mx = fmax(mx, m2_all[j]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-  if (lane == 0) red[warp] = mx;
-  __syncthreads();
-  double gm = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) gm = fmax(gm, red[w]);
-  const double eps = var_smoothing * gm;
-  __syncthreads();
-  // the FP32 tables feature-major, gauss_cpad(C) classes per feature
-  const int CP = gauss_cpad(C);
-  for (int k = threadIdx.x; k < CP * F_pad; k += blockDim.x) {
-    const int j = k / CP, c = k % CP;
-    if (j >= F || c >= C) {
-      g_mu[k] = 0.f;
-      g_ivar[k] = 0.f;
-      continue;
-    }
-    double v = var[(int64_t)c * F + j] + eps;
-    if (!(v > 0.0) || !isfinite(v)) atomicOr(status, ST_BAD_TABLE);
-    var[(int64_t)c * F + j] = v;
-    g_mu[k] = (float)mu[(int64_t)c * F + j];
-    g_ivar[k] = (float)(1.0 / v);
-  }
-  __syncthreads();
-  const double kTwoPi = 6.283185307179586476925;
-  __shared__ double red4[8];
-  for (int c = 0; c < C; ++c) {
-    // sum_j log(2 pi var_cj), and a4_c = sum_j m^2 v over the FP32 tables (a
-    // term of the CUDA-core scorer's rounding bound)
-    double s = 0.0, s4 = 0.0;
-    for (int j = threadIdx.x; j < F; j += blockDim.x) {
-      s += log(kTwoPi * var[(int64_t)c * F + j]);
-      const double mj = g_mu[(int64_t)j * CP + c];
-      s4 += mj * mj * (double)g_ivar[(int64_t)j * CP + c];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
-      s4 += __shfl_xor_sync(0xFFFFFFFFu, s4, off);
-    }
-    if (lane == 0) {
-      red[warp] = s;
-      red4[warp] = s4;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0, t4 = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        t += red[w];
-        t4 += red4[w];
-      }
-      g_const[C + c] = (float)t4;
-      if (!prior_given) {
-        if (nc[c] == 0) atomicOr(status, ST_BAD_LABEL);
-        log_pi[c] = nc[c] ? log((double)nc[c]) - log((double)n) : 0.0;
-      }
-      gconst[c] = log_pi[c] - 0.5 * t;
-      g_const[c] = (float)gconst[c];
-    }
-    __syncthreads();
-  }
-}
-
-nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld,
-                              const int32_t* y, const double* log_prior_dev, cudaStream_t st) {
-  const int C = m->C, F = m->F, S = C + 1;
-  ModelDev& d = m->d;
-  NB_TRY_CUDA(cudaMemsetAsync(d.nc, 0, sizeof(uint64_t) * C, st), "memset");
-  if (log_prior_dev && log_prior_dev != d.log_pi)
-    NB_TRY_CUDA(cudaMemcpyAsync(d.log_pi, log_prior_dev, sizeof(double) * C,
-                                cudaMemcpyDeviceToDevice, st),
-                "memcpy prior");
-  const int sms = num_sms();
-  const long long g = (n + 255) / 256;
-  count_launch();
-  k_label_hist<<<(unsigned)(g < sms * 4 ? g : sms * 4), 256, 0, st>>>(
-      y, n, C, reinterpret_cast<unsigned long long*>(d.nc), d.status);
-  NB_TRY_CUDA(cudaGetLastError(), "k_label_hist");
-  const int64_t chunk_rows = gauss_chunk_rows(n);
-  const int nchunk = (int)((n + chunk_rows - 1) / chunk_rows);
-  const size_t part_elems = (size_t)nchunk * S * F;
-  const size_t extra = (size_t)F * 2;   // mu_all, m2_all
-  void* scratch = nullptr;
-  NB_TRY_CUDA(cudaMallocAsync(&scratch, sizeof(double) * (part_elems + extra), st),
-              "cudaMallocAsync(gauss scratch)");
-  double* partial = static_cast<double*>(scratch);
-  double* mu_all = partial + part_elems;
-  double* m2_all = mu_all + F;
-  const int tile = gauss_tile(C);
-  const int smem = (int)(sizeof(double) * 8 * S * tile);
-  if (smem > kSmemOptIn)
-    NB_TRY_CUDA(cudaFuncSetAttribute(k_gauss_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem),
-                "cudaFuncSetAttribute");
-  dim3 grid(nchunk, (F + tile - 1) / tile);
-  const int rb = (S * F + 255) / 256;
-  for (int pass = 0; pass < 2; ++pass) {
-    count_launch();
-    k_gauss_partial<<<grid, 256, smem, st>>>(X, ld, n, F, C, y, pass, d.p0, mu_all, partial,
-                                             chunk_rows, tile, d.status);
-    NB_TRY_CUDA(cudaGetLastError(), "k_gauss_partial");
-    count_launch();
-    k_gauss_reduce<<<rb < 1024 ? rb : 1024, 256, 0, st>>>(
-        partial, nchunk, F, C, reinterpret_cast<unsigned long long*>(d.nc), n, pass, d.p0, mu_all,
-        d.p1, m2_all);
-    NB_TRY_CUDA(cudaGetLastError(), "k_gauss_reduce");
-  }
-  count_launch();
-  k_gauss_finalize<<<1, 256, 0, st>>>(m2_all, F, m->F_pad, C, m->var_smoothing,
-                                       reinterpret_cast<unsigned long long*>(d.nc), n,
-                                       log_prior_dev != nullptr, d.p0, d.p1, d.log_pi, d.gconst,
-                                       d.g_mu, d.g_ivar, d.g_const, d.status);
-  NB_TRY_CUDA(cudaGetLastError(), "k_gauss_finalize");
-  NB_TRY_CUDA(cudaFreeAsync(scratch, st), "cudaFreeAsync(gauss scratch)");
-  if (d.tcg_kc) return launch_derive_tcg(m, st);
   return NB_OK;
 }
 

@@ -143,6 +143,9 @@ struct nb_model {
   cudaStream_t stream;   // stream of the fit
   void* mem;
   size_t mem_bytes;
+  void* work;            // fit workspace kept between re-fits (see FitScratch), or nullptr
+  size_t work_bytes;
+  bool refit;            // the model has been fitted: later fits keep their workspace
   nbg::ModelDev d;
 };
 
@@ -153,9 +156,29 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt,
                                  int64_t n, int64_t ld, const int32_t* y,
                                  const nb_aux* aux, const double* log_prior_dev,
                                  cudaStream_t st);
-nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n,
-                              int64_t ld, const int32_t* y,
-                              const double* log_prior_dev, cudaStream_t st);
+// Gaussian fit (gauss_fit.cu): device scratch it needs, and the launches
+// (log priors, when given, already stand in the model's log_pi)
+size_t gauss_scratch_bytes(int64_t n, int F, int C);
+nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld,
+                              const int32_t* y, bool prior_given, void* scratch,
+                              cudaStream_t st);
+
+// Device scratch of a fit: the model's own workspace, kept between re-fits
+// (up to kKeepWork bytes; larger ones, the first fit's and those of a stream
+// being captured are allocated and freed in stream order).
+constexpr size_t kKeepWork = size_t(64) << 20;
+class FitScratch {
+ public:
+  FitScratch(nb_model* m, cudaStream_t st) : m_(m), st_(st) {}
+  ~FitScratch() { release(); }
+  nb_status take(size_t bytes, void** p);
+  nb_status release();
+
+ private:
+  nb_model* m_;
+  cudaStream_t st_;
+  void* own_ = nullptr;
+};
 
 struct ScoreOut {
   uint8_t* label;
@@ -228,39 +251,11 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
 // process-wide count of kernels this library has launched
 void count_launch();
 
-// Gaussian fit: rows per deterministic partial sum, features per block tile
-constexpr int kGChunkRows = 256;
-constexpr int kGTile = 64;
-// features per block tile of a fit with C classes: 64 up to 32 classes, 32
-// above (the block's shared partial sums, 8 (C + 1) tile doubles, must fit);
-// the tile changes which block sums a feature, not the order of its sums
-inline int gauss_tile(int C) { return C <= 32 ? kGTile : kGTile / 2; }
-// rows per partial sum of a fit of n rows: 32 for small fits (more blocks in
-// flight), else kGChunkRows; the partials are summed in chunk order, so the
-// result depends only on n (every Gaussian fit path uses this rule)
-inline int64_t gauss_chunk_rows(int64_t n) { return n <= 65536 ? 32 : kGChunkRows; }
-
 // ST_* bits of a status word -> status code and error text (first error wins)
 nb_status status_from_word(int w);
 
 // Looks up the allocation-free re-fit's device scratch for the current device
 // (noalloc.cu); under lazy module loading this is what commits it.
 nb_status noalloc_scratch_prepare();
-
-// Gaussian fit kernels (fit.cu)
-__global__ void k_label_hist(const int32_t* y, int64_t n, int C, unsigned long long* nc,
-                             int* status);
-__global__ void k_gauss_partial(const float* X, int64_t ld, int64_t n, int F, int C,
-                                const int32_t* y, int pass, const double* mu_c,
-                                const double* mu_all, double* partial, int64_t chunk_rows,
-                                int tile, int* status);
-__global__ void k_gauss_reduce(const double* partial, int nchunk, int F, int C,
-                               const unsigned long long* nc, int64_t n, int pass, double* mu_c,
-                               double* mu_all, double* m2_c, double* m2_all);
-__global__ void k_gauss_finalize(const double* m2_all, int F, int F_pad, int C,
-                                 double var_smoothing, const unsigned long long* nc, int64_t n,
-                                 int prior_given, const double* mu, double* var, double* log_pi,
-                                 double* gconst, float* g_mu, float* g_ivar, float* g_const,
-                                 int* status);
 
 }  // namespace nbg

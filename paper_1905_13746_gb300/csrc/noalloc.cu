@@ -1,7 +1,7 @@
 // Allocation-free Gaussian re-fit.
 //
 // nb_refit on a Gaussian model takes its per-chunk partial sums from
-// stream-ordered scratch (cudaMallocAsync / cudaFreeAsync).  Some callers
+// stream-ordered memory (cudaMallocAsync), which it keeps with the model.  Some callers
 // cannot allocate device memory at the point where they re-train: a thread
 // bound to a fixed memory budget whose pool must not grow, code running
 // between the instantiation and the replays of a CUDA graph, or an embedded
@@ -84,8 +84,9 @@ extern "C" nb_status nb_refit_gaussian_noalloc(nb_model* m, const float* X, int6
         set_error("nb_refit_gaussian_noalloc: log priors must be finite");
         return NB_EINVAL;
       }
-  // the same row chunks as nb_refit, so the partial sums and their order match
-  const int64_t chunk_rows = gauss_chunk_rows(n);
+  // the request's size is limited by 32-row (256-row above 65,536 rows) partial
+  // sums of C + 1 slots, the measure that the header states
+  const int64_t chunk_rows = n <= 65536 ? 32 : 256;
   const long long nchunk = (n + chunk_rows - 1) / chunk_rows;
   const size_t need = (size_t)nchunk * S * F + 2 * (size_t)F;
   if (need > kScratchDoubles) {
@@ -98,53 +99,21 @@ extern "C" nb_status nb_refit_gaussian_noalloc(nb_model* m, const float* X, int6
   nb_status s = scratch_for_current_device(&scratch);
   if (s != NB_OK) return s;
 
+  // the same kernels and row chunks as nb_refit, so the sums and their order
+  // match; their scratch is below `need` doubles for every accepted request
+  if (gauss_scratch_bytes(n, F, C) > sizeof(double) * kScratchDoubles) {
+    set_error("nb_refit_gaussian_noalloc: the fixed scratch is too small; use nb_refit");
+    return NB_EINVAL;
+  }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   m->var_smoothing = vs;
   m->stream = st;
   ModelDev& d = m->d;
-  double* partial = scratch;
-  double* mu_all = partial + (size_t)nchunk * S * F;
-  double* m2_all = mu_all + F;
-  NB_TRY_CUDA(cudaMemsetAsync(d.status, 0, sizeof(int), st), "memset(status)");
-  NB_TRY_CUDA(cudaMemsetAsync(d.nc, 0, sizeof(uint64_t) * C, st), "memset(nc)");
   if (prior)
     NB_TRY_CUDA(cudaMemcpyAsync(d.log_pi, prior, sizeof(double) * C, cudaMemcpyHostToDevice, st),
                 "memcpy(log prior)");
-  const int sms = num_sms();
-  const long long g = (n + 255) / 256;
-  count_launch();
-  k_label_hist<<<(unsigned)(g < sms * 4 ? g : sms * 4), 256, 0, st>>>(
-      y, n, C, reinterpret_cast<unsigned long long*>(d.nc), d.status);
-  NB_TRY_CUDA(cudaGetLastError(), "k_label_hist");
-  const int tile = gauss_tile(C);
-  const int smem = (int)(sizeof(double) * 8 * S * tile);
-  if (smem > kSmemOptIn)
-    NB_TRY_CUDA(cudaFuncSetAttribute(k_gauss_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem),
-                "cudaFuncSetAttribute");
-  const dim3 grid((unsigned)nchunk, (F + tile - 1) / tile);
-  const int rb = (S * F + 255) / 256;
-  for (int pass = 0; pass < 2; ++pass) {
-    count_launch();
-    k_gauss_partial<<<grid, 256, smem, st>>>(X, ld, n, F, C, y, pass, d.p0, mu_all, partial,
-                                             chunk_rows, tile, d.status);
-    NB_TRY_CUDA(cudaGetLastError(), "k_gauss_partial");
-    count_launch();
-    k_gauss_reduce<<<rb < 1024 ? rb : 1024, 256, 0, st>>>(
-        partial, (int)nchunk, F, C, reinterpret_cast<unsigned long long*>(d.nc), n, pass, d.p0,
-        mu_all, d.p1, m2_all);
-    NB_TRY_CUDA(cudaGetLastError(), "k_gauss_reduce");
-  }
-  count_launch();
-  k_gauss_finalize<<<1, 256, 0, st>>>(m2_all, F, m->F_pad, C, vs,
-                                       reinterpret_cast<unsigned long long*>(d.nc), n,
-                                       prior != nullptr, d.p0, d.p1, d.log_pi, d.gconst, d.g_mu,
-                                       d.g_ivar, d.g_const, d.status);
-  NB_TRY_CUDA(cudaGetLastError(), "k_gauss_finalize");
-  if (d.tcg_kc) {
-    s = launch_derive_tcg(m, st);
-    if (s != NB_OK) return s;
-  }
+  s = launch_fit_gaussian(m, X, n, ld, y, prior != nullptr, scratch, st);
+  if (s != NB_OK) return s;
   if (!(opts && opts->no_sync)) {
     int w = 0;
     NB_TRY_CUDA(cudaMemcpyAsync(&w, d.status, sizeof(int), cudaMemcpyDeviceToHost, st),

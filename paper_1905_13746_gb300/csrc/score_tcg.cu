@@ -609,22 +609,28 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_score_tcg(const __grid_consta
 // One thread per feature j (nks * TG_FS of them): m_j = the mean of the class
 // means, rounded to FP32 (the expansion uses that FP32 value), the eight limb
 // values of every class in one 16-byte record, the per-feature maxima.
-__global__ void k_derive_tcg(const double* mu, const double* var, int C, int F, int Cp, int nks,
-                             uint8_t* wlay, float* ctr, float* bmax, float* amax, TcgHeader* hdr) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per feature, lanes over the classes: FP64 division is slow on this
+// part, and one thread per feature took all Cp classes one after another on
+// F / 256 SMs (C = 64, F = 256: 108 us).
+__global__ void __launch_bounds__(256) k_derive_tcg(const double* mu, const double* var, int C,
+                                                    int F, int Cp, int nks, uint8_t* wlay,
+                                                    float* ctr, float* bmax, float* amax,
+                                                    TcgHeader* hdr) {
+  const int lane = threadIdx.x & 31, j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  pdl_wait();
   if (j >= nks * TG_FS) return;
   double m = 0.0;
-  if (j < F) {
-    for (int c = 0; c < C; ++c) m += mu[(int64_t)c * F + j];
-    m /= (double)C;
-  }
-  const float mf = (float)m;
+  if (j < F)
+    for (int c = lane; c < C; c += 32) m += mu[(int64_t)c * F + j];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xFFFFFFFFu, m, off);
+  const float mf = (float)(m / (double)C);
   const double md = (double)mf;
   const int ks = j / TG_FS, jj = j % TG_FS;
   uint8_t* stage = wlay + (size_t)ks * Cp * (2 * TG_KS);
   double bm = 0.0, am = 0.0;
   bool ok = true;
-  for (int c = 0; c < Cp; ++c) {
+  for (int c = lane; c < Cp; c += 32) {
     __half h[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) h[t] = __float2half_rn(0.f);
@@ -646,7 +652,13 @@ __global__ void k_derive_tcg(const double* mu, const double* var, int C, int F, 
     *reinterpret_cast<uint4*>(stage + (c >> 3) * (16 * TG_KS) + jj * 128 + (c & 7) * 16) =
         *reinterpret_cast<const uint4*>(h);
   }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    bm = fmax(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, off));
+    am = fmax(am, __shfl_xor_sync(0xFFFFFFFFu, am, off));
+  }
   if (!ok) hdr->bad = 1;   // a weight outside the FP16 range: every row to FP64
+  if (lane != 0) return;
   ctr[j] = j < F ? mf : 0.f;
   bmax[j] = (float)(bm * (1.0 + 1.0 / 1048576.0));
   amax[j] = (float)(am * (1.0 + 1.0 / 1048576.0));
@@ -659,6 +671,7 @@ __global__ void __launch_bounds__(256) k_derive_tcg_k(const double* mu, const do
                                                       int F, float* kc, TcgHeader* hdr) {
   __shared__ double red[8];
   const int c = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  pdl_wait();
   double s = 0.0, w = 0.0;
   for (int j = threadIdx.x; j < F; j += blockDim.x) {
     const double d = mu[(int64_t)c * F + j] - (double)ctr[j];
@@ -692,18 +705,18 @@ __global__ void __launch_bounds__(256) k_derive_tcg_k(const double* mu, const do
 nb_status launch_derive_tcg(nb_model* m, cudaStream_t st) {
   const int nks = (m->F + TG_FS - 1) / TG_FS;
   const int Cp = tc_classes_padded(m->C);
-  NB_TRY_CUDA(cudaMemsetAsync(m->d.tcg_hdr, 0, sizeof(TcgHeader), st), "memset(tcg header)");
+  // the header's flag was cleared by k_gauss_mean
   count_launch();
-  k_derive_tcg<<<(nks * TG_FS + 255) / 256, 256, 0, st>>>(m->d.p0, m->d.p1, m->C, m->F, Cp, nks,
-                                                           m->d.tc_w, m->d.tcg_ctr,
-                                                           m->d.tcg_bmax, m->d.tcg_amax,
-                                                           m->d.tcg_hdr);
-  NB_TRY_CUDA(cudaGetLastError(), "k_derive_tcg");
+  NB_TRY_CUDA(launch_pdl(k_derive_tcg, dim3(nks * TG_FS / 8), dim3(256), 0, st,
+                         (const double*)m->d.p0, (const double*)m->d.p1, m->C, m->F, Cp, nks,
+                         m->d.tc_w, m->d.tcg_ctr, m->d.tcg_bmax, m->d.tcg_amax, m->d.tcg_hdr),
+              "k_derive_tcg");
   count_launch();
-  k_derive_tcg_k<<<m->C, 256, 0, st>>>(m->d.p0, m->d.p1, m->d.gconst, m->d.tcg_ctr,
-                                       m->d.tcg_bmax, m->d.tcg_amax, m->F, m->d.tcg_kc,
-                                       m->d.tcg_hdr);
-  NB_TRY_CUDA(cudaGetLastError(), "k_derive_tcg_k");
+  NB_TRY_CUDA(launch_pdl(k_derive_tcg_k, dim3(m->C), dim3(256), 0, st, (const double*)m->d.p0,
+                         (const double*)m->d.p1, (const double*)m->d.gconst,
+                         (const float*)m->d.tcg_ctr, (const float*)m->d.tcg_bmax,
+                         (const float*)m->d.tcg_amax, m->F, m->d.tcg_kc, m->d.tcg_hdr),
+              "k_derive_tcg_k");
   return NB_OK;
 }
 
