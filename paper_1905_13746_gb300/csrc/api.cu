@@ -68,6 +68,7 @@ static nb_status alloc_model(nb_model* m) {
   const size_t o_c2 = take(sizeof(C2Header));
   const size_t o_delta = take(sizeof(float) * Fp);
   const size_t o_dq = take(sizeof(int32_t) * Fp);
+  const size_t o_dp = take(sizeof(int32_t) * Fp);
   const size_t o_limbs = take(7 * Fp);   // three limb planes + packed limb words
   const size_t o_il0 = take(sizeof(float) * Fp);
   const size_t o_il1 = take(sizeof(float) * Fp);
@@ -109,6 +110,7 @@ static nb_status alloc_model(nb_model* m) {
   d.c2 = reinterpret_cast<C2Header*>(b + o_c2);
   d.delta = reinterpret_cast<float*>(b + o_delta);
   d.delta_q = reinterpret_cast<int32_t*>(b + o_dq);
+  d.delta_p = reinterpret_cast<int32_t*>(b + o_dp);
   d.limbs = reinterpret_cast<uint4*>(b + o_limbs);
   d.il[0] = reinterpret_cast<float4*>(b + o_il0);
   d.il[1] = reinterpret_cast<float4*>(b + o_il1);
@@ -450,9 +452,12 @@ extern "C" void nb_model_free(nb_model* m) {
 
 static nb_path score_path(const nb_model* m, const void* X, nb_dtype dtype, int64_t ld,
                           int recheck) {
-  const bool aligned = ((reinterpret_cast<uintptr_t>(X) & 15) == 0) &&
-                       ((ld * elem_size(dtype)) % 16 == 0);
-  if (m->kind == NB_MULTINOMIAL && m->C == 2 && aligned) return NB_PATH_TWO_CLASS;
+  // two classes: 16-byte aligned rows of any type, and wider elements at any
+  // row pitch (bytes at an odd pitch stay with the general scorer)
+  if (m->kind == NB_MULTINOMIAL && m->C == 2 &&
+      (c2_aligned(X, dtype, ld) || (elem_size(dtype) >= 2 &&
+                                    reinterpret_cast<uintptr_t>(X) % elem_size(dtype) == 0)))
+    return NB_PATH_TWO_CLASS;
   if (tc_eligible(m, dtype, X, ld)) return NB_PATH_TENSOR;
   if (dtype == NB_F32 && tcg_eligible(m, X, ld, recheck)) return NB_PATH_TENSOR_GAUSS;
   return NB_PATH_GENERAL;

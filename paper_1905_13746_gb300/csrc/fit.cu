@@ -409,94 +409,6 @@ __global__ void __launch_bounds__(256) k_finalize_mn(const unsigned long long* c
     log_theta[(int64_t)c * F + j] = log((double)counts[(int64_t)c * F + j] + alpha) - log_den;
 }
 
-// two-class tables: Delta (FP64 -> FP32, fixed point + limbs), b, interleaved
-// copies for the scorer's 16-byte vectors.  One block.
-__global__ void __launch_bounds__(1024) k_derive_c2(const double* log_theta, const double* log_pi,
-                                                    int F, int F_pad, int nvec8, C2Header* hdr,
-                                                    float* delta, int32_t* delta_q, uint4* limbs,
-                                                    float4* il4, float4* il8, float4* il16,
-                                                    int* status) {
-  __shared__ double red[1024];
-  double mx = 0.0;
-  for (int j = threadIdx.x; j < F; j += blockDim.x) {
-    const double d = log_theta[F + j] - log_theta[j];
-    mx = fmax(mx, fabs(d));
-    if (!isfinite(d)) atomicOr(status, ST_BAD_TABLE);
-  }
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  const double maxabs64 = red[0];
-  int S = 0;
-  if (maxabs64 > 0.0) {
-    int e;
-    frexp(maxabs64, &e);   // maxabs64 < 2^e
-    S = 22 - e;
-  }
-  const double scale = ldexp(1.0, S);
-  float mx32 = 0.f;
-  for (int j = threadIdx.x; j < F_pad; j += blockDim.x) {
-    const double d = j < F ? log_theta[F + j] - log_theta[j] : 0.0;
-    const float d32 = (float)d;
-    mx32 = fmaxf(mx32, fabsf(d32));
-    delta[j] = d32;
-    const int32_t q = (int32_t)llrint(d * scale);   // |q| <= 2^22
-    delta_q[j] = q;
-    // balanced base-256 digits q = q2*65536 + q1*256 + q0, each in [-128, 127]
-    const int32_t q0 = ((q + 128) & 255) - 128;
-    const int32_t r1 = (q - q0) >> 8;
-    const int32_t q1 = ((r1 + 128) & 255) - 128;
-    const int32_t q2 = (r1 - q1) >> 8;
-    // u8 vectors hold 16 features; limb L of vector v is slot L * nvec8 + v,
-    // byte (j % 16) of it
-    const int v = j >> 4, b = j & 15;
-    unsigned char* L = reinterpret_cast<unsigned char*>(limbs);
-    L[((size_t)0 * nvec8 + v) * 16 + b] = (unsigned char)(q0 & 255);
-    L[((size_t)1 * nvec8 + v) * 16 + b] = (unsigned char)(q1 & 255);
-    L[((size_t)2 * nvec8 + v) * 16 + b] = (unsigned char)(q2 & 255);
-    // the same limbs packed into one word per feature (overflow entries)
-    reinterpret_cast<uint32_t*>(L + (size_t)3 * F_pad)[j] =
-        (uint32_t)(q0 & 255) | ((uint32_t)(q1 & 255) << 8) | ((uint32_t)(q2 & 255) << 16);
-    // FP32 tables for 4 / 8 / 16 elements per vector: quad q of vector v is
-    // slot q * (F_pad / EPV) + v
-    {
-      float* t = reinterpret_cast<float*>(il4);
-      const int epv = 4, vv = j / epv, e = j % epv;
-      t[((size_t)(e >> 2) * (F_pad / epv) + vv) * 4 + (e & 3)] = d32;
-    }
-    {
-      float* t = reinterpret_cast<float*>(il8);
-      const int epv = 8, vv = j / epv, e = j % epv;
-      t[((size_t)(e >> 2) * (F_pad / epv) + vv) * 4 + (e & 3)] = d32;
-    }
-    {
-      float* t = reinterpret_cast<float*>(il16);
-      const int epv = 16, vv = j / epv, e = j % epv;
-      t[((size_t)(e >> 2) * (F_pad / epv) + vv) * 4 + (e & 3)] = d32;
-    }
-  }
-  __shared__ float redf[1024];
-  redf[threadIdx.x] = mx32;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) redf[threadIdx.x] = fmaxf(redf[threadIdx.x], redf[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double b = log_pi[1] - log_pi[0];
-    hdr->b = (float)b;
-    hdr->b64 = b;
-    hdr->maxabs = redf[0];
-    hdr->S = S;
-    hdr->inv_scale = (float)ldexp(1.0, -S);
-    hdr->maxabs_q = (float)maxabs64;
-    hdr->pad = 0;
-  }
-}
-
 // Two-class finish of the fit in one launch (Sec. 4 likelihoods, Laplace
 // smoothing).  FP64 is slow on this part and the kernel is one chain of
 // latencies, so the work is spread thin and overlapped: a block of 4 kFinF
@@ -514,8 +426,8 @@ constexpr int kFinT = 4 * kFinF;   // threads per block
 __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     const unsigned long long* counts, const unsigned long long* nc, int64_t n, int F, int F_pad,
     int nvec8, double alpha, int prior_given, double* log_theta, double* log_pi, C2Header* hdr,
-    float* delta, int32_t* delta_q, uint4* limbs, float4* il4, float4* il8, float4* il16,
-    float* w, float* bias, float* wmax, unsigned long long* fin, int* status) {
+    float* delta, int32_t* delta_q, int32_t* delta_p, uint4* limbs, float4* il4, float4* il8,
+    float4* il16, float* w, float* bias, float* wmax, unsigned long long* fin, int* status) {
   constexpr int NT = kFinT, NL = 2 * kFinF;   // NL threads take the per-feature logs
   __shared__ unsigned long long part[2][2];
   __shared__ double ld[2];
@@ -658,6 +570,7 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
       if (jj >= F_pad) continue;
       const int32_t q = (int32_t)llrint(dd[u] * scale);   // |q| <= 2^22
       delta_q[jj] = q;
+      delta_p[jj] = (int32_t)llrint(dd[u] * scale * 256.0);   // |.| <= 2^30
       // balanced base-256 digits q = q2*65536 + q1*256 + q0, each in [-128, 127]
       const int32_t q0 = ((q + 128) & 255) - 128;
       const int32_t r1 = (q - q0) >> 8;
@@ -857,7 +770,7 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
                            0, st, reinterpret_cast<const unsigned long long*>(d.counts),
                            reinterpret_cast<const unsigned long long*>(d.nc), (int64_t)n, F,
                            m->F_pad, m->nvec8, m->alpha, (int)(log_prior_dev != nullptr), d.p0,
-                           d.log_pi, d.c2, d.delta, d.delta_q, d.limbs, d.il[0], d.il[1],
+                           d.log_pi, d.c2, d.delta, d.delta_q, d.delta_p, d.limbs, d.il[0], d.il[1],
                            d.il[2], d.w, d.bias, d.wmax, d.fin, d.status),
                 "k_fit_finish_c2");
     return NB_OK;
@@ -867,12 +780,6 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
       reinterpret_cast<unsigned long long*>(d.counts), reinterpret_cast<unsigned long long*>(d.nc),
       n, F, m->alpha, log_prior_dev != nullptr, d.p0, d.log_pi, d.status);
   NB_TRY_CUDA(cudaGetLastError(), "k_finalize_mn");
-  if (C == 2) {
-    count_launch();
-    k_derive_c2<<<1, 1024, 0, st>>>(d.p0, d.log_pi, F, m->F_pad, m->nvec8, d.c2, d.delta,
-                                    d.delta_q, d.limbs, d.il[0], d.il[1], d.il[2], d.status);
-    NB_TRY_CUDA(cudaGetLastError(), "k_derive_c2");
-  }
   NB_TRY_CUDA(cudaMemsetAsync(d.wmax, 0, sizeof(float), st), "memset");
   {
     const int blocks = (m->F_pad + 255) / 256;

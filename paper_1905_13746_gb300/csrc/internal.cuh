@@ -104,6 +104,7 @@ struct ModelDev {
   C2Header* c2;        // 1
   float* delta;        // F_pad      FP32 Delta, plain order
   int32_t* delta_q;    // F_pad      fixed-point Delta
+  int32_t* delta_p;    // F_pad      fixed-point Delta, eight bits finer (step 2^-(S+8))
   uint4* limbs;        // 3 * nvec8  int8 limbs of delta_q, interleaved (u8 path), then
                        //            F_pad packed words (limb l in byte l)
   float4* il[3];       // interleaved FP32 quads for 4/8/16 elements per vector
@@ -190,6 +191,10 @@ struct ScoreOut {
   bool counted = false;   // the scorer counted its marked rows into n_rechecked
 };
 
+// 16-byte aligned rows (base and pitch)
+inline bool c2_aligned(const void* X, nb_dtype dt, int64_t ld) {
+  return (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ld * elem_size(dt)) % 16 == 0;
+}
 nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt,
                         int64_t n, int64_t ld, const nb_aux* aux,
                         const ScoreOut& o, cudaStream_t st);

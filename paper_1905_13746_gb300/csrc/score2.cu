@@ -275,6 +275,238 @@ __global__ void __launch_bounds__(256) k_score2_fp(const S2Args a) {
 }
 
 // ---------------------------------------------------------------------------
+// F32, U16 and BF16 counts in the log-posterior mode: exact integer sums
+// ---------------------------------------------------------------------------
+// FP32 sums of rows row0 .. row0 + 3 (rows past the end repeat the last one),
+// 32 lanes per row.  Lane k (k < 4) receives row k's sum and |x| total.
+template <int DT>
+__device__ __forceinline__ void float_rows4(const S2Args& a, int64_t row0, float& s_out,
+                                            float& t_out) {
+  using Dec = Decode<DT>;
+  constexpr int EPV = Dec::EPV;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int r = 0; r < 4; ++r) {
+    const char* rp = a.X + min(row0 + r, a.n - 1) * a.ld_bytes;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, tf = 0.f;
+    for (int v = lane; v < a.nvec_row; v += 32) {
+      float val[EPV];
+      Dec::run(ld_stream16(rp + (int64_t)v * 16), val);
+      const float4* w4 = reinterpret_cast<const float4*>(a.delta) + (int64_t)v * (EPV / 4);
+#pragma unroll
+      for (int q = 0; q < EPV / 4; ++q) {
+        const float4 w = __ldg(w4 + q);
+        const float ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float x = v * EPV + 4 * q + e < a.F ? val[4 * q + e] : 0.f;
+          acc[e] = fmaf(x, ww[e], acc[e]);
+          tf += fabsf(x);
+        }
+      }
+    }
+    float s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      tf += __shfl_xor_sync(0xFFFFFFFFu, tf, off);
+    }
+    if (lane == r) {
+      s_out = s;
+      t_out = tf;
+    }
+  }
+}
+
+__device__ __forceinline__ void c2_float_store(const S2Args& a, const C2Header& h, int64_t row,
+                                               float s, float T) {
+  const float d = s + h.b;
+  const float k = (float)a.k_base;
+  const float gam = k * 5.9604645e-8f / (1.f - k * 5.9604645e-8f);
+  const float A = T * h.maxabs * 1.001f;
+  const float tau = gam * (A + fabsf(h.b)) * 1.01f + 1e-12f * (A + fabsf(h.b)) + 1e-30f;
+  if (c2_store(a.label, a.margin, a.logpost, a.want_lp, a.recheck, row, d, tau) && a.marks)
+    atomicAdd(a.marks, 1ull);
+}
+
+__device__ __forceinline__ void c2_fix_store(const S2Args& a, const C2Header& h, int64_t row,
+                                             long long D, float T) {
+  float d, tau;
+  fix_result(D, T, h, d, tau);
+  if (c2_store(a.label, a.margin, a.logpost, a.want_lp, a.recheck, row, d, tau) && a.marks)
+    atomicAdd(a.marks, 1ull);
+}
+
+// Short rows of 16-bit values: a group of LPR lanes sums four rows at a time;
+// the fixed-point table sits in shared memory.  Only if a row of a group holds
+// something else than counts are the group's rows read again for the FP32
+// sums.  Bound by about 9 operations a value (F = 128: 2.8 TB/s).
+template <int DT, int LPR>
+__global__ void __launch_bounds__(256) k_score2_fix(const S2Args a) {
+  using Dec = Decode<DT>;
+  constexpr int EPV = Dec::EPV, R = 4, SUBS = 32 / LPR, RPW = SUBS * R;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t bar;
+  if (!stage_table(smem_raw, a.table, a.table_bytes, &bar, a.status, ST_TIMEOUT)) return;
+  const int4* tab = reinterpret_cast<const int4*>(smem_raw);
+  const C2Header h = *a.hdr;
+  const int lane = threadIdx.x & 31, sub = lane / LPR, li = lane % LPR;
+  const int nv = a.nvec_row;
+  const int64_t ntiles = (a.n + RPW - 1) / RPW;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles;
+       t += nwarps) {
+    const int64_t row0 = t * RPW + (int64_t)sub * R;
+    const char* rp[R];
+    FixSum fix[R];
+    float tf[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {   // rows past the end repeat the last one and store nothing
+      rp[r] = a.X + min(row0 + r, a.n - 1) * a.ld_bytes;
+      tf[r] = 0.f;
+    }
+#pragma unroll 2
+    for (int v = li; v < nv; v += LPR) {
+      uint4 x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = ld_stream16(rp[r] + (int64_t)v * 16);
+      int q[EPV];
+#pragma unroll
+      for (int k = 0; k < EPV / 4; ++k) {
+        const int4 d = tab[v * (EPV / 4) + k];
+        q[4 * k] = d.x;
+        q[4 * k + 1] = d.y;
+        q[4 * k + 2] = d.z;
+        q[4 * k + 3] = d.w;
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float val[EPV];
+        Dec::run(x[r], val);
+        if (v == nv - 1) {
+#pragma unroll
+          for (int e = 0; e < EPV; ++e)
+            if (v * EPV + e >= a.F) val[e] = 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < EPV; ++e) {
+          fix_add(fix[r], val[e], q[e]);
+          tf[r] += val[e];
+        }
+      }
+    }
+    unsigned bad[R], any = 0u;   // per row: the groups whose row is no row of counts
+#pragma unroll
+    for (int r = 0; r < R; ++r) any |= bad[r] = __ballot_sync(0xFFFFFFFFu, fix[r].bad != 0u);
+    const long long D = sum4_transposed<LPR>(fix[0].D, fix[1].D, fix[2].D, fix[3].D, li);
+    const float T = sum4_transposed<LPR>(tf[0], tf[1], tf[2], tf[3], li);
+    const int mr = li / (LPR / 4);   // this lane's quarter holds row mr of the group
+    const unsigned gmask = LPR == 32 ? 0xFFFFFFFFu : ((1u << (LPR & 31)) - 1u) << (sub * LPR);
+    const unsigned mybad = (mr == 0 ? bad[0] : mr == 1 ? bad[1] : mr == 2 ? bad[2] : bad[3]) & gmask;
+    if (li % (LPR / 4) == 0 && row0 + mr < a.n && mybad == 0u) c2_fix_store(a, h, row0 + mr, D, T);
+    if (any) {
+#pragma unroll 1
+      for (int g = 0; g < SUBS; ++g) {
+        const unsigned gm = LPR == 32 ? 0xFFFFFFFFu : ((1u << (LPR & 31)) - 1u) << (g * LPR);
+        if (!(any & gm)) continue;
+        const int64_t r0 = t * RPW + (int64_t)g * R;
+        float s = 0.f, tt = 0.f;
+        float_rows4<DT>(a, r0, s, tt);
+        const unsigned lb = (lane == 0 ? bad[0] : lane == 1 ? bad[1] : lane == 2 ? bad[2] : bad[3]) & gm;
+        if (lane < R && lb && r0 + lane < a.n) c2_float_store(a, h, r0 + lane, s, tt);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// F32, U16 and BF16 rows of any alignment (a row width or a base that is no
+// multiple of 16 bytes)
+// ---------------------------------------------------------------------------
+// A warp takes four rows at a time; lane l reads elements l, l + 32, ... of
+// each with element-wise loads (a row's 32 loads cover 64 or 128 consecutive
+// bytes), U elements of each row in flight, and each entry of the Delta
+// tables, which stay in L1, once for the four rows.  FIX: exact sums, the FP32
+// ones only where a row holds something else than counts.  Without FIX (label
+// and OFF modes) the FP32 sums.
+// 100,003 rows of 1,003 F32 counts (401 MB), log-posterior mode, labels only:
+// 76 us for the whole call; 3.57 ms as 2 of the 64 class columns of the general
+// scorer's 64 x 64 tiles (1.08 ms) and every row in FP64 on top (2.5 ms).
+// 249,252 rows (1 GB): 158 us in the label mode (93% of the measured HBM rate),
+// 190 us (78%) in the log-posterior mode.
+template <int DT>
+__device__ __forceinline__ float any_load(const char* rp, int j) {
+  if (DT == NB_F32) {
+    float v;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(rp + (int64_t)j * 4));
+    return v;
+  }
+  unsigned short h;
+  asm volatile("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=h"(h) : "l"(rp + (int64_t)j * 2));
+  return DT == NB_U16 ? (float)h : __uint_as_float((uint32_t)h << 16);
+}
+
+template <int DT, bool FIX>
+__global__ void __launch_bounds__(256) k_score2_any(const S2Args a) {
+  constexpr int R = 4, U = 8;   // rows, elements in flight per row and lane
+  const int lane = threadIdx.x & 31;
+  const C2Header h = *a.hdr;
+  const int64_t ntiles = (a.n + R - 1) / R;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles;
+       t += nwarps) {
+    const char* rp[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)   // rows past the end repeat the last one and store nothing
+      rp[r] = a.X + min(t * R + r, a.n - 1) * a.ld_bytes;
+    // every element once: add(row, value, element)
+    auto sweep = [&](auto&& table, auto&& add) {
+      for (int j = lane; j < a.F; j += 32 * U) {
+        float x[U][R];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int r = 0; r < R; ++r) x[u][r] = j + 32 * u < a.F ? any_load<DT>(rp[r], j + 32 * u) : 0.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const auto w = table(j + 32 * u < a.F ? j + 32 * u : 0);
+#pragma unroll
+          for (int r = 0; r < R; ++r) add(r, x[u][r], w);
+        }
+      }
+    };
+    const int64_t row = t * R + lane / 8;   // eight lanes hold each row's sums
+    bool todo = true;
+    if (FIX) {
+      FixSum fix[R];
+      float tf[R] = {0.f, 0.f, 0.f, 0.f};
+      sweep([&](int j) { return __ldg(a.delta_p + j); },
+            [&](int r, float x, int q) {
+              fix_add(fix[r], x, q);
+              tf[r] += x;
+            });
+      unsigned bad = 0u;   // bit r: row r is no row of counts
+#pragma unroll
+      for (int r = 0; r < R; ++r) bad |= (__ballot_sync(0xFFFFFFFFu, fix[r].bad != 0u) != 0u) << r;
+      const long long D = sum4_transposed<32>(fix[0].D, fix[1].D, fix[2].D, fix[3].D, lane);
+      const float T = sum4_transposed<32>(tf[0], tf[1], tf[2], tf[3], lane);
+      todo = (bad >> (lane / 8)) & 1u;
+      if (lane % 8 == 0 && row < a.n && !todo) c2_fix_store(a, h, row, D, T);
+      if (!bad) continue;
+    }
+    float s[R] = {0.f, 0.f, 0.f, 0.f}, tf[R] = {0.f, 0.f, 0.f, 0.f};
+    sweep([&](int j) { return __ldg(a.delta + j); },
+          [&](int r, float x, float w) {
+            s[r] = fmaf(x, w, s[r]);
+            tf[r] += fabsf(x);
+          });
+    const float S = sum4_transposed<32>(s[0], s[1], s[2], s[3], lane);
+    const float T = sum4_transposed<32>(tf[0], tf[1], tf[2], tf[3], lane);
+    if (lane % 8 == 0 && row < a.n && todo) c2_float_store(a, h, row, S, T);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // launcher
 // ---------------------------------------------------------------------------
 template <typename K>
@@ -360,6 +592,13 @@ static nb_status dispatch_dt(nb_dtype dt, S2Args& a, int smem, cudaStream_t st) 
   return NB_EINVAL;
 }
 
+// The exact-sum kernel on short rows: 4 or 8 lanes per row, at most 16 vectors.
+template <int DT>
+static nb_status launch_fix(const S2Args& a, int smem, cudaStream_t st) {
+  if (a.nvec_row > 8) return launch_persistent(k_score2_fix<DT, 8>, smem, (a.n + 15) / 16, a, st);
+  return launch_persistent(k_score2_fix<DT, 4>, smem, (a.n + 31) / 32, a, st);
+}
+
 nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                         const nb_aux* aux, const ScoreOut& o, cudaStream_t st) {
   const int es = elem_size(dt);
@@ -372,6 +611,7 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   a.hdr = m->d.c2;
   a.delta_q = m->d.delta_q;
   a.delta = m->d.delta;
+  a.delta_p = m->d.delta_p;
   a.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
   a.ovf_col = aux ? aux->ovf_col : nullptr;
   a.ovf_add = aux ? aux->ovf_add : nullptr;
@@ -396,6 +636,32 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   }
   a.table_bytes = (uint32_t)smem;
   if (n == 0) return NB_OK;
+  const bool fp = dt == NB_F32 || dt == NB_U16 || dt == NB_BF16;
+  const bool fix = fp && o.recheck == NB_RECHECK_LP;
+  if (!c2_aligned(X, dt, ld)) {   // F32, U16 or BF16 (see score_path)
+    a.k_base = (m->F + 31) / 32 + 5 + 2;   // serial FMAs, reduction, weight and final roundings
+    const int64_t tiles = (n + 3) / 4;
+    switch (dt) {
+      case NB_F32:
+        return fix ? launch_persistent(k_score2_any<NB_F32, true>, 0, tiles, a, st)
+                   : launch_persistent(k_score2_any<NB_F32, false>, 0, tiles, a, st);
+      case NB_U16:
+        return fix ? launch_persistent(k_score2_any<NB_U16, true>, 0, tiles, a, st)
+                   : launch_persistent(k_score2_any<NB_U16, false>, 0, tiles, a, st);
+      default:
+        return fix ? launch_persistent(k_score2_any<NB_BF16, true>, 0, tiles, a, st)
+                   : launch_persistent(k_score2_any<NB_BF16, false>, 0, tiles, a, st);
+    }
+  }
+  // 16-bit rows of at most 16 vectors, which the pipelined kernel spreads over
+  // 32 lanes (1M BF16 files: F = 64 52 us against 127, F = 128 93 against 159;
+  // at F = 256 175 against 146 and at 1,024 291 against 211, so longer rows
+  // stay there).  F32 rows stay with the FP32 sums, which batches share.
+  if (fix && es == 2 && a.nvec_row <= 16) {
+    a.table = m->d.delta_p;
+    a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row
+    return dt == NB_U16 ? launch_fix<NB_U16>(a, smem, st) : launch_fix<NB_BF16>(a, smem, st);
+  }
   const nb_tile_config& cfg = m->tile;
   if (cfg.variant != NB_VARIANT_REGISTER) {
     // overflow slices are staged by bulk copies only from 16-byte aligned arrays

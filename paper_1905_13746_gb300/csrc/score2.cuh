@@ -23,6 +23,7 @@ struct S2Args {
   const C2Header* hdr;
   const int32_t* delta_q;   // plain fixed-point table (overflow entries)
   const float* delta;       // plain FP32 table (overflow entries)
+  const int32_t* delta_p;   // plain fixed-point table of step 2^-(S+8)
   const int64_t* ovf_ptr;
   const uint16_t* ovf_col;
   const uint16_t* ovf_add;
@@ -172,6 +173,46 @@ struct Decode<NB_FP8E4M3> {
 };
 
 // ---------------------------------------------------------------------------
+// F32, U16 and BF16 counts as exact integers (log-posterior mode)
+// ---------------------------------------------------------------------------
+// FP32 sums carry a rounding bound of gamma_k sum |x| |Delta|; with one
+// accumulator per 32 elements it is too loose for the log-posterior test on
+// almost every row, and the FP64 recheck of all rows costs more than the
+// scoring (2.5 ms against 1.1 ms for 100,000 rows of 1,003 counts).  The
+// kernels for rows of any alignment and for short 16-bit rows therefore sum a
+// fixed-point Delta exactly, D = sum x P in int64 with P = round(Delta 2^(S+8)),
+// |P| <= 2^30 (eight bits finer than the u8 path's, so that the result is the
+// FP64 one to FP32 rounding).  With u = x + 2^23 in FP32, x is an integer in
+// [0, 2^23) exactly when u lies in [2^23, 2^24) and u - 2^23 has x's bits; x is
+// then u's low 23 bits.  D cannot wrap below a total of 2^33 counts
+// (fix_result).  A row with any other value takes FP32 sums and their bound.
+// The integer sums do not depend on the order of the additions.
+struct FixSum {
+  long long D = 0;
+  uint32_t bad = 0u;   // non-zero: a value that is no count below 2^23
+};
+
+__device__ __forceinline__ void fix_add(FixSum& f, float x, int q) {
+  const float u = x + 8388608.f;
+  const uint32_t ub = __float_as_uint(u);
+  f.bad |= (__float_as_uint(u - 8388608.f) ^ __float_as_uint(x)) | ((ub & 0xFF800000u) ^ 0x4B000000u);
+  f.D += (long long)(int)(ub & 0x007FFFFFu) * (long long)q;
+}
+
+// Log-odds and bound of a row from its exact sum; T is the FP32 sum of the
+// counts.  The bound holds the quantisation of Delta (half a step per count)
+// and slack for the FP64 reference's own rounding; a total at which D could
+// have wrapped sends the row to FP64.
+__device__ __forceinline__ void fix_result(long long D, float T, const C2Header& h, float& d,
+                                           float& tau) {
+  const double step = __hiloint2double((1023 - h.S - 8) << 20, 0);   // 2^-(S+8)
+  d = (float)((double)D * step + h.b64);
+  T *= 1.001f;
+  tau = T < 4e9f ? 0.5f * T * (float)step * 1.0001f + 1e-12f * (T * h.maxabs + fabsf(h.b)) + 1e-30f
+                 : INFINITY;
+}
+
+// ---------------------------------------------------------------------------
 // FP8 E4M3 counts as exact integers
 // ---------------------------------------------------------------------------
 // Magic pair of a row with row scale 2^e: (M, M) in FP16, M = 2^(10 - e), for
@@ -269,21 +310,21 @@ __device__ __forceinline__ uint32_t fp8_lane_total(uint32_t tt, const Fp8Check& 
   return fp8_check_ok(c, m2) ? tt : 16777216u;
 }
 
-// Sums four int32 values over the LPR lanes of a lane group (LPR = 4 .. 32,
-// a power of two) with log2(LPR) + 1 shuffles instead of 4 log2(LPR): the
-// first two steps halve the set of values each lane carries.  Returns the lane's share: lanes [0, LPR/4) of
-// the group hold the sum of a0, then a1, a2 and a3 by quarter.  Integer sums
-// are exact, so the order does not matter.
-template <int LPR>
-__device__ __forceinline__ int sum4_transposed(int a0, int a1, int a2, int a3, int li) {
+// Sums four values over the LPR lanes of a lane group (LPR = 4 .. 32, a power
+// of two) with log2(LPR) + 1 shuffles instead of 4 log2(LPR): the first two
+// steps halve the set of values each lane carries.  Returns the lane's share:
+// lanes [0, LPR/4) of the group hold the sum of a0, then a1, a2 and a3 by
+// quarter.  Integer sums are exact, so the order does not matter.
+template <int LPR, typename T>
+__device__ __forceinline__ T sum4_transposed(T a0, T a1, T a2, T a3, int li) {
   const bool h1 = (li & (LPR / 2)) != 0;
-  int k0 = h1 ? a2 : a0, k1 = h1 ? a3 : a1;
-  const int s0 = h1 ? a0 : a2, s1 = h1 ? a1 : a3;
+  T k0 = h1 ? a2 : a0, k1 = h1 ? a3 : a1;
+  const T s0 = h1 ? a0 : a2, s1 = h1 ? a1 : a3;
   k0 += __shfl_xor_sync(0xFFFFFFFFu, s0, LPR / 2);
   k1 += __shfl_xor_sync(0xFFFFFFFFu, s1, LPR / 2);
   const bool h2 = (li & (LPR / 4)) != 0;
-  int k = h2 ? k1 : k0;
-  const int s = h2 ? k0 : k1;
+  T k = h2 ? k1 : k0;
+  const T s = h2 ? k0 : k1;
   k += __shfl_xor_sync(0xFFFFFFFFu, s, LPR / 4);
 #pragma unroll
   for (int off = LPR / 8; off > 0; off >>= 1) k += __shfl_xor_sync(0xFFFFFFFFu, k, off);
