@@ -32,8 +32,9 @@
 // C = 64, F = 256: re-fit on 64,000 rows (65.5 MB), scoring of 200,000 and
 // reading the parameters: 4.90 -> 0.84 ms, of which the fit was 3.45 ms of
 // device time with FP64 sums in shared memory, 32-row chunks (266 MB of
-// partials, mapped anew by every call) and a one-block finish; C = 2, F = 64,
-// 2,000 + 10,000 rows: 365 -> 136 us.
+// partials, mapped anew by every call) and a one-block finish, and is 0.12 ms
+// now (passes 34 and 42 us, reductions 7 and 15, finish 10, tensor-core tables
+// 16); C = 2, F = 64, 2,000 + 10,000 rows: 365 -> 136 us (fit 38).
 #include <math.h>
 
 #include "device.cuh"

@@ -20,7 +20,7 @@ namespace nbg {
 
 // FP64 tables of one model
 struct RModel {
-  int kind, C;
+  int C;
   const double* p0;       // log theta | mu
   const double* p1;       // var
   const double* log_pi;
@@ -31,7 +31,7 @@ struct RModel {
 struct RView {
   const char* X;
   int64_t ld;   // elements
-  int dtype, F;
+  int F;
   const int64_t* ovf_ptr;
   const uint16_t* ovf_col;
   const uint16_t* ovf_add;
@@ -42,72 +42,91 @@ struct RView {
   const int32_t* cols;   // feature j is stored column cols[j] (nullptr: column j)
 };
 
-__device__ __forceinline__ double load_x(int dtype, const char* rp, int j, double scale) {
-  switch (dtype) {
-    case NB_F32: return (double)reinterpret_cast<const float*>(rp)[j];
-    case NB_U16: return (double)reinterpret_cast<const uint16_t*>(rp)[j];
-    case NB_U8: return (double)reinterpret_cast<const uint8_t*>(rp)[j];
-    case NB_BF16: {
-      const uint32_t b = reinterpret_cast<const uint16_t*>(rp)[j];
-      return (double)__uint_as_float(b << 16);
+template <int DT>
+__device__ __forceinline__ double load_x(const char* rp, int j, double scale) {
+  if (DT == NB_F32) return (double)reinterpret_cast<const float*>(rp)[j];
+  if (DT == NB_U16) return (double)reinterpret_cast<const uint16_t*>(rp)[j];
+  if (DT == NB_U8) return (double)reinterpret_cast<const uint8_t*>(rp)[j];
+  if (DT == NB_BF16) {
+    const uint32_t b = reinterpret_cast<const uint16_t*>(rp)[j];
+    return (double)__uint_as_float(b << 16);
+  }
+  const uint16_t b = reinterpret_cast<const uint8_t*>(rp)[j];
+  return (double)e4m3x2_to_f32(b).x * scale;
+}
+
+// Sums of classes c0 .. c0 + nc - 1 (nc <= CB) over the features j = lane,
+// lane + 32, ... of one row, in ascending order per lane.  U features are
+// loaded at a time, then their CB table entries together: the loads, not the
+// FP64 additions, are what a marked row waits for (one feature at a time, 57
+// marked rows of 4,096 counts took 130 us).
+template <int DT, int KIND, int CB, int U>
+__device__ __forceinline__ void recheck_sums(const RView& v, const RModel& md, const char* rp,
+                                             double scale, int c0, int nc, double (&acc)[CB]) {
+  const int lane = threadIdx.x & 31, F = v.F;
+  const double* t0 = md.p0 + (int64_t)c0 * F;   // log theta | mu
+  const double* t1 = KIND == NB_GAUSSIAN ? md.p1 + (int64_t)c0 * F : nullptr;
+  for (int j0 = lane; j0 < F; j0 += 32 * U) {
+    double x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 32 * u;
+      x[u] = j < F ? load_x<DT>(rp, v.cols ? v.cols[j] : j, scale) : 0.0;
     }
-    default: {
-      const uint16_t b = reinterpret_cast<const uint8_t*>(rp)[j];
-      return (double)e4m3x2_to_f32(b).x * scale;
+    double w[U][CB], z[KIND == NB_GAUSSIAN ? U : 1][KIND == NB_GAUSSIAN ? CB : 1];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 32 * u;
+      // a zero count adds nothing to a multinomial score (log theta is finite
+      // for alpha > 0)
+      const bool need = j < F && (KIND == NB_GAUSSIAN || x[u] != 0.0);
+#pragma unroll
+      for (int k = 0; k < CB; ++k) {
+        w[u][k] = need && k < nc ? t0[(int64_t)k * F + j] : 0.0;
+        if (KIND == NB_GAUSSIAN) z[u][k] = need && k < nc ? t1[(int64_t)k * F + j] : 1.0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j0 + 32 * u >= F || (KIND == NB_MULTINOMIAL && x[u] == 0.0)) continue;
+#pragma unroll
+      for (int k = 0; k < CB; ++k) {
+        if (KIND == NB_MULTINOMIAL) {
+          acc[k] = fma(x[u], w[u][k], acc[k]);
+        } else {
+          const double dx = x[u] - w[u][k];
+          acc[k] += dx * dx / z[u][k];
+        }
+      }
     }
   }
 }
 
 // The whole warp recomputes row r of v with model md; lane 0 writes outputs.
-// Each lane sums its features j = lane, lane + 32, ... in ascending order for
-// eight classes at a time (the row's value loaded once for the eight, eight
-// independent FMA chains); a zero count adds nothing to a multinomial score
-// (log theta is finite for alpha > 0) and is skipped.  Per class the lane's
-// sum and the butterfly over the lanes are those of one class at a time.
+// The row's value is loaded once for CB classes; per class the lane's sum and
+// the butterfly over the lanes are those of one class at a time.
+template <int DT, int KIND, int CB, int U>
 __device__ __forceinline__ void recheck_row(const RView& v, const RModel& md, int64_t r,
                                             int want_lp, double* s_sh) {
   const int lane = threadIdx.x & 31;
-  const int es = v.dtype == NB_F32 ? 4 : ((v.dtype == NB_U16 || v.dtype == NB_BF16) ? 2 : 1);
+  constexpr int es = DT == NB_F32 ? 4 : ((DT == NB_U16 || DT == NB_BF16) ? 2 : 1);
   const char* rp = v.X + r * v.ld * es;
-  const double scale =
-      (v.dtype == NB_FP8E4M3 && v.row_exp) ? ldexp(1.0, (int)v.row_exp[r]) : 1.0;
-  constexpr int CB = 8;
+  const double scale = (DT == NB_FP8E4M3 && v.row_exp) ? ldexp(1.0, (int)v.row_exp[r]) : 1.0;
   for (int c0 = 0; c0 < md.C; c0 += CB) {
     const int nc = md.C - c0 < CB ? md.C - c0 : CB;
     double acc[CB];
 #pragma unroll
     for (int k = 0; k < CB; ++k) acc[k] = 0.0;
-    if (md.kind == NB_MULTINOMIAL) {
+    recheck_sums<DT, KIND, CB, U>(v, md, rp, scale, c0, nc, acc);
+    if (DT == NB_U8 && KIND == NB_MULTINOMIAL && v.ovf_ptr) {
       const double* lt = md.p0 + (int64_t)c0 * v.F;
-      for (int j = lane; j < v.F; j += 32) {
-        const double x = load_x(v.dtype, rp, v.cols ? v.cols[j] : j, scale);
-        if (x == 0.0) continue;
+      for (int64_t e = v.ovf_ptr[r] + lane; e < v.ovf_ptr[r + 1]; e += 32) {
+        const int j = v.ovf_col[e];
+        if (j >= v.F) continue;
+        const double add = (double)v.ovf_add[e];
 #pragma unroll
         for (int k = 0; k < CB; ++k)
-          if (k < nc) acc[k] = fma(x, lt[(int64_t)k * v.F + j], acc[k]);
-      }
-      if (v.dtype == NB_U8 && v.ovf_ptr) {
-        for (int64_t e = v.ovf_ptr[r] + lane; e < v.ovf_ptr[r + 1]; e += 32) {
-          const int j = v.ovf_col[e];
-          if (j >= v.F) continue;
-          const double add = (double)v.ovf_add[e];
-#pragma unroll
-          for (int k = 0; k < CB; ++k)
-            if (k < nc) acc[k] = fma(add, lt[(int64_t)k * v.F + j], acc[k]);
-        }
-      }
-    } else {
-      const double* mu = md.p0 + (int64_t)c0 * v.F;
-      const double* var = md.p1 + (int64_t)c0 * v.F;
-      for (int j = lane; j < v.F; j += 32) {
-        const double x = load_x(v.dtype, rp, j, scale);
-#pragma unroll
-        for (int k = 0; k < CB; ++k) {
-          if (k < nc) {
-            const double dx = x - mu[(int64_t)k * v.F + j];
-            acc[k] += dx * dx / var[(int64_t)k * v.F + j];
-          }
-        }
+          if (k < nc) acc[k] = fma(add, lt[(int64_t)k * v.F + j], acc[k]);
       }
     }
 #pragma unroll
@@ -120,26 +139,51 @@ __device__ __forceinline__ void recheck_row(const RView& v, const RModel& md, in
       for (int k = 0; k < CB; ++k) {
         const int c = c0 + k;
         if (k < nc)
-          s_sh[c] = md.kind == NB_MULTINOMIAL ? md.log_pi[c] + acc[k] : md.gconst[c] - 0.5 * acc[k];
+          s_sh[c] = KIND == NB_MULTINOMIAL ? md.log_pi[c] + acc[k] : md.gconst[c] - 0.5 * acc[k];
       }
     }
   }
   __syncwarp();
-  if (lane == 0) {
-    int best = 0;
-    for (int c = 1; c < md.C; ++c)
-      if (s_sh[c] > s_sh[best]) best = c;
-    double second = -INFINITY;
-    for (int c = 0; c < md.C; ++c)
-      if (c != best && s_sh[c] > second) second = s_sh[c];
-    v.label[r] = (uint8_t)best;
-    v.margin[r] = (float)(s_sh[best] - second);
-    if (want_lp) {
-      double sum = 0.0;
-      for (int c = 0; c < md.C; ++c) sum += exp(s_sh[c] - s_sh[best]);
-      const double lse = s_sh[best] + log(sum);
-      for (int c = 0; c < md.C; ++c) v.logpost[r * md.C + c] = (float)(s_sh[c] - lse);
+  // the lanes share the classes: arg-max (lowest index among the maxima; class
+  // 0 when its score is NaN or none is a number), second best, log-sum-exp (an
+  // FP64 exponential per class: one lane alone took them one after another)
+  double b = -INFINITY;
+  int best = 0x7FFFFFFF;
+  for (int c = lane; c < md.C; c += 32) {
+    const double sc = s_sh[c];
+    if (sc > b || (sc == b && c < best)) {
+      b = sc;
+      best = c;
     }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const double ob = __shfl_xor_sync(0xFFFFFFFFu, b, off);
+    const int oi = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+    if (ob > b || (ob == b && oi < best)) {
+      b = ob;
+      best = oi;
+    }
+  }
+  if (best >= md.C || s_sh[0] != s_sh[0]) best = 0;
+  const double sb = s_sh[best];
+  double second = -INFINITY, sum = 0.0;
+  for (int c = lane; c < md.C; c += 32) {
+    if (c != best && s_sh[c] > second) second = s_sh[c];
+    if (want_lp) sum += exp(s_sh[c] - sb);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    second = fmax(second, __shfl_xor_sync(0xFFFFFFFFu, second, off));
+    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+  }
+  if (lane == 0) {
+    v.label[r] = (uint8_t)best;
+    v.margin[r] = (float)(sb - second);
+  }
+  if (want_lp) {
+    const double lse = sb + log(sum);
+    for (int c = lane; c < md.C; c += 32) v.logpost[r * md.C + c] = (float)(s_sh[c] - lse);
   }
   __syncwarp();
 }
@@ -154,6 +198,8 @@ struct RArgs {
   unsigned long long* n_rechecked;
 };
 
+// CB classes and U features in flight: 16 table entries per lane either way.
+template <int DT, int KIND, int CB>
 __global__ void __launch_bounds__(256) k_recheck(const RArgs a) {
   __shared__ double s_sh[8][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -172,11 +218,27 @@ __global__ void __launch_bounds__(256) k_recheck(const RArgs a) {
     while (m) {
       const int src = __ffs(m) - 1;
       m &= m - 1;
-      recheck_row(a.v, a.md, base + src, a.want_lp, s_sh[warp]);
+      recheck_row<DT, KIND, CB, 16 / CB>(a.v, a.md, base + src, a.want_lp, s_sh[warp]);
       ++cnt;
     }
   }
   if (lane == 0 && cnt && a.n_rechecked && !a.counted) atomicAdd(a.n_rechecked, cnt);
+}
+
+using RKernel = void (*)(RArgs);
+template <int DT>
+static RKernel recheck_kernel(int C) {
+  return C == 2 ? (RKernel)k_recheck<DT, NB_MULTINOMIAL, 2> : (RKernel)k_recheck<DT, NB_MULTINOMIAL, 8>;
+}
+static RKernel recheck_kernel(nb_kind kind, nb_dtype dt, int C) {
+  if (kind == NB_GAUSSIAN) return k_recheck<NB_F32, NB_GAUSSIAN, 4>;
+  switch (dt) {
+    case NB_U8: return recheck_kernel<NB_U8>(C);
+    case NB_U16: return recheck_kernel<NB_U16>(C);
+    case NB_F32: return recheck_kernel<NB_F32>(C);
+    case NB_BF16: return recheck_kernel<NB_BF16>(C);
+    default: return recheck_kernel<NB_FP8E4M3>(C);
+  }
 }
 
 nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
@@ -187,7 +249,6 @@ nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t 
   RArgs a{};
   a.v.X = static_cast<const char*>(X);
   a.v.ld = ld;
-  a.v.dtype = dt;
   a.v.F = m->F;
   a.v.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
   a.v.ovf_col = aux ? aux->ovf_col : nullptr;
@@ -196,7 +257,7 @@ nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t 
   a.v.label = o.label;
   a.v.margin = o.margin;
   a.v.logpost = o.logpost;
-  a.md = RModel{m->kind, m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
+  a.md = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
   a.n = n;
   a.want_lp = o.want_lp;
   a.counted = o.counted ? 1 : 0;
@@ -209,7 +270,7 @@ nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t 
   a.rows = rows;
   const int64_t blocks = ((n + rows - 1) / rows + 7) / 8;
   count_launch();
-  NB_TRY_CUDA(launch_pdl(k_recheck, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0,
+  NB_TRY_CUDA(launch_pdl(recheck_kernel(m->kind, dt, m->C), dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0,
                          st, a),
               "k_recheck launch");
   return NB_OK;
@@ -223,10 +284,11 @@ struct RSegArgs {
   const SegGroup* groups;
   const SegHeader* hdr;
   RModel md[kSegMaxModels];
-  int dtype, F, want_lp;
+  int F, want_lp;
   unsigned long long* n_rechecked;
 };
 
+template <int DT, int CB>
 __global__ void __launch_bounds__(256) k_recheck_seg(const RSegArgs a) {
   __shared__ double s_sh[8][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -249,9 +311,8 @@ __global__ void __launch_bounds__(256) k_recheck_seg(const RSegArgs a) {
     RView v;
     v.cols = nullptr;
     v.X = G.X;
-    v.dtype = a.dtype;
     v.F = a.F;
-    const int es = a.dtype == NB_F32 ? 4 : ((a.dtype == NB_U16 || a.dtype == NB_BF16) ? 2 : 1);
+    constexpr int es = DT == NB_F32 ? 4 : ((DT == NB_U16 || DT == NB_BF16) ? 2 : 1);
     v.ld = G.ld_bytes / es;
     v.ovf_ptr = G.ovf_ptr;
     v.ovf_col = G.ovf_col;
@@ -263,11 +324,18 @@ __global__ void __launch_bounds__(256) k_recheck_seg(const RSegArgs a) {
     while (m) {
       const int src = __ffs(m) - 1;
       m &= m - 1;
-      recheck_row(v, a.md[G.model], base + src, a.want_lp, s_sh[warp]);
+      recheck_row<DT, NB_MULTINOMIAL, CB, 16 / CB>(v, a.md[G.model], base + src, a.want_lp,
+                                                  s_sh[warp]);
       ++cnt;
     }
   }
   if (lane == 0 && cnt && a.n_rechecked) atomicAdd(a.n_rechecked, cnt);
+}
+
+using RSegKernel = void (*)(RSegArgs);
+template <int DT>
+static RSegKernel recheck_seg_kernel(bool two) {
+  return two ? (RSegKernel)k_recheck_seg<DT, 2> : (RSegKernel)k_recheck_seg<DT, 8>;
 }
 
 nb_status launch_recheck_seg(const SegGroup* groups, const SegHeader* hdr,
@@ -278,14 +346,19 @@ nb_status launch_recheck_seg(const SegGroup* groups, const SegHeader* hdr,
   a.hdr = hdr;
   for (int i = 0; i < n_models && i < kSegMaxModels; ++i) {
     const nb_model* m = models[i];
-    a.md[i] = RModel{m->kind, m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
+    a.md[i] = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
   }
-  a.dtype = dt;
   a.F = F;
   a.want_lp = want_lp;
   a.n_rechecked = reinterpret_cast<unsigned long long*>(n_rechecked);
+  const bool two = models[0]->C == 2;   // the two-class list holds nothing else
+  const RSegKernel k = dt == NB_U8     ? recheck_seg_kernel<NB_U8>(two)
+                       : dt == NB_F32  ? recheck_seg_kernel<NB_F32>(two)
+                       : dt == NB_U16  ? recheck_seg_kernel<NB_U16>(two)
+                       : dt == NB_BF16 ? recheck_seg_kernel<NB_BF16>(two)
+                                       : recheck_seg_kernel<NB_FP8E4M3>(two);
   count_launch();
-  k_recheck_seg<<<num_sms() * 4, 256, 0, st>>>(a);
+  k<<<num_sms() * 4, 256, 0, st>>>(a);
   NB_TRY_CUDA(cudaGetLastError(), "k_recheck_seg launch");
   return NB_OK;
 }
@@ -340,7 +413,6 @@ __global__ void __launch_bounds__(256) k_recheck_gw(const RGwArgs a) {
       RView v;
       v.X = reinterpret_cast<const char*>(a.X);
       v.ld = a.ld;
-      v.dtype = NB_U8;
       v.F = a.k;
       v.ovf_ptr = nullptr;
       v.ovf_col = nullptr;
@@ -350,7 +422,7 @@ __global__ void __launch_bounds__(256) k_recheck_gw(const RGwArgs a) {
       v.margin = a.margin;
       v.logpost = a.logpost;
       v.cols = a.cols + (int64_t)g * a.k;
-      recheck_row(v, a.md[g], r, a.want_lp, s_sh[warp]);
+      recheck_row<NB_U8, NB_MULTINOMIAL, 2, 8>(v, a.md[g], r, a.want_lp, s_sh[warp]);
       ++cnt;
     }
   }
@@ -375,7 +447,7 @@ nb_status launch_recheck_gw(const unsigned char* X, int64_t ld, int64_t n, const
   a.cols = cols;
   for (int i = 0; i < n_models && i < kSegMaxModels; ++i) {
     const nb_model* m = models[i];
-    a.md[i] = RModel{m->kind, m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
+    a.md[i] = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
   }
   a.label = label;
   a.margin = margin;

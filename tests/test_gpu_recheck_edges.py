@@ -1,0 +1,35 @@
+"""The FP64 recheck at the edges of its feature batches and class blocks, and FP8
+rows narrower than a lane group.
+
+Files of all classes come from one profile, so that margins are tiny and the
+scorers mark most rows; the rechecked rows must match the FP64 oracle (labels
+equal, log posteriors within 1e-5).  A warp takes 32 x 8 features of two classes
+or 32 x 2 of eight at a time.
+"""
+import numpy as np
+import pytest
+import torch
+
+from _common import compare, count_matrix, oracle_mn, stored, to_np
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+nb = pytest.importorskip("paper_1905_13746_gb300")
+
+
+@pytest.mark.parametrize("fmt", ["u8ovf", "u16", "f32", "bf16", "fp8"])
+@pytest.mark.parametrize("C,F", [(2, 1), (2, 33), (2, 255), (2, 257), (2, 1000), (3, 63), (9, 65),
+                                 (33, 100), (70, 40)])
+def test_near_ties_of_one_profile(fmt, C, F):
+    p = np.repeat(synth.dirichlet_profiles(5, 1, F, 2.0), C, axis=0)
+    n = 40 * C + 400
+    labels = (np.arange(n) % C).astype(np.int32)
+    X, y, _ = count_matrix(17 + F, n, F, C=C, mu=4.0, sigma=1.0, p=p, labels=labels,
+                           clip=16 if fmt == "fp8" else 255)
+    f, vals = stored(X, fmt)
+    model = nb.fit(f, torch.from_numpy(y).cuda(), C)
+    res = to_np(nb.score(model, f))
+    _, ref = oracle_mn(vals, y, C, vals)
+    compare(res, ref)
