@@ -127,8 +127,10 @@ typedef struct nb_model nb_model;
 typedef struct nb_server nb_server;
 
 /* Kernel configuration of a model's scorer.
- *   variant  two classes: NB_VARIANT_AUTO: TMA-pipelined kernel when the row
- *            fits a stage, else the register-streaming kernel;
+ *   variant  two classes: NB_VARIANT_AUTO: the TMA-pipelined kernel when the
+ *            row fits a stage, else the register-streaming kernel; U8 and
+ *            FP8E4M3 rows, whose results no shape changes, take the one that
+ *            measured faster for their width unless a stage shape is given;
  *            NB_VARIANT_PIPELINED / NB_VARIANT_REGISTER: force one.
  *            3..64 classes with U8, FP8E4M3 or BF16 storage, X 16-byte
  *            aligned and ld * element size a multiple of 16:

@@ -624,7 +624,8 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
   a.status = m->d.sstatus;
   int smem;
-  if (dt == NB_U8 || dt == NB_FP8E4M3) {   // fixed-point limbs, exact sums
+  const bool limbs = dt == NB_U8 || dt == NB_FP8E4M3;   // fixed-point limbs, exact sums
+  if (limbs) {
     a.nvec_tab = m->nvec8;
     a.table = m->d.limbs;
     smem = 3 * m->nvec8 * 16;
@@ -662,8 +663,33 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
     a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row
     return dt == NB_U16 ? launch_fix<NB_U16>(a, smem, st) : launch_fix<NB_BF16>(a, smem, st);
   }
+  // u8 and FP8 rows: the sums are exact, so the kernel and its shape change no
+  // result, and the faster one is taken where none is asked for.  Dense rows
+  // stream through registers: over F = 64 .. 6,000 that is the fastest or
+  // within 4% of it (u8, against the pipelined kernel's default shape: 1M files
+  // of F = 64 24 / 121 us, 256 56 / 162, 512 90 / 147; 586,000 of 1,024
+  // 102 / 106; 293,000 of 2,048 102 / 139; FP8: 36 / 225, 90 / 231, 167 / 248,
+  // 198 / 207, 195 / 238).  With an overflow list the pipelined kernel, whose
+  // producer fetches the entries ahead, wins where the row fills its lanes:
+  // 16 vectors (two rows per pass: F = 256 127 against 143 us), 32 (512:
+  // 163 / 173), 52 to 64 (two rows: 900 148 / 165, 1,024 116 / 143) and up to
+  // 128 (1,500 143 / 150, 2,048 103 / 118); elsewhere registers (F = 64
+  // 48 / 225, 384 158 / 225, 640 192 / 225, 3,072 117 us).  The default shape
+  // took 226 us at F = 256, 144 at 1,024 and 146 at 2,048.  Two stages of 48 rows; shorter ones while the call has fewer than
+  // three tiles per block.
   const nb_tile_config& cfg = m->tile;
-  if (cfg.variant != NB_VARIANT_REGISTER) {
+  nb_tile_config shape = cfg;
+  bool pipe = cfg.variant != NB_VARIANT_REGISTER;
+  if (limbs && cfg.variant == NB_VARIANT_AUTO && cfg.stages == 0 && cfg.rows_per_stage == 0 &&
+      cfg.rows_per_warp == 0) {
+    const int nv = a.nvec_row;
+    pipe = a.ovf_ptr != nullptr && (nv == 16 || nv == 32 || (nv >= 52 && nv <= 128));
+    shape.rows_per_warp = nv == 16 || (nv > 32 && nv <= 64) ? 2 : 1;
+    shape.stages = 2;
+    const int64_t blocks = (int64_t)num_sms() * 2;
+    shape.rows_per_stage = n >= 3 * 48 * blocks ? 48 : (n >= 3 * 24 * blocks ? 24 : 16);
+  }
+  if (pipe) {
     // overflow slices are staged by bulk copies only from 16-byte aligned arrays
     S2Args ap = a;
     const int epv = 16 / es;
@@ -671,12 +697,11 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
     const bool side_ok = !a.ovf_ptr || ((reinterpret_cast<uintptr_t>(a.ovf_col) & 15) == 0 &&
                                         (reinterpret_cast<uintptr_t>(a.ovf_add) & 15) == 0);
     const nb_status s =
-        launch_score2_pipe(ap, dt, cfg.stages, cfg.rows_per_stage, cfg.rows_per_warp,
+        launch_score2_pipe(ap, dt, shape.stages, shape.rows_per_stage, shape.rows_per_warp,
                            side_ok ? 1 : 0, st);
     if (s != NB_EUNSUPPORTED || cfg.variant == NB_VARIANT_PIPELINED) return s;
   }
-  const int lpr = (dt == NB_U8 || dt == NB_FP8E4M3) ? pick_lpr_u8(a.nvec_row)
-                                                    : pick_lpr(a.nvec_row);
+  const int lpr = limbs ? pick_lpr_u8(a.nvec_row) : pick_lpr(a.nvec_row);
   {
     const int epv = 16 / es;
     const int per_lane = (a.nvec_row + lpr - 1) / lpr;

@@ -305,9 +305,12 @@ __device__ __forceinline__ int limb_byte_sum(const uint4& q) {
 }
 
 // The lane's count total, or 2^24 when one of its values failed the check
-// (which sends the row to the FP64 recheck, see c2_tau_u8).
+// (which sends the row to the FP64 recheck, see c2_tau_u8).  A lane that read
+// no vector (rows narrower than the lane group) has nothing to fail: without
+// that case every row of fewer than 32 vectors went to FP64 from the pipelined
+// kernel (1M files of F = 256: 13.3 ms).
 __device__ __forceinline__ uint32_t fp8_lane_total(uint32_t tt, const Fp8Check& c, uint32_t m2) {
-  return fp8_check_ok(c, m2) ? tt : 16777216u;
+  return fp8_check_ok(c, m2) || (c.orv == 0u && c.andv == 0xFFFFFFFFu) ? tt : 16777216u;
 }
 
 // Sums four values over the LPR lanes of a lane group (LPR = 4 .. 32, a power

@@ -33,3 +33,18 @@ def test_near_ties_of_one_profile(fmt, C, F):
     res = to_np(nb.score(model, f))
     _, ref = oracle_mn(vals, y, C, vals)
     compare(res, ref)
+
+
+@pytest.mark.parametrize("F", [5, 16, 17, 64, 100, 256, 384, 500])
+def test_narrow_fp8_rows_of_counts_need_no_recheck(F):
+    """Lanes without a vector of their own do not send a row to FP64."""
+    X, y, _ = count_matrix(50 + F, 800, F, clip=16)
+    f, vals = stored(X, "fp8")
+    model = nb.fit(f, torch.from_numpy(y).cuda(), 2)
+    _, ref = oracle_mn(vals, y, 2, vals)
+    for cfg in [(nb.NB_VARIANT_AUTO, 0, 0, 0), (nb.NB_VARIANT_PIPELINED, 2, 16, 1),
+                (nb.NB_VARIANT_PIPELINED, 2, 16, 2), (nb.NB_VARIANT_REGISTER, 0, 0, 0)]:
+        model.set_tile_config(*cfg)
+        res = to_np(nb.score(model, f, recheck=nb.NB_RECHECK_OFF))
+        assert res["n_rechecked"] == 0, cfg     # no row the fast path cannot compute
+        compare(to_np(nb.score(model, f)), ref)
