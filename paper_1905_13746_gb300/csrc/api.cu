@@ -83,6 +83,7 @@ static nb_status alloc_model(nb_model* m) {
   const size_t o_tcw = take(tc ? tc_w_bytes(m->C, m->F) : 0);
   const size_t o_tcq = take(tc ? sizeof(int32_t) * C * F : 0);
   const size_t o_tch = take(tc ? sizeof(TcHeader) : 0);
+  const size_t o_wm = take(tc ? sizeof(double) * F : 0);
   const bool tg = tcg_tables(m->kind, m->C, m->F);
   const int F8 = (m->F + kTcgFS - 1) / kTcgFS * kTcgFS;
   const size_t o_tgw = take(tg ? tcg_w_bytes(m->C, m->F) : 0);
@@ -124,6 +125,7 @@ static nb_status alloc_model(nb_model* m) {
   d.tc_w = tc ? reinterpret_cast<uint8_t*>(b + o_tcw) : nullptr;
   d.tc_q = tc ? reinterpret_cast<int32_t*>(b + o_tcq) : nullptr;
   d.tc_hdr = tc ? reinterpret_cast<TcHeader*>(b + o_tch) : nullptr;
+  d.wmean = tc ? reinterpret_cast<double*>(b + o_wm) : nullptr;
   if (tg) d.tc_w = reinterpret_cast<uint8_t*>(b + o_tgw);
   d.tcg_kc = tg ? reinterpret_cast<float*>(b + o_tgk) : nullptr;
   d.tcg_ctr = tg ? reinterpret_cast<float*>(b + o_tgc) : nullptr;

@@ -5,16 +5,21 @@
 //   N_cj = sum_{i : y_i = c} x_ij          exact, uint64
 //   log theta_cj = log(N_cj + alpha) - log(N_c + alpha F)       FP64
 //   log pi_c = log n_c - log n  (or the supplied log prior)     FP64
-// The count reduction first buckets the row indices by class, so that a warp
-// sums runs of rows of one class in registers and adds each feature's total
-// to N_cj with one 64-bit atomic per run; integer sums do not depend on the
-// order of the additions, so the counts are exact and reproducible.
+// The counts come from fit2.cu (two classes) or counts_rows.cu (any class
+// count).  What those do not take -- more classes
+// than the shared memory of an SM holds sums for, rows that start between
+// 4-byte words, or NB_VARIANT_REGISTER -- is counted here: the row indices are
+// bucketed by class, a warp sums runs of rows of one class in registers and
+// adds each feature's total to N_cj with one 64-bit atomic per run.  Integer
+// sums do not depend on the order of the additions, so the counts are exact
+// and reproducible.
 // The Gaussian fit is in gauss_fit.cu.
 #include <cuda_fp16.h>
 #include <math.h>
 
 #include "device.cuh"
 #include "internal.cuh"
+#include "log64.cuh"
 
 namespace nbg {
 
@@ -366,34 +371,33 @@ __global__ void k_counts_ovf(const int64_t* ptr, const uint16_t* col, const uint
 }
 
 // ---------------------------------------------------------------------------
-// FP64 finalize of the general-C tables
+// General-C finish (Sec. 4 likelihoods, Laplace smoothing)
 // ---------------------------------------------------------------------------
-// General-C finish (Sec. 4 likelihoods, Laplace smoothing): block (c, t)
-// writes log theta_cj for the kFinTile features of tile t.  Every block sums
-// the class total N_c from the exact counts (they sit in L2) and one thread
-// takes log(N_c + alpha F): FP64 is slow on this part, so the per-feature
-// logs are spread over C * F / kFinTile blocks rather than C.
-constexpr int kFinTile = 512;
-
-__global__ void __launch_bounds__(256) k_finalize_mn(const unsigned long long* counts,
-                                                     const unsigned long long* nc, int64_t n,
-                                                     int F, double alpha, int prior_given,
-                                                     double* log_theta, double* log_pi,
-                                                     int* status) {
+// Class totals: block c sums N_c from the exact counts and takes
+// log(N_c + alpha F) into log_den[c], and log pi_c.
+__global__ void __launch_bounds__(256) k_class_totals(const unsigned long long* counts,
+                                                      const unsigned long long* nc, int64_t n,
+                                                      int F, double alpha, int prior_given,
+                                                      double* log_den, double* log_pi, float* bias,
+                                                      float* wmax, int* status) {
   const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ unsigned long long part[8];
-  __shared__ double log_den;
+  pdl_wait();
   unsigned long long s = 0;
-  for (int j = tid; j < F; j += blockDim.x) s += counts[(int64_t)c * F + j];
+#pragma unroll 8
+  for (int j = tid; j < F; j += 256) s += counts[(int64_t)c * F + j];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
   if (lane == 0) part[warp] = s;
   __syncthreads();
   if (tid == 0) {
     unsigned long long t = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += part[k];
-    log_den = log((double)t + alpha * (double)F);
-    if (blockIdx.y == 0 && !prior_given) {
+    for (int k = 0; k < 8; ++k) t += part[k];
+    log_den[c] = log((double)t + alpha * (double)F);
+    if (c == 0) *wmax = 0.f;
+  }
+  if (tid == 32) {
+    if (!prior_given) {
       if (nc[c] == 0) {
         atomicOr(status, ST_BAD_LABEL);
         log_pi[c] = 0.0;
@@ -401,12 +405,65 @@ __global__ void __launch_bounds__(256) k_finalize_mn(const unsigned long long* c
         log_pi[c] = log((double)nc[c]) - log((double)n);
       }
     }
+    bias[c] = (float)log_pi[c];
   }
+}
+
+// Tables of 32 features and all classes per block (lane: feature; each warp
+// every eighth class): log theta_cj, the mean over the classes, the centred
+// FP32 weights w_cj = log theta_cj - mean_c log theta_cj (the class-independent
+// shift cancels in the margin and the log posterior) and max |w|.  FP64 bounds
+// it, hence log64 (log64.cuh), and one kernel for log theta and weights.
+// C = 64, F = 8,192: totals 7, this kernel 28 and the tensor-core tables 9 us;
+// log theta, weights and tensor-core tables in kernels of their own took 52, 28
+// and 37 us (FP64 logarithms in the first, 8,192 threads in the others).
+__global__ void __launch_bounds__(256) k_finish_mn(const unsigned long long* counts, int C, int F,
+                                                   int F_pad, double alpha, const double* log_den,
+                                                   double* log_theta, double* wmean, float* w,
+                                                   float* wmax, int* status) {
+  extern __shared__ __align__(16) double lt[];   // [C][32]
+  __shared__ double sum[8][32];
+  __shared__ float red[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = blockIdx.x * 32 + lane;
+  pdl_wait();
+  double s = 0.0;
+  if (j < F) {
+#pragma unroll 4
+    for (int c = warp; c < C; c += 8) {
+      const int64_t at = (int64_t)c * F + j;
+      const double v = log64((double)counts[at] + alpha) - log_den[c];
+      log_theta[at] = v;
+      lt[c * 32 + lane] = v;
+      s += v;
+    }
+  }
+  sum[warp][lane] = s;
   __syncthreads();
-  const int j0 = blockIdx.y * kFinTile;
-  const int j1 = min(F, j0 + kFinTile);
-  for (int j = j0 + tid; j < j1; j += blockDim.x)
-    log_theta[(int64_t)c * F + j] = log((double)counts[(int64_t)c * F + j] + alpha) - log_den;
+  double m = 0.0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) m += sum[k][lane];
+  m /= (double)C;
+  if (warp == 0 && j < F && wmean) wmean[j] = m;
+  float mx = 0.f;
+  for (int c = warp; c < C; c += 8) {
+    float v32 = 0.f;
+    if (j < F) {
+      const double v = lt[c * 32 + lane] - m;
+      if (!isfinite(v)) atomicOr(status, ST_BAD_TABLE);
+      v32 = (float)v;
+    }
+    w[(int64_t)c * F_pad + j] = v32;   // F_pad is a multiple of 32
+    mx = fmaxf(mx, fabsf(v32));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+  if (lane == 0) red[warp] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) mx = fmaxf(mx, red[k]);
+    atomicMax(reinterpret_cast<int*>(wmax), __float_as_int(mx));   // non-negative: ordered as ints
+  }
 }
 
 // Two-class finish of the fit in one launch (Sec. 4 likelihoods, Laplace
@@ -605,41 +662,6 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
   }
 }
 
-// general-C tables: w_cj = log theta_cj - mean_c log theta_cj (FP32), bias_c =
-// log pi_c (FP32), wmax = max |w|.  The class-independent shift cancels in
-// the margin and the log posterior.
-__global__ void k_derive_general(const double* log_theta, const double* log_pi, int C, int F,
-                                 int F_pad, float* w, float* bias, float* wmax, int* status) {
-  float mx = 0.f;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < F_pad; j += gridDim.x * blockDim.x) {
-    if (j >= F) {
-      for (int c = 0; c < C; ++c) w[(int64_t)c * F_pad + j] = 0.f;
-      continue;
-    }
-    double m = 0.0;
-    for (int c = 0; c < C; ++c) m += log_theta[(int64_t)c * F + j];
-    m /= (double)C;
-    for (int c = 0; c < C; ++c) {
-      const double v = log_theta[(int64_t)c * F + j] - m;
-      if (!isfinite(v)) atomicOr(status, ST_BAD_TABLE);
-      const float v32 = (float)v;
-      w[(int64_t)c * F_pad + j] = v32;
-      mx = fmaxf(mx, fabsf(v32));
-    }
-  }
-  // block max then one atomic (non-negative floats compare as ints)
-  __shared__ float red[256];
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicMax(reinterpret_cast<int*>(wmax), __float_as_int(red[0]));
-  if (blockIdx.x == 0)
-    for (int c = threadIdx.x; c < C; c += blockDim.x) bias[c] = (float)log_pi[c];
-}
-
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -679,7 +701,13 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
   if (C == 2 && m->tile.variant != NB_VARIANT_REGISTER)
     piped = launch_fit2_pipe(m, X, dt, n, ld, y, aux, st);
   if (piped != NB_OK && piped != NB_EUNSUPPORTED) return piped;
-  if (n > 0 && piped != NB_OK) {
+  bool rows = false;   // counted by k_counts_rows: the overflow list is still to be added
+  if (n > 0 && piped != NB_OK && m->tile.variant != NB_VARIANT_REGISTER) {
+    const nb_status s = launch_counts_rows(m, X, dt, n, ld, y, aux, st);
+    if (s != NB_OK && s != NB_EUNSUPPORTED) return s;
+    rows = s == NB_OK;
+  }
+  if (n > 0 && piped != NB_OK && !rows) {
     const long long g = (n + 255) / 256;
     const unsigned hb = (unsigned)(g < sms * 4 ? g : sms * 4);
     count_launch();
@@ -689,9 +717,10 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
 
     // scratch: offsets, cursors, run bases, bucketed row indices
     const size_t small = sizeof(long long) * (size_t)(C + 1) * 3;
+    FitScratch fs(m, st);
     void* scratch = nullptr;
-    NB_TRY_CUDA(cudaMallocAsync(&scratch, small + sizeof(int32_t) * (size_t)n, st),
-                "cudaMallocAsync(fit scratch)");
+    const nb_status ss = fs.take(small + sizeof(int32_t) * (size_t)n, &scratch);
+    if (ss != NB_OK) return ss;
     long long* offs = static_cast<long long*>(scratch);
     unsigned long long* cursor = reinterpret_cast<unsigned long long*>(offs + (C + 1));
     long long* item_base = offs + 2 * (C + 1);
@@ -740,11 +769,11 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
       case NB_BF16: s = run_counts<NB_BF16>(a, nwork, st); break;
       case NB_FP8E4M3: s = run_counts<NB_FP8E4M3>(a, nwork, st); break;
     }
-    if (s != NB_OK) {
-      cudaFreeAsync(scratch, st);
-      return s;
-    }
-    NB_TRY_CUDA(cudaFreeAsync(scratch, st), "cudaFreeAsync(fit scratch)");
+    if (s != NB_OK) return s;
+    s = fs.release();
+    if (s != NB_OK) return s;
+  }
+  if (n > 0 && piped != NB_OK) {
     if (dt == NB_U8 && aux && aux->ovf_ptr) {
       const size_t bins = sizeof(unsigned int) * (size_t)C * F;
       const int use_smem = bins <= 96 * 1024;
@@ -776,18 +805,21 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
     return NB_OK;
   }
   count_launch();
-  k_finalize_mn<<<dim3(C, (F + kFinTile - 1) / kFinTile), 256, 0, st>>>(
-      reinterpret_cast<unsigned long long*>(d.counts), reinterpret_cast<unsigned long long*>(d.nc),
-      n, F, m->alpha, log_prior_dev != nullptr, d.p0, d.log_pi, d.status);
-  NB_TRY_CUDA(cudaGetLastError(), "k_finalize_mn");
-  NB_TRY_CUDA(cudaMemsetAsync(d.wmax, 0, sizeof(float), st), "memset");
-  {
-    const int blocks = (m->F_pad + 255) / 256;
-    count_launch();
-    k_derive_general<<<blocks < 1024 ? blocks : 1024, 256, 0, st>>>(
-        d.p0, d.log_pi, C, F, m->F_pad, d.w, d.bias, d.wmax, d.status);
-    NB_TRY_CUDA(cudaGetLastError(), "k_derive_general");
-  }
+  NB_TRY_CUDA(launch_pdl(k_class_totals, dim3((unsigned)C), dim3(256), 0, st,
+                         reinterpret_cast<const unsigned long long*>(d.counts),
+                         reinterpret_cast<const unsigned long long*>(d.nc), (int64_t)n, F, m->alpha,
+                         (int)(log_prior_dev != nullptr), d.gconst, d.log_pi, d.bias, d.wmax,
+                         d.status),
+              "k_class_totals");
+  const int smem = (int)(sizeof(double) * 32 * C);
+  if (smem > kSmemOptIn)
+    NB_TRY_CUDA(cudaFuncSetAttribute(k_finish_mn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                "cudaFuncSetAttribute(k_finish_mn)");
+  count_launch();
+  NB_TRY_CUDA(launch_pdl(k_finish_mn, dim3((unsigned)(m->F_pad / 32)), dim3(256), (size_t)smem, st,
+                         reinterpret_cast<const unsigned long long*>(d.counts), C, F, m->F_pad,
+                         m->alpha, (const double*)d.gconst, d.p0, d.wmean, d.w, d.wmax, d.status),
+              "k_finish_mn");
   if (d.tc_w) return launch_derive_tc(m, st);
   return NB_OK;
 }

@@ -95,7 +95,8 @@ struct ModelDev {
   double* p0;          // C x F      log theta (multinomial) | mu (Gaussian)
   double* p1;          // C x F      var (Gaussian)
   double* log_pi;      // C
-  double* gconst;      // C          Gaussian: log pi_c - 1/2 sum_j log(2 pi var_cj)
+  double* gconst;      // C          Gaussian: log pi_c - 1/2 sum_j log(2 pi var_cj);
+                       //            multinomial: log(N_c + alpha F)
   int* status;         // 1 int: ST_* bits raised while fitting (cleared by each fit)
   int* sstatus;        // 1 int: ST_* bits raised by scoring calls (kept until
                        // nb_model_check reports them)
@@ -116,6 +117,7 @@ struct ModelDev {
   uint8_t* tc_w;       // ceil(F/64) stages x 3*Cp x 64 FP16 limbs (MMA operand layout)
   int32_t* tc_q;       // C x F fixed-point weights
   TcHeader* tc_hdr;    // 1
+  double* wmean;       // F          mean_c log theta_cj
   // Gaussian FP32 tables
   float* g_mu;         // F_pad x gauss_cpad(C), feature-major (classes past C: 0)
   float* g_ivar;       // same layout, 1 / var
@@ -200,6 +202,8 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt,
                         const ScoreOut& o, cudaStream_t st);
 nb_status launch_fit2_pipe(nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                            const int32_t* y, const nb_aux* aux, cudaStream_t st);
+nb_status launch_counts_rows(nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
+                             const int32_t* y, const nb_aux* aux, cudaStream_t st);
 struct S2Args;
 nb_status launch_score2_pipe(const S2Args& a, nb_dtype dt, int stages, int rows_per_stage,
                              int rows_per_warp, int stage_entries, cudaStream_t st);

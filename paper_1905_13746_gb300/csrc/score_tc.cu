@@ -1033,8 +1033,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
 // ---------------------------------------------------------------------------
 // tables: fixed-point weights and their FP16 limbs in the MMA operand layout
 // ---------------------------------------------------------------------------
-__global__ void k_derive_tc(const double* log_theta, int C, int F, int Cp, int nks,
-                            const float* wmax, uint8_t* wlay, int32_t* q, TcHeader* hdr) {
+// A thread takes eight consecutive features of one class: one 16-byte record of
+// each limb (eight features are adjacent in a core matrix's row), 64 bytes of
+// log theta read.
+__global__ void __launch_bounds__(256) k_derive_tc(const double* log_theta, const double* wmean,
+                                                   int C, int F, int Cp, int nks,
+                                                   const float* wmax, uint8_t* wlay, int32_t* q,
+                                                   TcHeader* hdr) {
+  pdl_wait();
   const int N = 3 * Cp;
   // |w| <= wmax (1 + 2^-24) < 2^e; then |Q| = |round(w 2^S)| <= 2^22
   const float wm = *wmax;
@@ -1049,49 +1055,55 @@ __global__ void k_derive_tc(const double* log_theta, int C, int F, int Cp, int n
     hdr->pad = 0;
   }
   const double sc = ldexp(1.0, S);
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nks * TC_KS;
-       j += gridDim.x * blockDim.x) {
-    double m = 0.0;
-    if (j < F) {
-      for (int c = 0; c < C; ++c) m += log_theta[(size_t)c * F + j];
-      m /= (double)C;
-    }
-    const int ks = j / TC_KS, kk = j % TC_KS;
-    uint8_t* stage = wlay + (size_t)ks * N * 128;
-    for (int c = 0; c < Cp; ++c) {
-      int Q = 0;
-      if (c < C && j < F) {
-        const double w = log_theta[(size_t)c * F + j] - m;
-        Q = isfinite(w) ? (int)rint(w * sc) : 0;
-        q[(size_t)c * F + j] = Q;
-      }
-      const int q0 = ((Q + 128) & 255) - 128;
-      const int Q1 = (Q - q0) >> 8;
-      const int q1 = ((Q1 + 128) & 255) - 128;
-      const int q2 = (Q1 - q1) >> 8;
-      const int limb[3] = {q0, q1, q2};
+  const int t = blockIdx.x * 256 + threadIdx.x, per = nks * (TC_KS / 8);
+  const int c = t / per, j0 = t % per * 8;
+  if (c >= Cp) return;
+  __align__(16) __half2 limb[3][4];
+  int Q[8];
 #pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        const int n = l * Cp + c;
-        __half* p = reinterpret_cast<__half*>(stage + (n >> 3) * 1024 + (kk >> 3) * 128 +
-                                              (n & 7) * 16 + (kk & 7) * 2);
-        *p = __int2half_rn(limb[l]);
-      }
+  for (int k = 0; k < 8; ++k) {
+    const int j = j0 + k;
+    Q[k] = 0;
+    if (c < C && j < F) {
+      const double w = log_theta[(size_t)c * F + j] - wmean[j];
+      Q[k] = isfinite(w) ? (int)rint(w * sc) : 0;
+      q[(size_t)c * F + j] = Q[k];
     }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k += 2) {
+    int v[2][3];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      v[h][0] = ((Q[k + h] + 128) & 255) - 128;
+      const int Q1 = (Q[k + h] - v[h][0]) >> 8;
+      v[h][1] = ((Q1 + 128) & 255) - 128;
+      v[h][2] = (Q1 - v[h][1]) >> 8;
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+      limb[l][k / 2] = __halves2half2(__int2half_rn(v[0][l]), __int2half_rn(v[1][l]));
+  }
+  const int ks = j0 / TC_KS, kk = j0 % TC_KS;
+  uint8_t* stage = wlay + (size_t)ks * N * 128;
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    const int n = l * Cp + c;
+    *reinterpret_cast<uint4*>(stage + (n >> 3) * 1024 + (kk >> 3) * 128 + (n & 7) * 16) =
+        *reinterpret_cast<const uint4*>(limb[l]);
   }
 }
 
 nb_status launch_derive_tc(nb_model* m, cudaStream_t st) {
-  const int nks = (m->F + TC_KS - 1) / TC_KS;
-  const int threads = 256;
-  const int blocks = (nks * TC_KS + threads - 1) / threads;
+  const int nks = (m->F + TC_KS - 1) / TC_KS, Cp = tc_classes_padded(m->C);
+  const long long threads = (long long)Cp * nks * (TC_KS / 8);
   count_launch();
-  k_derive_tc<<<blocks, threads, 0, st>>>(m->d.p0, m->C, m->F, tc_classes_padded(m->C), nks,
-                                          m->d.wmax, m->d.tc_w, m->d.tc_q, m->d.tc_hdr);
-  NB_TRY_CUDA(cudaGetLastError(), "k_derive_tc");
+  NB_TRY_CUDA(launch_pdl(k_derive_tc, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st,
+                         (const double*)m->d.p0, (const double*)m->d.wmean, m->C, m->F, Cp, nks,
+                         (const float*)m->d.wmax, m->d.tc_w, m->d.tc_q, m->d.tc_hdr),
+              "k_derive_tc");
   return NB_OK;
 }
-
 
 // ---------------------------------------------------------------------------
 // launch
