@@ -107,9 +107,10 @@ typedef struct {
  *                       recomputed in FP64: a two-class u8 row whose stored
  *                       counts total 2^24 or more (its int32 limb sums could
  *                       wrap), tensor-core rows of 2^17 or more counts beyond
- *                       the scorer's exact-redo capacity (FP8 and BF16 rows:
- *                       all of them) and FP8 / BF16 rows outside the
- *                       tensor-core scorer's count check;
+ *                       the scorer's exact-redo capacity (262,144 per call;
+ *                       FP8 and BF16 rows 4,096; none in a batch) and FP8 /
+ *                       BF16 rows outside the tensor-core scorer's count
+ *                       check;
  *   NB_RECHECK_LABEL -- rows whose margin is within the rigorous error bound
  *                       of the fast path are recomputed in FP64, so every
  *                       label equals the FP64 decision;

@@ -520,12 +520,12 @@ extern "C" nb_status nb_score_group(const nb_model* m, const void* X, nb_dtype d
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (n_rechecked) NB_TRY_CUDA(cudaMemsetAsync(n_rechecked, 0, sizeof(int64_t), st), "memset");
   ScoreOut o{label, margin, logpost, n_rechecked, want_lp, recheck};
+  // the scorers count the rows they mark, so the recheck can skip its scan when
+  // there are none
+  o.counted = n_rechecked != nullptr;
   nb_status s;
   switch (score_path(m, X, dtype, ld, recheck)) {
     case NB_PATH_TWO_CLASS:
-      // the two-class scorers count the rows they mark, so the recheck can
-      // skip its scan when there are none
-      o.counted = n_rechecked != nullptr;
       s = launch_score2(m, X, dtype, n, ld, aux, o, st);
       break;
     case NB_PATH_TENSOR: s = launch_score_tc(m, X, dtype, n, ld, aux, o, st); break;

@@ -45,10 +45,10 @@ struct nb_batch {
   size_t maps_off = 0;
   // two-class launch plan
   PipeArgs plan{};
-  int kv = 0, rpw = 1, ncw = 0, smem = 0;
+  int kv = 0, smem = 0;
   SegArgs seg{};
   // work lists
-  size_t bytes = 0;
+  size_t bytes = 0, copy_bytes = 0;   // lists; with the counter behind them
   void* dev = nullptr;
   void* host[2] = {nullptr, nullptr};
   cudaEvent_t done[2] = {nullptr, nullptr};
@@ -66,41 +66,44 @@ static SegGroup* list_of(void* base, int fam, int max_groups) {
          (size_t)fam * max_groups;
 }
 
-// The launches of one call (work list already on the device).
-static nb_status batch_launch(nb_batch* b, cudaStream_t st) {
+// The launches of one call (work list already on the device and *counter
+// cleared).  `groups`: the lists' group counts where the host knows them (an
+// empty list is not launched), else nullptr.  The two-class launch comes after
+// the tensor-core one, programmatically: its blocks fill the SMs that run out of
+// 256-row units first.
+static nb_status batch_launch(nb_batch* b, const int* groups, cudaStream_t st) {
   SegHeader* dh = hdr_of(b->dev);
-  NB_TRY_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(int64_t), st), "memset(counter)");
-  if (!b->fam[0].empty()) {
-    SegArgs a = b->seg;
-    a.groups = list_of(b->dev, 0, b->max_groups);
-    a.hdr = dh;
-    int grid = 0;
-    nb_status s =
-        launch_score2_seg(a, b->plan, b->dtype, b->kv, b->rpw, b->ncw, b->smem, &grid, st);
-    if (s != NB_OK) return s;
-  }
-  if (!b->fam[1].empty()) {
+  unsigned long long* marks = reinterpret_cast<unsigned long long*>(b->counter);
+  auto has = [&](int f) { return !b->fam[f].empty() && (!groups || groups[f] > 0); };
+  if (has(1)) {
     nb_status s = launch_score_gen_seg(list_of(b->dev, 1, b->max_groups), dh + 1,
                                        b->fam[1].data(), (int)b->fam[1].size(), b->dtype, b->F,
-                                       b->want_lp, b->recheck, b->status, st);
+                                       b->want_lp, b->recheck, marks, b->status, st);
     if (s != NB_OK) return s;
   }
-  if (!b->fam[2].empty()) {
+  if (has(2)) {
     nb_status s = launch_score_tc_seg(list_of(b->dev, 2, b->max_groups), dh + 2,
                                       static_cast<char*>(b->dev) + b->maps_off,
                                       b->fam[2].data(), (int)b->fam[2].size(), b->dtype, b->F,
-                                      b->want_lp, b->recheck, b->status, st);
+                                      b->want_lp, b->recheck, marks, b->status, st);
+    if (s != NB_OK) return s;
+  }
+  if (has(0)) {
+    SegArgs a = b->seg;
+    a.groups = list_of(b->dev, 0, b->max_groups);
+    a.hdr = dh;
+    a.marks = marks;
+    nb_status s = launch_score2_seg(a, b->plan, b->dtype, b->kv, b->smem, st);
     if (s != NB_OK) return s;
   }
   // also under NB_RECHECK_OFF: rows a scorer could not compute at all are marked
-  for (int f = 0; f < kFamilies; ++f) {
-    if (b->fam[f].empty()) continue;
-    nb_status s = launch_recheck_seg(list_of(b->dev, f, b->max_groups), dh + f,
-                                     b->fam[f].data(), (int)b->fam[f].size(), b->dtype, b->F,
-                                     b->want_lp, b->counter, st);
-    if (s != NB_OK) return s;
-  }
-  return NB_OK;
+  RecheckList lists[kFamilies];
+  int n = 0;
+  for (int f = 0; f < kFamilies; ++f)
+    if (has(f))
+      lists[n++] = RecheckList{list_of(b->dev, f, b->max_groups), dh + f, b->fam[f].data(),
+                               (int)b->fam[f].size()};
+  return launch_recheck_seg(lists, n, b->dtype, b->F, b->want_lp, marks, st);
 }
 
 namespace nbg {
@@ -120,7 +123,8 @@ nb_status batch_device_list(nb_batch* b, SegHeader** hdr, SegGroup** list0, int6
 
 // The batch's launches on a work list already written on the device.
 nb_status batch_launch_device(nb_batch* b, cudaStream_t st, int64_t* n_rechecked) {
-  nb_status s = batch_launch(b, st);
+  NB_TRY_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(int64_t), st), "memset(counter)");
+  nb_status s = batch_launch(b, nullptr, st);
   if (s != NB_OK) return s;
   if (n_rechecked)
     NB_TRY_CUDA(cudaMemcpyAsync(n_rechecked, b->counter, sizeof(int64_t),
@@ -202,20 +206,22 @@ nb_status nbg::batch_create(const nb_model* const* models, int n_models, nb_dtyp
   }
   if (!b->fam[0].empty()) {
     nb_status s = seg2_plan(dtype, F, b->F_pad, max_ld * es, (int)b->fam[0].size(), plain,
-                            &b->plan, &b->kv, &b->rpw, &b->ncw, &b->smem);
+                            &b->plan, &b->kv, &b->smem);
     if (s != NB_OK) return fail(s);
   }
   b->maps_off = (kFamilies * sizeof(SegHeader) + kFamilies * (size_t)max_groups * sizeof(SegGroup) +
                  127) / 128 * 128;
   b->bytes = b->maps_off + (b->fam[2].empty() ? 0 : (size_t)max_groups * kTcMapBytes);
+  // the counter follows the lists: the list's copy clears it
+  b->copy_bytes = b->bytes + sizeof(int64_t);
   cudaError_t e = cudaMalloc(&b->dev, b->bytes + 64);
   if (e != cudaSuccess) return fail(cuda_status(e, "cudaMalloc(batch)"));
   b->counter = reinterpret_cast<int64_t*>(static_cast<char*>(b->dev) + b->bytes);
   b->status = reinterpret_cast<int*>(static_cast<char*>(b->dev) + b->bytes + 16);
   for (int i = 0; i < 2; ++i) {
-    e = cudaMallocHost(&b->host[i], b->bytes);
+    e = cudaMallocHost(&b->host[i], b->copy_bytes);
     if (e != cudaSuccess) return fail(cuda_status(e, "cudaMallocHost(batch)"));
-    memset(b->host[i], 0, b->bytes);
+    memset(b->host[i], 0, b->copy_bytes);
     e = cudaEventCreateWithFlags(&b->done[i], cudaEventDisableTiming);
     if (e != cudaSuccess) return fail(cuda_status(e, "cudaEventCreate"));
   }
@@ -324,9 +330,10 @@ extern "C" nb_status nb_batch_score(nb_batch* b, const nb_group* groups, int n_g
   if (b->captured) {
     NB_TRY_CUDA(cudaGraphLaunch(b->exec[b->cur], st), "cudaGraphLaunch");
   } else {
-    NB_TRY_CUDA(cudaMemcpyAsync(b->dev, h, b->bytes, cudaMemcpyHostToDevice, st),
+    NB_TRY_CUDA(cudaMemcpyAsync(b->dev, h, b->copy_bytes, cudaMemcpyHostToDevice, st),
                 "memcpy(work list)");
-    nb_status s = batch_launch(b, st);
+    const int counts[kFamilies] = {hh[0].n_groups, hh[1].n_groups, hh[2].n_groups};
+    nb_status s = batch_launch(b, counts, st);
     if (s != NB_OK) return s;
   }
   NB_TRY_CUDA(cudaEventRecord(b->done[b->cur], st), "cudaEventRecord");
@@ -357,8 +364,8 @@ extern "C" nb_status nb_batch_capture(nb_batch* b, void* cuda_stream) {
     cudaGraph_t graph = nullptr;
     NB_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal),
                 "cudaStreamBeginCapture");
-    cudaError_t e = cudaMemcpyAsync(b->dev, b->host[i], b->bytes, cudaMemcpyHostToDevice, st);
-    nb_status s = e == cudaSuccess ? batch_launch(b, st) : cuda_status(e, "memcpy(capture)");
+    cudaError_t e = cudaMemcpyAsync(b->dev, b->host[i], b->copy_bytes, cudaMemcpyHostToDevice, st);
+    nb_status s = e == cudaSuccess ? batch_launch(b, nullptr, st) : cuda_status(e, "memcpy(capture)");
     cudaError_t e2 = cudaStreamEndCapture(st, &graph);
     if (s != NB_OK) {
       if (graph) cudaGraphDestroy(graph);

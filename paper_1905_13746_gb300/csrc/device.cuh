@@ -13,6 +13,11 @@ namespace nbg {
 // while the previous kernel on its stream drains; it calls pdl_wait() before it
 // reads anything that kernel wrote (the wait returns at once when there is no
 // such kernel).
+// pdl_trigger() in every block of a kernel lets the programmatic launch that
+// follows it start while the kernel runs, on resources that it leaves free.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // 16-byte streaming load: read once, do not keep in L1.

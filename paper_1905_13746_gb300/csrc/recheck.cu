@@ -277,89 +277,104 @@ nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t 
 }
 
 // ---------------------------------------------------------------------------
-// segmented recheck: warps take contiguous ranges of 32-row chunks of a group
-// list and walk its groups
+// segmented recheck: warps take contiguous ranges of 32-row chunks of each
+// group list of a batch and walk its groups
 // ---------------------------------------------------------------------------
+constexpr int kRSegLists = 3;
+
 struct RSegArgs {
-  const SegGroup* groups;
-  const SegHeader* hdr;
-  RModel md[kSegMaxModels];
-  int F, want_lp;
-  unsigned long long* n_rechecked;
+  struct List {
+    const SegGroup* groups;
+    const SegHeader* hdr;
+    int model0;            // its models start here in md
+    int two;               // two-class models
+  } list[kRSegLists];
+  RModel md[2 * kSegMaxModels];   // the two-class models and the many-class ones
+  int n_lists, F, want_lp;
+  const unsigned long long* marks;   // rows that the scorers marked
 };
 
-template <int DT, int CB>
+template <int DT>
 __global__ void __launch_bounds__(256) k_recheck_seg(const RSegArgs a) {
   __shared__ double s_sh[8][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n_groups = a.hdr->n_groups;
-  const long long chunks = a.hdr->chunks;
+  pdl_wait();   // the scorers' labels and mark count
+  if (*a.marks == 0ull) return;
   const long long W = (long long)gridDim.x * 8, w = (long long)blockIdx.x * 8 + warp;
-  const long long c0 = chunks * w / W, c1 = chunks * (w + 1) / W;
-  if (c0 >= c1 || n_groups == 0) return;
-  const SegGroup* gr = a.groups;
-  int g = seg_find(n_groups, c0, [gr](int i) { return gr[i].chunk0; });
-  unsigned long long cnt = 0;
-  for (long long c = c0; c < c1; ++c) {
-    while (g + 1 < n_groups && gr[g + 1].chunk0 <= c) ++g;
-    const SegGroup& G = gr[g];
-    const long long base = (c - G.chunk0) * 32;
-    const long long row = base + lane;
-    const bool f = row < G.n && G.label[row] == kLabelRecheck;
-    unsigned m = __ballot_sync(0xFFFFFFFFu, f);
-    if (!m) continue;
-    RView v;
-    v.cols = nullptr;
-    v.X = G.X;
-    v.F = a.F;
-    constexpr int es = DT == NB_F32 ? 4 : ((DT == NB_U16 || DT == NB_BF16) ? 2 : 1);
-    v.ld = G.ld_bytes / es;
-    v.ovf_ptr = G.ovf_ptr;
-    v.ovf_col = G.ovf_col;
-    v.ovf_add = G.ovf_add;
-    v.row_exp = G.row_exp;
-    v.label = G.label;
-    v.margin = G.margin;
-    v.logpost = G.logpost;
-    while (m) {
-      const int src = __ffs(m) - 1;
-      m &= m - 1;
-      recheck_row<DT, NB_MULTINOMIAL, CB, 16 / CB>(v, a.md[G.model], base + src, a.want_lp,
-                                                  s_sh[warp]);
-      ++cnt;
+  for (int f = 0; f < a.n_lists; ++f) {
+    const RSegArgs::List& L = a.list[f];
+    const int n_groups = L.hdr->n_groups;
+    const long long chunks = L.hdr->chunks;
+    const long long c0 = chunks * w / W, c1 = chunks * (w + 1) / W;
+    if (c0 >= c1 || n_groups == 0) continue;
+    const SegGroup* gr = L.groups;
+    int g = seg_find(n_groups, c0, [gr](int i) { return gr[i].chunk0; });
+    for (long long c = c0; c < c1; ++c) {
+      while (g + 1 < n_groups && gr[g + 1].chunk0 <= c) ++g;
+      const SegGroup& G = gr[g];
+      const long long base = (c - G.chunk0) * 32;
+      const long long row = base + lane;
+      const bool mk = row < G.n && G.label[row] == kLabelRecheck;
+      unsigned m = __ballot_sync(0xFFFFFFFFu, mk);
+      if (!m) continue;
+      RView v;
+      v.cols = nullptr;
+      v.X = G.X;
+      v.F = a.F;
+      constexpr int es = DT == NB_F32 ? 4 : ((DT == NB_U16 || DT == NB_BF16) ? 2 : 1);
+      v.ld = G.ld_bytes / es;
+      v.ovf_ptr = G.ovf_ptr;
+      v.ovf_col = G.ovf_col;
+      v.ovf_add = G.ovf_add;
+      v.row_exp = G.row_exp;
+      v.label = G.label;
+      v.margin = G.margin;
+      v.logpost = G.logpost;
+      const RModel& md = a.md[L.model0 + G.model];
+      while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        if (L.two)
+          recheck_row<DT, NB_MULTINOMIAL, 2, 8>(v, md, base + src, a.want_lp, s_sh[warp]);
+        else
+          recheck_row<DT, NB_MULTINOMIAL, 8, 2>(v, md, base + src, a.want_lp, s_sh[warp]);
+      }
     }
   }
-  if (lane == 0 && cnt && a.n_rechecked) atomicAdd(a.n_rechecked, cnt);
 }
 
-using RSegKernel = void (*)(RSegArgs);
-template <int DT>
-static RSegKernel recheck_seg_kernel(bool two) {
-  return two ? (RSegKernel)k_recheck_seg<DT, 2> : (RSegKernel)k_recheck_seg<DT, 8>;
-}
-
-nb_status launch_recheck_seg(const SegGroup* groups, const SegHeader* hdr,
-                             const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                             int want_lp, int64_t* n_rechecked, cudaStream_t st) {
+nb_status launch_recheck_seg(const RecheckList* lists, int n_lists, nb_dtype dt, int F, int want_lp,
+                             const unsigned long long* marks, cudaStream_t st) {
   RSegArgs a{};
-  a.groups = groups;
-  a.hdr = hdr;
-  for (int i = 0; i < n_models && i < kSegMaxModels; ++i) {
-    const nb_model* m = models[i];
-    a.md[i] = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
+  int at = 0;
+  for (int f = 0; f < n_lists && a.n_lists < kRSegLists; ++f) {
+    const RecheckList& l = lists[f];
+    if (l.n_models < 1) continue;
+    // the many-class lists share their models' order but not their number: each
+    // list brings its own entries
+    if (at + l.n_models > 2 * kSegMaxModels) {
+      set_error("recheck: too many models");
+      return NB_EINVAL;
+    }
+    RSegArgs::List& L = a.list[a.n_lists++];
+    L = {l.groups, l.hdr, at, l.models[0]->C == 2 ? 1 : 0};
+    for (int i = 0; i < l.n_models; ++i) {
+      const nb_model* m = l.models[i];
+      a.md[at++] = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
+    }
   }
+  if (a.n_lists == 0) return NB_OK;
   a.F = F;
   a.want_lp = want_lp;
-  a.n_rechecked = reinterpret_cast<unsigned long long*>(n_rechecked);
-  const bool two = models[0]->C == 2;   // the two-class list holds nothing else
-  const RSegKernel k = dt == NB_U8     ? recheck_seg_kernel<NB_U8>(two)
-                       : dt == NB_F32  ? recheck_seg_kernel<NB_F32>(two)
-                       : dt == NB_U16  ? recheck_seg_kernel<NB_U16>(two)
-                       : dt == NB_BF16 ? recheck_seg_kernel<NB_BF16>(two)
-                                       : recheck_seg_kernel<NB_FP8E4M3>(two);
+  a.marks = marks;
+  void (*k)(RSegArgs) = dt == NB_U8     ? k_recheck_seg<NB_U8>
+                        : dt == NB_F32  ? k_recheck_seg<NB_F32>
+                        : dt == NB_U16  ? k_recheck_seg<NB_U16>
+                        : dt == NB_BF16 ? k_recheck_seg<NB_BF16>
+                                        : k_recheck_seg<NB_FP8E4M3>;
   count_launch();
-  k<<<num_sms() * 4, 256, 0, st>>>(a);
-  NB_TRY_CUDA(cudaGetLastError(), "k_recheck_seg launch");
+  NB_TRY_CUDA(launch_pdl(k, dim3((unsigned)(num_sms() * 4)), dim3(256), 0, st, a),
+              "k_recheck_seg launch");
   return NB_OK;
 }
 

@@ -1,18 +1,25 @@
-// Segmented persistent two-class scorer: one launch scores a whole batch of
+// Segmented persistent two-class scorers: one launch scores a whole batch of
 // file groups of uneven size (1 .. 50,000 files and more), several resident
 // models, under a captured CUDA graph (the paper's groups, Sec. 3 / Sec. 4,
 // classified with their group's model).
 //
 // The launch reads its work list from device memory (header + one descriptor
-// per group, see seg.cuh), so a graph captured once serves every batch.  The
-// persistent grid splits the list's tiles (RS rows of one group) into
-// contiguous ranges per block; the producer warp walks the groups of its range
-// and streams each tile's rows and overflow slice into shared-memory stages
-// (pipe.cuh).  Every model's Delta table is staged once per block; a consumer
-// warp reloads its register slice when the stage's group uses another model.
-// Finished rows keep their group and are finalised 32 at a time.  The
-// per-row arithmetic is the single-group kernel's (32 lanes per row), so a
-// group gives the same bits alone and inside any batch.
+// per group, see seg.cuh), so a graph captured once serves every batch, and
+// every model's Delta table is staged in shared memory once per block.
+//
+// u8 rows (k_score2_seg_u8) stream through registers as in k_score2_u8: the
+// list's 32-row chunks are cut into units of the rows that a warp takes at a
+// time, and each warp takes a contiguous range of units, walking the groups.
+// The sums are exact integers, so a group gives the same bits alone and inside
+// any batch.
+//
+// F32 rows (k_score2_seg) go through the stage pipeline of pipe.cuh: the grid
+// splits the list's tiles (RS rows of one group) into contiguous ranges per
+// block; the producer warp walks the groups of its range and streams each
+// tile's rows into shared-memory stages; a consumer warp reloads its register
+// slice of the table when the stage's group uses another model; finished rows
+// keep their group and are finalised 32 at a time.  The per-row arithmetic is
+// the single-group kernel's (32 lanes per row).
 #include "pipe.cuh"
 #include "score2.cuh"
 #include "seg.cuh"
@@ -59,14 +66,13 @@ struct SegSrc {
   }
 };
 
-template <int DT, int KV, int RPW, int NCW>
-__global__ void __launch_bounds__((NCW + 1) * 32, NCW == 8 ? 2 : 1)
-    k_score2_seg(const SegArgs a, PipeArgs p) {
-  constexpr int LPR = 32 / RPW;   // lanes per row: RPW rows per warp pass
+constexpr int kSegNCW = 8;   // consumer warps (two blocks per SM)
+
+template <int KV>
+__global__ void __launch_bounds__((kSegNCW + 1) * 32, 2) k_score2_seg(const SegArgs a, PipeArgs p) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ uint64_t full[kMaxStages], empty[kMaxStages], tabbar;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = lane / LPR, li = lane % LPR;
   const int n_groups = a.hdr->n_groups;
   const long long tiles = a.hdr->tiles;
   const long long t0 = tiles * blockIdx.x / gridDim.x;
@@ -76,13 +82,13 @@ __global__ void __launch_bounds__((NCW + 1) * 32, NCW == 8 ? 2 : 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.S; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], NCW);
+      mbar_init(&empty[s], kSegNCW);
     }
     mbar_init(&tabbar, 1);
   }
   __syncthreads();
 
-  if (warp == NCW) {
+  if (warp == kSegNCW) {
     pipe_stage_tables(sm, a.tables, a.n_models, a.table_bytes, a.table_stride, &tabbar);
     if (ntl > 0) {
       SegSrc src{a.groups, n_groups, t0, p.RS, 0, TileInfo{}, 0};
@@ -93,54 +99,31 @@ __global__ void __launch_bounds__((NCW + 1) * 32, NCW == 8 ? 2 : 1)
   }
 
   // ------------------------------------------------------------- consumers
-  using Dec = Decode<DT>;
-  constexpr int EPV = Dec::EPV, QPV = EPV / 4;
   if (!mbar_wait_bounded(&tabbar, 0)) {
     if (lane == 0) atomicOr(a.status, ST_TIMEOUT);
     return;
   }
   const int nv = a.nvec_row, nt = a.nvec_tab;
-  uint4 q0[KV], q1[KV], q2[KV];
-  float4 wq[KV][QPV];
+  float4 wq[KV];
   int cur_g = -1, cur_m = -1;
   long long ld_bytes = 0;
-  const signed char* limb = nullptr;
-  const int keep = a.F * (16 / EPV) - 16 * (nv - 1);
-  uint32_t tm[4];
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    int vb = keep - 4 * w;
-    vb = vb < 0 ? 0 : (vb > 4 ? 4 : vb);
-    tm[w] = vb >= 4 ? 0xFFFFFFFFu : ((1u << (8 * vb)) - 1u);
-  }
-  const int tail_v = a.F < nv * EPV ? nv - 1 : -1;
+  const int tail_v = a.F < nv * 4 ? nv - 1 : -1;
 
-  int ra0 = 0, ra1 = 0, ra2 = 0;
-  uint32_t rt = 0;
   float rs = 0.f, rtf = 0.f;
   long long rrow = -1;
   int rgrp = 0, nres = 0;
+  unsigned marks = 0;
 
   auto finish = [&]() {
     if (lane < nres) {
       const SegGroup& G = a.groups[rgrp];
       const C2Header& H = *a.chdr[G.model];
-      if (DT == NB_U8) {
-        const long long D = ((long long)ra2 << 16) + ((long long)ra1 << 8) + (long long)ra0;
-        const float Dsum = (float)D * H.inv_scale;
-        const float d = Dsum + H.b;
-        const float tau = c2_tau_u8((float)rt, Dsum, H.b, H.inv_scale, H.maxabs);
-        c2_store(G.label, G.margin, G.logpost, a.want_lp, a.recheck, rrow, d, tau);
-      } else {
-        float scale = 1.f;
-        if (DT == NB_FP8E4M3 && G.row_exp) scale = exp2f((float)G.row_exp[rrow]);
-        const float d = rs * scale + H.b;
-        const float kk = (float)a.k_base;
-        const float gam = kk * 5.9604645e-8f / (1.f - kk * 5.9604645e-8f);
-        const float A = rtf * scale * H.maxabs * 1.001f;
-        const float tau = gam * (A + fabsf(H.b)) * 1.01f + 1e-12f * (A + fabsf(H.b)) + 1e-30f;
-        c2_store(G.label, G.margin, G.logpost, a.want_lp, a.recheck, rrow, d, tau);
-      }
+      const float d = rs + H.b;
+      const float kk = (float)a.k_base;
+      const float gam = kk * 5.9604645e-8f / (1.f - kk * 5.9604645e-8f);
+      const float A = rtf * H.maxabs * 1.001f;
+      const float tau = gam * (A + fabsf(H.b)) * 1.01f + 1e-12f * (A + fabsf(H.b)) + 1e-30f;
+      marks += c2_store(G.label, G.margin, G.logpost, a.want_lp, a.recheck, rrow, d, tau);
     }
     nres = 0;
   };
@@ -157,8 +140,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, NCW == 8 ? 2 : 1)
     const int nr = mp->nr;
     const long long row0 = mp->row0;
     const int g = mp->group;
-    const int in_smem = mp->in_smem;
-    const long long ebase = mp->ebase;
     if (g != cur_g) {
       cur_g = g;
       const SegGroup& G = a.groups[g];
@@ -166,176 +147,244 @@ __global__ void __launch_bounds__((NCW + 1) * 32, NCW == 8 ? 2 : 1)
       const int m = G.model;
       if (m != cur_m) {
         cur_m = m;
-        const unsigned char* tb = sm + (size_t)m * a.table_stride;
-        limb = reinterpret_cast<const signed char*>(tb);
+        const float4* tab = reinterpret_cast<const float4*>(sm + (size_t)m * a.table_stride);
 #pragma unroll
         for (int kv = 0; kv < KV; ++kv) {
-          const int v = li + LPR * kv;
-          if (DT == NB_U8) {
-            const uint4* tab = reinterpret_cast<const uint4*>(tb);
-            const uint4 z = make_uint4(0, 0, 0, 0);
-            q0[kv] = v < nv ? tab[v] : z;
-            q1[kv] = v < nv ? tab[nt + v] : z;
-            q2[kv] = v < nv ? tab[2 * nt + v] : z;
-          } else {
-            const float4* tab = reinterpret_cast<const float4*>(tb);
-#pragma unroll
-            for (int q = 0; q < QPV; ++q)
-              wq[kv][q] = v < nv ? tab[q * nt + v] : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
+          const int v = lane + 32 * kv;
+          wq[kv] = v < nv ? tab[v] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
     }
-    const SegGroup& G = a.groups[g];
-    const long long* sp = reinterpret_cast<const long long*>(st + p.ptr_off);
-    const uint16_t* scol = reinterpret_cast<const uint16_t*>(st + p.col_off);
-    const uint16_t* sadd = reinterpret_cast<const uint16_t*>(st + p.add_off);
-    for (int r0 = warp * RPW; r0 < nr; r0 += NCW * RPW) {
-      if (nres + RPW > 32) finish();
-      const int r = r0 + grp;             // this lane group's row
-      const bool valid = r < nr;
-      const unsigned char* rp = st + (size_t)(valid ? r : 0) * ld_bytes;
-      int c0[2] = {0, 0}, c1[2] = {0, 0}, c2[2] = {0, 0};   // even / odd vector chains
-      uint32_t ct[2] = {0u, 0u};
+    for (int r = warp; r < nr; r += kSegNCW) {
+      if (nres == 32) finish();
+      const unsigned char* rp = st + (size_t)r * ld_bytes;
       float acc[4] = {0.f, 0.f, 0.f, 0.f}, tf = 0.f;
 #pragma unroll
       for (int kv = 0; kv < KV; ++kv) {
-        const int v = li + LPR * kv, e = kv & 1;
+        const int v = lane + 32 * kv;
         if (v < nv) {
-          uint4 x = *reinterpret_cast<const uint4*>(rp + (size_t)v * 16);
-          if (DT == NB_U8) {
-            if (v == tail_v) {
-              x.x &= tm[0]; x.y &= tm[1]; x.z &= tm[2]; x.w &= tm[3];
-            }
-            c0[e] = dp4a_us(x.x, q0[kv].x, c0[e]);
-            c1[e] = dp4a_us(x.x, q1[kv].x, c1[e]);
-            c2[e] = dp4a_us(x.x, q2[kv].x, c2[e]);
-            ct[e] = dp4a_uu(x.x, 0x01010101u, ct[e]);
-            c0[e] = dp4a_us(x.y, q0[kv].y, c0[e]);
-            c1[e] = dp4a_us(x.y, q1[kv].y, c1[e]);
-            c2[e] = dp4a_us(x.y, q2[kv].y, c2[e]);
-            ct[e] = dp4a_uu(x.y, 0x01010101u, ct[e]);
-            c0[e] = dp4a_us(x.z, q0[kv].z, c0[e]);
-            c1[e] = dp4a_us(x.z, q1[kv].z, c1[e]);
-            c2[e] = dp4a_us(x.z, q2[kv].z, c2[e]);
-            ct[e] = dp4a_uu(x.z, 0x01010101u, ct[e]);
-            c0[e] = dp4a_us(x.w, q0[kv].w, c0[e]);
-            c1[e] = dp4a_us(x.w, q1[kv].w, c1[e]);
-            c2[e] = dp4a_us(x.w, q2[kv].w, c2[e]);
-            ct[e] = dp4a_uu(x.w, 0x01010101u, ct[e]);
-          } else {
-            float val[EPV];
-            Dec::run(x, val);
-            if (v == tail_v) {
+          const float4 x = *reinterpret_cast<const float4*>(rp + (size_t)v * 16);
+          float val[4] = {x.x, x.y, x.z, x.w};
+          if (v == tail_v) {
 #pragma unroll
-              for (int e = 0; e < EPV; ++e)
-                if (v * EPV + e >= a.F) val[e] = 0.f;
-            }
-#pragma unroll
-            for (int q = 0; q < QPV; ++q) {
-              acc[0] = fmaf(val[4 * q + 0], wq[kv][q].x, acc[0]);
-              acc[1] = fmaf(val[4 * q + 1], wq[kv][q].y, acc[1]);
-              acc[2] = fmaf(val[4 * q + 2], wq[kv][q].z, acc[2]);
-              acc[3] = fmaf(val[4 * q + 3], wq[kv][q].w, acc[3]);
-              tf += fabsf(val[4 * q + 0]) + fabsf(val[4 * q + 1]) + fabsf(val[4 * q + 2]) +
-                    fabsf(val[4 * q + 3]);
-            }
+            for (int e = 0; e < 4; ++e)
+              if (v * 4 + e >= a.F) val[e] = 0.f;
           }
+          acc[0] = fmaf(val[0], wq[kv].x, acc[0]);
+          acc[1] = fmaf(val[1], wq[kv].y, acc[1]);
+          acc[2] = fmaf(val[2], wq[kv].z, acc[2]);
+          acc[3] = fmaf(val[3], wq[kv].w, acc[3]);
+          tf += fabsf(val[0]) + fabsf(val[1]) + fabsf(val[2]) + fabsf(val[3]);
         }
       }
-      int a0 = c0[0] + c0[1], a1 = c1[0] + c1[1], a2 = c2[0] + c2[1];
-      uint32_t tt = ct[0] + ct[1];
-      if (DT == NB_U8 && G.ovf_ptr && valid) {
-        const long long k0 = sp[r], k1 = sp[r + 1];
-        for (long long e = k0 + li; e < k1; e += LPR) {
-          const uint32_t col = in_smem ? scol[e - ebase] : G.ovf_col[e];
-          const int add = in_smem ? sadd[e - ebase] : G.ovf_add[e];
+      float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+        tf += __shfl_xor_sync(0xFFFFFFFFu, tf, off);
+      }
+      if (lane == nres) {   // lane j holds the j-th finished row
+        rs = sum;
+        rtf = tf;
+        rrow = row0 + r;
+        rgrp = g;
+      }
+      ++nres;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    if (nres == 32) finish();
+  }
+  finish();
+  if (marks) atomicAdd(a.marks, (unsigned long long)marks);
+}
+
+// ---------------------------------------------------------------------------
+// u8 rows: a group of LPR lanes per row, R rows per group
+// ---------------------------------------------------------------------------
+// Bound by memory latency: a call gives each warp only a few units.  32 groups of
+// 62,000 files in all, F = 2,048 (127 MB): 38 us; 53 us through shared-memory
+// stages with one block of 12 consumer warps per SM.
+template <int LPR, int R>
+__global__ void __launch_bounds__(256, 2) k_score2_seg_u8(const SegArgs a) {
+  constexpr int RPW = 32 / LPR * R, UPC = 32 / RPW;   // rows per unit, units per 32-row chunk
+  static_assert(RPW <= 32, "a unit lies inside a chunk");
+  extern __shared__ __align__(128) unsigned char sm[];
+  __shared__ uint64_t bar;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_expect_tx(&bar, a.table_bytes * (uint32_t)a.n_models);
+    for (int i = 0; i < a.n_models; ++i)
+      for (uint32_t off = 0; off < a.table_bytes; off += 32768)
+        bulk_g2s(sm + (size_t)i * a.table_stride + off, static_cast<const char*>(a.tables[i]) + off,
+                 a.table_bytes - off < 32768 ? a.table_bytes - off : 32768, &bar);
+  }
+  __syncthreads();
+  const bool ok = mbar_wait_bounded(&bar, 0);
+  if (!ok) atomicOr(a.status, ST_TIMEOUT);
+  if (__syncthreads_and(ok) == 0) return;
+
+  const int lane = threadIdx.x & 31, sub = lane / LPR, li = lane % LPR;
+  const int nv = a.nvec_row, nt = a.nvec_tab, n_groups = a.hdr->n_groups;
+  const long long units = a.hdr->chunks * UPC;
+  const long long W = (long long)gridDim.x * 8, w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const long long u0 = units * w / W, u1 = units * (w + 1) / W;
+  const SegGroup* gr = a.groups;
+  // byte masks of the last (partial) vector
+  const int keep = a.F - 16 * (nv - 1);
+  uint32_t tm[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    int vb = keep - 4 * q;
+    vb = vb < 0 ? 0 : (vb > 4 ? 4 : vb);
+    tm[q] = vb >= 4 ? 0xFFFFFFFFu : ((1u << (8 * vb)) - 1u);
+  }
+  unsigned marks = 0;
+  // the range's first group: the last whose first chunk is not past it (the
+  // lanes look at 32 groups at a time: one memory latency, not a search's six)
+  int g = -1;
+  if (u0 < u1) {
+    const long long first = u0 / UPC;
+    for (int k = 0; k < n_groups; k += 32) {
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, k + lane < n_groups && gr[k + lane].chunk0 <= first);
+      g += __popc(m);
+      if (m != 0xFFFFFFFFu) break;
+    }
+  }
+  for (long long u = u0; u < u1; ++u) {
+    const long long chunk = u / UPC;
+    while (g + 1 < n_groups && gr[g + 1].chunk0 <= chunk) ++g;
+    const SegGroup& G = gr[g];
+    const long long n = G.n, ld = G.ld_bytes;
+    const uint4* tab = reinterpret_cast<const uint4*>(sm + (size_t)G.model * a.table_stride);
+    const long long row0 = (chunk - G.chunk0) * 32 + (u - chunk * UPC) * RPW + sub * R;
+    const char* rp[R];
+    int acc0[R], acc1[R], acc2[R];
+    uint32_t tot[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {   // rows past the end repeat the last one and store nothing
+      rp[r] = G.X + (row0 + r < n ? row0 + r : n - 1) * ld;
+      acc0[r] = acc1[r] = acc2[r] = 0;
+      tot[r] = 0u;
+    }
+#pragma unroll 4
+    for (int v = li; v < nv; v += LPR) {
+      uint4 x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = ld_stream16(rp[r] + (long long)v * 16);
+      const uint4 q0 = tab[v], q1 = tab[nt + v], q2 = tab[2 * nt + v];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        uint32_t b[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
+        if (v == nv - 1) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) b[q] &= tm[q];
+        }
+        const uint32_t l0[4] = {q0.x, q0.y, q0.z, q0.w}, l1[4] = {q1.x, q1.y, q1.z, q1.w},
+                       l2[4] = {q2.x, q2.y, q2.z, q2.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc0[r] = dp4a_us(b[q], l0[q], acc0[r]);
+          acc1[r] = dp4a_us(b[q], l1[q], acc1[r]);
+          acc2[r] = dp4a_us(b[q], l2[q], acc2[r]);
+          tot[r] = dp4a_uu(b[q], 0x01010101u, tot[r]);
+        }
+      }
+    }
+    if (G.ovf_ptr) {
+      const signed char* limb = reinterpret_cast<const signed char*>(tab);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (row0 + r >= n) continue;
+        const int64_t k1 = G.ovf_ptr[row0 + r + 1];
+        for (int64_t k = G.ovf_ptr[row0 + r] + li; k < k1; k += LPR) {
+          const uint32_t col = G.ovf_col[k];
+          const int add = G.ovf_add[k];
           if (col < (uint32_t)a.F) {
-            const int vv = col >> 4, b = col & 15;
-            a0 += add * (int)limb[(size_t)vv * 16 + b];
-            a1 += add * (int)limb[((size_t)nt + vv) * 16 + b];
-            a2 += add * (int)limb[((size_t)2 * nt + vv) * 16 + b];
-            tt += (uint32_t)add;
+            const size_t at = (size_t)(col >> 4) * 16 + (col & 15);
+            acc0[r] += add * (int)limb[at];
+            acc1[r] += add * (int)limb[(size_t)nt * 16 + at];
+            acc2[r] += add * (int)limb[(size_t)nt * 32 + at];
+            tot[r] += (uint32_t)add;
           } else {
             atomicOr(a.status, ST_OVF_RANGE);
           }
         }
       }
-      // lane nres + j takes row r0 + j of this pass from its group's first lane
-      const int src = (lane - nres) * LPR;
-      const bool take = lane >= nres && lane < nres + RPW && r0 + (lane - nres) < nr;
-      const int sl = take ? src : 0;
-      if (DT == NB_U8) {
-        // the group's four sums end up in its four lane quarters
-        const int k4 = sum4_transposed<LPR>(a0, a1, a2, (int)tt, li);
-        const int s0 = __shfl_sync(0xFFFFFFFFu, k4, sl);
-        const int s1 = __shfl_sync(0xFFFFFFFFu, k4, sl + LPR / 4);
-        const int s2 = __shfl_sync(0xFFFFFFFFu, k4, sl + LPR / 2);
-        const uint32_t st_ = (uint32_t)__shfl_sync(0xFFFFFFFFu, k4, sl + 3 * LPR / 4);
-        if (take) {
-          ra0 = s0, ra1 = s1, ra2 = s2, rt = st_;
-        }
-      } else {
-        float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-#pragma unroll
-        for (int off = LPR / 2; off > 0; off >>= 1) {
-          sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-          tf += __shfl_xor_sync(0xFFFFFFFFu, tf, off);
-        }
-        const float ss = __shfl_sync(0xFFFFFFFFu, sum, sl);
-        const float stf = __shfl_sync(0xFFFFFFFFu, tf, sl);
-        if (take) {
-          rs = ss, rtf = stf;
-        }
-      }
-      if (take) {
-        rrow = row0 + r0 + (lane - nres);
-        rgrp = g;
-      }
-      nres += (nr - r0) < RPW ? (nr - r0) : RPW;
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s]);
-    if (nres + RPW > 32) finish();
+    const C2Header& H = *a.chdr[G.model];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      long long D = ((long long)acc2[r] << 16) + ((long long)acc1[r] << 8) + (long long)acc0[r];
+#pragma unroll
+      for (int off = LPR / 2; off > 0; off >>= 1) {
+        D += __shfl_xor_sync(0xFFFFFFFFu, D, off);
+        tot[r] += __shfl_xor_sync(0xFFFFFFFFu, tot[r], off);
+      }
+      if (row0 + r < n && r % LPR == li) {
+        const float Dsum = (float)D * H.inv_scale;
+        const float d = Dsum + H.b;
+        const float tau = c2_tau_u8((float)tot[r], Dsum, H.b, H.inv_scale, H.maxabs);
+        marks += c2_store(G.label, G.margin, G.logpost, a.want_lp, a.recheck, row0 + r, d, tau);
+      }
+    }
   }
-  finish();
+  if (marks) atomicAdd(a.marks, (unsigned long long)marks);
+  // launched programmatically after the many-class kernel, whose output this
+  // one does not read: its completion has to imply that one's
+  pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
-template <int DT, int KV, int RPW, int NCW>
-static nb_status run_seg(const SegArgs& a, const PipeArgs& p, int smem, int* grid,
-                         cudaStream_t st) {
-  auto kern = k_score2_seg<DT, KV, RPW, NCW>;
+template <int KV>
+static nb_status run_seg(const SegArgs& a, const PipeArgs& p, int smem, cudaStream_t st) {
+  auto kern = k_score2_seg<KV>;
   if (smem > kSmemOptIn)
     NB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                 "cudaFuncSetAttribute(seg)");
   int occ = 0;
-  NB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, (NCW + 1) * 32, smem),
+  NB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, (kSegNCW + 1) * 32, smem),
               "occupancy(seg)");
   if (occ < 1) {
     set_error("segmented scorer does not fit on an SM");
     return NB_EUNSUPPORTED;
   }
-  *grid = num_sms() * occ;
   count_launch();
-  kern<<<*grid, (NCW + 1) * 32, smem, st>>>(a, p);
+  kern<<<num_sms() * occ, (kSegNCW + 1) * 32, smem, st>>>(a, p);
   NB_TRY_CUDA(cudaGetLastError(), "k_score2_seg launch");
   return NB_OK;
 }
 
-// Plan of a segmented two-class launch for rows of at most max_ld_bytes.
-// u8 rows of up to 16 (32) vectors take 8 (16) lanes per row, four (two) rows
-// per warp pass, so that short rows (a few hundred selected opcodes) keep all
-// lanes busy; exact integer sums make the result independent of the shape.
-// FP32 rows keep 32 lanes per row (their reduction order is that of the
-// single-group scorer).
+template <int LPR, int R>
+static nb_status run_seg_u8(const SegArgs& a, cudaStream_t st) {
+  auto kern = k_score2_seg_u8<LPR, R>;
+  const int smem = (int)(a.table_stride * (uint32_t)a.n_models);
+  if (smem > kSmemOptIn)
+    NB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                "cudaFuncSetAttribute(seg)");
+  int occ = 0;
+  NB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, smem),
+              "occupancy(seg)");
+  if (occ < 1) {
+    set_error("segmented scorer does not fit on an SM");
+    return NB_EUNSUPPORTED;
+  }
+  count_launch();
+  NB_TRY_CUDA(launch_pdl(kern, dim3((unsigned)(num_sms() * occ)), dim3(256), (size_t)smem, st, a),
+              "k_score2_seg_u8 launch");
+  return NB_OK;
+}
+
+// Plan of a segmented two-class launch for rows of at most max_ld_bytes: the
+// stages of the F32 kernel, and for both types the rows per tile of the work
+// list and the limits of what is accepted (tables and two stages in one
+// block's shared memory).
 //
 // Rows per stage: at most 48 when groups may carry side arrays (the producer's
 // lanes hold the overflow pointers of a tile), up to 240 for plain rows, so
 // that stages of short rows still move tens of KB.
 nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n_models,
-                    bool plain_rows, PipeArgs* p, int* kv_out, int* rpw_out, int* ncw_out,
-                    int* smem_out) {
+                    bool plain_rows, PipeArgs* p, int* kv_out, int* smem_out) {
   const int es = elem_size(dt);
   const int nvec_row = (F * es + 15) / 16;
   const int rpw = dt == NB_U8 ? (nvec_row <= 16 ? 4 : (nvec_row <= 32 ? 2 : 1)) : 1;
@@ -364,8 +413,6 @@ nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n
   S = S < 2 ? 2 : (S > kMaxStages ? kMaxStages : S);
   pipe_layout(*p, rs, S, max_ld_bytes, !plain_rows, false, stride * (uint32_t)n_models, 0);
   *kv_out = kv;
-  *rpw_out = rpw;
-  *ncw_out = ncw;
   *smem_out = (int)(p->stages_off + (uint32_t)p->S * p->stage_bytes);
   if (*smem_out > 220 * 1024) {
     set_error("batched two-class scoring: %d models do not fit in shared memory", n_models);
@@ -374,18 +421,27 @@ nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n
   return NB_OK;
 }
 
-nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int rpw,
-                            int ncw, int smem, int* grid, cudaStream_t st) {
-#define NB_SEG_CASE(D, K, R, N) \
-  if (dt == D && kv == K && rpw == R && ncw == N) return run_seg<D, K, R, N>(a, p, smem, grid, st);
-  NB_SEG_CASE(NB_U8, 1, 1, 8) NB_SEG_CASE(NB_U8, 2, 1, 8) NB_SEG_CASE(NB_U8, 3, 1, 12)
-  NB_SEG_CASE(NB_U8, 4, 1, 12)
-  NB_SEG_CASE(NB_U8, 1, 4, 12) NB_SEG_CASE(NB_U8, 2, 4, 12)
-  NB_SEG_CASE(NB_U8, 1, 2, 12) NB_SEG_CASE(NB_U8, 2, 2, 12)
-  NB_SEG_CASE(NB_F32, 1, 1, 8) NB_SEG_CASE(NB_F32, 2, 1, 8) NB_SEG_CASE(NB_F32, 3, 1, 8)
-  NB_SEG_CASE(NB_F32, 4, 1, 8) NB_SEG_CASE(NB_F32, 5, 1, 8) NB_SEG_CASE(NB_F32, 6, 1, 8)
-  NB_SEG_CASE(NB_F32, 7, 1, 8) NB_SEG_CASE(NB_F32, 8, 1, 8)
-#undef NB_SEG_CASE
+nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int smem,
+                            cudaStream_t st) {
+  if (dt == NB_U8) {   // lanes per row: about eight vectors each (see pick_lpr_u8), rows as there
+    const int nv = a.nvec_row;
+    if (nv <= 16) return run_seg_u8<2, 2>(a, st);
+    if (nv <= 32) return run_seg_u8<4, 4>(a, st);
+    if (nv <= 64) return run_seg_u8<8, 4>(a, st);
+    return run_seg_u8<16, 4>(a, st);
+  }
+  if (dt == NB_F32) {
+    switch (kv) {
+      case 1: return run_seg<1>(a, p, smem, st);
+      case 2: return run_seg<2>(a, p, smem, st);
+      case 3: return run_seg<3>(a, p, smem, st);
+      case 4: return run_seg<4>(a, p, smem, st);
+      case 5: return run_seg<5>(a, p, smem, st);
+      case 6: return run_seg<6>(a, p, smem, st);
+      case 7: return run_seg<7>(a, p, smem, st);
+      case 8: return run_seg<8>(a, p, smem, st);
+    }
+  }
   set_error("batched two-class scoring supports u8 and f32 storage");
   return NB_EUNSUPPORTED;
 }

@@ -43,6 +43,7 @@ struct GArgs {
   float* margin;
   float* logpost;
   int want_lp, recheck;
+  unsigned long long* marks;   // counts the rows marked for the recheck, or nullptr
   int* status;
 };
 
@@ -270,6 +271,7 @@ __device__ __forceinline__ void gen_tile(const GArgs& a, int64_t r0, float* gsm)
     if (lane == 0) {
       a.label[gr] = flag ? kLabelRecheck : (uint8_t)bi;
       a.margin[gr] = margin;
+      if (flag && a.marks) atomicAdd(a.marks, 1ull);
     }
     if (a.want_lp)
       for (int c = lane; c < a.C; c += 32)
@@ -311,6 +313,7 @@ struct GGArgs {
   float* margin;
   float* logpost;
   int want_lp, recheck;
+  unsigned long long* marks;   // counts the rows marked for the recheck, or nullptr
 };
 
 constexpr int kGaussWarps = 8;
@@ -512,6 +515,7 @@ __global__ void __launch_bounds__(kGaussWarps * 32, 2) k_score_gauss(const GGArg
         if (li == 0) {
           a.label[r] = fl ? kLabelRecheck : (uint8_t)bi;
           a.margin[r] = margin;
+          if (fl && a.marks) atomicAdd(a.marks, 1ull);
         }
         if (a.want_lp)
           for (int c = li; c < C; c += LPR) a.logpost[r * C + c] = (sr[c] - sb) - L;
@@ -566,6 +570,7 @@ struct GSegArgs {
   const SegHeader* hdr;
   GModel md[kSegMaxModels];
   int F, dtype, want_lp, recheck;
+  unsigned long long* marks;
   int* status;
 };
 
@@ -600,6 +605,7 @@ __global__ void __launch_bounds__(256) k_score_gen_seg(const GSegArgs s) {
     a.logpost = G.logpost;
     a.want_lp = s.want_lp;
     a.recheck = s.recheck;
+    a.marks = s.marks;
     a.status = s.status;
     gen_tile(a, (t - G.tile0) * GBM, gsm);
   }
@@ -607,8 +613,10 @@ __global__ void __launch_bounds__(256) k_score_gen_seg(const GSegArgs s) {
 
 nb_status launch_score_gen_seg(const SegGroup* groups, const SegHeader* hdr,
                                const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                               int want_lp, int recheck, int* status, cudaStream_t st) {
+                               int want_lp, int recheck, unsigned long long* marks, int* status,
+                               cudaStream_t st) {
   GSegArgs s{};
+  s.marks = marks;
   s.groups = groups;
   s.hdr = hdr;
   int C_max = 2;
@@ -661,6 +669,7 @@ nb_status launch_score_general(const nb_model* m, const void* X, nb_dtype dt, in
     a.logpost = o.logpost;
     a.want_lp = o.want_lp;
     a.recheck = o.recheck;
+    a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
     return launch_score_gauss(a, st);
   }
   const int es = elem_size(dt);
@@ -686,6 +695,7 @@ nb_status launch_score_general(const nb_model* m, const void* X, nb_dtype dt, in
   a.logpost = o.logpost;
   a.want_lp = o.want_lp;
   a.recheck = o.recheck;
+  a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
   a.status = m->d.sstatus;
   const int C_pad = ((m->C + 3) / 4) * 4;
   const int smem =

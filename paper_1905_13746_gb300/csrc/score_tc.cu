@@ -34,13 +34,15 @@
 // One weight stage (3 C_p limb rows x 64 features, one bulk copy) feeds the
 // MMAs of two 128-file tiles, which halves the weight traffic per file.
 //
-// Two launches of one kernel:
+// Passes:
 //   pass "pair"    units of 256 files (two 128-file tiles sharing each weight
 //                  stage), one FP32 accumulation per row in tensor memory
 //                  (2 x 192 columns) plus a ring of two A stages (128
 //                  columns); rows of 2^17 or more stored counts could have
 //                  rounded and are put on a list of heavy rows;
-//   pass "chunked" units of 128 listed heavy rows (read by the converter warps
+//   k_tc_heavy     up to kTcFew listed heavy rows on the CUDA cores, exact int64
+//                  sums against the 32-bit fixed-point weights;
+//   pass "chunked" more than those: units of 128 listed heavy rows (read by the converter warps
 //                  straight from global memory), accumulated in 512-feature
 //                  chunks (255 * 512 * 128 < 2^24: always exact) and joined in
 //                  exact int64 sums in tensor memory (2 columns per class).
@@ -81,6 +83,11 @@ constexpr uint32_t TC_RAW_BYTES = 2 * TC_M * TC_BOX;   // both tiles, 128 featur
 constexpr int TC_PD = 3;                   // row stages loaded ahead into registers
 constexpr long long TC_WAIT = 2000000000LL;
 constexpr int kTcHeavyCap = 262144;        // heavy rows one call redoes exactly
+// up to this many heavy rows go to the CUDA cores (k_tc_heavy) instead of the
+// chunked pass, which takes 153 us for any number of units up to one per SM (C =
+// 64, F = 8,192: one unit's 128 weight stages one after another) against 37 us
+// for the 130 heavy rows of 262,144
+constexpr int kTcFew = 4096;
 
 // Per-pass constants: H tiles per unit (two in the pair pass), P class parts
 // per row (the 16 warps cover H x 4 lane quadrants x P parts), BPT bytes of
@@ -123,6 +130,7 @@ struct TcArgs {
   long long* heavy;         // pair pass: rows of 2^17+ stored counts (g0 only), or nullptr
   unsigned long long* heavy_n;   // their count (may exceed heavy_cap)
   int heavy_cap;
+  unsigned long long* marks;     // counts the rows left for the FP64 recheck, or nullptr
   int* status;
 };
 
@@ -495,10 +503,13 @@ __device__ __forceinline__ bool tc_epilogue(const TcArgs& a, TcShared& sh, TcXch
   if (valid && part == 0) {
     G.label[grow] = (flag || heavy) ? kLabelRecheck : (uint8_t)Bi;
     G.margin[grow] = margin;
-    if (heavy && a.heavy) {
+    bool listed = false;
+    if (heavy && a.heavy && Tp < 4e9f) {   // an FP8 / BF16 row that failed its check has more
       const unsigned long long k = atomicAdd(a.heavy_n, 1ull);
-      if (k < (unsigned long long)a.heavy_cap) a.heavy[k] = grow;
+      listed = k < (unsigned long long)a.heavy_cap;
+      if (listed) a.heavy[k] = grow;
     }
+    if ((flag || heavy) && !listed && a.marks) atomicAdd(a.marks, 1ull);
   }
   if (a.want_lp && G.logpost) {
     // pass 2; a full chunk of 8 classes goes out as two 16-byte stores when the
@@ -582,6 +593,7 @@ __device__ __forceinline__ long long tc_units(const TcArgs& a) {
   if (MODE == 0) return a.groups ? a.hdr->tiles : a.units0;
   unsigned long long c = *a.heavy_n;
   if (c > (unsigned long long)a.heavy_cap) c = (unsigned long long)a.heavy_cap;
+  if (c <= (unsigned long long)kTcFew) return 0;   // k_tc_heavy took them
   return (long long)((c + TC_M - 1) / TC_M);
 }
 
@@ -601,7 +613,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
   uint8_t* B = raw + (MODE == 0 ? (size_t)TC_NRAW * TC_RAW_BYTES : 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_groups = a.groups ? a.hdr->n_groups : 1;
+  pdl_trigger();   // a batch's two-class launch may fill the SMs that run out of units
   const long long n_units = tc_units<MODE>(a);
+  if (MODE == 1 && n_units == 0) return;
   const long long my_units =
       n_units > (long long)blockIdx.x ? (n_units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
   const int nks = a.nks, F = a.F;
@@ -1157,6 +1171,237 @@ static nb_status run_tc(TcArgs& a, int maxN, long long units_hint, cudaStream_t 
   return NB_OK;
 }
 
+// ---------------------------------------------------------------------------
+// few heavy rows: exact sums on the CUDA cores
+// ---------------------------------------------------------------------------
+// An item is four listed rows against eight classes (32 int64 sums per thread,
+// each row's value read once for eight classes and each weight once for four
+// rows); the last of a row group's items finishes its rows, one warp per row.
+// Bound by the latency of the weight loads (from L2; two blocks per SM, 128
+// registers: 37 us for 130 rows, C = 64, F = 8,192; at 132 registers and one block
+// 55 us).
+struct TcHeavyArgs {
+  const char* X;
+  long long ld_bytes;
+  const int64_t* ovf_ptr;
+  const uint16_t* ovf_col;
+  const uint16_t* ovf_add;
+  const int8_t* row_exp;
+  TcModelArg M;
+  int F, want_lp, recheck;
+  const long long* heavy;
+  const unsigned long long* heavy_n;
+  int heavy_cap;
+  long long* sums;       // kTcFew x C
+  float* T;              // kTcFew: counts of the row, overflow entries included
+  unsigned int* done;    // kTcFew / 4, zero: finished items of a row group
+  uint8_t* label;
+  float* margin;
+  float* logpost;
+  unsigned long long* marks;
+};
+
+// values j .. j + V - 1 of a row as integer counts (checked by the pair pass)
+template <int DT, int V>
+__device__ __forceinline__ void heavy_counts(const char* rp, int j, int ex, int (&x)[V]) {
+  if constexpr (DT == NB_BF16) {
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+      x[k] = (int)__uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(rp) + j + k) << 16);
+  } else if constexpr (DT == NB_FP8E4M3) {
+    const float sc = exp2f((float)ex);
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+      x[k] = (int)(e4m3x2_to_f32((uint16_t)__ldg(reinterpret_cast<const uint8_t*>(rp) + j + k)).x * sc);
+  } else if constexpr (V == 4) {
+    const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(rp + j));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = (int)(w >> (8 * k) & 255u);
+  } else {
+    x[0] = (int)__ldg(reinterpret_cast<const uint8_t*>(rp) + j);
+  }
+}
+
+// V features per thread and step: 4 where F is a multiple of 4 (16-byte weight
+// loads), else 1
+template <int DT, int V>
+__global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
+  __shared__ long long red[8][32];
+  __shared__ unsigned int redT[8][4];
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();   // the pair pass's list
+  const long long n = (long long)min(*a.heavy_n, (unsigned long long)a.heavy_cap);
+  if (n == 0 || n > kTcFew) return;
+  const int C = a.M.C, F = a.F, ncb = (C + 7) / 8;
+  const long long items = (n + 3) / 4 * ncb;
+  for (long long item = blockIdx.x; item < items; item += gridDim.x) {
+    const long long rg = item / ncb;
+    const int cb = (int)(item % ncb) * 8;
+    const char* rp[4];
+    int ex[4];
+    long long row[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {   // rows past the end repeat the last one and store nothing
+      row[i] = a.heavy[min(4 * rg + i, n - 1)];
+      rp[i] = a.X + row[i] * a.ld_bytes;
+      ex[i] = DT == NB_FP8E4M3 && a.row_exp ? (int)a.row_exp[row[i]] : 0;
+    }
+    long long v[32];   // row i, class cb + c: v[8 i + c]
+    unsigned int T[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int p = 0; p < 32; ++p) v[p] = 0;
+    for (int j = V * tid; j < F; j += V * 256) {
+      int x[4][V];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        heavy_counts<DT, V>(rp[i], j, ex[i], x[i]);
+#pragma unroll
+        for (int k = 0; k < V; ++k) T[i] += (unsigned int)x[i][k];
+      }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        int q[V];
+        if constexpr (V == 4) {
+          int4 t = make_int4(0, 0, 0, 0);
+          if (cb + c < C) t = __ldg(reinterpret_cast<const int4*>(a.M.q + (long long)(cb + c) * F + j));
+          q[0] = t.x;
+          q[1] = t.y;
+          q[2] = t.z;
+          q[3] = t.w;
+        } else {
+          q[0] = cb + c < C ? __ldg(a.M.q + (long long)(cb + c) * F + j) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int k = 0; k < V; ++k) v[8 * i + c] += (long long)x[i][k] * (long long)q[k];
+      }
+    }
+    if (DT == NB_U8 && a.ovf_ptr) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        for (int64_t e = a.ovf_ptr[row[i]] + tid; e < a.ovf_ptr[row[i] + 1]; e += 256) {
+          const int j = a.ovf_col[e];
+          if (j >= F) continue;
+          const int add = a.ovf_add[e];
+          T[i] += (unsigned int)add;
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            if (cb + c < C) v[8 * i + c] += (long long)add * (long long)a.M.q[(long long)(cb + c) * F + j];
+        }
+    }
+    // reduce-scatter: lane l ends with value l of its warp
+#pragma unroll
+    for (int off = 16, m = 32; off > 0; off >>= 1, m >>= 1) {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int p = 0; p < m / 2; ++p) {
+        const long long send = up ? v[p] : v[p + m / 2], keep = up ? v[p + m / 2] : v[p];
+        v[p] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, off);
+      }
+    }
+    __syncthreads();   // the previous item's values are read
+    red[warp][lane] = v[0];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned int t = __reduce_add_sync(0xFFFFFFFFu, T[i]);
+      if (lane == 0) redT[warp][i] = t;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      long long t = 0;
+      for (int w = 0; w < 8; ++w) t += red[w][tid];
+      const int i = tid >> 3, c = cb + (tid & 7);
+      if (c < C) __stcg(&a.sums[(4 * rg + i) * C + c], t);
+      if (tid < 4) {
+        unsigned int tt = 0;
+        for (int w = 0; w < 8; ++w) tt += redT[w][tid];
+        if (cb == 0) __stcg(&a.T[4 * rg + tid], (float)tt);
+      }
+      __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&a.done[rg], 1u) == (unsigned)(ncb - 1);
+    __syncthreads();
+    if (!last || warp >= 4 || 4 * rg + warp >= n) continue;
+    // the row's scores, as in the chunked pass (the exact sum rounded once, one
+    // FMA with the prior), and the epilogue over the lanes
+    __threadfence();
+    const long long idx = 4 * rg + warp, r = a.heavy[idx];
+    const float sc = a.M.hdr->scale, Tt = __ldcg(&a.T[idx]);
+    float s[2];
+    float best = -INFINITY, emax = 0.f;
+    int bi = 0x7FFFFFFF;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = lane + 32 * h;
+      s[h] = -INFINITY;
+      if (c >= C) continue;
+      const long long q = __ldcg(&a.sums[idx * C + c]);
+      const float b = a.M.bias[c];
+      const float f = fmaf((float)(int)(q >> 24), 16777216.f, (float)(int)(q & 0xFFFFFF));
+      s[h] = fmaf(f, sc, b);
+      emax = fmaxf(emax, fabsf(b) + fabsf(f * sc) + fabsf(s[h]));
+      if (s[h] > best) {
+        best = s[h];
+        bi = c;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+      const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+      emax = fmaxf(emax, __shfl_xor_sync(0xFFFFFFFFu, emax, off));
+    }
+    float second = -INFINITY, se = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = lane + 32 * h;
+      if (c >= C) continue;
+      if (c != bi) second = fmaxf(second, s[h]);
+      se += expf(s[h] - best);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      second = fmaxf(second, __shfl_xor_sync(0xFFFFFFFFu, second, off));
+      se += __shfl_xor_sync(0xFFFFFFFFu, se, off);
+    }
+    const float lse = best + logf(se), margin = best - second;
+    // f = two roundings of the exact sum at most, s one more: e covers them (see
+    // tc_epilogue for the bound)
+    const float tau = 2.f * (Tt * a.M.hdr->tau_unit + 5.9604645e-8f * emax) * (1.f + 1.f / 1048576.f) + 1e-30f;
+    bool flag = false;
+    if (a.recheck != NB_RECHECK_OFF) {
+      flag = !(margin > tau);
+      if (a.recheck == NB_RECHECK_LP && tau > 5e-6f * fmaxf(1.f, margin)) flag = true;
+    }
+    if (lane == 0) {
+      a.label[r] = flag ? kLabelRecheck : (uint8_t)bi;
+      a.margin[r] = margin;
+      if (flag && a.marks) atomicAdd(a.marks, 1ull);
+    }
+    if (a.want_lp)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (lane + 32 * h < C) a.logpost[r * C + lane + 32 * h] = s[h] - lse;
+  }
+}
+
+template <int DT>
+static nb_status run_tc_heavy(const TcHeavyArgs& h, cudaStream_t st) {
+  // every weight row starts on 16 bytes when F is a multiple of 4
+  auto kern = h.F % 4 == 0 ? k_tc_heavy<DT, 4> : k_tc_heavy<DT, 1>;
+  count_launch();
+  NB_TRY_CUDA(launch_pdl(kern, dim3((unsigned)(num_sms() * 2)), dim3(256), 0, st, h),
+              "k_tc_heavy launch");
+  return NB_OK;
+}
+
 // cuTensorMapEncodeTiled from the driver, fetched once through the runtime
 static PFN_cuTensorMapEncodeTiled_v12000 tc_encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -1231,27 +1476,53 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
   a.want_lp = o.want_lp;
   a.recheck = o.recheck;
   a.status = m->d.sstatus;
-  if (!u8) {
-    // FP8 / BF16 rows: heavy or unchecked rows stay marked for the FP64 recheck
-    a.heavy = nullptr;
-    a.heavy_n = nullptr;
-    a.heavy_cap = 0;
-    return dt == NB_FP8E4M3 ? run_tc<0, NB_FP8E4M3>(a, a.models[0].N, a.units0, st)
-                            : run_tc<0, NB_BF16>(a, a.models[0].N, a.units0, st);
-  }
-  // the list of heavy rows (and its count) for the chunked pass: stream-ordered
-  // scratch of this call
-  const int cap = n < kTcHeavyCap ? (int)n : kTcHeavyCap;
-  void* scratch = nullptr;
-  NB_TRY_CUDA(cudaMallocAsync(&scratch, 16 + sizeof(long long) * (size_t)cap, st),
-              "cudaMallocAsync(heavy rows)");
-  a.heavy_n = static_cast<unsigned long long*>(scratch);
-  a.heavy = reinterpret_cast<long long*>(static_cast<char*>(scratch) + 16);
+  a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
+  // scratch of this call, stream-ordered: the count of heavy rows and the row
+  // groups' counters (cleared), the list, the sums of up to kTcFew rows.  FP8 and
+  // BF16 rows list no more than those (the chunked pass reads u8 rows only);
+  // what is not listed stays marked for the FP64 recheck.
+  const int most = u8 ? kTcHeavyCap : kTcFew;
+  const int cap = n < most ? (int)n : most, few = cap < kTcFew ? cap : kTcFew;
+  const size_t groups = ((size_t)few + 3) / 4, clear = 16 + 4 * (groups + 3) / 4 * 4;
+  const size_t o_list = (clear + 15) / 16 * 16, o_sums = o_list + 8 * (size_t)cap,
+               o_T = o_sums + 32 * groups * m->C;
+  char* scratch = nullptr;
+  NB_TRY_CUDA(cudaMallocAsync(&scratch, o_T + 16 * groups, st), "cudaMallocAsync(heavy rows)");
+  a.heavy_n = reinterpret_cast<unsigned long long*>(scratch);
+  a.heavy = reinterpret_cast<long long*>(scratch + o_list);
   a.heavy_cap = cap;
-  const cudaError_t me = cudaMemsetAsync(scratch, 0, 16, st);
+  TcHeavyArgs h{};
+  h.X = g.X;
+  h.ld_bytes = g.ld_bytes;
+  h.ovf_ptr = g.ovf_ptr;
+  h.ovf_col = g.ovf_col;
+  h.ovf_add = g.ovf_add;
+  h.row_exp = g.row_exp;
+  h.M = a.models[0];
+  h.F = a.F;
+  h.want_lp = o.want_lp;
+  h.recheck = o.recheck;
+  h.heavy = a.heavy;
+  h.heavy_n = a.heavy_n;
+  h.heavy_cap = cap;
+  h.sums = reinterpret_cast<long long*>(scratch + o_sums);
+  h.T = reinterpret_cast<float*>(scratch + o_T);
+  h.done = reinterpret_cast<unsigned int*>(scratch + 16);
+  h.label = o.label;
+  h.margin = o.margin;
+  h.logpost = o.logpost;
+  h.marks = a.marks;
+  const cudaError_t me = cudaMemsetAsync(scratch, 0, clear, st);
   nb_status s = me == cudaSuccess ? NB_OK : cuda_status(me, "memset(heavy count)");
-  if (s == NB_OK) s = run_tc<0, NB_U8>(a, a.models[0].N, a.units0, st);
-  if (s == NB_OK) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
+  if (s == NB_OK)
+    s = u8                   ? run_tc<0, NB_U8>(a, a.models[0].N, a.units0, st)
+        : dt == NB_FP8E4M3 ? run_tc<0, NB_FP8E4M3>(a, a.models[0].N, a.units0, st)
+                             : run_tc<0, NB_BF16>(a, a.models[0].N, a.units0, st);
+  if (s == NB_OK)
+    s = u8                   ? run_tc_heavy<NB_U8>(h, st)
+        : dt == NB_FP8E4M3 ? run_tc_heavy<NB_FP8E4M3>(h, st)
+                             : run_tc_heavy<NB_BF16>(h, st);
+  if (s == NB_OK && u8 && cap > kTcFew) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
   const cudaError_t fe = cudaFreeAsync(scratch, st);
   if (s != NB_OK) return s;
   NB_TRY_CUDA(fe, "cudaFreeAsync(heavy rows)");
@@ -1270,8 +1541,10 @@ bool tc_group_eligible(const nb_model* m, nb_dtype dt, const void* X, int64_t ld
 
 nb_status launch_score_tc_seg(const SegGroup* groups, const SegHeader* hdr, const void* maps,
                               const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                              int want_lp, int recheck, int* status, cudaStream_t st) {
+                              int want_lp, int recheck, unsigned long long* marks, int* status,
+                              cudaStream_t st) {
   TcArgs a{};
+  a.marks = marks;
   a.maps = static_cast<const CUtensorMap*>(maps);
   a.groups = groups;
   a.hdr = hdr;

@@ -91,6 +91,7 @@ struct TgArgs {
   float* margin;
   float* logpost;
   int want_lp, recheck;
+  unsigned long long* marks;   // counts the rows marked for the recheck, or nullptr
   int* status;
 };
 
@@ -580,6 +581,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_score_tcg(const __grid_consta
       if (valid) {
         a.label[grow] = flag ? kLabelRecheck : (uint8_t)bidx;
         a.margin[grow] = margin;
+        if (flag && a.marks) atomicAdd(a.marks, 1ull);
       }
       if (want_lp) {
         float* lp = a.logpost + (valid ? grow : 0) * a.C;
@@ -787,6 +789,7 @@ nb_status launch_score_tcg(const nb_model* m, const float* X, int64_t n, int64_t
   a.logpost = o.want_lp ? o.logpost : nullptr;
   a.want_lp = o.want_lp;
   a.recheck = o.recheck;
+  a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
   a.status = m->d.sstatus;
   const size_t smem = ((sizeof(TgShared) + 1023) / 1024) * 1024 + (size_t)TG_NRAW * TG_SLOT_BYTES +
                       (size_t)a.nb * a.Cp * (2 * TG_KS);

@@ -57,6 +57,7 @@ struct SegArgs {
   const C2Header* chdr[kSegMaxModels];
   uint32_t table_bytes, table_stride;
   int F, nvec_row, nvec_tab, want_lp, recheck, k_base;
+  unsigned long long* marks;   // counts the rows marked for the recheck
   int* status;
 };
 
@@ -64,21 +65,30 @@ struct PipeArgs;
 
 // launchers (score2_seg.cu, score_general.cu, recheck.cu)
 nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n_models,
-                    bool plain_rows, PipeArgs* p, int* kv_out, int* rpw_out, int* ncw_out,
-                    int* smem_out);
-nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int rpw,
-                            int ncw, int smem, int* grid, cudaStream_t st);
+                    bool plain_rows, PipeArgs* p, int* kv_out, int* smem_out);
+nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int smem,
+                            cudaStream_t st);
 nb_status launch_score_gen_seg(const SegGroup* groups, const SegHeader* hdr,
                                const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                               int want_lp, int recheck, int* status, cudaStream_t st);
+                               int want_lp, int recheck, unsigned long long* marks, int* status,
+                               cudaStream_t st);
 nb_status launch_score_tc_seg(const SegGroup* groups, const SegHeader* hdr, const void* maps,
                               const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                              int want_lp, int recheck, int* status, cudaStream_t st);
+                              int want_lp, int recheck, unsigned long long* marks, int* status,
+                              cudaStream_t st);
 nb_status tc_encode_rows(void* map, const void* X, int64_t n, int F, int64_t ld_bytes, int es);
 bool tc_group_eligible(const nb_model* m, nb_dtype dt, const void* X, int64_t ld);
 constexpr size_t kTcMapBytes = 128;
-nb_status launch_recheck_seg(const SegGroup* groups, const SegHeader* hdr,
-                             const nb_model* const* models, int n_models, nb_dtype dt, int F,
-                             int want_lp, int64_t* n_rechecked, cudaStream_t st);
+// One work list of a batch for the recheck: its groups, header and models.
+struct RecheckList {
+  const SegGroup* groups;
+  const SegHeader* hdr;
+  const nb_model* const* models;
+  int n_models;
+};
+// Recheck of all lists in one launch.  *marks: the rows that the scorers
+// marked (the launch ends at once when there are none).
+nb_status launch_recheck_seg(const RecheckList* lists, int n_lists, nb_dtype dt, int F, int want_lp,
+                             const unsigned long long* marks, cudaStream_t st);
 
 }  // namespace nbg
