@@ -264,6 +264,31 @@ static nb_status check_fit_args(nb_kind kind, const void* X, nb_dtype dtype, int
   return NB_OK;
 }
 
+// A page-locked buffer of the calling thread for small reads of device memory
+// (a copy to pageable memory costs the driver a staging copy and a wait each):
+// kPinned bytes, taken at the thread's first use and returned when it ends.
+// nullptr for more than that, or when there is none.
+constexpr size_t kPinned = 64 * 1024;
+struct PinnedBuffer {
+  void* p = nullptr;
+  bool tried = false;
+  ~PinnedBuffer() {
+    if (p) cudaFreeHost(p);
+  }
+};
+static void* pinned_staging(size_t bytes) {
+  static thread_local PinnedBuffer b;
+  if (bytes > kPinned) return nullptr;
+  if (!b.tried) {
+    b.tried = true;
+    if (cudaHostAlloc(&b.p, kPinned, cudaHostAllocPortable) != cudaSuccess) {
+      b.p = nullptr;
+      cudaGetLastError();
+    }
+  }
+  return b.p;
+}
+
 static nb_status fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld,
                               const int32_t* y, bool prior_given, cudaStream_t st) {
   FitScratch fs(m, st);
@@ -296,10 +321,11 @@ static nb_status fit_into(nb_model* m, const void* X, nb_dtype dtype, int64_t n,
   if (s != NB_OK) return s;
   if (!no_sync) {
     int w = 0;
-    NB_TRY_CUDA(cudaMemcpyAsync(&w, m->d.status, sizeof(int), cudaMemcpyDeviceToHost, st),
+    int* pin = static_cast<int*>(pinned_staging(sizeof(int)));
+    NB_TRY_CUDA(cudaMemcpyAsync(pin ? pin : &w, m->d.status, sizeof(int), cudaMemcpyDeviceToHost, st),
                 "memcpy(status)");
     NB_TRY_CUDA(cudaStreamSynchronize(st), "nb_fit sync");
-    return status_from_word(w);
+    return status_from_word(pin ? *pin : w);
   }
   return NB_OK;
 }
@@ -416,17 +442,29 @@ extern "C" nb_status nb_model_params(const nb_model* m, double* p0, double* p1, 
     set_error("nb_model_params: NULL model");
     return NB_EINVAL;
   }
-  NB_TRY_CUDA(cudaStreamSynchronize(m->stream), "sync");
+  if (p1 && m->kind != NB_GAUSSIAN) {
+    set_error("nb_model_params: only Gaussian models have variances");
+    return NB_EINVAL;
+  }
   const size_t cf = (size_t)m->C * m->F;
+  // the tables stand one after another (p0, p1, log pi): small models come over
+  // in one copy behind the fit
+  const char* first = reinterpret_cast<const char*>(m->d.p0);
+  const size_t span = reinterpret_cast<const char*>(m->d.log_pi + m->C) - first;
+  if (char* pin = static_cast<char*>(pinned_staging(span))) {
+    NB_TRY_CUDA(cudaMemcpyAsync(pin, first, span, cudaMemcpyDeviceToHost, m->stream), "memcpy");
+    NB_TRY_CUDA(cudaStreamSynchronize(m->stream), "sync");
+    if (p0) memcpy(p0, pin, sizeof(double) * cf);
+    if (p1) memcpy(p1, pin + (reinterpret_cast<const char*>(m->d.p1) - first), sizeof(double) * cf);
+    if (log_pi)
+      memcpy(log_pi, pin + (reinterpret_cast<const char*>(m->d.log_pi) - first), sizeof(double) * m->C);
+    return NB_OK;
+  }
+  NB_TRY_CUDA(cudaStreamSynchronize(m->stream), "sync");
   if (p0)
     NB_TRY_CUDA(cudaMemcpy(p0, m->d.p0, sizeof(double) * cf, cudaMemcpyDeviceToHost), "memcpy");
-  if (p1) {
-    if (m->kind != NB_GAUSSIAN) {
-      set_error("nb_model_params: only Gaussian models have variances");
-      return NB_EINVAL;
-    }
+  if (p1)
     NB_TRY_CUDA(cudaMemcpy(p1, m->d.p1, sizeof(double) * cf, cudaMemcpyDeviceToHost), "memcpy");
-  }
   if (log_pi)
     NB_TRY_CUDA(cudaMemcpy(log_pi, m->d.log_pi, sizeof(double) * m->C, cudaMemcpyDeviceToHost),
                 "memcpy");
