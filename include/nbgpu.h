@@ -108,7 +108,7 @@ typedef struct {
  *                       counts total 2^24 or more (its int32 limb sums could
  *                       wrap), tensor-core rows of 2^17 or more counts beyond
  *                       the scorer's exact-redo capacity (262,144 per call;
- *                       FP8 and BF16 rows 4,096; none in a batch) and FP8 /
+ *                       FP8 and BF16 rows 1,024; none in a batch) and FP8 /
  *                       BF16 rows outside the tensor-core scorer's count
  *                       check;
  *   NB_RECHECK_LABEL -- rows whose margin is within the rigorous error bound

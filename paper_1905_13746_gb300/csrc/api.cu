@@ -84,6 +84,7 @@ static nb_status alloc_model(nb_model* m) {
   const size_t o_tcq = take(tc ? sizeof(int32_t) * C * F : 0);
   const size_t o_tch = take(tc ? sizeof(TcHeader) : 0);
   const size_t o_wm = take(tc ? sizeof(double) * F : 0);
+  const size_t o_tcs = take(tc ? tc_scratch_bytes(m->C) : 0);
   const bool tg = tcg_tables(m->kind, m->C, m->F);
   const int F8 = (m->F + kTcgFS - 1) / kTcgFS * kTcgFS;
   const size_t o_tgw = take(tg ? tcg_w_bytes(m->C, m->F) : 0);
@@ -126,6 +127,11 @@ static nb_status alloc_model(nb_model* m) {
   d.tc_q = tc ? reinterpret_cast<int32_t*>(b + o_tcq) : nullptr;
   d.tc_hdr = tc ? reinterpret_cast<TcHeader*>(b + o_tch) : nullptr;
   d.wmean = tc ? reinterpret_cast<double*>(b + o_wm) : nullptr;
+  d.tc_scratch = tc ? b + o_tcs : nullptr;
+  if (tc && cudaEventCreateWithFlags(&m->slot.end, cudaEventDisableTiming) != cudaSuccess) {
+    m->slot.end = nullptr;   // scoring calls then allocate their scratch
+    cudaGetLastError();
+  }
   if (tg) d.tc_w = reinterpret_cast<uint8_t*>(b + o_tgw);
   d.tcg_kc = tg ? reinterpret_cast<float*>(b + o_tgk) : nullptr;
   d.tcg_ctr = tg ? reinterpret_cast<float*>(b + o_tgc) : nullptr;
@@ -134,6 +140,14 @@ static nb_status alloc_model(nb_model* m) {
   d.tcg_hdr = tg ? reinterpret_cast<TcgHeader*>(b + o_tgh) : nullptr;
   return NB_OK;
 }
+
+// A query of an event or an allocation of host memory may end a capture that runs
+// on some other stream (they count as unsafe there); these touch nothing captured.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 
 // A fit right after a synchronisation pays the driver for mapping pool memory
 // again when its scratch was returned to the pool before it (some 100 us and
@@ -168,6 +182,47 @@ nb_status FitScratch::release() {
   void* p = own_;
   own_ = nullptr;
   NB_TRY_CUDA(cudaFreeAsync(p, st_), "cudaFreeAsync(fit scratch)");
+  return NB_OK;
+}
+
+nb_status ScoreScratch::take(size_t bytes, char* kept, size_t kept_bytes, char** p) {
+  *p = nullptr;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  NB_TRY_CUDA(cudaStreamIsCapturing(st_, &cs), "cudaStreamIsCapturing");
+  ScoreSlot& k = m_->slot;
+  if (kept && k.end && bytes <= kept_bytes && cs == cudaStreamCaptureStatusNone) {
+    NB_TRY_CUDA(cudaStreamGetId(st_, &id_), "cudaStreamGetId");
+    std::lock_guard<std::mutex> lk(k.mu);
+    bool free = !k.busy && (!k.used || k.stream_id == id_);
+    if (!k.busy && !free) {
+      const RelaxedCapture relaxed;
+      free = cudaEventQuery(k.end) == cudaSuccess;
+      cudaGetLastError();   // cudaErrorNotReady is no error of this call
+    }
+    if (free) {
+      k.busy = slot_ = true;
+      *p = kept;
+      return NB_OK;
+    }
+  }
+  NB_TRY_CUDA(cudaMallocAsync(&own_, bytes, st_), "cudaMallocAsync(score scratch)");
+  *p = static_cast<char*>(own_);
+  return NB_OK;
+}
+
+nb_status ScoreScratch::release() {
+  if (slot_) {
+    ScoreSlot& k = m_->slot;
+    std::lock_guard<std::mutex> lk(k.mu);
+    slot_ = k.busy = false;
+    k.used = true;
+    k.stream_id = id_;
+    NB_TRY_CUDA(cudaEventRecord(k.end, st_), "cudaEventRecord(score scratch)");
+  }
+  if (!own_) return NB_OK;
+  void* p = own_;
+  own_ = nullptr;
+  NB_TRY_CUDA(cudaFreeAsync(p, st_), "cudaFreeAsync(score scratch)");
   return NB_OK;
 }
 
@@ -281,6 +336,7 @@ static void* pinned_staging(size_t bytes) {
   if (bytes > kPinned) return nullptr;
   if (!b.tried) {
     b.tried = true;
+    const RelaxedCapture relaxed;
     if (cudaHostAlloc(&b.p, kPinned, cudaHostAllocPortable) != cudaSuccess) {
       b.p = nullptr;
       cudaGetLastError();
@@ -373,6 +429,7 @@ extern "C" nb_status nb_fit(nb_kind kind, const void* X, nb_dtype dtype, int64_t
   else s = cuda_status(e, "memset(model)");
   if (s != NB_OK) {
     cudaStreamSynchronize(m->stream);
+    if (m->slot.end) cudaEventDestroy(m->slot.end);
     cudaFree(m->mem);
     delete m;
     return s;
@@ -486,6 +543,7 @@ extern "C" void nb_model_free(nb_model* m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
   if (m->work) cudaFree(m->work);
+  if (m->slot.end) cudaEventDestroy(m->slot.end);
   cudaFree(m->mem);
   delete m;
 }

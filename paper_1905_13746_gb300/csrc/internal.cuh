@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "nbgpu.h"
 
 namespace nbg {
@@ -118,6 +120,7 @@ struct ModelDev {
   int32_t* tc_q;       // C x F fixed-point weights
   TcHeader* tc_hdr;    // 1
   double* wmean;       // F          mean_c log theta_cj
+  char* tc_scratch;    // tc_scratch_bytes(C): heavy rows of one scoring call (ScoreScratch)
   // Gaussian FP32 tables
   float* g_mu;         // F_pad x gauss_cpad(C), feature-major (classes past C: 0)
   float* g_ivar;       // same layout, 1 / var
@@ -129,6 +132,15 @@ struct ModelDev {
   float* tcg_bmax;     // ... max_c |B_cj|
   float* tcg_amax;     // ... max_c |A_cj|
   TcgHeader* tcg_hdr;  // 1
+};
+
+// The model's scratch for one scoring call at a time: whether a call holds it,
+// and the stream and end of the last call that did.
+struct ScoreSlot {
+  std::mutex mu;
+  bool busy = false, used = false;
+  unsigned long long stream_id = 0;
+  cudaEvent_t end = nullptr;
 };
 
 }  // namespace nbg
@@ -149,6 +161,7 @@ struct nb_model {
   void* work;            // fit workspace kept between re-fits (see FitScratch), or nullptr
   size_t work_bytes;
   bool refit;            // the model has been fitted: later fits keep their workspace
+  mutable nbg::ScoreSlot slot;
   nbg::ModelDev d;
 };
 
@@ -165,6 +178,24 @@ size_t gauss_scratch_bytes(int64_t n, int F, int C);
 nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld,
                               const int32_t* y, bool prior_given, void* scratch,
                               cudaStream_t st);
+
+// Device scratch of a scoring call: the model's own when no other call can be
+// using it on the GPU (the last one was on this stream or has finished), else,
+// and on a stream being captured, memory allocated and freed in stream order.
+class ScoreScratch {
+ public:
+  ScoreScratch(const nb_model* m, cudaStream_t st) : m_(m), st_(st) {}
+  ~ScoreScratch() { release(); }
+  nb_status take(size_t bytes, char* kept, size_t kept_bytes, char** p);
+  nb_status release();
+
+ private:
+  const nb_model* m_;
+  cudaStream_t st_;
+  unsigned long long id_ = 0;
+  void* own_ = nullptr;
+  bool slot_ = false;
+};
 
 // Device scratch of a fit: the model's own workspace, kept between re-fits
 // (up to kKeepWork bytes; larger ones, the first fit's and those of a stream
@@ -222,6 +253,7 @@ inline size_t tc_w_bytes(int C, int F) {
 inline bool tc_tables(nb_kind kind, int C, int F) {
   return kind == NB_MULTINOMIAL && C >= 3 && C <= kTcMaxC && F <= kTcMaxF;
 }
+size_t tc_scratch_bytes(int C);
 bool tc_eligible(const nb_model* m, nb_dtype dt, const void* X, int64_t ld);
 nb_status launch_derive_tc(nb_model* m, cudaStream_t st);
 

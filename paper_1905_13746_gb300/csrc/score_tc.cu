@@ -87,7 +87,7 @@ constexpr int kTcHeavyCap = 262144;        // heavy rows one call redoes exactly
 // chunked pass, which takes 153 us for any number of units up to one per SM (C =
 // 64, F = 8,192: one unit's 128 weight stages one after another) against 37 us
 // for the 130 heavy rows of 262,144
-constexpr int kTcFew = 4096;
+constexpr int kTcFew = 1024;
 
 // Per-pass constants: H tiles per unit (two in the pair pass), P class parts
 // per row (the 16 warps cover H x 4 lane quadrants x P parts), BPT bytes of
@@ -127,7 +127,7 @@ struct TcArgs {
   int F, nks, want_lp, recheck;
   int pf;                   // stages between the L2 prefetch of a row's bytes and their load
   uint32_t b_bytes;         // bytes of one weight stage slot (largest model)
-  long long* heavy;         // pair pass: rows of 2^17+ stored counts (g0 only), or nullptr
+  int* heavy;               // pair pass: rows of 2^17+ stored counts (g0 only), or nullptr
   unsigned long long* heavy_n;   // their count (may exceed heavy_cap)
   int heavy_cap;
   unsigned long long* marks;     // counts the rows left for the FP64 recheck, or nullptr
@@ -507,7 +507,7 @@ __device__ __forceinline__ bool tc_epilogue(const TcArgs& a, TcShared& sh, TcXch
     if (heavy && a.heavy && Tp < 4e9f) {   // an FP8 / BF16 row that failed its check has more
       const unsigned long long k = atomicAdd(a.heavy_n, 1ull);
       listed = k < (unsigned long long)a.heavy_cap;
-      if (listed) a.heavy[k] = grow;
+      if (listed) a.heavy[k] = (int)grow;   // row coordinates of the tensor map are 32-bit
     }
     if ((flag || heavy) && !listed && a.marks) atomicAdd(a.marks, 1ull);
   }
@@ -1189,7 +1189,7 @@ struct TcHeavyArgs {
   const int8_t* row_exp;
   TcModelArg M;
   int F, want_lp, recheck;
-  const long long* heavy;
+  const int* heavy;
   const unsigned long long* heavy_n;
   int heavy_cap;
   long long* sums;       // kTcFew x C
@@ -1444,6 +1444,21 @@ static nb_status tc_row_map(CUtensorMap* map, const void* X, int64_t n, int F, i
   return NB_OK;
 }
 
+// Scratch of a call: the count of heavy rows and the row groups' counters
+// (cleared by each call), the list, the sums and totals of `few` rows.
+struct TcScratch {
+  size_t clear, list, sums, T, bytes;
+  TcScratch(int cap, int few, int C) {
+    const size_t groups = ((size_t)few + 3) / 4;
+    clear = 16 + 4 * groups;
+    list = (clear + 15) / 16 * 16;
+    sums = (list + 4 * (size_t)cap + 15) / 16 * 16;
+    T = sums + 32 * groups * C;
+    bytes = T + 16 * groups;
+  }
+};
+size_t tc_scratch_bytes(int C) { return TcScratch(kTcHeavyCap, kTcFew, C).bytes; }
+
 nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                           const nb_aux* aux, const ScoreOut& o, cudaStream_t st) {
   TcArgs a{};
@@ -1477,19 +1492,17 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
   a.recheck = o.recheck;
   a.status = m->d.sstatus;
   a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
-  // scratch of this call, stream-ordered: the count of heavy rows and the row
-  // groups' counters (cleared), the list, the sums of up to kTcFew rows.  FP8 and
-  // BF16 rows list no more than those (the chunked pass reads u8 rows only);
+  // FP8 and BF16 rows list no more than those (the chunked pass reads u8 rows only);
   // what is not listed stays marked for the FP64 recheck.
   const int most = u8 ? kTcHeavyCap : kTcFew;
   const int cap = n < most ? (int)n : most, few = cap < kTcFew ? cap : kTcFew;
-  const size_t groups = ((size_t)few + 3) / 4, clear = 16 + 4 * (groups + 3) / 4 * 4;
-  const size_t o_list = (clear + 15) / 16 * 16, o_sums = o_list + 8 * (size_t)cap,
-               o_T = o_sums + 32 * groups * m->C;
+  const TcScratch lay(cap, few, m->C);
+  ScoreScratch ss(m, st);
   char* scratch = nullptr;
-  NB_TRY_CUDA(cudaMallocAsync(&scratch, o_T + 16 * groups, st), "cudaMallocAsync(heavy rows)");
+  nb_status s = ss.take(lay.bytes, m->d.tc_scratch, tc_scratch_bytes(m->C), &scratch);
+  if (s != NB_OK) return s;
   a.heavy_n = reinterpret_cast<unsigned long long*>(scratch);
-  a.heavy = reinterpret_cast<long long*>(scratch + o_list);
+  a.heavy = reinterpret_cast<int*>(scratch + lay.list);
   a.heavy_cap = cap;
   TcHeavyArgs h{};
   h.X = g.X;
@@ -1505,15 +1518,14 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
   h.heavy = a.heavy;
   h.heavy_n = a.heavy_n;
   h.heavy_cap = cap;
-  h.sums = reinterpret_cast<long long*>(scratch + o_sums);
-  h.T = reinterpret_cast<float*>(scratch + o_T);
+  h.sums = reinterpret_cast<long long*>(scratch + lay.sums);
+  h.T = reinterpret_cast<float*>(scratch + lay.T);
   h.done = reinterpret_cast<unsigned int*>(scratch + 16);
   h.label = o.label;
   h.margin = o.margin;
   h.logpost = o.logpost;
   h.marks = a.marks;
-  const cudaError_t me = cudaMemsetAsync(scratch, 0, clear, st);
-  nb_status s = me == cudaSuccess ? NB_OK : cuda_status(me, "memset(heavy count)");
+  NB_TRY_CUDA(cudaMemsetAsync(scratch, 0, lay.clear, st), "memset(heavy count)");
   if (s == NB_OK)
     s = u8                   ? run_tc<0, NB_U8>(a, a.models[0].N, a.units0, st)
         : dt == NB_FP8E4M3 ? run_tc<0, NB_FP8E4M3>(a, a.models[0].N, a.units0, st)
@@ -1523,10 +1535,8 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
         : dt == NB_FP8E4M3 ? run_tc_heavy<NB_FP8E4M3>(h, st)
                              : run_tc_heavy<NB_BF16>(h, st);
   if (s == NB_OK && u8 && cap > kTcFew) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
-  const cudaError_t fe = cudaFreeAsync(scratch, st);
-  if (s != NB_OK) return s;
-  NB_TRY_CUDA(fe, "cudaFreeAsync(heavy rows)");
-  return NB_OK;
+  const nb_status f = ss.release();
+  return s != NB_OK ? s : f;
 }
 
 // tensor map of a group's rows (es bytes per feature) for a batch work list

@@ -1,5 +1,5 @@
 """Many-class rows of 2^17 and more counts: the exact sums on the CUDA cores (up to
-4,096 such rows a call) and, above that for u8, the chunked tensor-core pass.
+1,024 such rows a call) and, above that for u8, the chunked tensor-core pass.
 
 A row's sums are exact integers, so labels equal the FP64 oracle's and the log
 posteriors lie within the library's 1e-5; none of these rows needs FP64 unless the
@@ -49,7 +49,7 @@ def test_few_heavy_rows_are_exact(fmt, F, C, every):
     del yd
 
 
-@pytest.mark.parametrize("n", [4096, 4100])
+@pytest.mark.parametrize("n", [1024, 1030])
 def test_the_limit_between_the_two_passes(n):
     X, y = _heavy("u8", n, 520, 5, 1, seed=3)
     f, vals = stored(X, "u8")
@@ -57,3 +57,20 @@ def test_the_limit_between_the_two_passes(n):
     _, ref = oracle_mn(vals, y, 5, vals)
     res = to_np(nb.score(model, f))
     compare(res, ref)
+
+
+def test_calls_on_two_streams_do_not_share_scratch():
+    """A model's own scratch serves one call at a time; a second stream gets other memory."""
+    X, y = _heavy("u8", 3000, 520, 5, 3, seed=8)
+    f, vals = stored(X, "u8")
+    model = nb.fit(f, torch.from_numpy(y).cuda(), 5)
+    _, ref = oracle_mn(vals, y, 5, vals)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = []
+    for k in range(9):
+        with torch.cuda.stream(streams[k % 3]):
+            outs.append(nb.score(model, f, stream=streams[k % 3]))
+    torch.cuda.synchronize()
+    for o in outs:
+        compare(to_np(o), ref)
