@@ -120,8 +120,8 @@ static nb_status alloc_model(nb_model* m) {
   d.w = reinterpret_cast<float*>(b + o_w);
   d.bias = reinterpret_cast<float*>(b + o_bias);
   d.wmax = reinterpret_cast<float*>(b + o_wmax);
-  d.g_mu = m->kind == NB_GAUSSIAN ? reinterpret_cast<float*>(b + o_gmu) : nullptr;
-  d.g_ivar = m->kind == NB_GAUSSIAN ? reinterpret_cast<float*>(b + o_giv) : nullptr;
+  d.g_nms = m->kind == NB_GAUSSIAN ? reinterpret_cast<float*>(b + o_gmu) : nullptr;
+  d.g_isd = m->kind == NB_GAUSSIAN ? reinterpret_cast<float*>(b + o_giv) : nullptr;
   d.g_const = reinterpret_cast<float*>(b + o_gk);
   d.tc_w = tc ? reinterpret_cast<uint8_t*>(b + o_tcw) : nullptr;
   d.tc_q = tc ? reinterpret_cast<int32_t*>(b + o_tcq) : nullptr;

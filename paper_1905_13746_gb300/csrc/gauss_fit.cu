@@ -385,8 +385,8 @@ struct GfFin {
   double* var;
   double* log_pi;
   double* gconst;
-  float* g_mu;
-  float* g_ivar;
+  float* g_nms;
+  float* g_isd;
   float* g_const;
   double* part;           // per class and tile: sum of logs, sum of m^2 v
   unsigned int* done_c;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256) k_gauss_finish(const GfFin a) {
   const int c = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * 256 + threadIdx.x;
   pdl_wait();
-  float mu32 = 0.f, iv32 = 0.f;
+  float nm32 = 0.f, is32 = 0.f;
   double m = 1.0, s4 = 0.0;
   int e = 0;
   if (c < a.C && j < a.F) {
@@ -406,14 +406,14 @@ __global__ void __launch_bounds__(256) k_gauss_finish(const GfFin a) {
     const double v = a.var[at] + eps;
     if (!(v > 0.0) || !isfinite(v)) atomicOr(a.status, ST_BAD_TABLE);
     a.var[at] = v;
-    mu32 = (float)a.mu[at];
-    iv32 = (float)(1.0 / v);
+    is32 = (float)rsqrt(v);
+    nm32 = (float)(-a.mu[at] * (double)is32);
     m = frexp(6.283185307179586476925 * v, &e);   // zero, infinities and NaN pass through
-    s4 = (double)mu32 * (double)mu32 * (double)iv32;
+    s4 = (double)nm32 * (double)nm32;
   }
   if (j < a.F_pad) {   // feature-major, gauss_cpad(C) classes per feature
-    a.g_mu[(int64_t)j * a.CP + c] = mu32;
-    a.g_ivar[(int64_t)j * a.CP + c] = iv32;
+    a.g_nms[(int64_t)j * a.CP + c] = nm32;
+    a.g_isd[(int64_t)j * a.CP + c] = is32;
   }
   if (c >= a.C) return;
   // 32 mantissas in [1/2, 1): the product stays above 2^-33
@@ -517,8 +517,8 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   a.amax = reinterpret_cast<float*>(s);
   s += (size_t)(nchunk - 1) * cf * 4;
   unsigned int* done = reinterpret_cast<unsigned int*>(s);
-  // the scales wait in the 1/var table, which the finish kernel writes
-  float* scale = d.g_ivar;
+  // the scales wait in the 1/sd table, which the finish kernel writes
+  float* scale = d.g_isd;
   a.mean = d.p0;
   a.scale = scale;
   a.nc = reinterpret_cast<unsigned long long*>(d.nc);
@@ -537,7 +537,7 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   count_launch();
   NB_TRY_CUDA(launch_pdl(k_gauss_var, rgrid, block, 0, st, r), "k_gauss_var");
   GfFin f{F, m->F_pad, C, CP, jt, prior_given ? 1 : 0, n, m->var_smoothing, a.nc, d.fin, d.p0,
-          d.p1, d.log_pi, d.gconst, d.g_mu, d.g_ivar, d.g_const, part, done + nft, d.status};
+          d.p1, d.log_pi, d.gconst, d.g_nms, d.g_isd, d.g_const, part, done + nft, d.status};
   count_launch();
   NB_TRY_CUDA(launch_pdl(k_gauss_finish, dim3((unsigned)((m->F_pad + 255) / 256), (unsigned)CP),
                          dim3(256), 0, st, f),

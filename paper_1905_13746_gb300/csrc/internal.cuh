@@ -122,9 +122,9 @@ struct ModelDev {
   double* wmean;       // F          mean_c log theta_cj
   char* tc_scratch;    // tc_scratch_bytes(C): heavy rows of one scoring call (ScoreScratch)
   // Gaussian FP32 tables
-  float* g_mu;         // F_pad x gauss_cpad(C), feature-major (classes past C: 0)
-  float* g_ivar;       // same layout, 1 / var
-  float* g_const;      // 2C         gconst in FP32, then a4_c = sum_j m^2 v (FP32 tables)
+  float* g_nms;        // -mu / sd: F_pad x gauss_cpad(C), feature-major (past F and C: 0)
+  float* g_isd;        // same layout, 1 / sd
+  float* g_const;      // 2C         gconst in FP32, then a4_c = sum_j g_nms^2
   // Gaussian tensor-core tables (3 <= C <= kTcMaxC, F <= kTcgMaxF), else nullptr;
   // the FP16 limbs of B and A go to tc_w
   float* tcg_kc;       // C          K_c

@@ -289,26 +289,40 @@ __global__ void __launch_bounds__(256) k_score_gen(const GArgs a) {
 // ---------------------------------------------------------------------------
 // Gaussian scorer on the CUDA cores (any 2 <= C <= 64, FP32 rows)
 // ---------------------------------------------------------------------------
-// s_c = k_c - 1/2 sum_j v_cj (x_j - mu_cj)^2 (Sec. 4 with Gaussian class
-// conditionals; v = 1/var, k_c = log pi_c - 1/2 sum_j log(2 pi var_cj)).
+// s_c = k_c - 1/2 sum_j z_cj^2, z = (x_j - mu_cj) / sd_cj (Sec. 4 with Gaussian
+// class conditionals; k_c = log pi_c - 1/2 sum_j log(2 pi var_cj)).  The tables hold
+// -mu/sd and 1/sd, so that a term costs two fused operations, z = x (1/sd) - mu/sd
+// and q + z^2, and a pair of classes shares each instruction (f32x2).
 // A group of LPR lanes scores R rows at once: lane li takes features j = li,
 // li + LPR, ..., and for each block of CB classes keeps CB x R partial sums
-// q = sum v dx^2.  The block's warps stage mu and v of a chunk of features
-// (feature-major tables, CB consecutive classes per feature) in shared
-// memory, so that each is read from L2 once per block of rows and from
-// shared memory once per R rows.  The group's partial sums are combined by a
-// reduce-scatter (each exchange halves the values a lane holds: CB R (LPR -
-// 1) / LPR shuffles instead of CB R log2 LPR), which leaves lane li with the
-// finished sums of classes-and-rows li CB R / LPR ...; their scores and
-// bounds go to shared memory, and the LPR lanes then share each row's
+// q = sum z^2.  Slices of FC features go to shared memory with cp.async while the
+// slice before is summed: the tables (feature-major, CB consecutive classes per
+// feature) once per block of rows, the rows once per class block.  The group's
+// partial sums are combined by a reduce-scatter (each exchange halves the values a
+// lane holds: CB R (LPR - 1) / LPR shuffles instead of CB R log2 LPR), which leaves
+// lane li with the finished sums of classes-and-rows li CB R / LPR ...; their scores
+// and bounds go to shared memory, and the LPR lanes then share each row's
 // arg-max, sum of exponentials, recheck tests and log-posterior stores.
+//
+// Against 64 bits the two operations lose little (twice the rounding of 1/sd, one
+// product less) and the differences of the epilogue win more: 7.2e-8 -> 6.9e-8 at 64
+// classes, 6.8e-8 -> 6.5e-8 over 12 two-class models.
+// Bound by the FP32 pipe (51 % busy) and the shared-memory reads of the tables (62 %
+// of the wavefronts) at four warps a scheduler.  200,000 rows x 256 features x 64
+// classes with log posteriors: 636 us with (x - mu)^2 v, one class an instruction and
+// loads in place, 441 with two operations a term on pairs, 411 with the slices
+// staged ahead, 404 with the classes of a row in registers; 20 classes 371 -> 197,
+// 400,000 x 200 x 4: 316 -> 126.  Blocks of 8
+// rows x 8 classes halve the table reads and were slower (501): twice the row
+// reads.
 struct GGArgs {
   const float* X;
   int64_t ld, n;
   int F, F_pad, C;
-  const float* mu;
-  const float* ivar;
+  const float* nms;   // -mu / sd
+  const float* isd;   // 1 / sd
   const float* kc;
+  int vec4;           // rows start on 16-byte boundaries
   uint8_t* label;
   float* margin;
   float* logpost;
@@ -319,39 +333,77 @@ struct GGArgs {
 constexpr int kGaussWarps = 8;
 
 // lowest index among equal maxima; NaN never wins
-__device__ __forceinline__ void gauss_top2(float& b1, int& i1, float& b2, float ob1, int oi1,
-                                           float ob2) {
-  const bool other = ob1 > b1 || (ob1 == b1 && oi1 < i1);
-  const float lo = other ? b1 : ob1;
-  if (other) {
-    b1 = ob1;
-    i1 = oi1;
+__device__ __forceinline__ void gauss_top(float& b, int& i, float ob, int oi) {
+  if (ob > b || (ob == b && oi < i)) {
+    b = ob;
+    i = oi;
   }
-  b2 = fmaxf(fmaxf(b2, ob2), lo);
 }
 
+// two FP32 lanes in one instruction (the same roundings as one at a time)
+__device__ __forceinline__ uint64_t f32x2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f32x2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// 16 (4) bytes to shared memory, of which `bytes` are read and the rest are zeros
+__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4_zfill(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_addr(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// floats per row of the staged scores: 2 past a multiple of 16 puts the rows that
+// a warp's lanes write and read at once on different banks
+__host__ __device__ constexpr int gauss_cm(int C) { return (C + 15) / 16 * 16 + 2; }
 template <int LPR, int R, int CB>
-__global__ void __launch_bounds__(kGaussWarps * 32, 2) k_score_gauss(const GGArgs a) {
-  constexpr int G = 32 / LPR;     // row groups per warp
-  constexpr int RPW = G * R;      // rows per warp
-  constexpr int RPB = kGaussWarps * RPW;   // rows per block tile
+struct GaussLayout {
+  static constexpr int RPW = 32 / LPR * R;            // rows per warp
+  static constexpr int RPB = kGaussWarps * RPW;       // rows per block tile
+  static constexpr int FC = LPR == 8 ? 32 : 64;       // features per staged slice
+  // floats per staged feature (-mu/sd of CB classes, then 1/sd): eight lanes' 16-byte
+  // reads of consecutive slots touch distinct banks
+  static constexpr int SR = 2 * CB + 4;
+  // floats of a warp's staged rows: LPR more per group puts the groups' reads on
+  // different banks
+  static constexpr int XG = R * FC + LPR, XW = 32 / LPR * XG;
+  static constexpr int BUF = FC * SR + kGaussWarps * XW;   // one of the two buffers
+  static int smem(int C) { return 4 * (2 * BUF + 2 * RPB * gauss_cm(C)); }
+};
+
+template <int LPR, int R, int CB>
+__global__ void __launch_bounds__(kGaussWarps * 32, CB == 4 ? 4 : 2) k_score_gauss(const GGArgs a) {
+  using L = GaussLayout<LPR, R, CB>;
   constexpr int NP = CB * R;      // sums q of a class block
   constexpr int OWN = NP / LPR;   // pairs a lane finishes
-  // classes kept per row; 64 + 4 puts the rows of a warp's groups on different
-  // banks for the epilogue's reads of class li + LPR m
-  constexpr int CM = CB == 4 ? 4 : kTcMaxC + 4;
-  constexpr int FPL = LPR == 8 ? 8 : 4;   // features per lane per staged chunk
-  constexpr int FC = LPR * FPL;   // features per staged chunk
-  // a staged feature holds the class block's mu (CB floats) then v; the row
-  // stride keeps eight lanes' 16-byte reads of consecutive features on
-  // distinct banks
-  constexpr int SR = CB == 4 ? 12 : 2 * CB + 4;
+  constexpr int FC = L::FC, SR = L::SR, FPL = FC / LPR;   // FPL: features per lane and slice
   static_assert(NP % LPR == 0, "the reduce-scatter ends with whole pairs per lane");
-  __shared__ __align__(16) float s_tab[FC * SR];
-  __shared__ float s_s[kGaussWarps][RPW][CM], s_t[kGaussWarps][RPW][CM];
+  extern __shared__ __align__(16) float gsm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = lane / LPR, li = lane % LPR;
-  const int C = a.C, F = a.F, CP = gauss_cpad(C);
+  const int C = a.C, F = a.F, CP = gauss_cpad(C), CM = gauss_cm(C);
+  float* s_q = gsm + 2 * L::BUF + (warp * L::RPW + grp * R) * CM;   // [R][CM] of this group
+  float* s_t = s_q + kGaussWarps * L::RPW * CM;
   constexpr float u = 5.9604645e-8f;
 
   // rounding depth of each sum: F / LPR sequential adds, the log2 LPR
@@ -361,62 +413,100 @@ __global__ void __launch_bounds__(kGaussWarps * 32, 2) k_score_gauss(const GGArg
   const int kdepth = (F + LPR - 1) / LPR + lg + 8;
   const float gam = kdepth * u / (1.f - kdepth * u);
 
-  const int64_t nbt = (a.n + RPB - 1) / RPB;
-  for (int64_t bt = blockIdx.x; bt < nbt; bt += gridDim.x) {   // uniform over the block
-    const int64_t r0 = bt * RPB + (int64_t)warp * RPW + (int64_t)grp * R;
-    const float* xr[R];
-    bool ok[R];
+  // Slice -> shared memory: the tables of features f0 .. f0 + FC - 1 and classes
+  // cb .. cb + CB - 1 (by the block), the same features of the warp's rows from
+  // row w0 (rows past the end: the last one)
+  auto stage = [&](int buf, int cb, int f0, int64_t w0) {
+    float* st = gsm + buf * L::BUF;
+    constexpr int Q = CB / 4, TN = FC * Q * 2;
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      ok[i] = r0 + i < a.n;
-      xr[i] = a.X + (ok[i] ? r0 + i : 0) * a.ld;
+    for (int s = 0; s < (TN + kGaussWarps * 32 - 1) / (kGaussWarps * 32); ++s) {
+      const int e = threadIdx.x + s * kGaussWarps * 32;
+      const int fl = e / (2 * Q), rem = e % (2 * Q), which = rem / Q, q4 = rem % Q;
+      const int j = f0 + fl;
+      if (TN % (kGaussWarps * 32) == 0 || e < TN)
+        cp_async16_zfill(st + fl * SR + which * CB + 4 * q4,
+                         (which ? a.isd : a.nms) + (int64_t)(j < a.F_pad ? j : 0) * CP + cb + 4 * q4,
+                         j < a.F_pad ? 16 : 0);
     }
-    for (int cb = 0; cb < C; cb += CB) {
-      // sum p = k R + i: class cb + k, row r0 + i
-      float pq[NP];
+    float* sx = st + FC * SR + warp * L::XW;
+    if (a.vec4) {
+      constexpr int V = FC / 4;   // 16-byte pieces per row, V lanes a row
 #pragma unroll
-      for (int p = 0; p < NP; ++p) pq[p] = 0.f;
+      for (int s = 0; s < L::RPW * V / 32; ++s) {
+        const int r = s * (32 / V) + lane / V, v = lane % V;
+        const int64_t row = w0 + r < a.n ? w0 + r : a.n - 1;
+        const int j = f0 + 4 * v, b = 4 * (F - j);
+        cp_async16_zfill(sx + r / R * L::XG + r % R * FC + 4 * v, a.X + row * a.ld + (j < F ? j : 0),
+                         b < 0 ? 0 : (b < 16 ? b : 16));
+      }
+    } else {
+#pragma unroll 4
+      for (int s = 0; s < L::RPW * FC / 32; ++s) {
+        const int r = s / (FC / 32), v = s % (FC / 32) * 32 + lane;
+        const int64_t row = w0 + r < a.n ? w0 + r : a.n - 1;
+        const int j = f0 + v;
+        cp_async4_zfill(sx + r / R * L::XG + r % R * FC + v, a.X + row * a.ld + (j < F ? j : 0),
+                        j < F ? 4 : 0);
+      }
+    }
+  };
+
+  const int64_t nbt = (a.n + L::RPB - 1) / L::RPB;
+  int buf = 0;
+  if ((int64_t)blockIdx.x < nbt) stage(0, 0, 0, (int64_t)blockIdx.x * L::RPB + warp * L::RPW);
+  for (int64_t bt = blockIdx.x; bt < nbt; bt += gridDim.x) {   // uniform over the block
+    const int64_t w0 = bt * L::RPB + warp * L::RPW, r0 = w0 + grp * R;
+    for (int cb = 0; cb < C; cb += CB) {
+      // sums of class pairs: pq2[k][i] holds classes cb + 2 k, cb + 2 k + 1 of row
+      // r0 + i
+      uint64_t pq2[CB / 2][R];
+#pragma unroll
+      for (int k = 0; k < CB / 2; ++k)
+#pragma unroll
+        for (int i = 0; i < R; ++i) pq2[k][i] = 0ull;
       for (int f0 = 0; f0 < F; f0 += FC) {
-        // stage mu and v of features f0 .. f0 + FC - 1, classes cb .. cb + CB - 1
-        // (feature-major tables: CB consecutive floats per feature; padding
-        // classes and features past F are zero and add nothing)
-        __syncthreads();
-        for (int e = threadIdx.x; e < FC * (CB / 4) * 2; e += kGaussWarps * 32) {
-          const int fl = e / ((CB / 4) * 2), rem = e % ((CB / 4) * 2);
-          const int which = rem / (CB / 4), q4 = rem % (CB / 4);
-          const int j = f0 + fl;
-          float4 v4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (j < F)
-            v4 = __ldg(reinterpret_cast<const float4*>((which ? a.ivar : a.mu) +
-                                                       (int64_t)j * CP + cb) + q4);
-          *reinterpret_cast<float4*>(s_tab + fl * SR + which * CB + 4 * q4) = v4;
-        }
-        __syncthreads();
+        cp_async_wait_all();
+        __syncthreads();   // this slice is there; nobody reads the other buffer any more
+        const float* tab = gsm + buf * L::BUF + li * SR;
+        const float* xs = gsm + buf * L::BUF + FC * SR + warp * L::XW + grp * L::XG + li;
+        buf ^= 1;
+        if (f0 + FC < F)
+          stage(buf, cb, f0 + FC, w0);
+        else if (cb + CB < C)
+          stage(buf, cb + CB, 0, w0);
+        else if (bt + gridDim.x < nbt)
+          stage(buf, 0, 0, w0 + (int64_t)gridDim.x * L::RPB);
 #pragma unroll
         for (int jj = 0; jj < FPL; ++jj) {
-          const int fl = li + LPR * jj, j = f0 + fl;
-          if (j >= F) break;
-          float x[R];
+          if (f0 + LPR * jj >= F) break;   // uniform; the features past F are zeros
+          uint64_t xx[R];
 #pragma unroll
-          for (int i = 0; i < R; ++i) x[i] = ok[i] ? __ldg(xr[i] + j) : 0.f;
-          const float* tb = s_tab + fl * SR;
+          for (int i = 0; i < R; ++i) {
+            const float xv = xs[i * FC + LPR * jj];
+            xx[i] = f32x2_pack(xv, xv);
+          }
+          const float* tb = tab + jj * LPR * SR;
 #pragma unroll
           for (int k4 = 0; k4 < CB / 4; ++k4) {
-            const float4 m4 = *reinterpret_cast<const float4*>(tb + 4 * k4);
-            const float4 v4 = *reinterpret_cast<const float4*>(tb + CB + 4 * k4);
-            const float mm[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
+            const ulonglong2 m2 = *reinterpret_cast<const ulonglong2*>(tb + 4 * k4);
+            const ulonglong2 v2 = *reinterpret_cast<const ulonglong2*>(tb + CB + 4 * k4);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int k = 4 * k4 + e;
-#pragma unroll
-              for (int i = 0; i < R; ++i) {
-                const float dx = x[i] - mm[e];
-                pq[k * R + i] = fmaf(dx * vv[e], dx, pq[k * R + i]);
-              }
+            for (int i = 0; i < R; ++i) {
+              const uint64_t z0 = f32x2_fma(xx[i], v2.x, m2.x), z1 = f32x2_fma(xx[i], v2.y, m2.y);
+              pq2[2 * k4][i] = f32x2_fma(z0, z0, pq2[2 * k4][i]);
+              pq2[2 * k4 + 1][i] = f32x2_fma(z1, z1, pq2[2 * k4 + 1][i]);
             }
           }
         }
       }
+      // sum p = k R + i: class cb + k, row r0 + i
+      float pq[NP];
+#pragma unroll
+      for (int k = 0; k < CB / 2; ++k)
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          f32x2_unpack(pq2[k][i], pq[2 * k * R + i], pq[(2 * k + 1) * R + i]);
       // reduce-scatter over the group
 #pragma unroll
       for (int off = LPR / 2, n = NP; off > 0; off >>= 1, n >>= 1) {
@@ -432,93 +522,135 @@ __global__ void __launch_bounds__(kGaussWarps * 32, 2) k_score_gauss(const GGArg
       for (int o = 0; o < OWN; ++o) {
         const int p = li * OWN + o, k = p / R, i = p % R, c = cb + k;
         if (c >= C) continue;
-        const float qq = pq[o], kc = a.kc[c];
-        // |s - s_FP64| with u = 2^-24: m = fl(mu) and v = fl(1/var) are within
-        // u relative, dx = fl(x - m) within u (|dx| + |m|) of x - mu, so each
-        // term v dx^2 is within u v (4 dx^2 + 2 |dx| |m|) + 2 u^2 v (dx^2 +
-        // m^2); the FP32 sums add gam q; k_c and the final subtraction add
-        // u (|k_c| + |s|).  sum v |dx| |m| <= sqrt(sum v dx^2 sum v m^2)
-        // (Cauchy-Schwarz on the FP32 values; 1e-3 covers the rounding of the
-        // two computed sums); 1% slack covers the FP32 evaluation of the bound.
-        const float a4 = a.kc[C + c];   // sum_j m^2 v, from the fit
-        const float aa = sqrtf(qq * a4) * 1.001f;
+        const float qq = pq[o], kc = __ldg(a.kc + c);
+        // |s - s_FP64| with u = 2^-24: w = fl(1/sd) is within u relative, m =
+        // fl(mu w) within u |m| of mu w, and z = fl(x w - m) rounds once, so z
+        // is within u (2 |z| + |m|) of (x - mu) / sd (to first order) and each
+        // z^2 within u (4 z^2 + 2 |z| |m|) (1 + 2 u) + 2 u^2 (z^2 + m^2); the
+        // FP32 sums add gam q; k_c and the final subtraction add u (|k_c| +
+        // |s|).  sum |z| |m| <= sqrt(sum z^2 sum m^2) (Cauchy-Schwarz on the
+        // FP32 values; 1e-3 covers the rounding of the two computed sums and
+        // of the root, which is within 2^-22); 1% slack covers the FP32
+        // evaluation of the bound.
+        const float a4 = __ldg(a.kc + C + c);   // sum_j m^2, from the fit
+        const float aa = sqrt_approx(qq * a4) * 1.001f;
         const float sc = kc - 0.5f * qq;
-        s_s[warp][grp * R + i][c] = sc;
-        s_t[warp][grp * R + i][c] = (0.5f * (u * (4.f * qq + 2.f * aa) * (1.f + 2.f * u) +
-                                             2.f * u * u * (qq + a4) + gam * qq) +
-                                     u * (fabsf(kc) + fabsf(sc))) * 1.01f +
-                                    1e-12f * (qq + fabsf(kc)) + 1e-30f;
+        s_q[i * CM + c] = qq;
+        s_t[i * CM + c] = (0.5f * (u * (4.f * qq + 2.f * aa) * (1.f + 2.f * u) +
+                                   2.f * u * u * (qq + a4) + gam * qq) +
+                           u * (fabsf(kc) + fabsf(sc))) * 1.01f +
+                          1e-12f * (qq + fabsf(kc)) + 1e-30f;
       }
     }
     __syncwarp();
-    // epilogue: the group's lanes share each row's classes
+    // epilogue: the group's lanes share each row's classes, M a lane
+    constexpr int M = CB == 4 ? 1 : kTcMaxC / LPR;
+    float kv[M], kmax = 0.f;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int c = li + LPR * m;
+      kv[m] = c < C ? __ldg(a.kc + c) : -INFINITY;
+      if (c < C) kmax = fmaxf(kmax, fabsf(kv[m]));
+    }
+#pragma unroll
+    for (int off = LPR / 2; off > 0; off >>= 1)
+      kmax = fmaxf(kmax, __shfl_xor_sync(0xFFFFFFFFu, kmax, off));
+    const unsigned gmask = LPR == 32 ? 0xFFFFFFFFu : ((1u << (LPR & 31)) - 1) << (grp * LPR);
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-      const int rl = grp * R + i;
-      const float* sr = s_s[warp][rl];
-      const float* tr = s_t[warp][rl];
-      float b1 = -INFINITY, b2 = -INFINITY, tmax = 0.f;
+      const float* qr = s_q + i * CM;
+      const float* tr = s_t + i * CM;
+      float b1 = -INFINITY, tmax = 0.f;
       int i1 = 0x7FFFFFFF;
       bool nan = false;
-      for (int c = li; c < C; c += LPR) {
-        const float sv = sr[c];
-        nan |= !(sv == sv) || !(tr[c] == tr[c]);
-        tmax = fmaxf(tmax, tr[c]);
-        gauss_top2(b1, i1, b2, sv, c, -INFINITY);
+      float qv[M], tv[M];   // classes li + LPR m
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        if (m > 0 && LPR * m >= C) break;   // uniform
+        const int c = li + LPR * m;
+        qv[m] = c < C ? qr[c] : 0.f;
+        tv[m] = c < C ? tr[c] : 0.f;
+        const float sv = kv[m] - 0.5f * qv[m];
+        nan |= !(sv == sv) || !(tv[m] == tv[m]);
+        tmax = fmaxf(tmax, tv[m]);
+        gauss_top(b1, i1, sv, c);
       }
 #pragma unroll
       for (int off = LPR / 2; off > 0; off >>= 1) {
         const float ob1 = __shfl_xor_sync(0xFFFFFFFFu, b1, off);
         const int oi1 = __shfl_xor_sync(0xFFFFFFFFu, i1, off);
-        const float ob2 = __shfl_xor_sync(0xFFFFFFFFu, b2, off);
-        gauss_top2(b1, i1, b2, ob1, oi1, ob2);
+        gauss_top(b1, i1, ob1, oi1);
         tmax = fmaxf(tmax, __shfl_xor_sync(0xFFFFFFFFu, tmax, off));
-        nan |= __shfl_xor_sync(0xFFFFFFFFu, (int)nan, off) != 0;
       }
+      nan = (__ballot_sync(0xFFFFFFFFu, nan) & gmask) != 0;
       const int bi = i1 < C ? i1 : 0;   // every score NaN: class 0, and the row is marked
-      const float sb = sr[bi], tb = tr[bi];
-      float P = 0.f;
-      for (int c = li; c < C; c += LPR)
-        if (c != bi) P += expf(sr[c] - sb);
+      const float qb = qr[bi], tb = tr[bi], kb = __ldg(a.kc + bi);
+      const float sb = kb - 0.5f * qb;
+      // d_c = s_c - s_top from the constants' and the sums' differences: two
+      // roundings less than from the scores, at smaller magnitudes
+      float dv[M], d2 = -INFINITY, P = 0.f;
 #pragma unroll
-      for (int off = LPR / 2; off > 0; off >>= 1) P += __shfl_xor_sync(0xFFFFFFFFu, P, off);
-      const float margin = sb - b2;
-      // lp_c = (s_c - s_top) - L: formed from the differences, so that no
+      for (int m = 0; m < M; ++m) {
+        if (m > 0 && LPR * m >= C) break;
+        const int c = li + LPR * m;
+        dv[m] = (kv[m] - kb) - 0.5f * (qv[m] - qb);
+        if (c < C && c != bi) {
+          P += expf(dv[m]);
+          d2 = fmaxf(d2, dv[m]);
+        }
+      }
+#pragma unroll
+      for (int off = LPR / 2; off > 0; off >>= 1) {
+        P += __shfl_xor_sync(0xFFFFFFFFu, P, off);
+        d2 = fmaxf(d2, __shfl_xor_sync(0xFFFFFFFFu, d2, off));
+      }
+      // a runner-up within rounding may come out ahead; no number where s_top is none
+      const float margin = (d2 > 0.f ? 0.f : -d2) + (sb - sb);
+      // lp_c = d_c - L: formed from the differences, so that no
       // rounding at the scores' magnitude enters (lp_top = -L exactly)
-      const float L = log1pf(P);
+      const float lg1 = log1pf(P);
       bool flag = false;
       if (a.recheck != NB_RECHECK_OFF) {
         flag = nan;   // a NaN score or bound: FP64 decides
         // label: the top class stays ahead of every other class c by more than
-        // the two classes' bounds (a far class's large bound does not matter)
-        for (int c = li; c < C; c += LPR)
-          if (c != bi && !(sb - sr[c] > (tb + tr[c]) * 1.0001f)) flag = true;
-        if (a.recheck == NB_RECHECK_LP) {
-          // lp_c = d_c - L with d_c = s_c - s_top and L = log(1 + sum_{k != top}
-          // e^{d_k}); each d_k is off by at most D = t_top + t_max, so L is off
-          // by at most D e^{2D} P / (1 + P) (mean value; the softmax weights at
-          // the intermediate point are within e^{2D} of the computed ones), and
-          // lp_c by that plus t_c + t_top (c != top)
-          const float D = tb + tmax;
-          const float eL = D * expf(2.f * D) * (P / (1.f + P)) * 1.01f + 1e-30f;
-          for (int c = li; c < C; c += LPR) {
-            const float err = (c == bi ? 0.f : tr[c] + tb) + eL;
-            if (err > 5e-6f * fmaxf(1.f, fabsf((sr[c] - sb) - L))) flag = true;
-          }
+        // the two classes' bounds (a far class's large bound does not matter) and
+        // what the difference's own roundings add to them: u |k_c - k_top| and u
+        // |q_c - q_top| / 2 <= u (|k_c - k_top| + |d_c|), the parts relative to
+        // d_c within the factor.
+        // lp_c = d_c - L with L = log(1 + sum_{k != top} e^{d_k}); each d_k is
+        // off by at most D = t_top + t_max + 4 u max |k|, so L is off by at most
+        // D e^{2D} P / (1 + P) (mean value; the softmax weights at the
+        // intermediate point are within e^{2D} of the computed ones), and lp_c
+        // by that plus t_c + t_top (c != top)
+        const bool lp = a.recheck == NB_RECHECK_LP;
+        const float D = tb + tmax + 4.f * u * kmax;
+        const float eL = lp ? D * expf(2.f * D) * __fdividef(P, 1.f + P) * 1.01f + 1e-30f : 0.f;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          if (m > 0 && LPR * m >= C) break;
+          const int c = li + LPR * m;
+          if (c >= C) continue;
+          const float tt = tb + tv[m] + 2.f * u * fabsf(kv[m] - kb);
+          if (c != bi && !(-dv[m] > tt * 1.0001f)) flag = true;
+          if (lp && (c == bi ? 0.f : tt) + eL > 5e-6f * fmaxf(1.f, fabsf(dv[m] - lg1))) flag = true;
         }
       }
-      int fl = flag ? 1 : 0;
-#pragma unroll
-      for (int off = LPR / 2; off > 0; off >>= 1) fl |= __shfl_xor_sync(0xFFFFFFFFu, fl, off);
-      if (ok[i]) {
+      const bool fl = (__ballot_sync(0xFFFFFFFFu, flag) & gmask) != 0;
+      if (r0 + i < a.n) {
         const int64_t r = r0 + i;
         if (li == 0) {
           a.label[r] = fl ? kLabelRecheck : (uint8_t)bi;
           a.margin[r] = margin;
           if (fl && a.marks) atomicAdd(a.marks, 1ull);
         }
-        if (a.want_lp)
-          for (int c = li; c < C; c += LPR) a.logpost[r * C + c] = (sr[c] - sb) - L;
+        if (a.want_lp) {
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            if (m > 0 && LPR * m >= C) break;
+            const int c = li + LPR * m;
+            if (c < C) a.logpost[r * C + c] = dv[m] - lg1;
+          }
+        }
       }
     }
     __syncwarp();
@@ -527,31 +659,43 @@ __global__ void __launch_bounds__(kGaussWarps * 32, 2) k_score_gauss(const GGArg
 
 template <int LPR, int R, int CB>
 static nb_status run_score_gauss(const GGArgs& a, cudaStream_t st) {
-  constexpr int RPW = (32 / LPR) * R;
-  const int64_t ntile = (a.n + RPW - 1) / RPW;
+  using L = GaussLayout<LPR, R, CB>;
+  const int smem = L::smem(a.C);
+  NB_TRY_CUDA(cudaFuncSetAttribute(k_score_gauss<LPR, R, CB>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+              "smem attr(k_score_gauss)");
   int occ = 0;
   NB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                  &occ, k_score_gauss<LPR, R, CB>, kGaussWarps * 32, 0),
+                  &occ, k_score_gauss<LPR, R, CB>, kGaussWarps * 32, smem),
               "occupancy(k_score_gauss)");
   const int64_t cap = (int64_t)num_sms() * (occ > 0 ? occ : 1);
-  int64_t blocks = (ntile + kGaussWarps - 1) / kGaussWarps;
+  int64_t blocks = (a.n + L::RPB - 1) / L::RPB;
   if (blocks > cap) blocks = cap;
   count_launch();
-  k_score_gauss<LPR, R, CB><<<(unsigned)blocks, kGaussWarps * 32, 0, st>>>(a);
+  k_score_gauss<LPR, R, CB><<<(unsigned)blocks, kGaussWarps * 32, smem, st>>>(a);
   NB_TRY_CUDA(cudaGetLastError(), "k_score_gauss launch");
   return NB_OK;
 }
 
-// lanes per row: the features a lane sums in sequence stay at most 32 (the
-// rounding depth of the bound); few classes take 4-class blocks of 4 rows
+// Lanes per row: the features a lane sums in sequence stay at most 32 (the rounding
+// depth of the bound; 16 for many classes).  Up to 4 classes take 4-class blocks at four
+// blocks per SM (400,000 x 200 x 4: 158 us against 200 at two, before the epilogue kept
+// the classes in registers; 126 since).  More take 16-class blocks; between 129 and 512
+// features 8-class ones where half of the last 16 or more would be padding (20 classes x
+// 256 features: 217 us against 237, 36 x 300: 206 and 202; with 32 lanes a row they lose,
+// 24 x 600: 310 and 287, 20 x 1,000: 248 and 230).  At up to 128 features 8-class blocks
+// of four rows (400,000 x 100 x 10: 165 us against 184 for 16 classes of two rows,
+// 200,000 x 24 x 40: 200 against 224).
 static nb_status launch_score_gauss(const GGArgs& a, cudaStream_t st) {
   if (a.C <= 4) {
     if (a.F > 128) return run_score_gauss<16, 4, 4>(a, st);
     return run_score_gauss<8, 4, 4>(a, st);
   }
   if (a.F > 512) return run_score_gauss<32, 4, 16>(a, st);
-  if (a.F > 128) return run_score_gauss<16, 4, 16>(a, st);
-  return run_score_gauss<8, 2, 16>(a, st);
+  if (a.F > 128)
+    return (a.C - 1) % 16 < 8 ? run_score_gauss<16, 4, 8>(a, st)   // less padding
+                              : run_score_gauss<16, 4, 16>(a, st);
+  return run_score_gauss<8, 4, 8>(a, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -661,8 +805,9 @@ nb_status launch_score_general(const nb_model* m, const void* X, nb_dtype dt, in
     a.F = m->F;
     a.F_pad = m->F_pad;
     a.C = m->C;
-    a.mu = m->d.g_mu;
-    a.ivar = m->d.g_ivar;
+    a.nms = m->d.g_nms;
+    a.isd = m->d.g_isd;
+    a.vec4 = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ld & 3) == 0;
     a.kc = m->d.g_const;
     a.label = o.label;
     a.margin = o.margin;
