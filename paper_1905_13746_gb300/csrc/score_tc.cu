@@ -188,6 +188,12 @@ __device__ __forceinline__ uint32_t u8x2_to_f16x2(uint32_t w, uint32_t sel) {
   return r;
 }
 
+// two bytes of w -> FP16 subnormals x 2^-24: one permutation, and as exact (the
+// tensor cores keep subnormals; the epilogue multiplies by 2^24)
+__device__ __forceinline__ uint32_t u8x2_to_f16x2_sub(uint32_t w, uint32_t sel) {
+  return __byte_perm(w, 0u, sel);
+}
+
 // two E4M3 values (the low 16 bits of w) -> two exact FP16 values
 __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t w) {
   uint32_t r;
@@ -254,6 +260,7 @@ __device__ __forceinline__ bool tc_wait(TcShared& sh, uint64_t* bar, uint32_t pa
 // guards); the warp follows the outcome together
 __device__ __forceinline__ bool tc_wait_warp(TcShared& sh, uint64_t* bar, uint32_t parity,
                                              int* status) {
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;   // no clock read
   const bool mine = tc_wait_sleep(bar, parity);
   const bool all = __all_sync(0xFFFFFFFFu, mine) != 0;
   if (!all && (threadIdx.x & 31) == 0) {
@@ -321,7 +328,8 @@ __device__ __forceinline__ void tc_scores8(const SegGroup& G, const TcModelArg& 
                                            uint32_t lane_base, int h, int cb, bool any_ovf,
                                            long long k0, long long k1, float rsc, float (&s)[8],
                                            float (&e)[8], float& added) {
-  const float sc = M.hdr->scale * rsc;   // rsc: the row's power-of-two scale (FP8 rows)
+  // rsc: the accumulators' power-of-two scale (an FP8 row's, a u8 pair pass's 2^24)
+  const float sc = M.hdr->scale * rsc;
   added = 0.f;
   if (MODE == 0) {
     // the three limbs' loads in flight together, one wait
@@ -369,7 +377,7 @@ __device__ __forceinline__ void tc_scores8(const SegGroup& G, const TcModelArg& 
         if (j < F) o += (long long)G.ovf_add[k] * (long long)M.q[(long long)(cb + i) * F + j];
       }
       // the sum joins the score with two roundings (the conversion, the add)
-      const float t = (float)o * sc;
+      const float t = (float)o * M.hdr->scale;   // u8 rows have no scale of their own
       const float si = s[i] + t;
       e[i] += fabsf(t) + fabsf(si);
       s[i] = si;
@@ -818,222 +826,231 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
       return idx < n_heavy ? a.heavy[idx] : -1;
     };
 
-    // chunked pass: the listed rows' bytes come from global memory, TC_PD - 1
-    // A stages ahead of the conversion
-    long long l_i = 0;
-    int l_ka = 0, l_g = 0;
-    long long l_row = (MODE == 1 && total > 0) ? row_of(0, l_g) : -1;
-    const unsigned char* l_rp =
-        l_row >= 0 ? reinterpret_cast<const unsigned char*>(tc_group(a, l_g).X) +
-                         l_row * tc_group(a, l_g).ld_bytes
-                   : nullptr;
-    auto load_next = [&](uint4& dst) {
-      const int f = PS::KA * l_ka + PS::BPT * part;
-      // the same bytes a.pf stages on are fetched into L2 now
-      if (l_rp && f + PS::KA * a.pf < F)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(l_rp + f + PS::KA * a.pf));
-      uint4 x = make_uint4(0, 0, 0, 0);
-      if (l_rp && f < F) {
-        x = ld_stream16(l_rp + f);
-        if (f + 16 > F) {   // zero the bytes past F
-          const int keep = F - f;
-          uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int vb = keep - 4 * k;
-            w[k] &= vb >= 4 ? 0xFFFFFFFFu : (vb <= 0 ? 0u : ((1u << (8 * vb)) - 1u));
-          }
-          x = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-      dst = x;
-      if (++l_ka == nka) {
-        l_ka = 0;
-        if (++l_i < my_units) {
-          l_row = row_of(l_i, l_g);
-          const SegGroup& G = tc_group(a, l_g);
-          l_rp = l_row >= 0 ? reinterpret_cast<const unsigned char*>(G.X) + l_row * G.ld_bytes
-                            : nullptr;
-        } else {
-          l_rp = nullptr;
-        }
-      }
-    };
-    uint4 buf[MODE == 1 ? TC_PD : 1];
-    if constexpr (MODE == 1) {
-#pragma unroll
-      for (int d = 0; d < TC_PD - 1; ++d)
-        if (d < total) load_next(buf[d]);
-    }
-    long long ri = 0;   // pair pass: row stages consumed
     const uint32_t raw_s = smem_addr(raw) + (uint32_t)(h * TC_M * TC_BOX);
     const int rr = 32 * qd + lane;   // row within the tile
     constexpr int RAW_A = BOXF / PS::KA;     // A stages per row stage
     constexpr int NVT = PS::NV * ES;         // 16-byte chunks per thread per A stage
     constexpr int CPA = PS::KA * ES / 16;    // 16-byte chunks of a row per A stage
-    // FP8 / BF16 rows: the magic pair of the count check, and the row's flag
-    // and scale (set at the start of each unit)
-    uint32_t m2 = 0x64006400u, bad = 0u;
-    float rsc = 1.f;
-
-    // consumer state
-    long long c_i = 0;
-    int c_ka = 0, kc = 0;
-    uint32_t T = 0;
-    for (long long base = 0; base < total && ok; base += TC_PD) {
-#pragma unroll
-      for (int d = 0; d < TC_PD; ++d) {
-        if (base + d >= total || !ok) break;
-        if (tc_aborted(sh)) {
-          ok = false;
-          break;
+    if constexpr (MODE == 0) {
+      // Pair pass: a row stage at a time.  Its bytes are read and converted (RAW_A A
+      // stages), the row stage is handed back, and the A stages go to tensor memory as
+      // their slots come free.
+      static_assert(PS::NA == 2 && TC_NRAW == 2, "slot and phase from the counters' low bits");
+      const int nrs = (nka + RAW_A - 1) / RAW_A;
+      uint32_t as = 0, rs = 0;   // A stages written, row stages read
+      for (long long it = 0; it < my_units && ok; ++it) {
+        uint32_t T = 0, m2 = 0x64006400u, bad = 0u;
+        float rsc = DT == NB_U8 ? 16777216.f : 1.f;   // u8: subnormals x 2^-24
+        if (DT == NB_FP8E4M3) {
+          // this thread's row scale (2^e, e in {0, 1}; any other exponent sends the
+          // row to the FP64 recheck)
+          int g = 0;
+          const long long r = row_of(it, g);
+          const int8_t* re = tc_group(a, g).row_exp;
+          const int e = (re && r >= 0) ? (int)re[r] : 0;
+          if (e == 1) {
+            m2 = 0x60006000u;
+            rsc = 2.f;
+          } else if (e != 0) {
+            bad = 1u;
+          }
         }
-        uint4 xv[NVT];
-        if constexpr (MODE == 1) {
-          if (base + d + TC_PD - 1 < total) load_next(buf[(d + TC_PD - 1) % TC_PD]);
-          xv[0] = buf[d];
-        } else {
-          // this thread's bytes of the A stage: 16-byte chunks of its row in
-          // the row stage, swizzled by the row (rows and features past the end
-          // arrive as zeros)
-          const uint32_t slot = (uint32_t)(ri % TC_NRAW);
-          if (c_ka % RAW_A == 0 &&
-              !tc_wait_warp(sh, &sh.raw_full[slot], (uint32_t)((ri / TC_NRAW) & 1), a.status)) {
+#pragma unroll 1
+        for (int k = 0; k < nrs; ++k, ++rs) {
+          if (tc_aborted(sh) ||
+              !tc_wait_warp(sh, &sh.raw_full[rs & 1], (rs >> 1) & 1, a.status)) {
             ok = false;
             break;
           }
+          // this thread's bytes of the row stage: 16-byte chunks of its row, swizzled
+          // by the row (rows and features past the end arrive as zeros)
+          const uint32_t src = raw_s + (rs & 1) * TC_RAW_BYTES + (uint32_t)(rr * TC_BOX);
+          uint32_t o[RAW_A][PS::COLS];
 #pragma unroll
-          for (int v = 0; v < NVT; ++v) {
-            const int c16 = CPA * (c_ka % RAW_A) + NVT * part + v;
-            xv[v] = lds16(raw_s + slot * TC_RAW_BYTES +
-                          (uint32_t)(rr * TC_BOX + ((c16 ^ (rr & 7)) << 4)));
-          }
-        }
-        if (DT != NB_U8 && c_ka == 0) {
-          // a new unit: this thread's row scale (FP8 rows: 2^e, e in {0, 1};
-          // any other exponent sends the row to the FP64 recheck)
-          bad = 0u;
-          m2 = 0x64006400u;
-          rsc = 1.f;
-          if (DT == NB_FP8E4M3) {
-            int g = 0;
-            const long long r = row_of(c_i, g);
-            const int8_t* re = tc_group(a, g).row_exp;
-            const int e = (re && r >= 0) ? (int)re[r] : 0;
-            if (e == 1) {
-              m2 = 0x60006000u;
-              rsc = 2.f;
-            } else if (e != 0) {
-              bad = 1u;
-            }
-          }
-        }
-        // convert this thread's values to FP16 pairs
-        uint32_t o[PS::COLS];
-        if constexpr (DT == NB_U8) {
+          for (int sub = 0; sub < RAW_A; ++sub) {
 #pragma unroll
-          for (int v = 0; v < NVT; ++v) {
-            const uint4 x = xv[v];
-            T = dp4a_uu(x.x, 0x01010101u, T);
-            T = dp4a_uu(x.y, 0x01010101u, T);
-            T = dp4a_uu(x.z, 0x01010101u, T);
-            T = dp4a_uu(x.w, 0x01010101u, T);
-            o[8 * v + 0] = u8x2_to_f16x2(x.x, 0x5140u);
-            o[8 * v + 1] = u8x2_to_f16x2(x.x, 0x7362u);
-            o[8 * v + 2] = u8x2_to_f16x2(x.y, 0x5140u);
-            o[8 * v + 3] = u8x2_to_f16x2(x.y, 0x7362u);
-            o[8 * v + 4] = u8x2_to_f16x2(x.z, 0x5140u);
-            o[8 * v + 5] = u8x2_to_f16x2(x.z, 0x7362u);
-            o[8 * v + 6] = u8x2_to_f16x2(x.w, 0x5140u);
-            o[8 * v + 7] = u8x2_to_f16x2(x.w, 0x7362u);
-          }
-        } else {
+            for (int v = 0; v < NVT; ++v) {
+              const uint4 x = lds16(src + (uint32_t)(((CPA * sub + NVT * part + v) ^ (rr & 7)) << 4));
+              const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-          for (int v = 0; v < NVT; ++v) {
-            const uint32_t w[4] = {xv[v].x, xv[v].y, xv[v].z, xv[v].w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if constexpr (DT == NB_FP8E4M3) {
-                o[8 * v + 2 * k] = e4m3x2_to_f16x2(w[k] & 0xFFFFu);
-                o[8 * v + 2 * k + 1] = e4m3x2_to_f16x2(w[k] >> 16);
-              } else {
-                o[4 * v + k] = bf16x2_to_f16x2(w[k]);
-                bad |= bf16x2_tiny(w[k]);
+              for (int q = 0; q < 4; ++q) {
+                if constexpr (DT == NB_U8) {
+                  T = dp4a_uu(w[q], 0x01010101u, T);
+                  o[sub][8 * v + 2 * q] = u8x2_to_f16x2_sub(w[q], 0x4140u);
+                  o[sub][8 * v + 2 * q + 1] = u8x2_to_f16x2_sub(w[q], 0x4342u);
+                } else if constexpr (DT == NB_FP8E4M3) {
+                  o[sub][8 * v + 2 * q] = e4m3x2_to_f16x2(w[q] & 0xFFFFu);
+                  o[sub][8 * v + 2 * q + 1] = e4m3x2_to_f16x2(w[q] >> 16);
+                } else {
+                  o[sub][4 * v + q] = bf16x2_to_f16x2(w[q]);
+                  bad |= bf16x2_tiny(w[q]);
+                }
               }
             }
-          }
-          // every value an integer count x = v 2^e below 1024: x sits in the
-          // low 10 bits of v + M; T sums M + x (at most 2^15 + 2^10 for each of
-          // 32 values per A stage: no wrap below 2^32 for F <= 8192)
+            // every value an integer count x = v 2^e below 1024: x sits in the low 10
+            // bits of v + M; T sums M + x (at most 2^15 + 2^10 for each of 32 values
+            // per A stage: no wrap below 2^32 for F <= 8192)
+            if constexpr (DT != NB_U8) {
 #pragma unroll
-          for (int k = 0; k < PS::COLS; ++k) f16x2_count_check(o[k], m2, T, bad);
-        }
-        if constexpr (MODE == 0) {
-          if (c_ka % RAW_A == RAW_A - 1 || c_ka == nka - 1) {   // done with the row stage
+              for (int q = 0; q < PS::COLS; ++q) f16x2_count_check(o[sub][q], m2, T, bad);
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.raw_empty[rs & 1]);
+#pragma unroll
+          for (int sub = 0; sub < RAW_A; ++sub) {
+            if (RAW_A * k + sub >= nka) break;
+            if (!tc_wait_warp(sh, &sh.a_empty[as & 1], ((as >> 1) & 1) ^ 1u, a.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            tmem_st16(lane_base + a_col + (as & 1) * (uint32_t)(PS::ACOLS * PS::H), o[sub]);
+            tmem_st_wait();
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.raw_empty[ri % TC_NRAW]);
-            ++ri;
+            if (lane == 0) mbar_arrive(&sh.a_full[as & 1]);
+            ++as;
+          }
+          if (!ok) break;
+        }
+        if (!ok) break;
+        if (!tc_wait_warp(sh, &sh.acc_full, (uint32_t)(it & 1), a.status)) break;
+        tc_fence_after();
+        int g = 0;
+        const long long r = row_of(it, g);
+        const SegGroup& G = tc_group(a, g);
+        // FP8 / BF16: the unit's check; then the counts' total without the bias M of
+        // each of the 2 COLS values of every A stage (RAW_A of every row stage)
+        if (DT != NB_U8)
+          T = bad != 0u ? 0xFFFFFFFFu
+                        : T - (m2 & 0xFFFFu) * (uint32_t)(2 * PS::COLS) * (uint32_t)(RAW_A * nrs);
+        if (!tc_epilogue<MODE>(a, sh, xe, G, a.models[G.model], r, xr, h, part, T, rsc, lane_base,
+                               ep))
+          break;
+        tc_fence_before();   // the accumulators are read: the next unit's MMAs may start
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.acc_empty);
+      }
+    } else {
+      // chunked pass: the listed rows' bytes come from global memory, TC_PD - 1
+      // A stages ahead of the conversion
+      long long l_i = 0;
+      int l_ka = 0, l_g = 0;
+      long long l_row = total > 0 ? row_of(0, l_g) : -1;
+      const unsigned char* l_rp =
+          l_row >= 0 ? reinterpret_cast<const unsigned char*>(tc_group(a, l_g).X) +
+                           l_row * tc_group(a, l_g).ld_bytes
+                     : nullptr;
+      auto load_next = [&](uint4& dst) {
+        const int f = PS::KA * l_ka + PS::BPT * part;
+        // the same bytes a.pf stages on are fetched into L2 now
+        if (l_rp && f + PS::KA * a.pf < F)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(l_rp + f + PS::KA * a.pf));
+        uint4 x = make_uint4(0, 0, 0, 0);
+        if (l_rp && f < F) {
+          x = ld_stream16(l_rp + f);
+          if (f + 16 > F) {   // zero the bytes past F
+            const int keep = F - f;
+            uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int vb = keep - 4 * k;
+              w[k] &= vb >= 4 ? 0xFFFFFFFFu : (vb <= 0 ? 0u : ((1u << (8 * vb)) - 1u));
+            }
+            x = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
-        const int aslot = (int)(ai % PS::NA);
-        if (!tc_wait_warp(sh, &sh.a_empty[aslot], (uint32_t)((ai / PS::NA) & 1) ^ 1u,
-                          a.status)) {
-          ok = false;
-          break;
+        dst = x;
+        if (++l_ka == nka) {
+          l_ka = 0;
+          if (++l_i < my_units) {
+            l_row = row_of(l_i, l_g);
+            const SegGroup& G = tc_group(a, l_g);
+            l_rp = l_row >= 0 ? reinterpret_cast<const unsigned char*>(G.X) + l_row * G.ld_bytes
+                              : nullptr;
+          } else {
+            l_rp = nullptr;
+          }
         }
-        tc_fence_after();
-        if constexpr (PS::COLS == 16) tmem_st16(lane_base + a_col + (uint32_t)(aslot * PS::ACOLS * PS::H), o);
-        else tmem_st8(lane_base + a_col + (uint32_t)(aslot * PS::ACOLS * PS::H), o);
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.a_full[aslot]);
-        ++ai;
-        const bool unit_end = c_ka == nka - 1;
-        if (++kc == chunk || unit_end) {
-          // the accumulation cycle is complete: drain (chunked) and / or run
-          // the epilogue of the unit
-          kc = 0;
-          if (!tc_wait_warp(sh, &sh.acc_full, (uint32_t)(ci & 1), a.status)) {
+      };
+      uint4 buf[TC_PD];
+#pragma unroll
+      for (int d = 0; d < TC_PD - 1; ++d)
+        if (d < total) load_next(buf[d]);
+      // consumer state
+      long long c_i = 0;
+      int c_ka = 0, kc = 0;
+      uint32_t T = 0;
+      for (long long base = 0; base < total && ok; base += TC_PD) {
+#pragma unroll
+        for (int d = 0; d < TC_PD; ++d) {
+          if (base + d >= total || !ok) break;
+          if (tc_aborted(sh)) {
+            ok = false;
+            break;
+          }
+          if (base + d + TC_PD - 1 < total) load_next(buf[(d + TC_PD - 1) % TC_PD]);
+          const uint4 x = buf[d];
+          // this thread's values as FP16 pairs
+          uint32_t o[PS::COLS];
+          T = dp4a_uu(x.x, 0x01010101u, T);
+          T = dp4a_uu(x.y, 0x01010101u, T);
+          T = dp4a_uu(x.z, 0x01010101u, T);
+          T = dp4a_uu(x.w, 0x01010101u, T);
+          o[0] = u8x2_to_f16x2(x.x, 0x5140u);
+          o[1] = u8x2_to_f16x2(x.x, 0x7362u);
+          o[2] = u8x2_to_f16x2(x.y, 0x5140u);
+          o[3] = u8x2_to_f16x2(x.y, 0x7362u);
+          o[4] = u8x2_to_f16x2(x.z, 0x5140u);
+          o[5] = u8x2_to_f16x2(x.z, 0x7362u);
+          o[6] = u8x2_to_f16x2(x.w, 0x5140u);
+          o[7] = u8x2_to_f16x2(x.w, 0x7362u);
+          const int aslot = (int)(ai % PS::NA);
+          if (!tc_wait_warp(sh, &sh.a_empty[aslot], (uint32_t)((ai / PS::NA) & 1) ^ 1u,
+                            a.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          if (MODE == 1) {
+          tmem_st8(lane_base + a_col + (uint32_t)(aslot * PS::ACOLS * PS::H), o);
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.a_full[aslot]);
+          ++ai;
+          const bool unit_end = c_ka == nka - 1;
+          if (++kc == chunk || unit_end) {
+            // the accumulation cycle is complete: drain (chunked) and / or run
+            // the epilogue of the unit
+            kc = 0;
+            if (!tc_wait_warp(sh, &sh.acc_full, (uint32_t)(ci & 1), a.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
             tc_drain_chunk(a.models[0].Cp, PS::CPP * part, PS::CPP, c_ka < chunk, lane_base);
             // the chunk's sums are in the int64 columns: the MMAs may go on
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.acc_empty);
-          }
-          if (unit_end) {
-            int g = 0;
-            const long long r = row_of(c_i, g);
-            const SegGroup& G = tc_group(a, g);
-            uint32_t Tu = T;
-            if (DT != NB_U8) {
-              // the unit's check; then the counts' total without the bias M of
-              // each of the 2 COLS values of every A stage
-              Tu = bad != 0u ? 0xFFFFFFFFu
-                        : T - (m2 & 0xFFFFu) * (uint32_t)(2 * PS::COLS) * (uint32_t)nka;
+            if (unit_end) {
+              int g = 0;
+              const long long r = row_of(c_i, g);
+              const SegGroup& G = tc_group(a, g);
+              if (!tc_epilogue<MODE>(a, sh, xe, G, a.models[G.model], r, xr, h, part, T, 1.f,
+                                     lane_base, ep)) {
+                ok = false;
+                break;
+              }
+              T = 0;
             }
-            if (!tc_epilogue<MODE>(a, sh, xe, G, a.models[G.model], r, xr, h, part, Tu, rsc,
-                                   lane_base, ep)) {
-              ok = false;
-              break;
-            }
-            T = 0;
+            ++ci;
           }
-          if (MODE == 0) {   // the accumulators are read: the next unit's MMAs may start
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.acc_empty);
+          if (++c_ka == nka) {
+            c_ka = 0;
+            ++c_i;
           }
-          ++ci;
-        }
-        if (++c_ka == nka) {
-          c_ka = 0;
-          ++c_i;
         }
       }
     }
