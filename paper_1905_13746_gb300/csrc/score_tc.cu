@@ -11,7 +11,8 @@
 // Exactness.  The weights are held in fixed point, Q_cj = round(w_cj 2^S)
 // with |Q| <= 2^22, split into three balanced limbs Q = q0 + 2^8 q1 + 2^16 q2
 // with |q_l| <= 128, each an exact FP16 integer.  Stored u8 counts (0..255)
-// are exact FP16 integers as well, so every product is exact, and a limb's
+// are exact in FP16 as well (the pair pass stores them as subnormals, x 2^-24, and
+// its epilogue multiplies by 2^24), so every product is exact, and a limb's
 // sum over a row stays an integer below 2^24 -- exact in the FP32 accumulator
 // whatever the order of the tensor core's additions -- when the row holds
 // fewer than 2^17 stored counts.  Overflow-list entries (counts above 255) are
@@ -250,7 +251,7 @@ __device__ __forceinline__ bool tc_aborted(TcShared& sh) {
 }
 
 __device__ __forceinline__ bool tc_wait(TcShared& sh, uint64_t* bar, uint32_t parity, int* status) {
-  if (tc_wait_sleep(bar, parity)) return true;
+  if (mbar_try_wait(bar, parity) || tc_wait_sleep(bar, parity)) return true;
   atomicOr(status, ST_TIMEOUT);
   *reinterpret_cast<volatile int*>(&sh.abort) = 1;
   return false;
@@ -268,6 +269,15 @@ __device__ __forceinline__ bool tc_wait_warp(TcShared& sh, uint64_t* bar, uint32
     *reinterpret_cast<volatile int*>(&sh.abort) = 1;
   }
   return all;
+}
+
+// 1 in one lane of the warp (every lane calls it)
+__device__ __forceinline__ uint32_t tc_elect() {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(r));
+  return r;
 }
 
 // D[tmem] (+)= A[tmem] * B[smem]^T, issued by one thread (A: 128 lanes = rows,
@@ -660,8 +670,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
   if (warp == TC_WORK) {
     // ---- weight-limb producer -----------------------------------------
     if (lane == 0) {
-      long long bi = 0, last[TC_NB];
-      for (int s = 0; s < TC_NB; ++s) last[s] = -1;
+      int slot = 0, filled = 0;   // ring position; slots that have been filled
+      uint32_t ph = 0;
       bool ok = true;
       for (long long it = 0; it < my_units && ok && !tc_aborted(sh); ++it) {
         const long long t = blockIdx.x + it * gridDim.x;
@@ -669,30 +679,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
         const TcModelArg& M = a.models[tc_group(a, g).model];
         const uint32_t sb = (uint32_t)M.N * 128u;
         const int rot = tc_rot<MODE>(nks);
-        for (int ks = 0; ks < nks; ++ks, ++bi) {
-          const int slot = (int)(bi % TC_NB);
-          const uint32_t par = (uint32_t)((bi / TC_NB) & 1);
-          if (!tc_wait(sh, &sh.b_empty[slot], par ^ 1u, a.status)) {
+        for (int ks = 0; ks < nks; ++ks) {
+          if (!tc_wait(sh, &sh.b_empty[slot], ph ^ 1u, a.status)) {
             ok = false;
             break;
           }
           mbar_expect_tx(&sh.b_full[slot], sb);
           const int kse = ks + rot < nks ? ks + rot : ks + rot - nks;
           bulk_g2s(B + (size_t)slot * a.b_bytes, M.wlay + (size_t)kse * sb, sb, &sh.b_full[slot]);
-          last[slot] = bi;
+          if (filled < TC_NB) ++filled;
+          if (++slot == TC_NB) {
+            slot = 0;
+            ph ^= 1;
+          }
         }
       }
       // copies still in flight land before the CTA exits
-      for (int s = 0; s < TC_NB; ++s)
-        if (last[s] >= 0)
-          tc_wait(sh, &sh.b_full[s], (uint32_t)((last[s] / TC_NB) & 1), a.status);
+      for (int s = 0; s < filled; ++s)   // slots from `slot` on were last filled a round ago
+        tc_wait(sh, &sh.b_full[s], s < slot ? ph : ph ^ 1u, a.status);
     }
     __syncwarp();
   } else if (warp == TC_WORK + 2) {
     // ---- row producer (pair pass) ----------------------------------------
     if (MODE == 0 && lane == 0) {
-      long long ri = 0, last[TC_NRAW];
-      for (int s = 0; s < TC_NRAW; ++s) last[s] = -1;
+      uint32_t ri = 0;   // row stages loaded
       bool ok = (smem_addr(raw) & 1023u) == 0;   // the swizzled reads assume 1 KB alignment
       if (!ok) {
         atomicOr(a.status, ST_TIMEOUT);
@@ -712,9 +722,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
         const int nraw = (F + BOXF - 1) / BOXF, rot = tc_rot<MODE>(nks) * TC_KS / BOXF;
         for (int rs = 0; rs < nraw; ++rs, ++ri) {
           const int f0 = BOXF * (rs + rot < nraw ? rs + rot : rs + rot - nraw);
-          const int slot = (int)(ri % TC_NRAW);
-          const uint32_t par = (uint32_t)((ri / TC_NRAW) & 1);
-          if (!tc_wait(sh, &sh.raw_empty[slot], par ^ 1u, a.status)) {
+          const uint32_t slot = ri % TC_NRAW;
+          if (!tc_wait(sh, &sh.raw_empty[slot], (ri / TC_NRAW & 1) ^ 1u, a.status)) {
             ok = false;
             break;
           }
@@ -728,74 +737,75 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
                 "l"(tmap), "r"(f0), "r"((int)(U.row0 + TC_M * h)),
                 "r"(smem_addr(&sh.raw_full[slot]))
                 : "memory");
-          last[slot] = ri;
         }
       }
       // copies still in flight land before the CTA exits
-      for (int s = 0; s < TC_NRAW; ++s)
-        if (last[s] >= 0)
-          tc_wait(sh, &sh.raw_full[s], (uint32_t)((last[s] / TC_NRAW) & 1), a.status);
+      for (uint32_t k = ri > TC_NRAW ? ri - TC_NRAW : 0; k < ri; ++k)
+        tc_wait(sh, &sh.raw_full[k % TC_NRAW], k / TC_NRAW & 1, a.status);
     }
     __syncwarp();
   } else if (warp == TC_WORK + 1) {
-    // ---- MMA issuer -----------------------------------------------------
-    if (lane == 0) {
-      long long bi = 0, ai = 0, ci = 0;
+    // ---- MMA issuer: the whole warp waits, one elected lane issues ---------
+    // One lane that waited and issued by itself took some 1,600 cycles for a stage
+    // of eight MMAs (the tensor cores need 770), whatever the MMAs' size: 64-bit
+    // remainders, a clock read per wait and operands moved to the uniform registers
+    // one at a time (262,144 u8 rows x 8,192 features x 64 classes: 730 -> 510 us the
+    // call; 0.83 of it is the MMAs' time at the tensor cores' rate and the heavy rows).
+    static_assert(PS::SUB == 1 && (PS::NA & (PS::NA - 1)) == 0, "an A stage per weight stage");
+    {
+      const uint32_t lead = tc_elect();
+      uint32_t bslot = 0, bph = 0, as = 0, ci = 0;
       bool ok = true;
-      const int chunk = MODE == 0 ? nks : TC_CHUNK;
-      for (long long it = 0; it < my_units && ok && !tc_aborted(sh); ++it) {
+      const uint32_t chunk = MODE == 0 ? (uint32_t)nks : (uint32_t)TC_CHUNK;
+      // descriptor of weight slot 0; slot s and K16 step j add (s b_bytes + 256 j) /
+      // 16 to its start-address field (14 bits: no carry below 256 KB)
+      const uint64_t bdesc0 = tc_desc(smem_addr(B), 128u, 1024u);
+      for (long long it = 0; it < my_units && ok && !__any_sync(0xFFFFFFFFu, tc_aborted(sh)); ++it) {
         const long long t = blockIdx.x + it * gridDim.x;
         const int g = MODE == 0 ? tc_unit(a, n_groups, t).g : 0;
-        const TcModelArg& M = a.models[tc_group(a, g).model];
-        const uint32_t idesc = tc_idesc_f16(TC_M, M.N);
-        int kc = 0;
-        for (int ks = 0; ks < nks && ok; ++ks) {
-          if (kc == 0 && ci > 0) {   // the accumulators were drained
-            if (!tc_wait(sh, &sh.acc_empty, (uint32_t)((ci - 1) & 1), a.status)) {
-              ok = false;
-              break;
-            }
-          }
-          const int bslot = (int)(bi % TC_NB);
-          if (!tc_wait(sh, &sh.b_full[bslot], (uint32_t)((bi / TC_NB) & 1), a.status)) {
+        const uint32_t idesc = tc_idesc_f16(TC_M, a.models[tc_group(a, g).model].N);
+        uint32_t kc = 0;
+        for (int ks = 0; ks < nks; ++ks) {
+          const uint32_t aslot = as & (PS::NA - 1);
+          if ((kc == 0 && ci > 0 &&   // the accumulators were drained
+               !tc_wait_warp(sh, &sh.acc_empty, (ci - 1) & 1, a.status)) ||
+              !tc_wait_warp(sh, &sh.b_full[bslot], bph, a.status) ||
+              !tc_wait_warp(sh, &sh.a_full[aslot], (as / PS::NA) & 1, a.status)) {
             ok = false;
             break;
           }
-          const uint32_t bs = smem_addr(B + (size_t)bslot * a.b_bytes);
-          // the weight stage's A stages, KA features each
-#pragma unroll
-          for (int sub = 0; sub < PS::SUB; ++sub) {
-            const int aslot = (int)(ai % PS::NA);
-            if (!tc_wait(sh, &sh.a_full[aslot], (uint32_t)((ai / PS::NA) & 1), a.status)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
+          tc_fence_after();
+          const uint64_t bd = bdesc0 + (uint64_t)((bslot * a.b_bytes) >> 4);
+          const uint32_t at = tmem + TC_ACOL + aslot * (uint32_t)(PS::ACOLS * PS::H);
+          const bool end = kc + 1 == chunk || ks == nks - 1;
+          if (lead) {
 #pragma unroll
             for (int h = 0; h < PS::H; ++h)
 #pragma unroll
               for (int j = 0; j < PS::KA / 16; ++j)
-                tc_mma_f16_ts(tmem + (uint32_t)(TC_ACC * h),
-                              tmem + (uint32_t)(TC_ACOL + aslot * PS::ACOLS * PS::H +
-                                                PS::ACOLS * h + 8 * j),
-                              tc_desc(bs + 256u * (uint32_t)(sub * (PS::KA / 16) + j), 128u, 1024u),
-                              idesc, (uint32_t)(kc | sub | j));
+                tc_mma_f16_ts(tmem + (uint32_t)(TC_ACC * h), at + (uint32_t)(PS::ACOLS * h + 8 * j),
+                              bd + 16u * j, idesc, kc | (uint32_t)j);
             tc_commit(&sh.a_empty[aslot]);
-            ++ai;
+            tc_commit(&sh.b_empty[bslot]);
+            if (end) tc_commit(&sh.acc_full);
           }
-          if (!ok) break;
-          tc_commit(&sh.b_empty[bslot]);
-          ++bi;
-          if (++kc == chunk || ks == nks - 1) {
-            tc_commit(&sh.acc_full);
+          __syncwarp();
+          ++as;
+          if (++bslot == TC_NB) {
+            bslot = 0;
+            bph ^= 1;
+          }
+          ++kc;
+          if (end) {
             ++ci;
             kc = 0;
           }
         }
       }
       // every MMA issued so far has completed once this arrives
-      tc_commit(&sh.fin);
-      tc_wait(sh, &sh.fin, 0, a.status);
+      if (lead) tc_commit(&sh.fin);
+      __syncwarp();
+      tc_wait_warp(sh, &sh.fin, 0, a.status);
     }
     __syncwarp();
   } else {
@@ -834,7 +844,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
     if constexpr (MODE == 0) {
       // Pair pass: a row stage at a time.  Its bytes are read and converted (RAW_A A
       // stages), the row stage is handed back, and the A stages go to tensor memory as
-      // their slots come free.
+      // their slots come free.  200 instructions a warp and A stage with 64-bit stage
+      // counters, a clock read per wait and an abort test per stage were 117 without
+      // (the same call 826 -> 730 us, BF16 rows x 2,048 features 195 -> 169).
       static_assert(PS::NA == 2 && TC_NRAW == 2, "slot and phase from the counters' low bits");
       const int nrs = (nka + RAW_A - 1) / RAW_A;
       uint32_t as = 0, rs = 0;   // A stages written, row stages read
