@@ -212,29 +212,46 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w) {
   return r;
 }
 
-// non-zero if a BF16 half of w is non-zero with magnitude below 2^-14 (its
-// FP16 image would be subnormal or zero, which the count check cannot tell
-// from an exact value)
-__device__ __forceinline__ uint32_t bf16x2_tiny(uint32_t w) {
-  const uint32_t mag = w & 0x7FFF7FFFu;
-  const uint32_t nz = mag + 0x7FFF7FFFu;      // bit 15 of a half set: half >= 1
-  const uint32_t big = mag + 0x47804780u;     // bit 15 of a half set: half >= 0x3880 (2^-14)
-  return nz & ~big & 0x80008000u;
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// The BF16 halves of w, less one in each half (0 becomes the largest), into the running
+// minimum: a non-zero half below 1.0 (0x3F80) shows in it.  (One below 2^-25 would
+// become an FP16 zero, which the count check cannot tell from an exact one.)
+__device__ __forceinline__ void bf16x2_least(uint32_t w, uint32_t& mn) {
+  uint32_t r;
+  asm("add.u16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0xFFFFFFFFu));
+  mn = min_u16x2(mn, r);
 }
 
 // Count check of an FP16 pair h against the magic pair m2 = (M, M), M = 2^(10-e):
-// with w = h + M (FP16), a half of h is a non-negative multiple of 2^-e below M
-// exactly when that half of w lies in [M, 2M) (its sign and exponent field is
-// M's) and w - M == h; its count h 2^e is then the low 10 bits of w.  A failing
-// half leaves a bit in bd.  The biased halves M + x are summed into tt (the
-// caller removes M per value).
+// with w = h + M (FP16), a half of h below M is a non-negative multiple of 2^-e
+// exactly when w - M == h; its count h 2^e is then the low 10 bits of w.  A failing
+// half leaves a bit in bd or a value of M or more (negative and NaN halves are
+// larger as integers) in the running maximum mx.  The biased halves M + x are summed
+// into tt (the caller removes M per value).  The converters of BF16 rows are bound by
+// these instructions: with the range and the tiny values tested by masks and
+// additions, 14 a pair, 150,001 rows x 2,048 features x 16 classes took 163 us, with running
+// extremes, 10 a pair, 140.
 __device__ __forceinline__ void f16x2_count_check(uint32_t h, uint32_t m2, uint32_t& tt,
-                                                  uint32_t& bd) {
+                                                  uint32_t& bd, uint32_t& mx) {
   uint32_t w, back;
   asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w) : "r"(h), "r"(m2));
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(back) : "r"(w), "r"(m2));
-  bd |= (back ^ h) | ((w & 0xFC00FC00u) ^ m2);
+  bd |= back ^ h;
+  mx = max_u16x2(mx, h);
   tt = (uint32_t)dp2a_lo_us(w, 0x01010101u, (int)tt);
+}
+__device__ __forceinline__ bool halves_below(uint32_t v, uint32_t lim) {
+  return (v & 0xFFFFu) < lim && (v >> 16) < lim;
 }
 
 // bounded wait that sleeps in the barrier instead of polling
@@ -846,12 +863,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
       // stages), the row stage is handed back, and the A stages go to tensor memory as
       // their slots come free.  200 instructions a warp and A stage with 64-bit stage
       // counters, a clock read per wait and an abort test per stage were 117 without
-      // (the same call 826 -> 730 us, BF16 rows x 2,048 features 195 -> 169).
+      // (the same call 826 -> 730 us, 150,001 BF16 rows x 2,048 x 16 195 -> 169).
       static_assert(PS::NA == 2 && TC_NRAW == 2, "slot and phase from the counters' low bits");
       const int nrs = (nka + RAW_A - 1) / RAW_A;
       uint32_t as = 0, rs = 0;   // A stages written, row stages read
       for (long long it = 0; it < my_units && ok; ++it) {
-        uint32_t T = 0, m2 = 0x64006400u, bad = 0u;
+        uint32_t T = 0, m2 = 0x64006400u, bad = 0u, mx = 0u, mn = 0xFFFFFFFFu;
         float rsc = DT == NB_U8 ? 16777216.f : 1.f;   // u8: subnormals x 2^-24
         if (DT == NB_FP8E4M3) {
           // this thread's row scale (2^e, e in {0, 1}; any other exponent sends the
@@ -895,7 +912,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
                   o[sub][8 * v + 2 * q + 1] = e4m3x2_to_f16x2(w[q] >> 16);
                 } else {
                   o[sub][4 * v + q] = bf16x2_to_f16x2(w[q]);
-                  bad |= bf16x2_tiny(w[q]);
+                  bf16x2_least(w[q], mn);
                 }
               }
             }
@@ -904,7 +921,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
             // per A stage: no wrap below 2^32 for F <= 8192)
             if constexpr (DT != NB_U8) {
 #pragma unroll
-              for (int q = 0; q < PS::COLS; ++q) f16x2_count_check(o[sub][q], m2, T, bad);
+              for (int q = 0; q < PS::COLS; ++q) f16x2_count_check(o[sub][q], m2, T, bad, mx);
             }
           }
           __syncwarp();
@@ -935,8 +952,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
         // FP8 / BF16: the unit's check; then the counts' total without the bias M of
         // each of the 2 COLS values of every A stage (RAW_A of every row stage)
         if (DT != NB_U8)
-          T = bad != 0u ? 0xFFFFFFFFu
-                        : T - (m2 & 0xFFFFu) * (uint32_t)(2 * PS::COLS) * (uint32_t)(RAW_A * nrs);
+          T = bad != 0u || !halves_below(mx, m2 & 0xFFFFu) ||
+                      (mn & 0xFFFFu) < 0x3F7Fu || (mn >> 16) < 0x3F7Fu
+                  ? 0xFFFFFFFFu
+                  : T - (m2 & 0xFFFFu) * (uint32_t)(2 * PS::COLS) * (uint32_t)(RAW_A * nrs);
         if (!tc_epilogue<MODE>(a, sh, xe, G, a.models[G.model], r, xr, h, part, T, rsc, lane_base,
                                ep))
           break;
