@@ -79,7 +79,7 @@ constexpr float TC_T_EXACT = 131072.f;     // 128 T < 2^24: one accumulation is 
 constexpr int TC_WORK = 16;                // converter / epilogue warps
 constexpr int TC_THREADS = (TC_WORK + 3) * 32;
 constexpr int TC_BOX = 128;                // features per TMA box (128-byte swizzle span)
-constexpr int TC_NRAW = 2;                 // row stages in shared memory (pair pass)
+constexpr int TC_NRAW = 4;                 // most row stages in shared memory (pair pass: 2 or 4)
 constexpr uint32_t TC_RAW_BYTES = 2 * TC_M * TC_BOX;   // both tiles, 128 features
 constexpr int TC_PD = 3;                   // row stages loaded ahead into registers
 constexpr long long TC_WAIT = 2000000000LL;
@@ -634,7 +634,8 @@ __device__ __forceinline__ long long tc_units(const TcArgs& a) {
 
 // DT: storage of the rows (NB_U8, NB_FP8E4M3 or NB_BF16; the chunked pass
 // takes u8 rows only).  A 128-byte row box holds BOXF features.
-template <int MODE, int DT>
+// RL: log2 of the pair pass's row stages in shared memory.
+template <int MODE, int DT, int RL>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constant__ TcArgs a) {
   using PS = TcPass<MODE>;
   static_assert(MODE == 0 || DT == NB_U8, "the chunked pass reads u8 rows");
@@ -645,7 +646,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
   TcXch& xe = *reinterpret_cast<TcXch*>(tc_smem + 1024);
   // 1 KB aligned: the swizzled row stages (pair pass only), then the weights
   uint8_t* raw = tc_smem + 1024 + ((sizeof(TcXch) + 1023) / 1024) * 1024;
-  uint8_t* B = raw + (MODE == 0 ? (size_t)TC_NRAW * TC_RAW_BYTES : 0);
+  uint8_t* B = raw + (MODE == 0 ? (size_t)TC_RAW_BYTES << RL : 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_groups = a.groups ? a.hdr->n_groups : 1;
   pdl_trigger();   // a batch's two-class launch may fill the SMs that run out of units
@@ -720,6 +721,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
     // ---- row producer (pair pass) ----------------------------------------
     if (MODE == 0 && lane == 0) {
       uint32_t ri = 0;   // row stages loaded
+      constexpr uint32_t raw_mask = (1u << RL) - 1;
       bool ok = (smem_addr(raw) & 1023u) == 0;   // the swizzled reads assume 1 KB alignment
       if (!ok) {
         atomicOr(a.status, ST_TIMEOUT);
@@ -739,8 +741,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
         const int nraw = (F + BOXF - 1) / BOXF, rot = tc_rot<MODE>(nks) * TC_KS / BOXF;
         for (int rs = 0; rs < nraw; ++rs, ++ri) {
           const int f0 = BOXF * (rs + rot < nraw ? rs + rot : rs + rot - nraw);
-          const uint32_t slot = ri % TC_NRAW;
-          if (!tc_wait(sh, &sh.raw_empty[slot], (ri / TC_NRAW & 1) ^ 1u, a.status)) {
+          const uint32_t slot = ri & raw_mask;
+          if (!tc_wait(sh, &sh.raw_empty[slot], (ri >> RL & 1) ^ 1u, a.status)) {
             ok = false;
             break;
           }
@@ -757,8 +759,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
         }
       }
       // copies still in flight land before the CTA exits
-      for (uint32_t k = ri > TC_NRAW ? ri - TC_NRAW : 0; k < ri; ++k)
-        tc_wait(sh, &sh.raw_full[k % TC_NRAW], k / TC_NRAW & 1, a.status);
+      for (uint32_t k = ri > raw_mask ? ri - raw_mask - 1 : 0; k < ri; ++k)
+        tc_wait(sh, &sh.raw_full[k & raw_mask], k >> RL & 1, a.status);
     }
     __syncwarp();
   } else if (warp == TC_WORK + 1) {
@@ -864,7 +866,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
       // their slots come free.  200 instructions a warp and A stage with 64-bit stage
       // counters, a clock read per wait and an abort test per stage were 117 without
       // (the same call 826 -> 730 us, 150,001 BF16 rows x 2,048 x 16 195 -> 169).
-      static_assert(PS::NA == 2 && TC_NRAW == 2, "slot and phase from the counters' low bits");
+      static_assert(PS::NA == 2, "slot and phase from the counter's low bits");
+      constexpr uint32_t raw_mask = (1u << RL) - 1;
       const int nrs = (nka + RAW_A - 1) / RAW_A;
       uint32_t as = 0, rs = 0;   // A stages written, row stages read
       for (long long it = 0; it < my_units && ok; ++it) {
@@ -887,13 +890,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
 #pragma unroll 1
         for (int k = 0; k < nrs; ++k, ++rs) {
           if (tc_aborted(sh) ||
-              !tc_wait_warp(sh, &sh.raw_full[rs & 1], (rs >> 1) & 1, a.status)) {
+              !tc_wait_warp(sh, &sh.raw_full[rs & raw_mask], (rs >> RL) & 1, a.status)) {
             ok = false;
             break;
           }
           // this thread's bytes of the row stage: 16-byte chunks of its row, swizzled
           // by the row (rows and features past the end arrive as zeros)
-          const uint32_t src = raw_s + (rs & 1) * TC_RAW_BYTES + (uint32_t)(rr * TC_BOX);
+          const uint32_t src = raw_s + (rs & raw_mask) * TC_RAW_BYTES + (uint32_t)(rr * TC_BOX);
           uint32_t o[RAW_A][PS::COLS];
 #pragma unroll
           for (int sub = 0; sub < RAW_A; ++sub) {
@@ -925,7 +928,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(&sh.raw_empty[rs & 1]);
+          if (lane == 0) mbar_arrive(&sh.raw_empty[rs & raw_mask]);
 #pragma unroll
           for (int sub = 0; sub < RAW_A; ++sub) {
             if (RAW_A * k + sub >= nka) break;
@@ -1190,16 +1193,16 @@ static TcModelArg tc_model_arg(const nb_model* m) {
 }
 
 // shared memory of a launch whose largest model has N limb rows
-static size_t tc_smem_bytes(int mode, int N) {
+constexpr size_t kTcMaxSmem = 227 * 1024;
+static size_t tc_smem_bytes(int mode, int N, int raw_lg) {
   return 1024 + ((sizeof(TcXch) + 1023) / 1024) * 1024 +
-         (mode == 0 ? (size_t)TC_NRAW * TC_RAW_BYTES : 0) + (size_t)TC_NB * (uint32_t)N * 128u;
+         (mode == 0 ? (size_t)TC_RAW_BYTES << raw_lg : 0) + (size_t)TC_NB * (uint32_t)N * 128u;
 }
 
-template <int MODE, int DT>
-static nb_status run_tc(TcArgs& a, int maxN, long long units_hint, cudaStream_t st) {
-  constexpr size_t kMax = 227 * 1024;
-  const size_t smem = tc_smem_bytes(MODE, maxN);
-  if (smem > kMax) {
+template <int MODE, int DT, int RL>
+static nb_status run_tc_rl(TcArgs& a, int maxN, long long units_hint, cudaStream_t st) {
+  const size_t smem = tc_smem_bytes(MODE, maxN, RL);
+  if (smem > kTcMaxSmem) {
     set_error("tensor-core scorer: shared memory %zu bytes exceeds the limit", smem);
     return NB_EUNSUPPORTED;
   }
@@ -1208,15 +1211,27 @@ static nb_status run_tc(TcArgs& a, int maxN, long long units_hint, cudaStream_t 
   // more than half the shared memory of an SM keeps one CTA (and one
   // tensor-memory allocation) per SM
   const size_t launch_smem = smem < 120 * 1024 ? 120 * 1024 : smem;
-  NB_TRY_CUDA(cudaFuncSetAttribute(k_score_tc<MODE, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  NB_TRY_CUDA(cudaFuncSetAttribute(k_score_tc<MODE, DT, RL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)launch_smem),
               "cudaFuncSetAttribute(k_score_tc)");
   long long grid = num_sms();
   if (units_hint > 0 && units_hint < grid) grid = units_hint;
   count_launch();
-  k_score_tc<MODE, DT><<<(unsigned)grid, TC_THREADS, launch_smem, st>>>(a);
+  k_score_tc<MODE, DT, RL><<<(unsigned)grid, TC_THREADS, launch_smem, st>>>(a);
   NB_TRY_CUDA(cudaGetLastError(), "k_score_tc launch");
   return NB_OK;
+}
+
+// Four row stages where the weight stages leave the room (N <= 132: up to 40
+// classes): with few classes the MMAs are short and the rows' latency shows (150,001
+// BF16 rows x 2,048 features x 16 classes 150 -> 131 us).
+template <int MODE, int DT>
+static nb_status run_tc(TcArgs& a, int maxN, long long units_hint, cudaStream_t st) {
+  if constexpr (MODE == 0) {
+    if (tc_smem_bytes(MODE, maxN, 2) <= kTcMaxSmem)
+      return run_tc_rl<MODE, DT, 2>(a, maxN, units_hint, st);
+  }
+  return run_tc_rl<MODE, DT, 1>(a, maxN, units_hint, st);
 }
 
 // ---------------------------------------------------------------------------
