@@ -175,7 +175,8 @@ typedef struct {
  *         FP8E4M3 with integer values); N_cj is accumulated exactly in
  *         uint64, then log theta and log prior in FP64 on the device.
  *         NB_GAUSSIAN: X holds real values (F32); class means and MLE
- *         variances are computed in FP64 by two deterministic passes.
+ *         variances are computed by two deterministic passes (paired FP32
+ *         sums over short runs of rows, FP64 from there on).
  *   y     int32 labels in [0, C) (device), n entries.
  *   C     2 <= C <= 255;  F >= 1.
  * On success *out owns device tables; free it with nb_model_free.  Errors:
@@ -188,8 +189,10 @@ NB_API nb_status nb_fit(nb_kind kind, const void* X, nb_dtype dtype, int64_t n,
 /* Re-trains an existing model in place on new data with the same F and C
  * (kind, C and F are the model's).  Allocates no model memory, so a training
  * loop or a timed benchmark step does not pay for cudaMalloc / cudaFree; the
- * count reduction still takes stream-ordered scratch (cudaMallocAsync).  The
- * model must not be in use by a score call on another stream meanwhile.
+ * scratch of the reduction is kept with the model between re-fits up to 64 MiB
+ * (taken stream-ordered, cudaMallocAsync, and kept from the first re-fit on;
+ * larger scratch, and that of a call on a stream being captured, is allocated
+ * and freed in stream order).  The model must not be in use by a score call on another stream meanwhile.
  * Same errors as nb_fit. */
 NB_API nb_status nb_refit(nb_model* model, const void* X, nb_dtype dtype, int64_t n,
                    int64_t ld, const int32_t* y, const nb_fit_opts* opts,

@@ -13,7 +13,7 @@
 //     three signed 8-bit limbs; dp4a accumulates x * limb exactly in int32, so
 //     the only error is the quantisation of Delta (<= 2^-S / 2 per count).
 //     FP8 E4M3 storage takes the same limbs: its values become exact integer
-//     counts (row scale 2^0 or 2^1, checked per value, see fp8_count_pairs)
+//     counts (row scale 2^0 or 2^1, checked per value, see fp8_biased_pairs)
 //     in 16-bit pairs, accumulated with dp2a.
 //   * f32 / u16 / bf16 storage: decode to FP32 and FMA against the FP32 Delta
 //     table, four accumulators per row per lane.
