@@ -41,7 +41,7 @@
 //                  (2 x 192 columns) plus a ring of two A stages (128
 //                  columns); rows of 2^17 or more stored counts could have
 //                  rounded and are put on a list of heavy rows;
-//   k_tc_heavy     up to kTcFew listed heavy rows on the CUDA cores, exact int64
+//   k_tc_heavy     up to kTcFewU8 (FP8, BF16: kTcFew) listed heavy rows on the CUDA cores, exact int64
 //                  sums against the 32-bit fixed-point weights;
 //   pass "chunked" more than those: units of 128 listed heavy rows (read by the converter warps
 //                  straight from global memory), accumulated in 512-feature
@@ -84,11 +84,12 @@ constexpr uint32_t TC_RAW_BYTES = 2 * TC_M * TC_BOX;   // both tiles, 128 featur
 constexpr int TC_PD = 3;                   // row stages loaded ahead into registers
 constexpr long long TC_WAIT = 2000000000LL;
 constexpr int kTcHeavyCap = 262144;        // heavy rows one call redoes exactly
-// up to this many heavy rows go to the CUDA cores (k_tc_heavy) instead of the
-// chunked pass, which takes 153 us for any number of units up to one per SM (C =
-// 64, F = 8,192: one unit's 128 weight stages one after another) against 37 us
-// for the 130 heavy rows of 262,144
-constexpr int kTcFew = 1024;
+// Up to this many heavy rows go to the CUDA cores (k_tc_heavy).  u8 rows beyond
+// kTcFewU8 take the chunked pass, 137 us for any number of units up to one per SM (C =
+// 64, F = 8,192: one unit's 128 weight stages one after another): k_tc_heavy takes 35 us
+// for 128 rows, 57 for 256, 116 for 512, 140 for 768, 192 for 1,024 there (C = 16, F =
+// 2,048: 15 against 33 at 768).  FP8 and BF16 rows beyond kTcFew go to FP64.
+constexpr int kTcFew = 1024, kTcFewU8 = 768;
 
 // Per-pass constants: H tiles per unit (two in the pair pass), P class parts
 // per row (the 16 warps cover H x 4 lane quadrants x P parts), BPT bytes of
@@ -628,7 +629,7 @@ __device__ __forceinline__ long long tc_units(const TcArgs& a) {
   if (MODE == 0) return a.groups ? a.hdr->tiles : a.units0;
   unsigned long long c = *a.heavy_n;
   if (c > (unsigned long long)a.heavy_cap) c = (unsigned long long)a.heavy_cap;
-  if (c <= (unsigned long long)kTcFew) return 0;   // k_tc_heavy took them
+  if (c <= (unsigned long long)kTcFewU8) return 0;   // k_tc_heavy took them
   return (long long)((c + TC_M - 1) / TC_M);
 }
 
@@ -1295,7 +1296,7 @@ __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_wait();   // the pair pass's list
   const long long n = (long long)min(*a.heavy_n, (unsigned long long)a.heavy_cap);
-  if (n == 0 || n > kTcFew) return;
+  if (n == 0 || n > (DT == NB_U8 ? kTcFewU8 : kTcFew)) return;
   const int C = a.M.C, F = a.F, ncb = (C + 7) / 8;
   const long long items = (n + 3) / 4 * ncb;
   for (long long item = blockIdx.x; item < items; item += gridDim.x) {
@@ -1597,7 +1598,7 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
     s = u8                   ? run_tc_heavy<NB_U8>(h, st)
         : dt == NB_FP8E4M3 ? run_tc_heavy<NB_FP8E4M3>(h, st)
                              : run_tc_heavy<NB_BF16>(h, st);
-  if (s == NB_OK && u8 && cap > kTcFew) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
+  if (s == NB_OK && u8 && cap > kTcFewU8) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
   const nb_status f = ss.release();
   return s != NB_OK ? s : f;
 }
