@@ -106,11 +106,13 @@ typedef struct {
  *                       rows that a fast path cannot compute at all are still
  *                       recomputed in FP64: a two-class u8 row whose stored
  *                       counts total 2^24 or more (its int32 limb sums could
- *                       wrap), tensor-core rows of 2^17 or more counts beyond
- *                       the scorer's exact-redo capacity (262,144 per call;
- *                       FP8 and BF16 rows 1,024; none in a batch) and FP8 /
- *                       BF16 rows outside the tensor-core scorer's count
- *                       check;
+ *                       wrap), tensor-core rows of 2^17 or more counts
+ *                       (U8 rows beyond the scorer's exact-redo capacity of
+ *                       262,144 a call, none in a batch; FP8 and BF16 rows:
+ *                       all of them, the first 1,024 of a call that is not
+ *                       captured as part of the scoring, without joining
+ *                       n_rechecked) and FP8 / BF16 rows outside the
+ *                       tensor-core scorer's count check;
  *   NB_RECHECK_LABEL -- rows whose margin is within the rigorous error bound
  *                       of the fast path are recomputed in FP64, so every
  *                       label equals the FP64 decision;

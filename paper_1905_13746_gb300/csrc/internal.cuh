@@ -244,6 +244,10 @@ nb_status launch_score_general(const nb_model* m, const void* X, nb_dtype dt,
 nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt,
                          int64_t n, int64_t ld, const nb_aux* aux,
                          const ScoreOut& o, cudaStream_t st);
+// The listed rows (FP8 or BF16, at most cap) in FP64.
+nb_status launch_recheck_list(const nb_model* m, const void* X, nb_dtype dt, int64_t ld,
+                              const nb_aux* aux, const ScoreOut& o, const int* list,
+                              const unsigned long long* count, int cap, cudaStream_t st);
 
 // many-class tensor-core scorer (score_tc.cu)
 inline int tc_classes_padded(int C) { return (C + 15) / 16 * 16; }

@@ -102,48 +102,51 @@ __device__ __forceinline__ void recheck_sums(const RView& v, const RModel& md, c
   }
 }
 
-// The whole warp recomputes row r of v with model md; lane 0 writes outputs.
-// The row's value is loaded once for CB classes; per class the lane's sum and
-// the butterfly over the lanes are those of one class at a time.
+// The whole warp sums classes c0 .. c0 + nc - 1 (nc <= CB) of row r of v; their
+// scores go to s_sh.  The row's value is loaded once for the CB classes; per class
+// the lane's sum and the butterfly over the lanes are those of one class at a
+// time, so that CB changes no bit.
 template <int DT, int KIND, int CB, int U>
-__device__ __forceinline__ void recheck_row(const RView& v, const RModel& md, int64_t r,
-                                            int want_lp, double* s_sh) {
+__device__ __forceinline__ void recheck_classes(const RView& v, const RModel& md, int64_t r,
+                                                int c0, int nc, double* s_sh) {
   const int lane = threadIdx.x & 31;
   constexpr int es = DT == NB_F32 ? 4 : ((DT == NB_U16 || DT == NB_BF16) ? 2 : 1);
   const char* rp = v.X + r * v.ld * es;
   const double scale = (DT == NB_FP8E4M3 && v.row_exp) ? ldexp(1.0, (int)v.row_exp[r]) : 1.0;
-  for (int c0 = 0; c0 < md.C; c0 += CB) {
-    const int nc = md.C - c0 < CB ? md.C - c0 : CB;
-    double acc[CB];
+  double acc[CB];
 #pragma unroll
-    for (int k = 0; k < CB; ++k) acc[k] = 0.0;
-    recheck_sums<DT, KIND, CB, U>(v, md, rp, scale, c0, nc, acc);
-    if (DT == NB_U8 && KIND == NB_MULTINOMIAL && v.ovf_ptr) {
-      const double* lt = md.p0 + (int64_t)c0 * v.F;
-      for (int64_t e = v.ovf_ptr[r] + lane; e < v.ovf_ptr[r + 1]; e += 32) {
-        const int j = v.ovf_col[e];
-        if (j >= v.F) continue;
-        const double add = (double)v.ovf_add[e];
+  for (int k = 0; k < CB; ++k) acc[k] = 0.0;
+  recheck_sums<DT, KIND, CB, U>(v, md, rp, scale, c0, nc, acc);
+  if (DT == NB_U8 && KIND == NB_MULTINOMIAL && v.ovf_ptr) {
+    const double* lt = md.p0 + (int64_t)c0 * v.F;
+    for (int64_t e = v.ovf_ptr[r] + lane; e < v.ovf_ptr[r + 1]; e += 32) {
+      const int j = v.ovf_col[e];
+      if (j >= v.F) continue;
+      const double add = (double)v.ovf_add[e];
 #pragma unroll
-        for (int k = 0; k < CB; ++k)
-          if (k < nc) acc[k] = fma(add, lt[(int64_t)k * v.F + j], acc[k]);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < CB; ++k) {
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xFFFFFFFFu, acc[k], off);
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < CB; ++k) {
-        const int c = c0 + k;
-        if (k < nc)
-          s_sh[c] = KIND == NB_MULTINOMIAL ? md.log_pi[c] + acc[k] : md.gconst[c] - 0.5 * acc[k];
-      }
+      for (int k = 0; k < CB; ++k)
+        if (k < nc) acc[k] = fma(add, lt[(int64_t)k * v.F + j], acc[k]);
     }
   }
-  __syncwarp();
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+    for (int k = 0; k < CB; ++k) acc[k] += __shfl_xor_sync(0xFFFFFFFFu, acc[k], off);
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < CB; ++k) {
+      const int c = c0 + k;
+      if (k < nc)
+        s_sh[c] = KIND == NB_MULTINOMIAL ? md.log_pi[c] + acc[k] : md.gconst[c] - 0.5 * acc[k];
+    }
+  }
+}
+
+// The whole warp writes row r's outputs from its scores.
+__device__ __forceinline__ void recheck_finish(const RView& v, const RModel& md, int64_t r,
+                                               int want_lp, const double* s_sh) {
+  const int lane = threadIdx.x & 31;
   // the lanes share the classes: arg-max (lowest index among the maxima; class
   // 0 when its score is NaN or none is a number), second best, log-sum-exp (an
   // FP64 exponential per class: one lane alone took them one after another)
@@ -185,6 +188,16 @@ __device__ __forceinline__ void recheck_row(const RView& v, const RModel& md, in
     const double lse = sb + log(sum);
     for (int c = lane; c < md.C; c += 32) v.logpost[r * md.C + c] = (float)(s_sh[c] - lse);
   }
+}
+
+// The whole warp recomputes row r of v with model md.
+template <int DT, int KIND, int CB, int U>
+__device__ __forceinline__ void recheck_row(const RView& v, const RModel& md, int64_t r,
+                                            int want_lp, double* s_sh) {
+  for (int c0 = 0; c0 < md.C; c0 += CB)
+    recheck_classes<DT, KIND, CB, U>(v, md, r, c0, md.C - c0 < CB ? md.C - c0 : CB, s_sh);
+  __syncwarp();
+  recheck_finish(v, md, r, want_lp, s_sh);
   __syncwarp();
 }
 
@@ -241,22 +254,28 @@ static RKernel recheck_kernel(nb_kind kind, nb_dtype dt, int C) {
   }
 }
 
+static RView view_of(const void* X, int64_t ld, int F, const nb_aux* aux, const ScoreOut& o) {
+  RView v{};
+  v.X = static_cast<const char*>(X);
+  v.ld = ld;
+  v.F = F;
+  v.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
+  v.ovf_col = aux ? aux->ovf_col : nullptr;
+  v.ovf_add = aux ? aux->ovf_add : nullptr;
+  v.row_exp = aux ? aux->row_exp : nullptr;
+  v.label = o.label;
+  v.margin = o.margin;
+  v.logpost = o.logpost;
+  return v;
+}
+
 nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                          const nb_aux* aux, const ScoreOut& o, cudaStream_t st) {
   // NB_RECHECK_OFF still recomputes the rows a scorer could not compute at all
   // (see NB_RECHECK_OFF in the header); in that mode nothing else is marked
   if (n == 0) return NB_OK;
   RArgs a{};
-  a.v.X = static_cast<const char*>(X);
-  a.v.ld = ld;
-  a.v.F = m->F;
-  a.v.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
-  a.v.ovf_col = aux ? aux->ovf_col : nullptr;
-  a.v.ovf_add = aux ? aux->ovf_add : nullptr;
-  a.v.row_exp = aux ? aux->row_exp : nullptr;
-  a.v.label = o.label;
-  a.v.margin = o.margin;
-  a.v.logpost = o.logpost;
+  a.v = view_of(X, ld, m->F, aux, o);
   a.md = RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst};
   a.n = n;
   a.want_lp = o.want_lp;
@@ -273,6 +292,50 @@ nb_status launch_recheck(const nb_model* m, const void* X, nb_dtype dt, int64_t 
   NB_TRY_CUDA(launch_pdl(recheck_kernel(m->kind, dt, m->C), dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0,
                          st, a),
               "k_recheck launch");
+  return NB_OK;
+}
+
+// ---------------------------------------------------------------------------
+// listed rows (FP8 and BF16 rows of 2^17 and more counts): a block per row, its
+// warps two classes each
+// ---------------------------------------------------------------------------
+// The bits of k_recheck, which gives a marked row to one warp: with few rows that
+// warp's loads, one batch of features after another for all classes, are what the
+// call waits for (BF16, F = 2,048, C = 16: 64 batches one after another, here 8).
+struct RListArgs {
+  RView v;
+  RModel md;
+  const int* list;
+  const unsigned long long* count;
+  int cap, want_lp;
+};
+
+template <int DT>
+__global__ void __launch_bounds__(256) k_recheck_list(const RListArgs a) {
+  __shared__ double s_sh[kTcMaxC];
+  const int warp = threadIdx.x >> 5;
+  pdl_wait();   // the scorer's list
+  const int n = (int)min(*a.count, (unsigned long long)a.cap);
+  for (int i = blockIdx.x; i < n; i += gridDim.x) {
+    const int64_t r = a.list[i];
+    for (int c0 = 2 * warp; c0 < a.md.C; c0 += 16)
+      recheck_classes<DT, NB_MULTINOMIAL, 2, 8>(a.v, a.md, r, c0, a.md.C - c0 < 2 ? 1 : 2, s_sh);
+    __syncthreads();
+    if (warp == 0) recheck_finish(a.v, a.md, r, a.want_lp, s_sh);
+    __syncthreads();
+  }
+}
+
+nb_status launch_recheck_list(const nb_model* m, const void* X, nb_dtype dt, int64_t ld,
+                              const nb_aux* aux, const ScoreOut& o, const int* list,
+                              const unsigned long long* count, int cap, cudaStream_t st) {
+  RListArgs a{view_of(X, ld, m->F, aux, o), RModel{m->C, m->d.p0, m->d.p1, m->d.log_pi, m->d.gconst},
+              list, count, cap, o.want_lp};
+  const int grid = num_sms() * 2;
+  count_launch();
+  NB_TRY_CUDA(launch_pdl(dt == NB_BF16 ? k_recheck_list<NB_BF16> : k_recheck_list<NB_FP8E4M3>,
+                         dim3((unsigned)(cap < grid ? cap : grid)), dim3(256), 0, st, a),
+              "k_recheck_list launch");
   return NB_OK;
 }
 

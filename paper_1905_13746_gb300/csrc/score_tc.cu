@@ -41,7 +41,7 @@
 //                  (2 x 192 columns) plus a ring of two A stages (128
 //                  columns); rows of 2^17 or more stored counts could have
 //                  rounded and are put on a list of heavy rows;
-//   k_tc_heavy     up to kTcFewU8 (FP8, BF16: kTcFew) listed heavy rows on the CUDA cores, exact int64
+//   k_tc_heavy     up to kTcFewU8 listed heavy u8 rows on the CUDA cores, exact int64
 //                  sums against the 32-bit fixed-point weights;
 //   pass "chunked" more than those: units of 128 listed heavy rows (read by the converter warps
 //                  straight from global memory), accumulated in 512-feature
@@ -84,11 +84,13 @@ constexpr uint32_t TC_RAW_BYTES = 2 * TC_M * TC_BOX;   // both tiles, 128 featur
 constexpr int TC_PD = 3;                   // row stages loaded ahead into registers
 constexpr long long TC_WAIT = 2000000000LL;
 constexpr int kTcHeavyCap = 262144;        // heavy rows one call redoes exactly
-// Up to this many heavy rows go to the CUDA cores (k_tc_heavy).  u8 rows beyond
-// kTcFewU8 take the chunked pass, 137 us for any number of units up to one per SM (C =
+// Up to kTcFewU8 heavy u8 rows go to the CUDA cores (k_tc_heavy).  More
+// take the chunked pass, 137 us for any number of units up to one per SM (C =
 // 64, F = 8,192: one unit's 128 weight stages one after another): k_tc_heavy takes 35 us
 // for 128 rows, 57 for 256, 116 for 512, 140 for 768, 192 for 1,024 there (C = 16, F =
-// 2,048: 15 against 33 at 768).  FP8 and BF16 rows beyond kTcFew go to FP64.
+// 2,048: 15 against 33 at 768).  FP8 and BF16 rows of this weight go to FP64 as in a
+// batch, where the library promises the same bits: up to kTcFew through the list
+// (k_recheck_list), the rest through the recheck's scan.
 constexpr int kTcFew = 1024, kTcFewU8 = 768;
 
 // Per-pass constants: H tiles per unit (two in the pair pass), P class parts
@@ -1250,34 +1252,24 @@ struct TcHeavyArgs {
   const int64_t* ovf_ptr;
   const uint16_t* ovf_col;
   const uint16_t* ovf_add;
-  const int8_t* row_exp;
   TcModelArg M;
   int F, want_lp, recheck;
   const int* heavy;
   const unsigned long long* heavy_n;
   int heavy_cap;
-  long long* sums;       // kTcFew x C
-  float* T;              // kTcFew: counts of the row, overflow entries included
-  unsigned int* done;    // kTcFew / 4, zero: finished items of a row group
+  long long* sums;       // kTcFewU8 x C
+  float* T;              // kTcFewU8: counts of the row, overflow entries included
+  unsigned int* done;    // kTcFewU8 / 4, zero: finished items of a row group
   uint8_t* label;
   float* margin;
   float* logpost;
   unsigned long long* marks;
 };
 
-// values j .. j + V - 1 of a row as integer counts (checked by the pair pass)
-template <int DT, int V>
-__device__ __forceinline__ void heavy_counts(const char* rp, int j, int ex, int (&x)[V]) {
-  if constexpr (DT == NB_BF16) {
-#pragma unroll
-    for (int k = 0; k < V; ++k)
-      x[k] = (int)__uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(rp) + j + k) << 16);
-  } else if constexpr (DT == NB_FP8E4M3) {
-    const float sc = exp2f((float)ex);
-#pragma unroll
-    for (int k = 0; k < V; ++k)
-      x[k] = (int)(e4m3x2_to_f32((uint16_t)__ldg(reinterpret_cast<const uint8_t*>(rp) + j + k)).x * sc);
-  } else if constexpr (V == 4) {
+// values j .. j + V - 1 of a row
+template <int V>
+__device__ __forceinline__ void heavy_counts(const char* rp, int j, int (&x)[V]) {
+  if constexpr (V == 4) {
     const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(rp + j));
 #pragma unroll
     for (int k = 0; k < 4; ++k) x[k] = (int)(w >> (8 * k) & 255u);
@@ -1288,7 +1280,7 @@ __device__ __forceinline__ void heavy_counts(const char* rp, int j, int ex, int 
 
 // V features per thread and step: 4 where F is a multiple of 4 (16-byte weight
 // loads), else 1
-template <int DT, int V>
+template <int V>
 __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
   __shared__ long long red[8][32];
   __shared__ unsigned int redT[8][4];
@@ -1296,20 +1288,18 @@ __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_wait();   // the pair pass's list
   const long long n = (long long)min(*a.heavy_n, (unsigned long long)a.heavy_cap);
-  if (n == 0 || n > (DT == NB_U8 ? kTcFewU8 : kTcFew)) return;
+  if (n == 0 || n > kTcFewU8) return;
   const int C = a.M.C, F = a.F, ncb = (C + 7) / 8;
   const long long items = (n + 3) / 4 * ncb;
   for (long long item = blockIdx.x; item < items; item += gridDim.x) {
     const long long rg = item / ncb;
     const int cb = (int)(item % ncb) * 8;
     const char* rp[4];
-    int ex[4];
     long long row[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {   // rows past the end repeat the last one and store nothing
       row[i] = a.heavy[min(4 * rg + i, n - 1)];
       rp[i] = a.X + row[i] * a.ld_bytes;
-      ex[i] = DT == NB_FP8E4M3 && a.row_exp ? (int)a.row_exp[row[i]] : 0;
     }
     long long v[32];   // row i, class cb + c: v[8 i + c]
     unsigned int T[4] = {0u, 0u, 0u, 0u};
@@ -1319,7 +1309,7 @@ __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
       int x[4][V];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        heavy_counts<DT, V>(rp[i], j, ex[i], x[i]);
+        heavy_counts<V>(rp[i], j, x[i]);
 #pragma unroll
         for (int k = 0; k < V; ++k) T[i] += (unsigned int)x[i][k];
       }
@@ -1342,7 +1332,7 @@ __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
           for (int k = 0; k < V; ++k) v[8 * i + c] += (long long)x[i][k] * (long long)q[k];
       }
     }
-    if (DT == NB_U8 && a.ovf_ptr) {
+    if (a.ovf_ptr) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         for (int64_t e = a.ovf_ptr[row[i]] + tid; e < a.ovf_ptr[row[i] + 1]; e += 256) {
@@ -1456,10 +1446,9 @@ __global__ void __launch_bounds__(256, 2) k_tc_heavy(const TcHeavyArgs a) {
   }
 }
 
-template <int DT>
 static nb_status run_tc_heavy(const TcHeavyArgs& h, cudaStream_t st) {
   // every weight row starts on 16 bytes when F is a multiple of 4
-  auto kern = h.F % 4 == 0 ? k_tc_heavy<DT, 4> : k_tc_heavy<DT, 1>;
+  auto kern = h.F % 4 == 0 ? k_tc_heavy<4> : k_tc_heavy<1>;
   count_launch();
   NB_TRY_CUDA(launch_pdl(kern, dim3((unsigned)(num_sms() * 2)), dim3(256), 0, st, h),
               "k_tc_heavy launch");
@@ -1521,7 +1510,7 @@ struct TcScratch {
     bytes = T + 16 * groups;
   }
 };
-size_t tc_scratch_bytes(int C) { return TcScratch(kTcHeavyCap, kTcFew, C).bytes; }
+size_t tc_scratch_bytes(int C) { return TcScratch(kTcHeavyCap, kTcFewU8, C).bytes; }
 
 nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                           const nb_aux* aux, const ScoreOut& o, cudaStream_t st) {
@@ -1556,11 +1545,23 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
   a.recheck = o.recheck;
   a.status = m->d.sstatus;
   a.marks = o.counted ? reinterpret_cast<unsigned long long*>(o.n_rechecked) : nullptr;
-  // FP8 and BF16 rows list no more than those (the chunked pass reads u8 rows only);
-  // what is not listed stays marked for the FP64 recheck.
+  auto pair_pass = [&]() {
+    return u8                 ? run_tc<0, NB_U8>(a, a.models[0].N, a.units0, st)
+           : dt == NB_FP8E4M3 ? run_tc<0, NB_FP8E4M3>(a, a.models[0].N, a.units0, st)
+                              : run_tc<0, NB_BF16>(a, a.models[0].N, a.units0, st);
+  };
+  if (!u8) {
+    // heavy FP8 and BF16 rows go to FP64; in a capture through the marks alone, so
+    // that the graph holds no memory node
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    NB_TRY_CUDA(cudaStreamIsCapturing(st, &cs), "cudaStreamIsCapturing");
+    if (cs != cudaStreamCaptureStatusNone) return pair_pass();
+  }
+  // FP8 and BF16 rows list no more than kTcFew; what is not listed stays marked for
+  // the FP64 recheck.
   const int most = u8 ? kTcHeavyCap : kTcFew;
-  const int cap = n < most ? (int)n : most, few = cap < kTcFew ? cap : kTcFew;
-  const TcScratch lay(cap, few, m->C);
+  const int cap = n < most ? (int)n : most;
+  const TcScratch lay(cap, !u8 ? 0 : (cap < kTcFewU8 ? cap : kTcFewU8), m->C);
   ScoreScratch ss(m, st);
   char* scratch = nullptr;
   nb_status s = ss.take(lay.bytes, m->d.tc_scratch, tc_scratch_bytes(m->C), &scratch);
@@ -1568,37 +1569,34 @@ nb_status launch_score_tc(const nb_model* m, const void* X, nb_dtype dt, int64_t
   a.heavy_n = reinterpret_cast<unsigned long long*>(scratch);
   a.heavy = reinterpret_cast<int*>(scratch + lay.list);
   a.heavy_cap = cap;
-  TcHeavyArgs h{};
-  h.X = g.X;
-  h.ld_bytes = g.ld_bytes;
-  h.ovf_ptr = g.ovf_ptr;
-  h.ovf_col = g.ovf_col;
-  h.ovf_add = g.ovf_add;
-  h.row_exp = g.row_exp;
-  h.M = a.models[0];
-  h.F = a.F;
-  h.want_lp = o.want_lp;
-  h.recheck = o.recheck;
-  h.heavy = a.heavy;
-  h.heavy_n = a.heavy_n;
-  h.heavy_cap = cap;
-  h.sums = reinterpret_cast<long long*>(scratch + lay.sums);
-  h.T = reinterpret_cast<float*>(scratch + lay.T);
-  h.done = reinterpret_cast<unsigned int*>(scratch + 16);
-  h.label = o.label;
-  h.margin = o.margin;
-  h.logpost = o.logpost;
-  h.marks = a.marks;
   NB_TRY_CUDA(cudaMemsetAsync(scratch, 0, lay.clear, st), "memset(heavy count)");
-  if (s == NB_OK)
-    s = u8                   ? run_tc<0, NB_U8>(a, a.models[0].N, a.units0, st)
-        : dt == NB_FP8E4M3 ? run_tc<0, NB_FP8E4M3>(a, a.models[0].N, a.units0, st)
-                             : run_tc<0, NB_BF16>(a, a.models[0].N, a.units0, st);
-  if (s == NB_OK)
-    s = u8                   ? run_tc_heavy<NB_U8>(h, st)
-        : dt == NB_FP8E4M3 ? run_tc_heavy<NB_FP8E4M3>(h, st)
-                             : run_tc_heavy<NB_BF16>(h, st);
-  if (s == NB_OK && u8 && cap > kTcFewU8) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
+  s = pair_pass();
+  if (s == NB_OK && u8) {
+    TcHeavyArgs h{};
+    h.X = g.X;
+    h.ld_bytes = g.ld_bytes;
+    h.ovf_ptr = g.ovf_ptr;
+    h.ovf_col = g.ovf_col;
+    h.ovf_add = g.ovf_add;
+    h.M = a.models[0];
+    h.F = a.F;
+    h.want_lp = o.want_lp;
+    h.recheck = o.recheck;
+    h.heavy = a.heavy;
+    h.heavy_n = a.heavy_n;
+    h.heavy_cap = cap;
+    h.sums = reinterpret_cast<long long*>(scratch + lay.sums);
+    h.T = reinterpret_cast<float*>(scratch + lay.T);
+    h.done = reinterpret_cast<unsigned int*>(scratch + 16);
+    h.label = o.label;
+    h.margin = o.margin;
+    h.logpost = o.logpost;
+    h.marks = a.marks;
+    s = run_tc_heavy(h, st);
+    if (s == NB_OK && cap > kTcFewU8) s = run_tc<1, NB_U8>(a, a.models[0].N, 0, st);
+  } else if (s == NB_OK) {
+    s = launch_recheck_list(m, X, dt, ld, aux, o, a.heavy, a.heavy_n, cap, st);
+  }
   const nb_status f = ss.release();
   return s != NB_OK ? s : f;
 }
