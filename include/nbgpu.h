@@ -177,8 +177,9 @@ typedef struct {
  *         FP8E4M3 with integer values); N_cj is accumulated exactly in
  *         uint64, then log theta and log prior in FP64 on the device.
  *         NB_GAUSSIAN: X holds real values (F32); class means and MLE
- *         variances are computed by two deterministic passes (paired FP32
- *         sums over short runs of rows, FP64 from there on).
+ *         variances are computed by two deterministic passes (FP32 sums with
+ *         two error terms over short runs of rows, rounded to FP64 once and
+ *         added in FP64: the accuracy of FP64 sums).
  *   y     int32 labels in [0, C) (device), n entries.
  *   C     2 <= C <= 255;  F >= 1.
  * On success *out owns device tables; free it with nb_model_free.  Errors:

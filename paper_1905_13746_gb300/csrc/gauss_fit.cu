@@ -4,13 +4,18 @@
 // every variance.
 //
 // What bounds it.  FP64 runs at about two lanes per clock and SM on this part
-// (an FP32 operation at 128), so the passes hold their sums in pairs of FP32
-// numbers with exact error terms (Knuth's two-sum, and the FMA product error):
-// about 48 bits per partial sum for ~12 (pass 1) and ~20 (pass 2) FP32
-// operations a value, where FP64 sums of each class and of all rows cost eight
-// slots of the FP64 pipe, i.e. 512 of an FP32 one.  FP64 is left to what is
-// done once per class and feature.  The overall variance behind eps comes from
-// the class moments (n_c, mu_c, var_c), not from sums of its own.
+// (an FP32 operation at 128), so a warp holds the sums of a run of rows in three
+// FP32 numbers, the sum, its error and the error of that, the first two joined
+// exactly (Knuth's two-sum, and the FMA product error): the run's sum is then
+// exact to about 2^-70 of its largest term and is rounded once, to FP64, for ~15
+// (pass 1) and ~40 (pass 2) FP32 operations a value, where FP64 sums of each class
+// and of all rows cost eight slots of the FP64 pipe, i.e. 512 of an FP32 one.
+// Sums of runs are added in FP64.  (Two numbers a sum, about 48 bits, cost 18 us
+// less at C = 64, F = 256 and left the variances 1e-14 off, where FP64 sums are 4e-16
+// off and these 2e-16.)  The additions are written as intrinsics: a product that the
+// compiler fused into one of them would break the error terms.  The overall
+// variance behind eps comes from the class moments (n_c, mu_c, var_c), not from sums
+// of its own.
 //
 // Pass 2 sums (x - K)^2 with K = fl32(mean) of the class and feature, and
 // var = S2 / n_c - (mean - K)^2; x - K is formed exactly as a pair.  Values
@@ -24,11 +29,11 @@
 // order of every sum is fixed), deals the sorted rows evenly to its 8 warps,
 // and each warp sums runs of one class in registers; a class that several
 // warps share is joined in warp order.  So no class count or class size leaves
-// warps idle, and a (chunk, class, feature) partial is 12 bytes.  Chunks are
-// sized for four blocks per SM; the partials are reduced by a block per class
-// and 32 features in a fixed order: the results are the same bits on every
-// run, and the same with any scratch (nb_refit and the allocation-free
-// re-fit).
+// warps idle, and a (chunk, class, feature) partial is 12 bytes (an FP64 sum and
+// the largest |x|).  Chunks are sized for four blocks per SM; the partials are
+// reduced by a block per class and 32 features in a fixed order: the results are
+// the same bits on every run, and the same with any scratch (nb_refit and the
+// allocation-free re-fit).
 // C = 64, F = 256: re-fit on 64,000 rows (65.5 MB), scoring of 200,000 and
 // reading the parameters: 4.90 -> 0.84 ms, of which the fit was 3.45 ms of
 // device time with FP64 sums in shared memory, 32-row chunks (266 MB of
@@ -51,8 +56,8 @@ struct GfArgs {
   int64_t ld, n;
   int F, C, rows;
   const int32_t* y;
-  float2* part0;        // C x F sums of chunk 0 ...
-  float2* part;         // ... and of chunks 1, 2, ...
+  double* part0;        // C x F sums of chunk 0 ...
+  double* part;         // ... and of chunks 1, 2, ...
   float* amax0;         // C x F max |x| of chunk 0 (pass 1)
   float* amax;          // ... and of the others
   const double* mean;   // C x F (pass 2)
@@ -61,44 +66,60 @@ struct GfArgs {
   int* status;
 };
 
-// (s, e) += x with the rounding error of s kept in e (Knuth)
-__device__ __forceinline__ void pair_add(float& s, float& e, float x) {
-  const float t = s + x;
-  const float b = t - s;
-  e += (s - (t - b)) + (x - b);
-  s = t;
+// s = a + b rounded, e = what the rounding lost (Knuth)
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float t = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
 }
 
 // One run's sums of this lane's feature.
 struct GfAcc {
-  float s = 0.f, e = 0.f;
+  float s = 0.f, e = 0.f, l = 0.f;
   unsigned int m = 0u;   // pass 1: max of |x| as bits (NaN above infinity)
+  __device__ __forceinline__ double sum() const { return (double)s + ((double)e + (double)l); }
 };
+
+// The FP64 sum of a run, or of several.
+struct GfSum {
+  double s = 0.0;
+  unsigned int m = 0u;
+};
+__device__ __forceinline__ void gf_join(GfSum& a, const GfSum& b) {
+  a.s += b.s;
+  a.m = max(a.m, b.m);
+}
 
 template <int PASS>
 __device__ __forceinline__ void gf_add(GfAcc& a, float x, float K, float sc) {
+  float r, t;
   if (PASS == 1) {
     a.m = max(a.m, __float_as_uint(x) & 0x7FFFFFFFu);
-    pair_add(a.s, a.e, x);
+    two_sum(a.s, x, a.s, r);
+    two_sum(a.e, r, a.e, t);
+    a.l = __fadd_rn(a.l, t);
   } else {
-    // d + dl = x sc - K exactly; its square joins as p + q + 2 d dl
-    const float xs = x * sc;
-    const float d = xs - K;
-    const float b = xs - d;
-    const float dl = (xs - (d + b)) + (b - K);
-    const float p = d * d;
-    const float q = fmaf(d, d, -p);
-    pair_add(a.s, a.e, p);
-    a.e += fmaf(2.f * d, dl, q);
+    // d + dl = x sc - K exactly; its square is p + q + w + (u + dl^2), u the
+    // product error of w
+    float d, dl, t2, t3, t4;
+    two_sum(__fmul_rn(x, sc), -K, d, dl);
+    const float p = __fmul_rn(d, d), q = __fmaf_rn(d, d, -p);
+    const float d2 = __fmul_rn(2.f, d), w = __fmul_rn(d2, dl);
+    const float u = __fmaf_rn(dl, dl, __fmaf_rn(d2, dl, -w));
+    two_sum(a.s, p, a.s, r);
+    two_sum(a.e, r, a.e, t2);
+    two_sum(a.e, q, a.e, t3);
+    two_sum(a.e, w, a.e, t4);
+    a.l = __fadd_rn(a.l, __fadd_rn(__fadd_rn(t2, t3), __fadd_rn(t4, u)));
   }
 }
 
 template <int PASS>
-__device__ __forceinline__ void gf_store(const GfArgs& a, int c, int j, const GfAcc& v) {
+__device__ __forceinline__ void gf_store(const GfArgs& a, int c, int j, const GfSum& v) {
   if (j >= a.F) return;
   const int64_t at = (int64_t)c * a.F + j;
   const int64_t off = blockIdx.x == 0 ? at : ((int64_t)(blockIdx.x - 1) * a.C) * a.F + at;
-  (blockIdx.x == 0 ? a.part0 : a.part)[off] = make_float2(v.s, v.e);
+  (blockIdx.x == 0 ? a.part0 : a.part)[off] = v.s;
   if (PASS == 1) {
     (blockIdx.x == 0 ? a.amax0 : a.amax)[off] = __uint_as_float(v.m);
     if (v.m >= 0x7F800000u) atomicOr(a.status, ST_BAD_VALUE);
@@ -110,7 +131,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
   extern __shared__ __align__(16) unsigned char gf_sm[];
   __shared__ uint16_t s_order[kGfMaxRows];
   __shared__ int s_off[kTcMaxC + 1];
-  __shared__ GfAcc s_frag[2 * kGfWarps][32];
+  __shared__ GfSum s_frag[2 * kGfWarps][32];
   __shared__ int s_fc[2 * kGfWarps];
   uint16_t* cnt = reinterpret_cast<uint16_t*>(gf_sm);   // [label group][class]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -207,20 +228,21 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
         if (pos + u < end) gf_add<PASS>(v, x[u], K, sc);
       pos = end;
     }
+    const GfSum sum{v.sum(), v.m};
     if (start == s_off[c] && end == s_off[c + 1]) {
-      gf_store<PASS>(a, c, j, v);
+      gf_store<PASS>(a, c, j, sum);
     } else {   // the class is shared with a neighbouring warp: slot 0 begins, slot 1 ends a share
       const int slot = 2 * warp + (start == a0 ? 0 : 1);
-      s_frag[slot][lane] = v;
+      s_frag[slot][lane] = sum;
       if (lane == 0) s_fc[slot] = c;
     }
   }
   // classes without rows in this chunk
   for (int k = warp; k < C; k += kGfWarps)
-    if (s_off[k] == s_off[k + 1]) gf_store<PASS>(a, k, j, GfAcc{});
+    if (s_off[k] == s_off[k + 1]) gf_store<PASS>(a, k, j, GfSum{});
   __syncthreads();
   if (warp == 0) {   // join the shared classes' pieces in order
-    GfAcc v;
+    GfSum v;
     int cur = -1;
     for (int k = 0; k < 2 * kGfWarps; ++k) {
       const int fc = s_fc[k];
@@ -230,10 +252,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
         v = s_frag[k][lane];
         cur = fc;
       } else {
-        const GfAcc o = s_frag[k][lane];
-        pair_add(v.s, v.e, o.s);
-        v.e += o.e;
-        v.m = max(v.m, o.m);
+        gf_join(v, s_frag[k][lane]);
       }
     }
     if (cur >= 0) gf_store<PASS>(a, cur, j, v);
@@ -255,33 +274,26 @@ struct GfRed {
   TcgHeader* tcg_hdr;       // cleared here when present
 };
 
-// the pair of this lane's (class, feature) over all chunks (valid in warp 0)
+// the sum of this lane's (class, feature) over all chunks (valid in warp 0)
 template <int PASS>
-__device__ __forceinline__ GfAcc gf_reduce(const GfRed& r, int c, int j) {
-  __shared__ GfAcc sh[kGfWarps][32];
+__device__ __forceinline__ GfSum gf_reduce(const GfRed& r, int c, int j) {
+  __shared__ GfSum sh[kGfWarps][32];
   const GfArgs& a = r.a;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  GfAcc v;
+  GfSum v;
   if (j < a.F) {
     const int64_t at = (int64_t)c * a.F + j, step = (int64_t)a.C * a.F;
 #pragma unroll 4
     for (int k = warp; k < r.nchunk; k += kGfWarps) {
       const int64_t off = k == 0 ? at : (int64_t)(k - 1) * step + at;
-      const float2 p = (k == 0 ? a.part0 : a.part)[off];
-      pair_add(v.s, v.e, p.x);
-      v.e += p.y;
+      v.s += (k == 0 ? a.part0 : a.part)[off];
       if (PASS == 1) v.m = max(v.m, __float_as_uint((k == 0 ? a.amax0 : a.amax)[off]));
     }
   }
   sh[warp][lane] = v;
   __syncthreads();
   if (warp == 0)
-    for (int k = 1; k < kGfWarps; ++k) {
-      const GfAcc o = sh[k][lane];
-      pair_add(v.s, v.e, o.s);
-      v.e += o.e;
-      v.m = max(v.m, o.m);
-    }
+    for (int k = 1; k < kGfWarps; ++k) gf_join(v, sh[k][lane]);
   return v;
 }
 
@@ -297,10 +309,10 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_mean(const GfRed r) {
       if (r.tcg_hdr) r.tcg_hdr->bad = 0;
     }
   }
-  const GfAcc v = gf_reduce<1>(r, c, j);
+  const GfSum v = gf_reduce<1>(r, c, j);
   if (threadIdx.x >= 32 || j >= a.F) return;
   const double nc = (double)a.nc[c];
-  double mean = nc > 0 ? ((double)v.s + (double)v.e) / nc : 0.0;
+  double mean = nc > 0 ? v.s / nc : 0.0;
   if (!isfinite(v.s) && v.m < 0x7F800000u) {
     // finite values whose FP32 sum overflowed (above 2^127 in all): FP64, row by row
     double t = 0.0;
@@ -322,12 +334,12 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_var(const GfRed r) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.y, j = blockIdx.x * 32 + lane;
   pdl_wait();
-  const GfAcc v = gf_reduce<2>(r, c, j);
+  const GfSum v = gf_reduce<2>(r, c, j);
   if (warp == 0 && j < a.F) {
     const int64_t at = (int64_t)c * a.F + j;
     const double nc = (double)a.nc[c], mean = r.mu[at], sc = (double)r.scale[at];
     const double dk = mean - (double)(float)mean;
-    double var = nc > 0 ? ((double)v.s + (double)v.e) / (nc * sc * sc) - dk * dk : 0.0;
+    double var = nc > 0 ? v.s / (nc * sc * sc) - dk * dk : 0.0;
     if (var < 0.0) var = 0.0;
     __stcg(&r.var[at], var);
   }
@@ -495,7 +507,7 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   const int64_t rows = gf_rows(n, F, C), nchunk = (n + rows - 1) / rows;
   const size_t cf = (size_t)C * F;
   const int nft = (F + 31) / 32, jt = (F + 255) / 256, CP = gauss_cpad(C);
-  // scratch: pairs and maxima of the chunks after the first, the finish
+  // scratch: sums and maxima of the chunks after the first, the finish
   // kernel's tile sums, counters.  The first chunk's go to the model's count
   // table (which a Gaussian model does not use) and, before the variances are
   // written there, to its variance table.
@@ -508,11 +520,11 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   a.C = C;
   a.rows = (int)rows;
   a.y = y;
-  a.part0 = reinterpret_cast<float2*>(d.counts);
+  a.part0 = reinterpret_cast<double*>(d.counts);
   a.amax0 = reinterpret_cast<float*>(d.p1);
   double* part = reinterpret_cast<double*>(s);
   s += 16 * (size_t)C * jt;
-  a.part = reinterpret_cast<float2*>(s);
+  a.part = reinterpret_cast<double*>(s);
   s += (size_t)(nchunk - 1) * cf * 8;
   a.amax = reinterpret_cast<float*>(s);
   s += (size_t)(nchunk - 1) * cf * 4;

@@ -1,0 +1,37 @@
+"""The Gaussian fit's class moments are as exact as FP64 sums.
+
+A run's sum is rounded to FP64 once; sums of runs are added in FP64: at most three pieces
+of a class per chunk, ceil(chunks / 8) chunks per warp, eight warps.  Every addition and
+the final divisions and subtraction round by at most 2^-53 of the sum of magnitudes, so
+a moment is within (additions + 4) 2^-53 of it (mean: of mean |x|; variance: of itself and
+of the square by which K, the FP32 mean, may miss the mean, at most 2^-48 of the mean's).
+The reference is summed in NumPy's long double (64 bits of mantissa or more).
+"""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+nb = pytest.importorskip("paper_1905_13746_gb300")
+
+
+@pytest.mark.parametrize("n,F,C,offset", [(700, 40, 2, 0.0), (4096, 400, 2, 10.0), (9000, 33, 5, 3.0),
+                                          (70_000, 40, 3, 100.0), (20_000, 64, 64, 5.0)])
+def test_moments_round_like_fp64_sums(n, F, C, offset):
+    rng = np.random.default_rng(n + F)
+    y = (np.arange(n) % C).astype(np.int32)
+    rng.shuffle(y)
+    X = (rng.normal(size=(n, F)) * rng.uniform(0.5, 3, F) + offset * rng.uniform(0, 1, F)).astype(np.float32)
+    mu, var, _ = nb.fit(torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), C,
+                        kind=nb.NB_GAUSSIAN, var_smoothing=0.0).params()
+    rows = 64 if n <= 65536 else 512          # the fewest rows of a chunk: the most chunks
+    adds = 3 + -(-n // rows) // 8 + 1 + 8
+    u = (adds + 4) * 2.0 ** -53
+    for c in range(C):
+        r = X[y == c].astype(np.longdouble)
+        m = r.mean(axis=0)
+        v = np.square(r - m).mean(axis=0)
+        assert (np.abs(mu[c] - m) <= u * np.abs(r).mean(axis=0)).all(), c
+        assert (np.abs(var[c] - v) <= u * (v + 2.0 ** -48 * m * m)).all(), \
+            (c, float(np.max(np.abs(var[c] - v) / v)), u)
