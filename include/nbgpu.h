@@ -134,7 +134,8 @@ typedef struct nb_server nb_server;
  *            row fits a stage, else the register-streaming kernel; U8 and
  *            FP8E4M3 rows, whose results no shape changes, take the one that
  *            measured faster for their width unless a stage shape is given;
- *            NB_VARIANT_PIPELINED / NB_VARIANT_REGISTER: force one.
+ *            NB_VARIANT_PIPELINED / NB_VARIANT_REGISTER: force one.  F32, U16
+ *            and BF16 rows off 16-byte boundaries have one kernel.
  *            3..64 classes with U8, FP8E4M3 or BF16 storage, X 16-byte
  *            aligned and ld * element size a multiple of 16:
  *            NB_VARIANT_AUTO / NB_VARIANT_PIPELINED take the tensor-core

@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     frexp(maxabs64, &e);   // maxabs64 < 2^e
     S = 22 - e;
   }
-  const double scale = ldexp(1.0, S);
+  const double scale = ldexp(1.0, S), fine_step = ldexp(1.0, -S - 8);
   // U features per thread at a time: their log theta loads all go out before
   // the byte stores of the limbs (which may alias them) hold the next ones up
   constexpr int U = 4;
@@ -627,7 +627,9 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
       if (jj >= F_pad) continue;
       const int32_t q = (int32_t)llrint(dd[u] * scale);   // |q| <= 2^22
       delta_q[jj] = q;
-      delta_p[jj] = (int32_t)llrint(dd[u] * scale * 256.0);   // |.| <= 2^30
+      const double fine = dd[u] * scale * 256.0, whole = rint(fine);   // |.| <= 2^30
+      delta_p[jj] = (int32_t)whole;
+      reinterpret_cast<float*>(delta_p)[F_pad + jj] = (float)((fine - whole) * fine_step);
       // balanced base-256 digits q = q2*65536 + q1*256 + q0, each in [-128, 127]
       const int32_t q0 = ((q + 128) & 255) - 128;
       const int32_t r1 = (q - q0) >> 8;

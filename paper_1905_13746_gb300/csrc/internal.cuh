@@ -107,7 +107,8 @@ struct ModelDev {
   C2Header* c2;        // 1
   float* delta;        // F_pad      FP32 Delta, plain order
   int32_t* delta_q;    // F_pad      fixed-point Delta
-  int32_t* delta_p;    // F_pad      fixed-point Delta, eight bits finer (step 2^-(S+8))
+  int32_t* delta_p;    // F_pad      fixed-point Delta, eight bits finer (step 2^-(S+8)), then
+                       //            F_pad floats: what it leaves of Delta
   uint4* limbs;        // 3 * nvec8  int8 limbs of delta_q, interleaved (u8 path), then
                        //            F_pad packed words (limb l in byte l)
   float4* il[3];       // interleaved FP32 quads for 4/8/16 elements per vector

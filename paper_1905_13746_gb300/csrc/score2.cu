@@ -330,11 +330,25 @@ __device__ __forceinline__ void c2_float_store(const S2Args& a, const C2Header& 
 }
 
 __device__ __forceinline__ void c2_fix_store(const S2Args& a, const C2Header& h, int64_t row,
-                                             long long D, float T) {
-  float d, tau;
-  fix_result(D, T, h, d, tau);
-  if (c2_store(a.label, a.margin, a.logpost, a.want_lp, a.recheck, row, d, tau) && a.marks)
+                                             long long D, float Rs, float T, int depth) {
+  double d;
+  float tau;
+  fix_result(D, Rs, T, depth, h, d, tau);
+  if (c2_store64(a.label, a.margin, a.logpost, a.want_lp, a.recheck, row, (float)d, d, tau) && a.marks)
     atomicAdd(a.marks, 1ull);
+}
+
+// The totals T of a group's four rows' counts and R of their residuals, by quarter as in
+// sum4_transposed.
+template <int LPR>
+__device__ __forceinline__ void fix_totals(const FixSum2 (&fix)[2], int li, float& T, float& R) {
+  float v[4];
+  f32x2_unpack(fix[0].t, v[0], v[1]);
+  f32x2_unpack(fix[1].t, v[2], v[3]);
+  T = sum4_transposed<LPR>(v[0], v[1], v[2], v[3], li);
+  f32x2_unpack(fix[0].r, v[0], v[1]);
+  f32x2_unpack(fix[1].r, v[2], v[3]);
+  R = sum4_transposed<LPR>(v[0], v[1], v[2], v[3], li);
 }
 
 // Short rows of 16-bit values: a group of LPR lanes sums four rows at a time;
@@ -342,13 +356,14 @@ __device__ __forceinline__ void c2_fix_store(const S2Args& a, const C2Header& h,
 // something else than counts are the group's rows read again for the FP32
 // sums.  Bound by about 9 operations a value (F = 128: 2.8 TB/s).
 template <int DT, int LPR>
-__global__ void __launch_bounds__(256) k_score2_fix(const S2Args a) {
+__global__ void __launch_bounds__(256, 3) k_score2_fix(const S2Args a) {
   using Dec = Decode<DT>;
   constexpr int EPV = Dec::EPV, R = 4, SUBS = 32 / LPR, RPW = SUBS * R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t bar;
   if (!stage_table(smem_raw, a.table, a.table_bytes, &bar, a.status, ST_TIMEOUT)) return;
   const int4* tab = reinterpret_cast<const int4*>(smem_raw);
+  const float4* res = reinterpret_cast<const float4*>(smem_raw + a.table_bytes / 2);
   const C2Header h = *a.hdr;
   const int lane = threadIdx.x & 31, sub = lane / LPR, li = lane % LPR;
   const int nv = a.nvec_row;
@@ -358,52 +373,58 @@ __global__ void __launch_bounds__(256) k_score2_fix(const S2Args a) {
        t += nwarps) {
     const int64_t row0 = t * RPW + (int64_t)sub * R;
     const char* rp[R];
-    FixSum fix[R];
-    float tf[R];
+    FixSum2 fix[R / 2];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {   // rows past the end repeat the last one and store nothing
+    for (int r = 0; r < R; ++r)   // rows past the end repeat the last one and store nothing
       rp[r] = a.X + min(row0 + r, a.n - 1) * a.ld_bytes;
-      tf[r] = 0.f;
-    }
 #pragma unroll 2
     for (int v = li; v < nv; v += LPR) {
       uint4 x[R];
 #pragma unroll
       for (int r = 0; r < R; ++r) x[r] = ld_stream16(rp[r] + (int64_t)v * 16);
       int q[EPV];
+      float qr[EPV];
 #pragma unroll
       for (int k = 0; k < EPV / 4; ++k) {
         const int4 d = tab[v * (EPV / 4) + k];
+        const float4 e = res[v * (EPV / 4) + k];
+        qr[4 * k] = e.x;
+        qr[4 * k + 1] = e.y;
+        qr[4 * k + 2] = e.z;
+        qr[4 * k + 3] = e.w;
         q[4 * k] = d.x;
         q[4 * k + 1] = d.y;
         q[4 * k + 2] = d.z;
         q[4 * k + 3] = d.w;
       }
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        float val[EPV];
-        Dec::run(x[r], val);
+      for (int r = 0; r < R; r += 2) {
+        float v0[EPV], v1[EPV];
+        Dec::run(x[r], v0);
+        Dec::run(x[r + 1], v1);
         if (v == nv - 1) {
 #pragma unroll
           for (int e = 0; e < EPV; ++e)
-            if (v * EPV + e >= a.F) val[e] = 0.f;
+            if (v * EPV + e >= a.F) v0[e] = v1[e] = 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < EPV; ++e) {
-          fix_add(fix[r], val[e], q[e]);
-          tf[r] += val[e];
-        }
+        for (int e = 0; e < EPV; ++e) fix_add(fix[r / 2], v0[e], v1[e], q[e], qr[e]);
       }
     }
-    unsigned bad[R], any = 0u;   // per row: the groups whose row is no row of counts
-#pragma unroll
-    for (int r = 0; r < R; ++r) any |= bad[r] = __ballot_sync(0xFFFFFFFFu, fix[r].bad != 0u);
-    const long long D = sum4_transposed<LPR>(fix[0].D, fix[1].D, fix[2].D, fix[3].D, li);
-    const float T = sum4_transposed<LPR>(tf[0], tf[1], tf[2], tf[3], li);
+    // per row: the groups whose row is no row of counts
+    const unsigned bad[R] = {__ballot_sync(0xFFFFFFFFu, fix[0].bad0()),
+                             __ballot_sync(0xFFFFFFFFu, fix[0].bad1()),
+                             __ballot_sync(0xFFFFFFFFu, fix[1].bad0()),
+                             __ballot_sync(0xFFFFFFFFu, fix[1].bad1())};
+    const unsigned any = bad[0] | bad[1] | bad[2] | bad[3];
+    const long long D = sum4_transposed<LPR>(fix[0].D0, fix[0].D1, fix[1].D0, fix[1].D1, li);
+    float T, Rs;
+    fix_totals<LPR>(fix, li, T, Rs);
     const int mr = li / (LPR / 4);   // this lane's quarter holds row mr of the group
     const unsigned gmask = LPR == 32 ? 0xFFFFFFFFu : ((1u << (LPR & 31)) - 1u) << (sub * LPR);
     const unsigned mybad = (mr == 0 ? bad[0] : mr == 1 ? bad[1] : mr == 2 ? bad[2] : bad[3]) & gmask;
-    if (li % (LPR / 4) == 0 && row0 + mr < a.n && mybad == 0u) c2_fix_store(a, h, row0 + mr, D, T);
+    if (li % (LPR / 4) == 0 && row0 + mr < a.n && mybad == 0u)
+      c2_fix_store(a, h, row0 + mr, D, Rs, T, EPV * ((nv + LPR - 1) / LPR) + 5);
     if (any) {
 #pragma unroll 1
       for (int g = 0; g < SUBS; ++g) {
@@ -430,7 +451,7 @@ __global__ void __launch_bounds__(256) k_score2_fix(const S2Args a) {
 // ones only where a row holds something else than counts.  Without FIX (label
 // and OFF modes) the FP32 sums.
 // 100,003 rows of 1,003 F32 counts (401 MB), log-posterior mode, labels only:
-// 76 us for the whole call; 3.57 ms as 2 of the 64 class columns of the general
+// 78 us for the whole call; 3.57 ms as 2 of the 64 class columns of the general
 // scorer's 64 x 64 tiles (1.08 ms) and every row in FP64 on top (2.5 ms).
 // 249,252 rows (1 GB): 158 us in the label mode (93% of the measured HBM rate),
 // 190 us (78%) in the log-posterior mode.
@@ -447,7 +468,7 @@ __device__ __forceinline__ float any_load(const char* rp, int j) {
 }
 
 template <int DT, bool FIX>
-__global__ void __launch_bounds__(256) k_score2_any(const S2Args a) {
+__global__ void __launch_bounds__(256, 3) k_score2_any(const S2Args a) {
   constexpr int R = 4, U = 8;   // rows, elements in flight per row and lane
   const int lane = threadIdx.x & 31;
   const C2Header h = *a.hdr;
@@ -459,7 +480,7 @@ __global__ void __launch_bounds__(256) k_score2_any(const S2Args a) {
 #pragma unroll
     for (int r = 0; r < R; ++r)   // rows past the end repeat the last one and store nothing
       rp[r] = a.X + min(t * R + r, a.n - 1) * a.ld_bytes;
-    // every element once: add(row, value, element)
+    // every element once: add(the rows' values, the tables' entry)
     auto sweep = [&](auto&& table, auto&& add) {
       for (int j = lane; j < a.F; j += 32 * U) {
         float x[U][R];
@@ -470,35 +491,39 @@ __global__ void __launch_bounds__(256) k_score2_any(const S2Args a) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const auto w = table(j + 32 * u < a.F ? j + 32 * u : 0);
-#pragma unroll
-          for (int r = 0; r < R; ++r) add(r, x[u][r], w);
+          add(x[u], w);
         }
       }
     };
     const int64_t row = t * R + lane / 8;   // eight lanes hold each row's sums
     bool todo = true;
     if (FIX) {
-      FixSum fix[R];
-      float tf[R] = {0.f, 0.f, 0.f, 0.f};
-      sweep([&](int j) { return __ldg(a.delta_p + j); },
-            [&](int r, float x, int q) {
-              fix_add(fix[r], x, q);
-              tf[r] += x;
+      FixSum2 fix[R / 2];
+      sweep([&](int j) { return make_int2(__ldg(a.delta_p + j), __float_as_int(__ldg(a.delta_r + j))); },
+            [&](const float (&x)[R], int2 q) {
+              fix_add(fix[0], x[0], x[1], q.x, __int_as_float(q.y));
+              fix_add(fix[1], x[2], x[3], q.x, __int_as_float(q.y));
             });
-      unsigned bad = 0u;   // bit r: row r is no row of counts
-#pragma unroll
-      for (int r = 0; r < R; ++r) bad |= (__ballot_sync(0xFFFFFFFFu, fix[r].bad != 0u) != 0u) << r;
-      const long long D = sum4_transposed<32>(fix[0].D, fix[1].D, fix[2].D, fix[3].D, lane);
-      const float T = sum4_transposed<32>(tf[0], tf[1], tf[2], tf[3], lane);
+      // bit r: row r is no row of counts
+      const unsigned bad = (__any_sync(0xFFFFFFFFu, fix[0].bad0()) ? 1u : 0u) |
+                           (__any_sync(0xFFFFFFFFu, fix[0].bad1()) ? 2u : 0u) |
+                           (__any_sync(0xFFFFFFFFu, fix[1].bad0()) ? 4u : 0u) |
+                           (__any_sync(0xFFFFFFFFu, fix[1].bad1()) ? 8u : 0u);
+      const long long D = sum4_transposed<32>(fix[0].D0, fix[0].D1, fix[1].D0, fix[1].D1, lane);
+      float T, Rs;
+      fix_totals<32>(fix, lane, T, Rs);
       todo = (bad >> (lane / 8)) & 1u;
-      if (lane % 8 == 0 && row < a.n && !todo) c2_fix_store(a, h, row, D, T);
+      if (lane % 8 == 0 && row < a.n && !todo) c2_fix_store(a, h, row, D, Rs, T, (a.F + 31) / 32 + 5);
       if (!bad) continue;
     }
     float s[R] = {0.f, 0.f, 0.f, 0.f}, tf[R] = {0.f, 0.f, 0.f, 0.f};
     sweep([&](int j) { return __ldg(a.delta + j); },
-          [&](int r, float x, float w) {
-            s[r] = fmaf(x, w, s[r]);
-            tf[r] += fabsf(x);
+          [&](const float (&x)[R], float w) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              s[r] = fmaf(x[r], w, s[r]);
+              tf[r] += fabsf(x[r]);
+            }
           });
     const float S = sum4_transposed<32>(s[0], s[1], s[2], s[3], lane);
     const float T = sum4_transposed<32>(tf[0], tf[1], tf[2], tf[3], lane);
@@ -612,6 +637,7 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   a.delta_q = m->d.delta_q;
   a.delta = m->d.delta;
   a.delta_p = m->d.delta_p;
+  a.delta_r = reinterpret_cast<const float*>(m->d.delta_p + m->F_pad);
   a.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
   a.ovf_col = aux ? aux->ovf_col : nullptr;
   a.ovf_add = aux ? aux->ovf_add : nullptr;
@@ -654,14 +680,18 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
                    : launch_persistent(k_score2_any<NB_BF16, false>, 0, tiles, a, st);
     }
   }
+  const nb_tile_config& cfg = m->tile;
+  const bool open = cfg.variant == NB_VARIANT_AUTO && cfg.stages == 0 && cfg.rows_per_stage == 0 &&
+                    cfg.rows_per_warp == 0;   // no kernel or shape is asked for
   // 16-bit rows of at most 16 vectors, which the pipelined kernel spreads over
   // 32 lanes (1M BF16 files: F = 64 52 us against 127, F = 128 93 against 159;
   // at F = 256 175 against 146 and at 1,024 291 against 211, so longer rows
   // stay there).  F32 rows stay with the FP32 sums, which batches share.
   if (fix && es == 2 && a.nvec_row <= 16) {
-    a.table = m->d.delta_p;
+    a.table = m->d.delta_p;   // and the residuals
+    a.table_bytes = 2 * smem;
     a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row
-    return dt == NB_U16 ? launch_fix<NB_U16>(a, smem, st) : launch_fix<NB_BF16>(a, smem, st);
+    return dt == NB_U16 ? launch_fix<NB_U16>(a, 2 * smem, st) : launch_fix<NB_BF16>(a, 2 * smem, st);
   }
   // u8 and FP8 rows: the sums are exact, so the kernel and its shape change no
   // result, and the faster one is taken where none is asked for.  Dense rows
@@ -677,11 +707,9 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   // 48 / 225, 384 158 / 225, 640 192 / 225, 3,072 117 us).  The default shape
   // took 226 us at F = 256, 144 at 1,024 and 146 at 2,048.  Two stages of 48 rows; shorter ones while the call has fewer than
   // three tiles per block.
-  const nb_tile_config& cfg = m->tile;
   nb_tile_config shape = cfg;
   bool pipe = cfg.variant != NB_VARIANT_REGISTER;
-  if (limbs && cfg.variant == NB_VARIANT_AUTO && cfg.stages == 0 && cfg.rows_per_stage == 0 &&
-      cfg.rows_per_warp == 0) {
+  if (limbs && open) {
     const int nv = a.nvec_row;
     pipe = a.ovf_ptr != nullptr && (nv == 16 || nv == 32 || (nv >= 52 && nv <= 128));
     shape.rows_per_warp = nv == 16 || (nv > 32 && nv <= 64) ? 2 : 1;

@@ -24,6 +24,7 @@ struct S2Args {
   const int32_t* delta_q;   // plain fixed-point table (overflow entries)
   const float* delta;       // plain FP32 table (overflow entries)
   const int32_t* delta_p;   // plain fixed-point table of step 2^-(S+8)
+  const float* delta_r;     // and its residuals
   const int64_t* ovf_ptr;
   const uint16_t* ovf_col;
   const uint16_t* ovf_add;
@@ -47,9 +48,8 @@ __device__ __forceinline__ float softplusf(float z) {
 // tau = +inf says that the fast path's sums are not valid for this row at all
 // (see c2_tau_u8): the row is marked in every recheck mode, NB_RECHECK_OFF
 // included.
-__device__ __forceinline__ bool c2_store(uint8_t* label, float* margin, float* logpost,
-                                         int want_lp, int recheck, int64_t row, float d,
-                                         float tau) {
+__device__ __forceinline__ bool c2_decide(uint8_t* label, float* margin, int recheck, int64_t row,
+                                          float d, float tau) {
   bool flag = !(tau < INFINITY);
   const float ad = fabsf(d);
   if (recheck != NB_RECHECK_OFF) {
@@ -58,9 +58,46 @@ __device__ __forceinline__ bool c2_store(uint8_t* label, float* margin, float* l
   }
   label[row] = flag ? kLabelRecheck : (d > 0.f ? 1 : 0);
   margin[row] = ad;
+  return flag;
+}
+
+__device__ __forceinline__ bool c2_store(uint8_t* label, float* margin, float* logpost,
+                                         int want_lp, int recheck, int64_t row, float d,
+                                         float tau) {
+  const bool flag = c2_decide(label, margin, recheck, row, d, tau);
   if (want_lp) {
     logpost[2 * row] = -softplusf(d);
     logpost[2 * row + 1] = -softplusf(-d);
+  }
+  return flag;
+}
+
+// log1p(exp(-x)) and x more than it, rounded once each.  Out of line: inlined, the
+// FP64 functions cost the kernels a third of their warps (128 registers for 80).
+static __device__ __noinline__ float2 softplus_near(double x) {
+  const double s = log1p(exp(-x));
+  return make_float2((float)s, (float)(x + s));
+}
+
+// c2_store of a log-odds known beyond FP32, d = (float)d64 (the exact sums of F32 and 16-bit
+// rows, which stand in for the FP64 recheck): each output is the FP64
+// one rounded once.  From |d| = 20 on log1p(exp(-|d|)) is below 3e-9 and FP32
+// takes it as exp(-|d|); few rows are nearer.
+__device__ __forceinline__ bool c2_store64(uint8_t* label, float* margin, float* logpost,
+                                           int want_lp, int recheck, int64_t row, float d,
+                                           double d64, float tau) {
+  const bool flag = c2_decide(label, margin, recheck, row, d, tau);
+  if (want_lp) {
+    float near, far = fabsf(d);   // -log posterior of the class decided for, and of the other
+    if (far < 20.f) {
+      const float2 nf = softplus_near(fabs(d64));
+      near = nf.x;
+      far = nf.y;
+    } else {
+      near = expf(-far);
+    }
+    logpost[2 * row] = -(d > 0.f ? far : near);
+    logpost[2 * row + 1] = -(d > 0.f ? near : far);
   }
   return flag;
 }
@@ -181,34 +218,54 @@ struct Decode<NB_FP8E4M3> {
 // scoring (2.5 ms against 1.1 ms for 100,000 rows of 1,003 counts).  The
 // kernels for rows of any alignment and for short 16-bit rows therefore sum a
 // fixed-point Delta exactly, D = sum x P in int64 with P = round(Delta 2^(S+8)),
-// |P| <= 2^30 (eight bits finer than the u8 path's, so that the result is the
-// FP64 one to FP32 rounding).  With u = x + 2^23 in FP32, x is an integer in
-// [0, 2^23) exactly when u lies in [2^23, 2^24) and u - 2^23 has x's bits; x is
+// |P| <= 2^30, and in FP32 what P leaves of Delta, at most half a step a count:
+// the result is the FP64 one to FP32 rounding.  (Without the residuals margins were off
+// by up to half a step a count, many FP32 units of a small one; they cost 74 -> 78 us
+// at 100,003 rows of 1,003 F32 counts, 149 -> 174 at 200,000 of 1,001 BF16 ones and
+// nothing on short 16-bit rows.)  With u = x + 2^23 in FP32, x is an integer in
+// [0, 2^23) exactly when x's bits lie below 2^23's and u - 2^23 has x's bits; x is
 // then u's low 23 bits.  D cannot wrap below a total of 2^33 counts
 // (fix_result).  A row with any other value takes FP32 sums and their bound.
 // The integer sums do not depend on the order of the additions.
-struct FixSum {
-  long long D = 0;
-  uint32_t bad = 0u;   // non-zero: a value that is no count below 2^23
+// Two rows at a time: a packed instruction serves both.
+struct FixSum2 {
+  long long D0 = 0, D1 = 0;
+  uint64_t r = 0, t = 0;           // FP32 pairs: the residuals' sums, the counts' totals
+  uint32_t off0 = 0u, off1 = 0u;   // non-zero: a value that is no integer
+  uint32_t max0 = 0u, max1 = 0u;   // largest value as bits (negative ones and NaN above infinity)
+  __device__ __forceinline__ bool bad0() const { return off0 != 0u || max0 >= 0x4B000000u; }
+  __device__ __forceinline__ bool bad1() const { return off1 != 0u || max1 >= 0x4B000000u; }
 };
 
-__device__ __forceinline__ void fix_add(FixSum& f, float x, int q) {
-  const float u = x + 8388608.f;
-  const uint32_t ub = __float_as_uint(u);
-  f.bad |= (__float_as_uint(u - 8388608.f) ^ __float_as_uint(x)) | ((ub & 0xFF800000u) ^ 0x4B000000u);
-  f.D += (long long)(int)(ub & 0x007FFFFFu) * (long long)q;
+__device__ __forceinline__ void fix_add(FixSum2& f, float x0, float x1, int q, float r) {
+  const uint64_t x = f32x2_pack(x0, x1), m = f32x2_pack(8388608.f, 8388608.f);
+  const uint64_t u = f32x2_add(x, m);
+  float u0, u1, v0, v1;
+  f32x2_unpack(u, u0, u1);
+  f32x2_unpack(f32x2_add(u, f32x2_pack(-8388608.f, -8388608.f)), v0, v1);
+  const uint32_t a0 = __float_as_uint(u0), a1 = __float_as_uint(u1);
+  f.off0 |= __float_as_uint(v0) ^ __float_as_uint(x0);
+  f.off1 |= __float_as_uint(v1) ^ __float_as_uint(x1);
+  f.max0 = max(f.max0, __float_as_uint(x0));
+  f.max1 = max(f.max1, __float_as_uint(x1));
+  f.D0 += (long long)(int)(a0 & 0x007FFFFFu) * (long long)q;
+  f.D1 += (long long)(int)(a1 & 0x007FFFFFu) * (long long)q;
+  f.t = f32x2_add(f.t, x);
+  f.r = f32x2_fma(x, f32x2_pack(r, r), f.r);
 }
 
-// Log-odds and bound of a row from its exact sum; T is the FP32 sum of the
-// counts.  The bound holds the quantisation of Delta (half a step per count)
-// and slack for the FP64 reference's own rounding; a total at which D could
-// have wrapped sends the row to FP64.
-__device__ __forceinline__ void fix_result(long long D, float T, const C2Header& h, float& d,
-                                           float& tau) {
+// Log-odds and bound of a row from its exact sum and the sum R of its residuals
+// (`depth` roundings deep); T is the FP32 sum of the counts.  The bound holds R's
+// rounding and that of the residuals, each at most half a step, and slack for the
+// FP64 reference's own rounding; a total at which D could have wrapped sends the row
+// to FP64.
+__device__ __forceinline__ void fix_result(long long D, float R, float T, int depth,
+                                           const C2Header& h, double& d, float& tau) {
   const double step = __hiloint2double((1023 - h.S - 8) << 20, 0);   // 2^-(S+8)
-  d = (float)((double)D * step + h.b64);
+  d = fma((double)D, step, (double)R) + h.b64;
   T *= 1.001f;
-  tau = T < 4e9f ? 0.5f * T * (float)step * 1.0001f + 1e-12f * (T * h.maxabs + fabsf(h.b)) + 1e-30f
+  tau = T < 4e9f ? T * (float)step * (float)(depth + 2) * 5.9604645e-8f +
+                       1e-12f * (T * h.maxabs + fabsf(h.b)) + 1e-30f
                  : INFINITY;
 }
 
