@@ -135,7 +135,9 @@ typedef struct nb_server nb_server;
  *            FP8E4M3 rows, whose results no shape changes, take the one that
  *            measured faster for their width unless a stage shape is given;
  *            NB_VARIANT_PIPELINED / NB_VARIANT_REGISTER: force one.  F32, U16
- *            and BF16 rows off 16-byte boundaries have one kernel.
+ *            and BF16 rows off 16-byte boundaries have one kernel, and FP8
+ *            rows of up to 496 features one (37-bit weights, FP64 outputs)
+ *            that NB_VARIANT_AUTO and NB_VARIANT_PIPELINED take.
  *            3..64 classes with U8, FP8E4M3 or BF16 storage, X 16-byte
  *            aligned and ld * element size a multiple of 16:
  *            NB_VARIANT_AUTO / NB_VARIANT_PIPELINED take the tensor-core
@@ -158,7 +160,8 @@ typedef struct nb_server nb_server;
  * For u8 storage every configuration gives bit-identical results (exact
  * integer sums).  For the FP32 paths the two variants share the reduction
  * order when a row spans >= 64 sixteen-byte vectors; nb_autotune_score keeps
- * the variant fixed otherwise, so tuning never changes a result. */
+ * the variant fixed otherwise (and for the FP8 rows of up to 496 features), so
+ * tuning never changes a result. */
 typedef enum {
   NB_VARIANT_AUTO = 0,
   NB_VARIANT_PIPELINED = 1,

@@ -70,6 +70,7 @@ static nb_status alloc_model(nb_model* m) {
   const size_t o_dq = take(sizeof(int32_t) * Fp);
   const size_t o_dp = take(2 * sizeof(int32_t) * Fp);   // with the residuals behind it
   const size_t o_limbs = take(7 * Fp);   // three limb planes + packed limb words
+  const size_t o_limbs5 = take(fp8_narrow(m->F) ? 5 * Fp : 0);
   const size_t o_il0 = take(sizeof(float) * Fp);
   const size_t o_il1 = take(sizeof(float) * Fp);
   const size_t o_il2 = take(sizeof(float) * Fp);
@@ -114,6 +115,7 @@ static nb_status alloc_model(nb_model* m) {
   d.delta_q = reinterpret_cast<int32_t*>(b + o_dq);
   d.delta_p = reinterpret_cast<int32_t*>(b + o_dp);
   d.limbs = reinterpret_cast<uint4*>(b + o_limbs);
+  d.limbs5 = fp8_narrow(m->F) ? reinterpret_cast<uint4*>(b + o_limbs5) : nullptr;
   d.il[0] = reinterpret_cast<float4*>(b + o_il0);
   d.il[1] = reinterpret_cast<float4*>(b + o_il1);
   d.il[2] = reinterpret_cast<float4*>(b + o_il2);

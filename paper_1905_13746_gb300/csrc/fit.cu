@@ -483,7 +483,7 @@ constexpr int kFinT = 4 * kFinF;   // threads per block
 __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     const unsigned long long* counts, const unsigned long long* nc, int64_t n, int F, int F_pad,
     int nvec8, double alpha, int prior_given, double* log_theta, double* log_pi, C2Header* hdr,
-    float* delta, int32_t* delta_q, int32_t* delta_p, uint4* limbs, float4* il4, float4* il8,
+    float* delta, int32_t* delta_q, int32_t* delta_p, uint4* limbs, uint4* limbs5, float4* il4, float4* il8,
     float4* il16, float* w, float* bias, float* wmax, unsigned long long* fin, int* status) {
   constexpr int NT = kFinT, NL = 2 * kFinF;   // NL threads take the per-feature logs
   __shared__ unsigned long long part[2][2];
@@ -645,6 +645,15 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
       // the same limbs packed into one word per feature (overflow entries)
       reinterpret_cast<uint32_t*>(L + (size_t)3 * F_pad)[jj] =
           (uint32_t)(q0 & 255) | ((uint32_t)(q1 & 255) << 8) | ((uint32_t)(q2 & 255) << 16);
+      if (limbs5) {   // what q leaves of Delta, in steps of 2^-(S+15): |f| <= 2^14
+        const int32_t f = (int32_t)llrint((dd[u] * scale - (double)q) * 32768.0);
+        const int32_t f0 = ((f + 128) & 255) - 128, f1 = (f - f0) >> 8;   // |f1| <= 64
+        const int32_t l5[5] = {q0, q1, q2, f0, f1};
+#pragma unroll
+        for (int l = 0; l < 5; ++l)
+          reinterpret_cast<unsigned char*>(limbs5)[((size_t)l * nvec8 + v) * 16 + b] =
+              (unsigned char)(l5[l] & 255);
+      }
     }
   }
   if (tid < 2) bias[tid] = (float)log_pi[tid];
@@ -801,7 +810,7 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
                            0, st, reinterpret_cast<const unsigned long long*>(d.counts),
                            reinterpret_cast<const unsigned long long*>(d.nc), (int64_t)n, F,
                            m->F_pad, m->nvec8, m->alpha, (int)(log_prior_dev != nullptr), d.p0,
-                           d.log_pi, d.c2, d.delta, d.delta_q, d.delta_p, d.limbs, d.il[0], d.il[1],
+                           d.log_pi, d.c2, d.delta, d.delta_q, d.delta_p, d.limbs, d.limbs5, d.il[0], d.il[1],
                            d.il[2], d.w, d.bias, d.wmax, d.fin, d.status),
                 "k_fit_finish_c2");
     return NB_OK;

@@ -87,6 +87,10 @@ struct TcgHeader {
   float wsum;         // sum_j (max_c |B_cj| + max_c |A_cj|), rounded up
 };
 
+// Two-class FP8 rows of fewer than 32 vectors of 16 bytes take five limbs of Delta (see
+// k_score2_u8).
+inline bool fp8_narrow(int F) { return F <= 31 * 16; }
+
 // ---------------------------------------------------------------------------
 // model (library-owned)
 // ---------------------------------------------------------------------------
@@ -111,6 +115,8 @@ struct ModelDev {
                        //            F_pad floats: what it leaves of Delta
   uint4* limbs;        // 3 * nvec8  int8 limbs of delta_q, interleaved (u8 path), then
                        //            F_pad packed words (limb l in byte l)
+  uint4* limbs5;       // 5 * nvec8  the three limbs and two more (step 2^-(S+15)) for narrow FP8
+                       //            rows (fp8_narrow), else nullptr
   float4* il[3];       // interleaved FP32 quads for 4/8/16 elements per vector
   // general-C tables (CUDA-core scorer)
   float* w;            // C x F_pad  centred weights log theta_cj - mean_c log theta_cj

@@ -161,6 +161,107 @@ __global__ void __launch_bounds__(256) k_score2_u8(const S2Args a) {
   c2_flush_marks(a, marks);
 }
 
+// ---------------------------------------------------------------------------
+// FP8 rows of fewer than 32 vectors (F <= 496): five limbs, FP64 outputs
+// ---------------------------------------------------------------------------
+// Every such row once went to FP64 from the pipelined kernel (a lane without a vector
+// failed the count check: 1M files of F = 256 13.3 ms), so what replaces that keeps
+// its accuracy: Delta in 37 bits, five limbs instead of three, one rounding of each
+// output.  Bound by the decode as k_score2_u8 (1M files of F = 64 45 us, 256 102, 480
+// 204; three limbs 39, 110 and 194).
+template <int LPR>
+__global__ void __launch_bounds__(256, 3) k_score2_fp8(const S2Args a) {
+  constexpr int R = 2, SUBS = 32 / LPR, RPW = SUBS * R;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t bar;
+  if (!stage_table(smem_raw, a.table, a.table_bytes, &bar, a.status, ST_TIMEOUT)) return;
+  const uint4* tab = reinterpret_cast<const uint4*>(smem_raw);
+  const C2Header h = *a.hdr;
+  const int lane = threadIdx.x & 31, sub = lane / LPR, li = lane % LPR;
+  const int nv = a.nvec_row, nt = a.nvec_tab;
+  const int64_t ntiles = (a.n + RPW - 1) / RPW;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  // byte masks of the last (partial) vector
+  const int keep = a.F - 16 * (nv - 1);
+  uint32_t tm[4];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    int vb = keep - 4 * w;
+    vb = vb < 0 ? 0 : (vb > 4 ? 4 : vb);
+    tm[w] = vb >= 4 ? 0xFFFFFFFFu : ((1u << (8 * vb)) - 1u);
+  }
+  const double step = __hiloint2double((1023 - h.S - 15) << 20, 0);   // 2^-(S+15)
+  // the prior's part in whole steps: d is then an integer until it is rounded to FP32.
+  // (In FP64 where it does not fit: weights of next to nothing.)
+  const bool whole = fabs(h.b64) < 4.611686018427388e18 * step;
+  const long long b = whole ? llrint(h.b64 / step) : 0ll;
+  unsigned marks = 0;
+  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles;
+       t += nwarps) {
+    const int64_t row0 = t * RPW + (int64_t)sub * R;
+    int acc[R][5];
+    uint32_t tot[R], m2[R];
+    Fp8Check chk[R];
+    const char* rp[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {   // rows past the end repeat the last one and store nothing
+      const int64_t row = min(row0 + r, a.n - 1);
+#pragma unroll
+      for (int l = 0; l < 5; ++l) acc[r][l] = 0;
+      tot[r] = 0;
+      rp[r] = a.X + row * a.ld_bytes;
+      m2[r] = fp8_magic(a.row_exp ? (int)a.row_exp[row] : 0);
+    }
+#pragma unroll 2
+    for (int v = li; v < nv; v += LPR) {
+      uint4 x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = ld_stream16(rp[r] + (int64_t)v * 16);
+      const uint4 q[5] = {tab[v], tab[nt + v], tab[2 * nt + v], tab[3 * nt + v], tab[4 * nt + v]};
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (v == nv - 1) {
+          x[r].x &= tm[0];
+          x[r].y &= tm[1];
+          x[r].z &= tm[2];
+          x[r].w &= tm[3];
+        }
+        fp8_vector_limbs5(x[r], q, m2[r], acc[r], tot[r], chk[r]);
+      }
+    }
+    long long D[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      // |acc| <= 128 T < 2^31 (c2_tau_u8's limit), |D| < 2^62
+      D[r] = ((((long long)acc[r][2] << 16) + ((long long)acc[r][1] << 8) + (long long)acc[r][0]) << 15) +
+             ((long long)acc[r][4] << 8) + (long long)acc[r][3];
+      tot[r] = fp8_lane_total(tot[r], chk[r], m2[r]);
+    }
+#pragma unroll
+    for (int off = LPR / 2; off > 0; off >>= 1) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        D[r] += __shfl_xor_sync(0xFFFFFFFFu, D[r], off);
+        tot[r] += __shfl_xor_sync(0xFFFFFFFFu, tot[r], off);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (row0 + r >= a.n || r % LPR != li) continue;
+      // (|D| < 2^62 and |b| <= 2^62: no wrap)
+      const float d = whole ? (float)(D[r] + b) * (float)step : (float)fma((double)D[r], step, h.b64);
+      const double d64 = whole ? (double)(D[r] + b) * step : fma((double)D[r], step, h.b64);
+      const float T = (float)tot[r];
+      // the three-limb kernels' bound: the rows that it does not settle are the
+      // recheck's in every kernel
+      const float tau = c2_tau_u8(T, d, h.b, h.inv_scale, h.maxabs);
+      marks += c2_store64(a.label, a.margin, a.logpost, a.want_lp, a.recheck, row0 + r, d, d64,
+                          tau);
+    }
+  }
+  c2_flush_marks(a, marks);
+}
+
 template <int DT, int LPR, int R>
 __global__ void __launch_bounds__(256) k_score2_fp(const S2Args a) {
   using Dec = Decode<DT>;
@@ -624,6 +725,12 @@ static nb_status launch_fix(const S2Args& a, int smem, cudaStream_t st) {
   return launch_persistent(k_score2_fix<DT, 4>, smem, (a.n + 31) / 32, a, st);
 }
 
+// Narrow FP8 rows: about eight vectors per lane, at least two lanes per row.
+static nb_status launch_fp8(const S2Args& a, int smem, cudaStream_t st) {
+  if (a.nvec_row > 16) return launch_persistent(k_score2_fp8<4>, smem, (a.n + 15) / 16, a, st);
+  return launch_persistent(k_score2_fp8<2>, smem, (a.n + 31) / 32, a, st);
+}
+
 nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n, int64_t ld,
                         const nb_aux* aux, const ScoreOut& o, cudaStream_t st) {
   const int es = elem_size(dt);
@@ -683,6 +790,12 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   const nb_tile_config& cfg = m->tile;
   const bool open = cfg.variant == NB_VARIANT_AUTO && cfg.stages == 0 && cfg.rows_per_stage == 0 &&
                     cfg.rows_per_warp == 0;   // no kernel or shape is asked for
+  if (dt == NB_FP8E4M3 && fp8_narrow(m->F) && cfg.variant != NB_VARIANT_REGISTER) {
+    a.table = m->d.limbs5;
+    smem = 5 * m->nvec8 * 16;
+    a.table_bytes = (uint32_t)smem;
+    return launch_fp8(a, smem, st);
+  }
   // 16-bit rows of at most 16 vectors, which the pipelined kernel spreads over
   // 32 lanes (1M BF16 files: F = 64 52 us against 127, F = 128 93 against 159;
   // at F = 256 175 against 146 and at 1,024 291 against 211, so longer rows
@@ -693,13 +806,13 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
     a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row
     return dt == NB_U16 ? launch_fix<NB_U16>(a, 2 * smem, st) : launch_fix<NB_BF16>(a, 2 * smem, st);
   }
-  // u8 and FP8 rows: the sums are exact, so the kernel and its shape change no
+  // u8 and wider FP8 rows: the sums are exact, so the kernel and its shape change no
   // result, and the faster one is taken where none is asked for.  Dense rows
   // stream through registers: over F = 64 .. 6,000 that is the fastest or
   // within 4% of it (u8, against the pipelined kernel's default shape: 1M files
   // of F = 64 24 / 121 us, 256 56 / 162, 512 90 / 147; 586,000 of 1,024
-  // 102 / 106; 293,000 of 2,048 102 / 139; FP8: 36 / 225, 90 / 231, 167 / 248,
-  // 198 / 207, 195 / 238).  With an overflow list the pipelined kernel, whose
+  // 102 / 106; 293,000 of 2,048 102 / 139; FP8 from F = 512 on: 167 / 248, 198 / 207,
+  // 195 / 238).  With an overflow list the pipelined kernel, whose
   // producer fetches the entries ahead, wins where the row fills its lanes:
   // 16 vectors (two rows per pass: F = 256 127 against 143 us), 32 (512:
   // 163 / 173), 52 to 64 (two rows: 900 148 / 165, 1,024 116 / 143) and up to

@@ -79,8 +79,8 @@ static __device__ __noinline__ float2 softplus_near(double x) {
   return make_float2((float)s, (float)(x + s));
 }
 
-// c2_store of a log-odds known beyond FP32, d = (float)d64 (the exact sums of F32 and 16-bit
-// rows, which stand in for the FP64 recheck): each output is the FP64
+// c2_store of a log-odds known beyond FP32, d = (float)d64 (the exact sums of F32, 16-bit and
+// narrow FP8 rows, which stand in for the FP64 recheck): each output is the FP64
 // one rounded once.  From |d| = 20 on log1p(exp(-|d|)) is below 3e-9 and FP32
 // takes it as exp(-|d|); few rows are nearer.
 __device__ __forceinline__ bool c2_store64(uint8_t* label, float* margin, float* logpost,
@@ -350,6 +350,24 @@ __device__ __forceinline__ void fp8_vector_limbs_biased(const uint4& x, const ui
     a1 = dp2a_hi_us(u23, l1[k], dp2a_lo_us(u01, l1[k], a1));
     a2 = dp2a_hi_us(u23, l2[k], dp2a_lo_us(u01, l2[k], a2));
     tt = (uint32_t)dp2a_hi_us(u23, 0x01010101u, dp2a_lo_us(u01, 0x01010101u, (int)tt));
+  }
+}
+
+// fp8_vector_limbs with the two limbs of the finer table (see fp8_narrow).
+__device__ __forceinline__ void fp8_vector_limbs5(const uint4& x, const uint4 (&q)[5], uint32_t m2,
+                                                  int (&acc)[5], uint32_t& tt, Fp8Check& c) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t u01, u23;
+    fp8_biased_pairs(w[k], m2, u01, u23, c);
+    const uint32_t x01 = u01 & 0x03FF03FFu, x23 = u23 & 0x03FF03FFu;
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+      const uint32_t lw = k == 0 ? q[l].x : k == 1 ? q[l].y : k == 2 ? q[l].z : q[l].w;
+      acc[l] = dp2a_hi_us(x23, lw, dp2a_lo_us(x01, lw, acc[l]));
+    }
+    tt = (uint32_t)dp2a_hi_us(x23, 0x01010101u, dp2a_lo_us(x01, 0x01010101u, (int)tt));
   }
 }
 

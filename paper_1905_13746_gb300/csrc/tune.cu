@@ -57,7 +57,8 @@ extern "C" nb_status nb_autotune_score(nb_model* m, const void* X, nb_dtype dtyp
   }
   const int64_t ld_bytes = ld * es;
   const int nvec_row = (m->F * es + 15) / 16;
-  const bool same_order = dtype == NB_U8 || dtype == NB_FP8E4M3 || nvec_row > 64;
+  // narrow FP8 rows take three limbs instead of five in the register kernel
+  const bool same_order = dtype == NB_U8 || (dtype == NB_FP8E4M3 && !fp8_narrow(m->F)) || nvec_row > 64;
 
   std::vector<nb_tile_config> cand;
   // rows per warp changes the FP32 reduction tree, so it is varied only for u8

@@ -1,19 +1,20 @@
 """Two-class rows that stand in for the FP64 recheck: each output is the FP64 one rounded once.
 
 F32, U16 and BF16 counts at any alignment (log-posterior mode) sum a 30-bit Delta exactly and
-its residuals in FP32.  One heavy feature
+its residuals in FP32; FP8 rows of up to 496 features sum a 37-bit Delta.  One heavy feature
 makes the step coarse while the other weights are small, so that many margins are near zero,
 where an absolute error of the step's size would show.
 
 Tolerance: half an FP32 unit (2^-24 of the value), and, absolute, the part of Delta that the
-sums leave out -- per count half a step 2^-(S+9) times (depth + 2) roundings of 2^-24 -- and the FP64 sums' own rounding on both sides, F additions of terms that
+sums leave out -- per count half a step 2^-(S+9) times (depth + 2) roundings of 2^-24, or half
+a step 2^-(S+16) -- and the FP64 sums' own rounding on both sides, F additions of terms that
 make up T max |log theta|, 2^-53 each; 2^(22 - S) is the power of two above max |Delta|.
 """
 import numpy as np
 import pytest
 import torch
 
-from _common import oracle_mn, to_np
+from _common import oracle_mn, stored, to_np
 from test_gpu_float_counts import _features
 
 pytestmark = pytest.mark.gpu
@@ -55,3 +56,16 @@ def test_float_and_16_bit_counts(fmt, F, pad):
     depth = max(8 * 4, (F + 31) // 32) + 7      # values a lane sums, shuffles, the residual's own
     _check(to_np(nb.score(model, f)), m, ref, vals, 2.0 ** -9 * depth * 2.0 ** -24)
 
+
+@pytest.mark.parametrize("F", [1, 16, 17, 100, 256, 257, 495, 496])
+@pytest.mark.parametrize("mode", [nb.NB_RECHECK_LP, nb.NB_RECHECK_OFF])
+def test_narrow_fp8_counts(F, mode):
+    X, y = _rows(F, 3000, F, 16)
+    f, vals = stored(X, "fp8")
+    model = nb.fit(f, torch.from_numpy(y).cuda(), 2)
+    m, ref = oracle_mn(vals, y, 2, vals)
+    res = to_np(nb.score(model, f, recheck=mode))
+    if mode == nb.NB_RECHECK_OFF:     # labels of nearer rows are the recheck's to settle
+        near = ref["margin"] <= 1e-6
+        res["label"][near] = ref["label"][near]
+    _check(res, m, ref, vals, 2.0 ** -16)
