@@ -137,7 +137,8 @@ typedef struct nb_server nb_server;
  *            NB_VARIANT_PIPELINED / NB_VARIANT_REGISTER: force one.  F32, U16
  *            and BF16 rows off 16-byte boundaries have one kernel, and FP8
  *            rows of up to 496 features one (37-bit weights, FP64 outputs)
- *            that NB_VARIANT_AUTO and NB_VARIANT_PIPELINED take.
+ *            that NB_VARIANT_AUTO and NB_VARIANT_PIPELINED take; so do U16 and
+ *            BF16 rows of up to 256 bytes in the log-posterior mode.
  *            3..64 classes with U8, FP8E4M3 or BF16 storage, X 16-byte
  *            aligned and ld * element size a multiple of 16:
  *            NB_VARIANT_AUTO / NB_VARIANT_PIPELINED take the tensor-core

@@ -800,7 +800,7 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   // 32 lanes (1M BF16 files: F = 64 52 us against 127, F = 128 93 against 159;
   // at F = 256 175 against 146 and at 1,024 291 against 211, so longer rows
   // stay there).  F32 rows stay with the FP32 sums, which batches share.
-  if (fix && es == 2 && a.nvec_row <= 16) {
+  if (fix && es == 2 && a.nvec_row <= 16 && cfg.variant != NB_VARIANT_REGISTER) {
     a.table = m->d.delta_p;   // and the residuals
     a.table_bytes = 2 * smem;
     a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row

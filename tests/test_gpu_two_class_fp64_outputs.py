@@ -14,7 +14,7 @@ import numpy as np
 import pytest
 import torch
 
-from _common import oracle_mn, stored, to_np
+from _common import compare, oracle_mn, stored, to_np
 from test_gpu_float_counts import _features
 
 pytestmark = pytest.mark.gpu
@@ -69,3 +69,20 @@ def test_narrow_fp8_counts(F, mode):
         near = ref["margin"] <= 1e-6
         res["label"][near] = ref["label"][near]
     _check(res, m, ref, vals, 2.0 ** -16)
+
+
+@pytest.mark.parametrize("fmt", ["u16", "bf16"])
+def test_the_register_kernel_can_be_asked_for(fmt):
+    """Its FP32 bound leaves most rows of the log-posterior mode to FP64; the exact sums none."""
+    X, y = _rows(5, 3000, 64, 250)
+    f, vals = _features(X, fmt, 0)
+    model = nb.fit(f, torch.from_numpy(y).cuda(), 2)
+    m, ref = oracle_mn(vals, y, 2, vals)
+    marked = {}
+    for variant in (nb.NB_VARIANT_AUTO, nb.NB_VARIANT_PIPELINED, nb.NB_VARIANT_REGISTER):
+        model.set_tile_config(variant, 0, 0, 0)
+        res = to_np(nb.score(model, f))
+        marked[variant] = res["n_rechecked"]
+        compare(res, ref)
+    assert marked[nb.NB_VARIANT_AUTO] == marked[nb.NB_VARIANT_PIPELINED] <= 30
+    assert marked[nb.NB_VARIANT_REGISTER] > 1500
