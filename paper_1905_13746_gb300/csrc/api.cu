@@ -330,7 +330,9 @@ struct PinnedBuffer {
   void* p = nullptr;
   bool tried = false;
   ~PinnedBuffer() {
-    if (p) cudaFreeHost(p);
+    if (!p) return;
+    const RelaxedCapture relaxed;   // a thread may end while another captures
+    cudaFreeHost(p);
   }
 };
 static void* pinned_staging(size_t bytes) {
