@@ -68,9 +68,9 @@ static SegGroup* list_of(void* base, int fam, int max_groups) {
 
 // The launches of one call (work list already on the device and *counter
 // cleared).  `groups`: the lists' group counts where the host knows them (an
-// empty list is not launched), else nullptr.  The two-class launch comes after
-// the tensor-core one, programmatically: its blocks fill the SMs that run out of
-// 256-row units first.
+// empty list is not launched), else nullptr.  The two-class launch comes directly
+// after the tensor-core one, programmatically where there is one: its blocks fill
+// the SMs that run out of 256-row units first.
 static nb_status batch_launch(nb_batch* b, const int* groups, cudaStream_t st) {
   SegHeader* dh = hdr_of(b->dev);
   unsigned long long* marks = reinterpret_cast<unsigned long long*>(b->counter);
@@ -93,7 +93,7 @@ static nb_status batch_launch(nb_batch* b, const int* groups, cudaStream_t st) {
     a.groups = list_of(b->dev, 0, b->max_groups);
     a.hdr = dh;
     a.marks = marks;
-    nb_status s = launch_score2_seg(a, b->plan, b->dtype, b->kv, b->smem, st);
+    nb_status s = launch_score2_seg(a, b->plan, b->dtype, b->kv, b->smem, has(2), st);
     if (s != NB_OK) return s;
   }
   // also under NB_RECHECK_OFF: rows a scorer could not compute at all are marked

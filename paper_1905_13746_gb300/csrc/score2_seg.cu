@@ -222,7 +222,10 @@ __global__ void __launch_bounds__(256, 2) k_score2_seg_u8(const SegArgs a) {
   __syncthreads();
   const bool ok = mbar_wait_bounded(&bar, 0);
   if (!ok) atomicOr(a.status, ST_TIMEOUT);
-  if (__syncthreads_and(ok) == 0) return;
+  if (__syncthreads_and(ok) == 0) {
+    pdl_wait();   // as at the end
+    return;
+  }
 
   const int lane = threadIdx.x & 31, sub = lane / LPR, li = lane % LPR;
   const int nv = a.nvec_row, nt = a.nvec_tab, n_groups = a.hdr->n_groups;
@@ -330,7 +333,7 @@ __global__ void __launch_bounds__(256, 2) k_score2_seg_u8(const SegArgs a) {
     }
   }
   if (marks) atomicAdd(a.marks, (unsigned long long)marks);
-  // launched programmatically after the many-class kernel, whose output this
+  // launched programmatically behind the many-class kernel, whose output this
   // one does not read: its completion has to imply that one's
   pdl_wait();
 }
@@ -355,8 +358,11 @@ static nb_status run_seg(const SegArgs& a, const PipeArgs& p, int smem, cudaStre
   return NB_OK;
 }
 
+// behind_tc: the many-class kernel is the launch before this one; it read the lists
+// and the cleared counter as this one does, and triggers this one while it runs.  Behind
+// anything else (the copy or the memset that settles those) an ordinary launch waits.
 template <int LPR, int R>
-static nb_status run_seg_u8(const SegArgs& a, cudaStream_t st) {
+static nb_status run_seg_u8(const SegArgs& a, bool behind_tc, cudaStream_t st) {
   auto kern = k_score2_seg_u8<LPR, R>;
   const int smem = (int)(a.table_stride * (uint32_t)a.n_models);
   if (smem > kSmemOptIn)
@@ -370,8 +376,13 @@ static nb_status run_seg_u8(const SegArgs& a, cudaStream_t st) {
     return NB_EUNSUPPORTED;
   }
   count_launch();
-  NB_TRY_CUDA(launch_pdl(kern, dim3((unsigned)(num_sms() * occ)), dim3(256), (size_t)smem, st, a),
-              "k_score2_seg_u8 launch");
+  const dim3 grid((unsigned)(num_sms() * occ));
+  if (behind_tc) {
+    NB_TRY_CUDA(launch_pdl(kern, grid, dim3(256), (size_t)smem, st, a), "k_score2_seg_u8 launch");
+  } else {
+    kern<<<grid, 256, smem, st>>>(a);
+    NB_TRY_CUDA(cudaGetLastError(), "k_score2_seg_u8 launch");
+  }
   return NB_OK;
 }
 
@@ -422,13 +433,13 @@ nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n
 }
 
 nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int smem,
-                            cudaStream_t st) {
+                            bool behind_tc, cudaStream_t st) {
   if (dt == NB_U8) {   // lanes per row: about eight vectors each (see pick_lpr_u8), rows as there
     const int nv = a.nvec_row;
-    if (nv <= 16) return run_seg_u8<2, 2>(a, st);
-    if (nv <= 32) return run_seg_u8<4, 4>(a, st);
-    if (nv <= 64) return run_seg_u8<8, 4>(a, st);
-    return run_seg_u8<16, 4>(a, st);
+    if (nv <= 16) return run_seg_u8<2, 2>(a, behind_tc, st);
+    if (nv <= 32) return run_seg_u8<4, 4>(a, behind_tc, st);
+    if (nv <= 64) return run_seg_u8<8, 4>(a, behind_tc, st);
+    return run_seg_u8<16, 4>(a, behind_tc, st);
   }
   if (dt == NB_F32) {
     switch (kv) {

@@ -67,7 +67,7 @@ struct PipeArgs;
 nb_status seg2_plan(nb_dtype dt, int F, int F_pad, long long max_ld_bytes, int n_models,
                     bool plain_rows, PipeArgs* p, int* kv_out, int* smem_out);
 nb_status launch_score2_seg(const SegArgs& a, const PipeArgs& p, nb_dtype dt, int kv, int smem,
-                            cudaStream_t st);
+                            bool behind_tc, cudaStream_t st);
 nb_status launch_score_gen_seg(const SegGroup* groups, const SegHeader* hdr,
                                const nb_model* const* models, int n_models, nb_dtype dt, int F,
                                int want_lp, int recheck, unsigned long long* marks, int* status,
