@@ -7,8 +7,8 @@
 // (an FP32 operation at 128), so a warp holds the sums of a run of rows in three
 // FP32 numbers, the sum, its error and the error of that, the first two joined
 // exactly (Knuth's two-sum, and the FMA product error): the run's sum is then
-// exact to about 2^-70 of its largest term and is rounded once, to FP64, for ~15
-// (pass 1) and ~40 (pass 2) FP32 operations a value, where FP64 sums of each class
+// exact to about 2^-70 of its largest term and is rounded once, to FP64, for ~8
+// (pass 1) and ~22 (pass 2) packed FP32 instructions a value, where FP64 sums of each class
 // and of all rows cost eight slots of the FP64 pipe, i.e. 512 of an FP32 one.
 // Sums of runs are added in FP64.  (Two numbers a sum, about 48 bits, cost 18 us
 // less at C = 64, F = 256 and left the variances 1e-14 off, where FP64 sums are 4e-16
@@ -68,18 +68,26 @@ struct GfArgs {
   int* status;
 };
 
+// Two rows at a time, one in each half of a packed instruction (the same roundings, half
+// the issue slots, which bound pass 2: 43 -> 53 us with one row an instruction).
+__device__ __forceinline__ uint64_t neg2(uint64_t a) {
+  return f32x2_fma(a, f32x2_pack(-1.f, -1.f), f32x2_pack(-0.f, -0.f));
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  return f32x2_fma(b, f32x2_pack(-1.f, -1.f), a);
+}
 // s = a + b rounded, e = what the rounding lost (Knuth)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float t = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+__device__ __forceinline__ void two_sum2(uint64_t a, uint64_t b, uint64_t& s, uint64_t& e) {
+  s = f32x2_add(a, b);
+  const uint64_t t = sub2(s, a);
+  e = f32x2_add(sub2(a, sub2(s, t)), sub2(b, t));
 }
 
-// One run's sums of this lane's feature.
+// One run's sums of this lane's feature, of its even and its odd rows.
 struct GfAcc {
-  float s = 0.f, e = 0.f, l = 0.f;
+  uint64_t s = 0, e = 0, l = 0;
   unsigned int m = 0u;   // pass 1: max of |x| as bits (NaN above infinity)
-  __device__ __forceinline__ double sum() const { return (double)s + ((double)e + (double)l); }
+  __device__ __forceinline__ double sum() const;
 };
 
 // The FP64 sum of a run, or of several.
@@ -92,27 +100,44 @@ __device__ __forceinline__ void gf_join(GfSum& a, const GfSum& b) {
   a.m = max(a.m, b.m);
 }
 
+// Both halves joined (as exactly as a row is), then one rounding to FP64.
+__device__ __forceinline__ double GfAcc::sum() const {
+  float s0, s1, e0, e1, l0, l1, t[3];
+  f32x2_unpack(s, s0, s1);
+  f32x2_unpack(e, e0, e1);
+  f32x2_unpack(l, l0, l1);
+  auto two_sum = [](float a, float b, float& r) {
+    const float c = __fadd_rn(a, b), d = __fsub_rn(c, a);
+    r = __fadd_rn(__fsub_rn(a, __fsub_rn(c, d)), __fsub_rn(b, d));
+    return c;
+  };
+  s0 = two_sum(s0, s1, t[0]);
+  e0 = two_sum(e0, e1, t[1]);
+  e0 = two_sum(e0, t[0], t[2]);
+  l0 = __fadd_rn(__fadd_rn(l0, l1), __fadd_rn(t[1], t[2]));
+  return (double)s0 + ((double)e0 + (double)l0);
+}
+
+// Pass 1: x the two rows' values.  Pass 2: x their values, scaled; nK = -K twice.
 template <int PASS>
-__device__ __forceinline__ void gf_add(GfAcc& a, float x, float K, float sc) {
-  float r, t;
+__device__ __forceinline__ void gf_add(GfAcc& a, uint64_t x, uint64_t nK) {
+  uint64_t r, t;
   if (PASS == 1) {
-    a.m = max(a.m, __float_as_uint(x) & 0x7FFFFFFFu);
-    two_sum(a.s, x, a.s, r);
-    two_sum(a.e, r, a.e, t);
-    a.l = __fadd_rn(a.l, t);
+    two_sum2(a.s, x, a.s, r);
+    two_sum2(a.e, r, a.e, t);
+    a.l = f32x2_add(a.l, t);
   } else {
-    // d + dl = x sc - K exactly; its square is p + q + w + (u + dl^2), u the
-    // product error of w
-    float d, dl, t2, t3, t4;
-    two_sum(__fmul_rn(x, sc), -K, d, dl);
-    const float p = __fmul_rn(d, d), q = __fmaf_rn(d, d, -p);
-    const float d2 = __fmul_rn(2.f, d), w = __fmul_rn(d2, dl);
-    const float u = __fmaf_rn(dl, dl, __fmaf_rn(d2, dl, -w));
-    two_sum(a.s, p, a.s, r);
-    two_sum(a.e, r, a.e, t2);
-    two_sum(a.e, q, a.e, t3);
-    two_sum(a.e, w, a.e, t4);
-    a.l = __fadd_rn(a.l, __fadd_rn(__fadd_rn(t2, t3), __fadd_rn(t4, u)));
+    // d + dl = x - K exactly; its square is p + q + w + u, u of w's product error and dl^2
+    uint64_t d, dl, t2, t3, t4;
+    two_sum2(x, nK, d, dl);
+    const uint64_t p = f32x2_mul(d, d), q = f32x2_fma(d, d, neg2(p));
+    const uint64_t d2 = f32x2_add(d, d), w = f32x2_mul(d2, dl);
+    const uint64_t u = f32x2_fma(dl, dl, f32x2_fma(d2, dl, neg2(w)));
+    two_sum2(a.s, p, a.s, r);
+    two_sum2(a.e, r, a.e, t2);
+    two_sum2(a.e, q, a.e, t3);
+    two_sum2(a.e, w, a.e, t4);
+    a.l = f32x2_add(a.l, f32x2_add(f32x2_add(t2, t3), f32x2_add(t4, u)));
   }
 }
 
@@ -211,23 +236,33 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
       sc = a.scale[at];
       K = (float)a.mean[at] * sc;
     }
+    const uint64_t nK = f32x2_pack(-K, -K);
     GfAcc v;
     constexpr int U = 8;   // rows in flight per lane
+    auto rows = [&](const float (&x)[U], int n) {   // a row past the run: nothing to add
+#pragma unroll
+      for (int u = 0; u < U; u += 2) {
+        if (u >= n) break;
+        if (PASS == 1) {
+          v.m = max(v.m, max(__float_as_uint(x[u]) & 0x7FFFFFFFu, __float_as_uint(x[u + 1]) & 0x7FFFFFFFu));
+          gf_add<PASS>(v, f32x2_pack(x[u], x[u + 1]), nK);
+        } else {
+          gf_add<PASS>(v, f32x2_pack(__fmul_rn(x[u], sc), u + 1 < n ? __fmul_rn(x[u + 1], sc) : K), nK);
+        }
+      }
+    };
     for (; pos + U <= end; pos += U) {
       float x[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) x[u] = in ? __ldg(xb + (int64_t)s_order[pos + u] * a.ld) : 0.f;
-#pragma unroll
-      for (int u = 0; u < U; ++u) gf_add<PASS>(v, x[u], K, sc);
+      rows(x, U);
     }
     if (pos < end) {
       float x[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
         x[u] = in && pos + u < end ? __ldg(xb + (int64_t)s_order[pos + u] * a.ld) : 0.f;
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (pos + u < end) gf_add<PASS>(v, x[u], K, sc);
+      rows(x, end - pos);
       pos = end;
     }
     GfSum sum{v.sum(), v.m};
