@@ -10,9 +10,10 @@
 // exact to about 2^-70 of its largest term and is rounded once, to FP64, for ~8
 // (pass 1) and ~22 (pass 2) packed FP32 instructions a value, where FP64 sums of each class
 // and of all rows cost eight slots of the FP64 pipe, i.e. 512 of an FP32 one.
-// Sums of runs are added in FP64.  (Two numbers a sum, about 48 bits, cost 18 us
-// less at C = 64, F = 256 and left the variances 1e-14 off, where FP64 sums are 4e-16
-// off and these 2e-16.)  The additions are written as intrinsics: a product that the
+// Sums of runs are added in FP64.  (Two numbers a sum, about 48 bits, took the fit of
+// 64,000 rows at C = 64, F = 256 110 us instead of 123, 447,355 rows at C = 3, F = 18
+// 86 instead of 99, and left the variances 1e-14 off, where FP64 sums are 4e-16 off and
+// these 2e-16.  Three numbers a sum in the reductions too, without FP64: 127 and 121.)  The additions are written as intrinsics: a product that the
 // compiler fused into one of them would break the error terms.  A run whose FP32 sum
 // overflows is summed again in FP64 by itself (400,000 rows of such values x 32
 // features: 55 ms while a feature's lane walked all rows instead).  The overall
@@ -40,8 +41,8 @@
 // reading the parameters: 4.90 -> 0.84 ms, of which the fit was 3.45 ms of
 // device time with FP64 sums in shared memory, 32-row chunks (266 MB of
 // partials, mapped anew by every call) and a one-block finish, and is 0.12 ms
-// now (passes 34 and 42 us, reductions 7 and 15, finish 10, tensor-core tables
-// 16); C = 2, F = 64, 2,000 + 10,000 rows: 365 -> 136 us (fit 38).
+// now (passes 37 and 52 us, reductions 8 and 19, finish 10, tensor-core tables
+// 16, each launch by itself); C = 2, F = 64, 2,000 rows: the fit 30 us.
 #include <math.h>
 
 #include "device.cuh"
@@ -51,7 +52,6 @@ namespace nbg {
 
 constexpr int kGfWarps = 8;
 constexpr int kGfMaxRows = 2048;              // rows per chunk (the sort's shared memory)
-constexpr int kGfGroups = kGfMaxRows / 32;    // 32-row label groups of a chunk
 
 struct GfArgs {
   const float* X;
@@ -69,7 +69,7 @@ struct GfArgs {
 };
 
 // Two rows at a time, one in each half of a packed instruction (the same roundings, half
-// the issue slots, which bound pass 2: 43 -> 53 us with one row an instruction).
+// the issue slots).
 __device__ __forceinline__ uint64_t neg2(uint64_t a) {
   return f32x2_fma(a, f32x2_pack(-1.f, -1.f), f32x2_pack(-0.f, -0.f));
 }
