@@ -68,7 +68,8 @@ static nb_status alloc_model(nb_model* m) {
   const size_t o_c2 = take(sizeof(C2Header));
   const size_t o_delta = take(sizeof(float) * Fp);
   const size_t o_dq = take(sizeof(int32_t) * Fp);
-  const size_t o_dp = take(2 * sizeof(int32_t) * Fp);   // with the residuals behind it
+  const size_t o_dpr = take(sizeof(int2) * Fp);
+  const size_t o_dp = take(fix_rows(m->F) ? 2 * sizeof(int32_t) * Fp : 0);
   const size_t o_limbs = take(7 * Fp);   // three limb planes + packed limb words
   const size_t o_limbs5 = take(fp8_narrow(m->F) ? 5 * Fp : 0);
   const size_t o_il0 = take(sizeof(float) * Fp);
@@ -113,7 +114,8 @@ static nb_status alloc_model(nb_model* m) {
   d.c2 = reinterpret_cast<C2Header*>(b + o_c2);
   d.delta = reinterpret_cast<float*>(b + o_delta);
   d.delta_q = reinterpret_cast<int32_t*>(b + o_dq);
-  d.delta_p = reinterpret_cast<int32_t*>(b + o_dp);
+  d.delta_pr = reinterpret_cast<int2*>(b + o_dpr);
+  d.delta_p = fix_rows(m->F) ? reinterpret_cast<int32_t*>(b + o_dp) : nullptr;
   d.limbs = reinterpret_cast<uint4*>(b + o_limbs);
   d.limbs5 = fp8_narrow(m->F) ? reinterpret_cast<uint4*>(b + o_limbs5) : nullptr;
   d.il[0] = reinterpret_cast<float4*>(b + o_il0);

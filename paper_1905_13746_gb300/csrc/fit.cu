@@ -483,7 +483,7 @@ constexpr int kFinT = 4 * kFinF;   // threads per block
 __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     const unsigned long long* counts, const unsigned long long* nc, int64_t n, int F, int F_pad,
     int nvec8, double alpha, int prior_given, double* log_theta, double* log_pi, C2Header* hdr,
-    float* delta, int32_t* delta_q, int32_t* delta_p, uint4* limbs, uint4* limbs5, float4* il4, float4* il8,
+    float* delta, int32_t* delta_q, int2* delta_pr, int32_t* delta_p, uint4* limbs, uint4* limbs5, float4* il4, float4* il8,
     float4* il16, float* w, float* bias, float* wmax, unsigned long long* fin, int* status) {
   constexpr int NT = kFinT, NL = 2 * kFinF;   // NL threads take the per-feature logs
   __shared__ unsigned long long part[2][2];
@@ -610,7 +610,8 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     frexp(maxabs64, &e);   // maxabs64 < 2^e
     S = 22 - e;
   }
-  const double scale = ldexp(1.0, S), fine_step = ldexp(1.0, -S - 8);
+  const double scale = ldexp(1.0, S);
+  const float fine_step = (float)ldexp(1.0, -S - 8);
   // U features per thread at a time: their log theta loads all go out before
   // the byte stores of the limbs (which may alias them) hold the next ones up
   constexpr int U = 4;
@@ -625,11 +626,15 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
     for (int u = 0; u < U; ++u) {
       const int jj = base + u * NT + tid;
       if (jj >= F_pad) continue;
-      const int32_t q = (int32_t)llrint(dd[u] * scale);   // |q| <= 2^22
+      const double ds = dd[u] * scale, fine = ds * 256.0;
+      const int32_t q = __double2int_rn(ds), p = __double2int_rn(fine);   // |q| <= 2^22, |p| <= 2^30
+      const float rest = (float)(fine - (double)p) * fine_step;   // a power of two: exact
       delta_q[jj] = q;
-      const double fine = dd[u] * scale * 256.0, whole = rint(fine);   // |.| <= 2^30
-      delta_p[jj] = (int32_t)whole;
-      reinterpret_cast<float*>(delta_p)[F_pad + jj] = (float)((fine - whole) * fine_step);
+      delta_pr[jj] = make_int2(p, __float_as_int(rest));
+      if (delta_p) {
+        delta_p[jj] = p;
+        reinterpret_cast<float*>(delta_p)[F_pad + jj] = rest;
+      }
       // balanced base-256 digits q = q2*65536 + q1*256 + q0, each in [-128, 127]
       const int32_t q0 = ((q + 128) & 255) - 128;
       const int32_t r1 = (q - q0) >> 8;
@@ -646,7 +651,7 @@ __global__ void __launch_bounds__(kFinT) k_fit_finish_c2(
       reinterpret_cast<uint32_t*>(L + (size_t)3 * F_pad)[jj] =
           (uint32_t)(q0 & 255) | ((uint32_t)(q1 & 255) << 8) | ((uint32_t)(q2 & 255) << 16);
       if (limbs5) {   // what q leaves of Delta, in steps of 2^-(S+15): |f| <= 2^14
-        const int32_t f = (int32_t)llrint((dd[u] * scale - (double)q) * 32768.0);
+        const int32_t f = (int32_t)llrint((ds - (double)q) * 32768.0);
         const int32_t f0 = ((f + 128) & 255) - 128, f1 = (f - f0) >> 8;   // |f1| <= 64
         const int32_t l5[5] = {q0, q1, q2, f0, f1};
 #pragma unroll
@@ -810,7 +815,7 @@ nb_status launch_fit_multinomial(nb_model* m, const void* X, nb_dtype dt, int64_
                            0, st, reinterpret_cast<const unsigned long long*>(d.counts),
                            reinterpret_cast<const unsigned long long*>(d.nc), (int64_t)n, F,
                            m->F_pad, m->nvec8, m->alpha, (int)(log_prior_dev != nullptr), d.p0,
-                           d.log_pi, d.c2, d.delta, d.delta_q, d.delta_p, d.limbs, d.limbs5, d.il[0], d.il[1],
+                           d.log_pi, d.c2, d.delta, d.delta_q, d.delta_pr, d.delta_p, d.limbs, d.limbs5, d.il[0], d.il[1],
                            d.il[2], d.w, d.bias, d.wmax, d.fin, d.status),
                 "k_fit_finish_c2");
     return NB_OK;

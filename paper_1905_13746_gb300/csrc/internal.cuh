@@ -87,6 +87,10 @@ struct TcgHeader {
   float wsum;         // sum_j (max_c |B_cj| + max_c |A_cj|), rounded up
 };
 
+// Two-class U16 and BF16 rows of up to 16 vectors of 16 bytes take the exact sums of
+// k_score2_fix.
+inline bool fix_rows(int F) { return F <= 16 * 8; }
+
 // Two-class FP8 rows of fewer than 32 vectors of 16 bytes take five limbs of Delta (see
 // k_score2_u8).
 inline bool fp8_narrow(int F) { return F <= 31 * 16; }
@@ -111,8 +115,10 @@ struct ModelDev {
   C2Header* c2;        // 1
   float* delta;        // F_pad      FP32 Delta, plain order
   int32_t* delta_q;    // F_pad      fixed-point Delta
-  int32_t* delta_p;    // F_pad      fixed-point Delta, eight bits finer (step 2^-(S+8)), then
-                       //            F_pad floats: what it leaves of Delta
+  int2* delta_pr;      // F_pad      fixed-point Delta, eight bits finer (step 2^-(S+8)), and in
+                       //            FP32 what it leaves of Delta
+  int32_t* delta_p;    // 2 F_pad    the same one after the other for short 16-bit rows
+                       //            (fix_rows), else nullptr
   uint4* limbs;        // 3 * nvec8  int8 limbs of delta_q, interleaved (u8 path), then
                        //            F_pad packed words (limb l in byte l)
   uint4* limbs5;       // 5 * nvec8  the three limbs and two more (step 2^-(S+15)) for narrow FP8

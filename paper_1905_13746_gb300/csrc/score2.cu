@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(256, 3) k_score2_fix(const S2Args a) {
 // ones only where a row holds something else than counts.  Without FIX (label
 // and OFF modes) the FP32 sums.
 // 100,003 rows of 1,003 F32 counts (401 MB), log-posterior mode, labels only:
-// 78 us for the whole call; 3.57 ms as 2 of the 64 class columns of the general
+// 76 us for the whole call; 3.57 ms as 2 of the 64 class columns of the general
 // scorer's 64 x 64 tiles (1.08 ms) and every row in FP64 on top (2.5 ms).
 // 249,252 rows (1 GB): 158 us in the label mode (93% of the measured HBM rate),
 // 190 us (78%) in the log-posterior mode.
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(256, 3) k_score2_any(const S2Args a) {
     bool todo = true;
     if (FIX) {
       FixSum2 fix[R / 2];
-      sweep([&](int j) { return make_int2(__ldg(a.delta_p + j), __float_as_int(__ldg(a.delta_r + j))); },
+      sweep([&](int j) { return __ldg(a.delta_pr + j); },
             [&](const float (&x)[R], int2 q) {
               fix_add(fix[0], x[0], x[1], q.x, __int_as_float(q.y));
               fix_add(fix[1], x[2], x[3], q.x, __int_as_float(q.y));
@@ -743,8 +743,7 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   a.hdr = m->d.c2;
   a.delta_q = m->d.delta_q;
   a.delta = m->d.delta;
-  a.delta_p = m->d.delta_p;
-  a.delta_r = reinterpret_cast<const float*>(m->d.delta_p + m->F_pad);
+  a.delta_pr = m->d.delta_pr;
   a.ovf_ptr = aux ? aux->ovf_ptr : nullptr;
   a.ovf_col = aux ? aux->ovf_col : nullptr;
   a.ovf_add = aux ? aux->ovf_add : nullptr;
@@ -800,7 +799,7 @@ nb_status launch_score2(const nb_model* m, const void* X, nb_dtype dt, int64_t n
   // 32 lanes (1M BF16 files: F = 64 52 us against 127, F = 128 93 against 159;
   // at F = 256 175 against 146 and at 1,024 291 against 211, so longer rows
   // stay there).  F32 rows stay with the FP32 sums, which batches share.
-  if (fix && es == 2 && a.nvec_row <= 16 && cfg.variant != NB_VARIANT_REGISTER) {
+  if (fix && es == 2 && fix_rows(m->F) && cfg.variant != NB_VARIANT_REGISTER) {
     a.table = m->d.delta_p;   // and the residuals
     a.table_bytes = 2 * smem;
     a.k_base = (4 / es) + 2 + 5 + 2;   // of the FP32 sums, 32 lanes per row

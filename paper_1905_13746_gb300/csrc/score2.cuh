@@ -23,8 +23,7 @@ struct S2Args {
   const C2Header* hdr;
   const int32_t* delta_q;   // plain fixed-point table (overflow entries)
   const float* delta;       // plain FP32 table (overflow entries)
-  const int32_t* delta_p;   // plain fixed-point table of step 2^-(S+8)
-  const float* delta_r;     // and its residuals
+  const int2* delta_pr;     // plain fixed-point table of step 2^-(S+8) and its FP32 residuals
   const int64_t* ovf_ptr;
   const uint16_t* ovf_col;
   const uint16_t* ovf_add;
@@ -220,9 +219,10 @@ struct Decode<NB_FP8E4M3> {
 // fixed-point Delta exactly, D = sum x P in int64 with P = round(Delta 2^(S+8)),
 // |P| <= 2^30, and in FP32 what P leaves of Delta, at most half a step a count:
 // the result is the FP64 one to FP32 rounding.  (Without the residuals margins were off
-// by up to half a step a count, many FP32 units of a small one; they cost 74 -> 78 us
-// at 100,003 rows of 1,003 F32 counts, 149 -> 174 at 200,000 of 1,001 BF16 ones and
-// nothing on short 16-bit rows.)  With u = x + 2^23 in FP32, x is an integer in
+// by up to half a step a count, many FP32 units of a small one; they cost 74 -> 76 us
+// at 100,003 rows of 1,003 F32 counts, 149 -> 153 at 200,000 of 1,001 BF16 ones, from
+// one table of entries by turns (78 and 174 from two), and nothing on short 16-bit
+// rows.)  With u = x + 2^23 in FP32, x is an integer in
 // [0, 2^23) exactly when x's bits lie below 2^23's and u - 2^23 has x's bits; x is
 // then u's low 23 bits.  D cannot wrap below a total of 2^33 counts
 // (fix_result).  A row with any other value takes FP32 sums and their bound.
