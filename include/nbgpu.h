@@ -200,8 +200,8 @@ NB_API nb_status nb_fit(nb_kind kind, const void* X, nb_dtype dtype, int64_t n,
  * scratch of the reduction is kept with the model between re-fits up to 64 MiB
  * (taken stream-ordered, cudaMallocAsync, and kept from the first re-fit on;
  * larger scratch, and that of a call on a stream being captured, is allocated
- * and freed in stream order).  The model must not be in use by a score call on another stream meanwhile.
- * Same errors as nb_fit. */
+ * and freed in stream order).  The model must not be in use by a score call on
+ * another stream meanwhile.  Same errors as nb_fit. */
 NB_API nb_status nb_refit(nb_model* model, const void* X, nb_dtype dtype, int64_t n,
                    int64_t ld, const int32_t* y, const nb_fit_opts* opts,
                    void* cuda_stream);
@@ -296,7 +296,8 @@ NB_API int nb_score_path(const nb_model* model, const void* X, nb_dtype dtype, i
  * rest), then one FP64 recheck launch per family -- independent of the number
  * of groups.  Each row's arithmetic
  * is that of nb_score_group, so a group's results are the same bits alone
- * and inside any batch.
+ * and inside any batch (but for the U8 rows of many-class models whose stored
+ * bytes total 2^17 or more: exact fixed-point sums alone, FP64 in a batch).
  *
  * nb_batch_create: models[0..n_models) (multinomial, all with the same F,
  *   n_models <= 128; the two-class models' tables, 3 bytes per feature (u8

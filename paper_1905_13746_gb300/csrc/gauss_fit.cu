@@ -8,17 +8,17 @@
 // FP32 numbers, the sum, its error and the error of that, the first two joined
 // exactly (Knuth's two-sum, and the FMA product error): the run's sum is then
 // exact to about 2^-70 of its largest term and is rounded once, to FP64, for ~8
-// (pass 1) and ~22 (pass 2) packed FP32 instructions a value, where FP64 sums of each class
-// and of all rows cost eight slots of the FP64 pipe, i.e. 512 of an FP32 one.
+// (pass 1) and ~22 (pass 2) packed FP32 instructions a value, where FP64 sums of each
+// class and of all rows cost eight slots of the FP64 pipe, i.e. 512 of an FP32 one.
 // Sums of runs are added in FP64.  (Two numbers a sum, about 48 bits, took the fit of
 // 64,000 rows at C = 64, F = 256 110 us instead of 123, 447,355 rows at C = 3, F = 18
 // 86 instead of 99, and left the variances 1e-14 off, where FP64 sums are 4e-16 off and
-// these 2e-16.  Three numbers a sum in the reductions too, without FP64: 127 and 121.)  The additions are written as intrinsics: a product that the
-// compiler fused into one of them would break the error terms.  A run whose FP32 sum
-// overflows is summed again in FP64 by itself (400,000 rows of such values x 32
-// features: 55 ms while a feature's lane walked all rows instead).  The overall
-// variance behind eps comes from the class moments (n_c, mu_c, var_c), not from sums
-// of its own.
+// these 2e-16.  Three numbers a sum in the reductions too, without FP64: 127 and 121.)
+// The additions are written as intrinsics: a product that the compiler fused into one
+// of them would break the error terms.  A run whose FP32 sum overflows is summed again
+// in FP64 by itself (400,000 rows of such values x 32 features: 55 ms while a feature's
+// lane walked all rows instead).  The overall variance behind eps comes from the class
+// moments (n_c, mu_c, var_c), not from sums of its own.
 //
 // Pass 2 sums (x - K)^2 with K = fl32(mean) of the class and feature, and
 // var = S2 / n_c - (mean - K)^2; x - K is formed exactly as a pair.  Values
@@ -506,7 +506,8 @@ __global__ void __launch_bounds__(256) k_gauss_finish(const GfFin a) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// Rows per chunk: four blocks per SM over chunks x feature tiles, but at least
+// Rows per chunk: four blocks per SM of this part (152, whatever the device: the
+// chunks fix the order of the sums) over chunks x feature tiles, but at least
 // eight rows per class (smaller chunks write more partials than they read
 // rows), at least 64 rows, 512 past 65,536 rows (the bound on the scratch that
 // the allocation-free re-fit's limit relies on), and what the sort can hold.

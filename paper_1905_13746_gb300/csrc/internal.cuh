@@ -162,7 +162,7 @@ struct nb_model {
   nb_kind kind;
   int C;
   int F;
-  int F_pad;        // F rounded up to a multiple of 16
+  int F_pad;        // F rounded up to a multiple of 32
   int nvec8;        // F_pad / 16 (u8 vectors of 16 bytes)
   double alpha;
   double var_smoothing;

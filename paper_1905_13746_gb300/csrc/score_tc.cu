@@ -350,9 +350,9 @@ __device__ __forceinline__ void tc_load_acc8(uint32_t lane_base, int h, int Cp, 
 // way (each rounding is within 2^-24 of its result, the prior's within 2^-24
 // of itself).  Pair pass: s = ((a0 sc + b) + a1 2^8 sc) + a2 2^16 sc from the
 // exact FP32 limb sums (sc = 2^-S: the products are exact, each FMA rounds
-// once), then + (float)(overflow sum) sc.  Chunked pass: the exact int64 sum
-// q (overflow entries included) is rounded once to FP32 and enters one FMA
-// with the prior.  `added` receives the overflow entries' counts.
+// once).  Chunked pass: the exact int64 sum q of the stored counts is rounded once
+// to FP32 and enters one FMA with the prior.  Both then add (float)(the overflow
+// entries' exact sum) sc.  `added` receives the overflow entries' counts.
 template <int MODE>
 __device__ __forceinline__ void tc_scores8(const SegGroup& G, const TcModelArg& M, int F,
                                            uint32_t lane_base, int h, int cb, bool any_ovf,
@@ -923,8 +923,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_score_tc(const __grid_constan
               }
             }
             // every value an integer count x = v 2^e below 1024: x sits in the low 10
-            // bits of v + M; T sums M + x (at most 2^15 + 2^10 for each of 32 values
-            // per A stage: no wrap below 2^32 for F <= 8192)
+            // bits of v + M; T sums M + x (at most 2^15 + 2^10 for each of this thread's
+            // F / 2 values, F <= 32,768: no wrap)
             if constexpr (DT != NB_U8) {
 #pragma unroll
               for (int q = 0; q < PS::COLS; ++q) f16x2_count_check(o[sub][q], m2, T, bad, mx);
@@ -1225,8 +1225,8 @@ static nb_status run_tc_rl(TcArgs& a, int maxN, long long units_hint, cudaStream
   return NB_OK;
 }
 
-// Four row stages where the weight stages leave the room (N <= 132: up to 40
-// classes): with few classes the MMAs are short and the rows' latency shows (150,001
+// Four row stages where the weight stages leave the room (N = 3 C_p <= 132, C_p in steps
+// of 16: up to 32 classes): with few classes the MMAs are short and the rows' latency shows (150,001
 // BF16 rows x 2,048 features x 16 classes 150 -> 131 us).
 template <int MODE, int DT>
 static nb_status run_tc(TcArgs& a, int maxN, long long units_hint, cudaStream_t st) {
