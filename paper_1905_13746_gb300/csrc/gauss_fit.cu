@@ -57,6 +57,7 @@ struct GfArgs {
   const float* X;
   int64_t ld, n;
   int F, C, rows;
+  unsigned nchunk;      // chunks of rows; block: (feature tile) x nchunk + chunk
   const int32_t* y;
   double* part0;        // C x F sums of chunk 0 ...
   double* part;         // ... and of chunks 1, 2, ...
@@ -142,13 +143,14 @@ __device__ __forceinline__ void gf_add(GfAcc& a, uint64_t x, uint64_t nK) {
 }
 
 template <int PASS>
-__device__ __forceinline__ void gf_store(const GfArgs& a, int c, int j, const GfSum& v) {
+__device__ __forceinline__ void gf_store(const GfArgs& a, unsigned chunk, int c, int j,
+                                         const GfSum& v) {
   if (j >= a.F) return;
   const int64_t at = (int64_t)c * a.F + j;
-  const int64_t off = blockIdx.x == 0 ? at : ((int64_t)(blockIdx.x - 1) * a.C) * a.F + at;
-  (blockIdx.x == 0 ? a.part0 : a.part)[off] = v.s;
+  const int64_t off = chunk == 0 ? at : ((int64_t)(chunk - 1) * a.C) * a.F + at;
+  (chunk == 0 ? a.part0 : a.part)[off] = v.s;
   if (PASS == 1) {
-    (blockIdx.x == 0 ? a.amax0 : a.amax)[off] = __uint_as_float(v.m);
+    (chunk == 0 ? a.amax0 : a.amax)[off] = __uint_as_float(v.m);
     if (v.m >= 0x7F800000u) atomicOr(a.status, ST_BAD_VALUE);
   }
 }
@@ -163,10 +165,12 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
   uint16_t* cnt = reinterpret_cast<uint16_t*>(gf_sm);   // [label group][class]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int C = a.C;
-  const int64_t r0 = (int64_t)blockIdx.x * a.rows;
+  // one grid dimension: the others end at 65,535, fewer than the tiles of 2.1M features
+  const unsigned chunk = blockIdx.x % a.nchunk, ft = blockIdx.x / a.nchunk;
+  const int64_t r0 = (int64_t)chunk * a.rows;
   const int nr = (int)min((int64_t)a.rows, a.n - r0);
   const int ng = (nr + 31) / 32;
-  const int j = blockIdx.y * 32 + lane;
+  const int j = (int)ft * 32 + lane;
   for (int k = threadIdx.x; k < ng * C; k += kGfWarps * 32) cnt[k] = 0;
   if (threadIdx.x < 2 * kGfWarps) s_fc[threadIdx.x] = -1;
   pdl_wait();   // the cleared counters, or the means of pass 1
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
     const int r = 32 * g + lane;
     int c = r < nr ? a.y[r0 + r] : -1;
     if (r < nr && (c < 0 || c >= C)) {
-      if (PASS == 1 && blockIdx.y == 0) atomicOr(a.status, ST_BAD_LABEL);
+      if (PASS == 1 && ft == 0) atomicOr(a.status, ST_BAD_LABEL);
       c = -1;
     }
     return c;
@@ -197,7 +201,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
         cnt[g * C + threadIdx.x] = (uint16_t)run;
         run += t;
       }
-      if (PASS == 1 && blockIdx.y == 0 && run) atomicAdd(&a.nc[threadIdx.x], (unsigned long long)run);
+      if (PASS == 1 && ft == 0 && run) atomicAdd(&a.nc[threadIdx.x], (unsigned long long)run);
     }
     // exclusive scan of the class totals over both warps
     int inc = run;
@@ -272,7 +276,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
       for (int k = start; k < end; ++k) sum.s += (double)__ldg(xb + (int64_t)s_order[k] * a.ld);
     }
     if (start == s_off[c] && end == s_off[c + 1]) {
-      gf_store<PASS>(a, c, j, sum);
+      gf_store<PASS>(a, chunk, c, j, sum);
     } else {   // the class is shared with a neighbouring warp: slot 0 begins, slot 1 ends a share
       const int slot = 2 * warp + (start == a0 ? 0 : 1);
       s_frag[slot][lane] = sum;
@@ -281,7 +285,7 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
   }
   // classes without rows in this chunk
   for (int k = warp; k < C; k += kGfWarps)
-    if (s_off[k] == s_off[k + 1]) gf_store<PASS>(a, k, j, GfSum{});
+    if (s_off[k] == s_off[k + 1]) gf_store<PASS>(a, chunk, k, j, GfSum{});
   __syncthreads();
   if (warp == 0) {   // join the shared classes' pieces in order
     GfSum v;
@@ -290,14 +294,14 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
       const int fc = s_fc[k];
       if (fc < 0) continue;
       if (fc != cur) {
-        if (cur >= 0) gf_store<PASS>(a, cur, j, v);
+        if (cur >= 0) gf_store<PASS>(a, chunk, cur, j, v);
         v = s_frag[k][lane];
         cur = fc;
       } else {
         gf_join(v, s_frag[k][lane]);
       }
     }
-    if (cur >= 0) gf_store<PASS>(a, cur, j, v);
+    if (cur >= 0) gf_store<PASS>(a, chunk, cur, j, v);
   }
 }
 
@@ -306,7 +310,6 @@ __global__ void __launch_bounds__(kGfWarps * 32) k_gauss_pass(const GfArgs a) {
 // ---------------------------------------------------------------------------
 struct GfRed {
   GfArgs a;
-  int nchunk;
   double* mu;               // C x F
   double* var;              // C x F
   float* scale;             // C x F
@@ -326,7 +329,7 @@ __device__ __forceinline__ GfSum gf_reduce(const GfRed& r, int c, int j) {
   if (j < a.F) {
     const int64_t at = (int64_t)c * a.F + j, step = (int64_t)a.C * a.F;
 #pragma unroll 4
-    for (int k = warp; k < r.nchunk; k += kGfWarps) {
+    for (int k = warp; k < (int)a.nchunk; k += kGfWarps) {
       const int64_t off = k == 0 ? at : (int64_t)(k - 1) * step + at;
       v.s += (k == 0 ? a.part0 : a.part)[off];
       if (PASS == 1) v.m = max(v.m, __float_as_uint((k == 0 ? a.amax0 : a.amax)[off]));
@@ -555,6 +558,7 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   a.F = F;
   a.C = C;
   a.rows = (int)rows;
+  a.nchunk = (unsigned)nchunk;
   a.y = y;
   a.part0 = reinterpret_cast<double*>(d.counts);
   a.amax0 = reinterpret_cast<float*>(d.p1);
@@ -571,9 +575,9 @@ nb_status launch_fit_gaussian(nb_model* m, const float* X, int64_t n, int64_t ld
   a.scale = scale;
   a.nc = reinterpret_cast<unsigned long long*>(d.nc);
   a.status = d.status;
-  GfRed r{a, (int)nchunk, d.p0, d.p1, scale, done, done + nft, d.fin, d.tcg_kc ? d.tcg_hdr : nullptr};
+  GfRed r{a, d.p0, d.p1, scale, done, done + nft, d.fin, d.tcg_kc ? d.tcg_hdr : nullptr};
   const int smem = (int)(sizeof(uint16_t) * ((rows + 31) / 32) * C);
-  const dim3 grid((unsigned)nchunk, (unsigned)nft), rgrid((unsigned)nft, (unsigned)C);
+  const dim3 grid((unsigned)(nchunk * nft)), rgrid((unsigned)nft, (unsigned)C);
   const dim3 block(kGfWarps * 32);
   count_launch();
   k_gauss_pass<1><<<grid, block, smem, st>>>(a);

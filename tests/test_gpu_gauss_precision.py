@@ -80,3 +80,20 @@ def test_overflowing_sums_cost_a_run_not_the_matrix():
             best = min(best, a.elapsed_time(b))
         times.append(best)
     assert times[1] <= 20 * times[0], times
+
+
+def test_more_features_than_a_grid_dimension_holds_tiles():
+    """2.1M features are 65,626 tiles of 32."""
+    F, n = 2_100_003, 6
+    rng = np.random.default_rng(3)
+    X = rng.normal(size=(n, F)).astype(np.float32)
+    y = np.array([0, 1, 0, 1, 1, 0], np.int32)
+    mu, var, _ = nb.fit(torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), 2,
+                        kind=nb.NB_GAUSSIAN, var_smoothing=0.0).params()
+    for c in range(2):
+        r = X[y == c].astype(np.longdouble)
+        m = r.mean(axis=0)
+        v = np.square(r - m).mean(axis=0)
+        u = 16 * 2.0 ** -53              # at most three pieces of one chunk
+        assert (np.abs(mu[c] - m) <= u * np.abs(r).mean(axis=0)).all()
+        assert (np.abs(var[c] - v) <= u * (v + 2.0 ** -48 * m * m)).all()
