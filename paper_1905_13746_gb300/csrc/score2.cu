@@ -193,8 +193,9 @@ __global__ void __launch_bounds__(256, 3) k_score2_fp8(const S2Args a) {
   const double step = __hiloint2double((1023 - h.S - 15) << 20, 0);   // 2^-(S+15)
   // the prior's part in whole steps: d is then an integer until it is rounded to FP32.
   // (In FP64 where it does not fit: weights of next to nothing.)
-  const bool whole = fabs(h.b64) < 4.611686018427388e18 * step;
-  const long long b = whole ? llrint(h.b64 / step) : 0ll;
+  const double bs = h.b64 * __hiloint2double((1023 + h.S + 15) << 20, 0);
+  const bool whole = fabs(bs) < 4.611686018427388e18;
+  const long long b = whole ? llrint(bs) : 0ll;
   unsigned marks = 0;
   for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles;
        t += nwarps) {

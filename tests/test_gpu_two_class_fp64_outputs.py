@@ -86,3 +86,15 @@ def test_the_register_kernel_can_be_asked_for(fmt):
         compare(res, ref)
     assert marked[nb.NB_VARIANT_AUTO] == marked[nb.NB_VARIANT_PIPELINED] <= 30
     assert marked[nb.NB_VARIANT_REGISTER] > 1500
+
+
+@pytest.mark.parametrize("F", [100, 490])
+def test_tuning_narrow_fp8_rows_changes_no_result(F):
+    X, y = _rows(F, 3000, F, 16)
+    f, vals = stored(X, "fp8")
+    model = nb.fit(f, torch.from_numpy(y).cuda(), 2)
+    before = to_np(nb.score(model, f))
+    assert model.autotune(f)[0][0] != nb.NB_VARIANT_REGISTER
+    after = to_np(nb.score(model, f))
+    for k in ("label", "margin", "lp"):
+        assert np.array_equal(before[k], after[k]), k
